@@ -10,6 +10,17 @@ void count_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memo
 
 jq_status check_launch() { return cudaGetLastError() == cudaSuccess ? JQ_OK : JQ_ERR_CUDA; }
 
+int device_sms()
+{
+    static std::atomic<int> sms[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if ((n = sms[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    sms[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 static jq_status check_shape(const jq_shape *s)
 {
     if (!s) return JQ_ERR_INVALID_ARG;

@@ -102,6 +102,7 @@ int heads_per_group(int L, int heads, int tiles_per_head, int sms);
 int score_sms();   // CTAs of the scoring kernel on the current device; 0 on error
 
 // Host-side bookkeeping.
+int device_sms();           // multiprocessors of the current device; 0 on error
 void count_launch(int n = 1);
 jq_status check_launch();   // cudaGetLastError -> JQ_OK / JQ_ERR_CUDA
 
