@@ -1,9 +1,9 @@
 """B200 (sm_100a) library for the per-layer KV-cache eviction pass of Judge Q (arXiv 2509.10798).
 
-Thin ctypes binding over libjq.so (C ABI in include/jq.h).  The functions here only marshal
-arguments: torch tensors supply device memory and the current CUDA stream, every step of the pass
-runs in the library's own kernels.  There is no CPU or PyTorch fallback: if libjq.so is missing or
-no CUDA device is present, the calls raise.
+Thin binding over libjq.so (C ABI in include/jq.h).  The functions here only marshal arguments (the ones called in a
+loop through the small C extension csrc/jq_pycall.c, the others through ctypes): torch tensors supply device memory and
+the current CUDA stream, every step of the pass runs in the library's own kernels.  There is no CPU or PyTorch fallback:
+if libjq.so or the extension is missing or no CUDA device is present, the calls raise.
 """
 import ctypes
 import os
@@ -154,10 +154,32 @@ def new_workspace(s, device="cuda", stream=None):
     return ws
 
 
+_fast = None
+
+
+def _calls():
+    """The C marshalling of the calls that are made in a loop, bound to the loaded library."""
+    global _fast
+    if _fast is None:
+        L = lib()
+        try:
+            from . import _jqcall
+        except ImportError as e:
+            raise RuntimeError("_jqcall is not built: run `python -m paper_2509_10798_b200.build` (%s)" % e) from e
+        _jqcall.bind({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in EXPORTS}, _stream_lookup())
+        _fast = _jqcall
+    return _fast
+
+
+def _stream_lookup():
+    """A callable that gives the current stream of the current device as an integer."""
+    C = _torch()._C
+    device, raw = C._cuda_getDevice, C._cuda_getCurrentRawStream
+    return lambda: raw(device())
+
+
 def score(K, Qwin, s, scores, ws, stream=None, fma=False):
-    fn = lib().jq_score_fma if fma else lib().jq_score
-    _raise("jq_score_fma" if fma else "jq_score",
-           fn(_ptr(K), _ptr(Qwin), ctypes.byref(s), _ptr(scores), _ptr(ws), ws.numel(), _stream(stream)))
+    _raise("jq_score_fma" if fma else "jq_score", (_fast or _calls()).score(K, Qwin, s, scores, ws, stream, fma))
 
 
 def score_static(K, Qwin, s, scores, stream=None):
@@ -176,38 +198,31 @@ def score_windowed(K, Qwin, Kwin, s, scores, ws, stream=None):
 
 def evict_layer_windowed(K, V, Qwin, Kwin, s, Kout, Vout, kept_idx, ws, stream=None):
     _raise("jq_evict_layer_windowed",
-           lib().jq_evict_layer_windowed(_ptr(K), _ptr(V), _ptr(Qwin), _ptr(Kwin), ctypes.byref(s), _ptr(Kout), _ptr(Vout),
-                                         _ptr(kept_idx), _ptr(ws), ws.numel(), _stream(stream)))
+           (_fast or _calls()).evict_layer_windowed(K, V, Qwin, Kwin, s, Kout, Vout, kept_idx, ws, stream))
 
 
 def evict_layer_window_kept(K, V, Qwin, Kwin, Vwin, s, Kout, Vout, kept_idx, ws, stream=None):
     """jq_evict_layer_window_kept: budget - w prefix rows chosen by the window-inclusive scores, then the w window rows."""
     _raise("jq_evict_layer_window_kept",
-           lib().jq_evict_layer_window_kept(_ptr(K), _ptr(V), _ptr(Qwin), _ptr(Kwin), _ptr(Vwin), ctypes.byref(s), _ptr(Kout),
-                                            _ptr(Vout), _ptr(kept_idx), _ptr(ws), ws.numel(), _stream(stream)))
+           (_fast or _calls()).evict_layer_window_kept(K, V, Qwin, Kwin, Vwin, s, Kout, Vout, kept_idx, ws, stream))
 
 
 def select_topk(scores, s, kept_idx, ws, pooled=None, stream=None):
-    _raise("jq_select_topk", lib().jq_select_topk(_ptr(scores), ctypes.byref(s), _ptr(kept_idx), _ptr(pooled),
-                                                  _ptr(ws), ws.numel(), _stream(stream)))
+    _raise("jq_select_topk", (_fast or _calls()).select_topk(scores, s, kept_idx, ws, pooled, stream))
 
 
 def compact_kv(K, V, kept_idx, s, Kout, Vout, stream=None):
-    _raise("jq_compact_kv", lib().jq_compact_kv(_ptr(K), _ptr(V), _ptr(kept_idx), ctypes.byref(s), _ptr(Kout),
-                                                _ptr(Vout), _stream(stream)))
+    _raise("jq_compact_kv", (_fast or _calls()).compact_kv(K, V, kept_idx, s, Kout, Vout, stream))
 
 
 def evict_layer(K, V, Qwin, s, Kout, Vout, kept_idx, ws, stream=None):
-    _raise("jq_evict_layer", lib().jq_evict_layer(_ptr(K), _ptr(V), _ptr(Qwin), ctypes.byref(s), _ptr(Kout),
-                                                  _ptr(Vout), _ptr(kept_idx), _ptr(ws), ws.numel(),
-                                                  _stream(stream)))
+    _raise("jq_evict_layer", (_fast or _calls()).evict_layer(K, V, Qwin, s, Kout, Vout, kept_idx, ws, stream))
 
 
 def evict_layer_host(hK, hV, hQwin, s, hKout, hVout, hkept_idx, dev_buf, stream=None):
     """Host-tensor variant: all h* are CPU tensors (pinned for asynchronous copies)."""
     _raise("jq_evict_layer_host",
-           lib().jq_evict_layer_host(_ptr(hK), _ptr(hV), _ptr(hQwin), ctypes.byref(s), _ptr(hKout), _ptr(hVout),
-                                     _ptr(hkept_idx), _ptr(dev_buf), dev_buf.numel(), _stream(stream)))
+           (_fast or _calls()).evict_layer_host(hK, hV, hQwin, s, hKout, hVout, hkept_idx, dev_buf, stream))
 
 
 def layers_workspace_bytes(s, nlayers):
@@ -227,11 +242,8 @@ def new_layers_workspace(s, nlayers, device="cuda", stream=None):
 
 def evict_layers(Ks, Vs, Qwins, s, Kout, Vout, kept_idx, ws, stream=None):
     """jq_evict_layers: Ks, Vs, Qwins are lists of per-layer CUDA tensors of shape `s`; the outputs are stacked."""
-    n = len(Ks)
-    arr = lambda ts: (ctypes.c_void_p * n)(*[t.data_ptr() for t in ts])
-    _raise("jq_evict_layers",
-           lib().jq_evict_layers(arr(Ks), arr(Vs), arr(Qwins), n, ctypes.byref(s), _ptr(Kout), _ptr(Vout), _ptr(kept_idx),
-                                 _ptr(ws), ws.numel(), _stream(stream)))
+    # (jq_evict_layers is jq_evict_ragged with one length and one budget)
+    _raise("jq_evict_layers", (_fast or _calls()).evict_ragged(Ks, Vs, Qwins, s, None, None, Kout, Vout, kept_idx, ws, stream))
 
 
 def _ints(xs):
@@ -260,11 +272,7 @@ def new_ragged_workspace(s, nunits, L=None, device="cuda", stream=None):
 def evict_ragged(Ks, Vs, Qwins, s, L, budget, Kout, Vout, kept_idx, ws, stream=None):
     """jq_evict_ragged: Ks, Vs, Qwins are lists of per-unit CUDA tensors; L, budget lists of ints (or None for
     s.L / s.budget everywhere); the outputs hold the units' blocks of Hkv * nkeep_u rows one after the other."""
-    n = len(Ks)
-    arr = lambda ts: (ctypes.c_void_p * n)(*[t.data_ptr() for t in ts])
-    _raise("jq_evict_ragged",
-           lib().jq_evict_ragged(arr(Ks), arr(Vs), arr(Qwins), n, ctypes.byref(s), _ints(L), _ints(budget), _ptr(Kout),
-                                 _ptr(Vout), _ptr(kept_idx), _ptr(ws), ws.numel(), _stream(stream)))
+    _raise("jq_evict_ragged", (_fast or _calls()).evict_ragged(Ks, Vs, Qwins, s, L, budget, Kout, Vout, kept_idx, ws, stream))
 
 
 def new_append_workspace(s, device="cuda", stream=None):
@@ -280,10 +288,7 @@ def new_append_workspace(s, device="cuda", stream=None):
 def evict_append(Kc, Vc, n_old, Knew, Vnew, Qrecent, s, kept_idx, ws, stream=None):
     """jq_evict_append: Kc, Vc [Hkv, cap, d] hold n_old retained rows per head; Knew, Vnew [Hkv, n_new, d] are appended and
     the cache is evicted again to s.budget rows (s.L = n_old + n_new), in place."""
-    n_new = 0 if Knew is None else int(Knew.shape[1])
-    _raise("jq_evict_append",
-           lib().jq_evict_append(_ptr(Kc), _ptr(Vc), int(Kc.shape[1]), int(n_old), _ptr(Knew), _ptr(Vnew), n_new, _ptr(Qrecent),
-                                 ctypes.byref(s), _ptr(kept_idx), _ptr(ws), ws.numel(), _stream(stream)))
+    _raise("jq_evict_append", (_fast or _calls()).evict_append(Kc, Vc, n_old, Knew, Vnew, Qrecent, s, kept_idx, ws, stream))
 
 
 def decode_workspace_bytes(Hkv, Hq, n):
@@ -292,8 +297,7 @@ def decode_workspace_bytes(Hkv, Hq, n):
 
 def decode_attention(Kc, Vc, q, out, ws, stream=None):
     """One decoding step over the pruned cache: Kc, Vc [Hkv,n,128] bf16, q [Hq,128] bf16 -> out [Hq,128] fp32."""
-    _raise("jq_decode_attention", lib().jq_decode_attention(_ptr(Kc), _ptr(Vc), _ptr(q), int(Kc.shape[0]), int(q.shape[0]),
-                                                            int(Kc.shape[1]), _ptr(out), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)))
+    _raise("jq_decode_attention", (_fast or _calls()).decode_attention(Kc, Vc, q, out, ws, stream))
 
 
 def hit_rate(cur_idx, ref_idx, rate, stream=None):

@@ -6,12 +6,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libjq.so")
 LIB_DEBUG = os.path.join(HERE, "libjq_debug.so")
+LIB_CALL = os.path.join(HERE, "_jqcall.so")   # the binding's C marshalling (csrc/jq_pycall.c)
 OBJDIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,7 +31,18 @@ def _deps():
     return glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
 
 
+def _build_call(force: bool):
+    src = os.path.join(CSRC, "jq_pycall.c")
+    if not force and os.path.exists(LIB_CALL) and os.path.getmtime(LIB_CALL) >= max(os.path.getmtime(p) for p in [src] + _deps()):
+        return
+    tmp = LIB_CALL + ".tmp%d" % os.getpid()
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-std=c11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), src, "-o", tmp], check=True)
+    os.replace(tmp, LIB_CALL)
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
+    _build_call(force)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     objdir = OBJDIR + ("_debug" if debug else "")
     lib = LIB_DEBUG if debug else LIB
