@@ -109,6 +109,10 @@ jq_status jq_evict_layer_windowed(const void *K, const void *V, const void *Qwin
     Workspace w;
     if ((rc = check_ws(s, ws, ws_bytes, &w)) != JQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
+    FusedSource src;
+    src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin;
+    bool taken;
+    if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     if ((rc = launch_score_tc(K, Qwin, *s, w.scores, w, st, Kwin)) != JQ_OK) return rc;
     return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);
 }
@@ -131,6 +135,10 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     jq_shape sp = *s;
     sp.budget = s->budget - s->w;
     const size_t row = (size_t)s->d * 2, np = (size_t)(sp.budget < s->L ? sp.budget : s->L), nt = np + (size_t)s->w;
+    FusedSource src;
+    src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin; src.Vwin = Vwin;
+    bool taken;
+    if ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
     if ((rc = launch_score_tc(K, Qwin, sp, w.scores, w, st, Kwin)) != JQ_OK) return rc;
     if ((rc = launch_select(w.scores, sp, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, 0, (int)nt)) != JQ_OK) return rc;
@@ -184,6 +192,10 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
     Workspace w;
     if ((rc = check_ws(s, ws, ws_bytes, &w)) != JQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
+    FusedSource src;
+    src.KA = K; src.VA = V; src.LA = s->L;
+    bool taken;
+    if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     if ((rc = launch_score_tc(K, Qwin, *s, w.scores, w, st)) != JQ_OK) return rc;
     return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);   // selects, then copies the kept rows
 }
@@ -359,6 +371,11 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     cudaStream_t st = (cudaStream_t)stream;
     const size_t row = (size_t)s->d * 2, nkeep = (size_t)(s->budget < s->L ? s->budget : s->L);
     char *Ktmp = (char *)ws + w.bytes, *Vtmp = Ktmp + align_up((size_t)s->Hkv * nkeep * row, 256);
+    // a short cache: one launch that reads the two parts where they are and moves the kept rows in place
+    FusedSource src;
+    src.KA = Kc; src.VA = Vc; src.LA = n_old; src.a_rows = cap; src.KB = Knew; src.VB = Vnew; src.LB = n_new; src.inplace = true;
+    bool taken;
+    if ((rc = launch_fused(*s, src, Qrecent, Kc, Vc, cap, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     // 1. the new rows go behind the retained ones, head by head (the cache keeps `cap` rows per head)
     if (n_new > 0) {
         if (cudaMemcpy2DAsync((char *)Kc + (size_t)n_old * row, (size_t)cap * row, Knew, (size_t)n_new * row, (size_t)n_new * row,

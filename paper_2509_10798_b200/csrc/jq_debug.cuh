@@ -14,7 +14,7 @@ struct DebugRecord {
     int kernel, site;                // of the first one
     long long index, extent;
 };
-enum { kDbgScore = 1, kDbgSelect = 2, kDbgGather = 3, kDbgDecode = 4 };
+enum { kDbgScore = 1, kDbgSelect = 2, kDbgGather = 3, kDbgDecode = 4, kDbgFused = 5 };
 
 #ifdef JQ_DEBUG
 DebugRecord *debug_record();   // host: device address of the record on the current device (nullptr on error)

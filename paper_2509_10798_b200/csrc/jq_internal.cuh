@@ -96,7 +96,8 @@ static inline size_t unit_tables_bytes(int nunits, int hpu)
            align_up((size_t)nunits * hpu * sizeof(GroupRec), 256) + align_up((size_t)nunits * hpu * sizeof(HeadRec), 256);
 }
 // One tensor map for a bf16 tensor [heads][rows][128], boxes of 64 columns x box_rows rows (host).
-bool make_tensor_map(void *map, const void *ptr, int rows, int heads, int box_rows);
+// (head_rows: rows between consecutive heads in memory when they are not packed).
+bool make_tensor_map(void *map, const void *ptr, int rows, int heads, int box_rows, int head_rows = 0);
 // Most KV heads of L keys that the scoring kernel takes as one group (tiles of a group are split over `sms` CTAs).
 int heads_per_group(int L, int heads, int tiles_per_head, int sms);
 int score_sms();   // CTAs of the scoring kernel on the current device; 0 on error
@@ -124,6 +125,17 @@ jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, fl
                         const Workspace &w, cudaStream_t st, const void *K = nullptr, const void *V = nullptr,
                         void *Kout = nullptr, void *Vout = nullptr, const UnitTables *tables = nullptr,
                         int src_head_rows = 0, int out_head_rows = 0);
+// The keys and values of a one-launch layer call: rows [0, LA) of every head in KA, VA (a_rows rows apart; 0: packed), rows
+// [LA, LA + LB) in KB, VB (packed), and the window's (Kwin: one more tile of the denominator; Vwin too: its rows are kept).
+struct FusedSource {
+    const void *KA = nullptr, *VA = nullptr, *KB = nullptr, *VB = nullptr, *Kwin = nullptr, *Vwin = nullptr;
+    int LA = 0, LB = 0, a_rows = 0;
+    bool inplace = false;   // the outputs are KA, VA themselves
+};
+// The whole pass in one launch, if the shape is one that this is the faster way for (*taken; else nothing is launched).
+// In place (Kout, Vout are KA, VA and out_head_rows is a_rows) the kept rows move to the head of the cache.
+jq_status launch_fused(const jq_shape &s, const FusedSource &src, const void *Q, void *Kout, void *Vout, int out_head_rows,
+                       int32_t *idx, const Workspace &w, cudaStream_t st, bool *taken);
 jq_status launch_gather(const void *K, const void *V, const int32_t *idx, const jq_shape &s,
                         void *Kout, void *Vout, cudaStream_t st);
 

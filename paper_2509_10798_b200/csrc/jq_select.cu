@@ -20,6 +20,7 @@
 //   4. (fused layer path only) the cluster copies the kept K and V rows of its head.
 // Everything is integer arithmetic on bit patterns, hence deterministic and exact.
 #include "jq_internal.cuh"
+#include "jq_pool.cuh"
 #include "jq_debug.cuh"
 #include <cooperative_groups.h>
 
@@ -55,19 +56,6 @@ struct SelCtl {
     int tot_gt, tot_eq;
     int scan[33];
 };
-
-__device__ __forceinline__ uint32_t order_key(float x)
-{
-    uint32_t b = __float_as_uint(x + 0.0f);  // -0 -> +0
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-__device__ __forceinline__ float max3f(float a, float b, float c)
-{
-    float y;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-    return y;
-}
 
 // Block-wide exclusive scan of one int per thread (1024 threads).
 __device__ __forceinline__ int block_excl_scan(int v, int *warp_sums)
@@ -504,33 +492,6 @@ __device__ __forceinline__ const float4 *stage_step(float4 *bufs, const float *_
     return cur;
 }
 
-// Pooled order keys (and values) of the four positions of quad `at` (0 .. 127) of the staged step.
-__device__ __forceinline__ void pooled_quad(const float4 *buf, int at, int radius, uint32_t (&key)[4], float (&best)[4])
-{
-    const float4 a = buf[at], b = buf[at + 1], c = buf[at + 2];
-    const float x[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
-    if (radius == 3) {
-        // window of 7: the four windows share x4..x7; the rest are running maxima of the three neighbours on either side
-        const float core = fmaxf(max3f(x[4], x[5], x[6]), x[7]);
-        const float l2 = fmaxf(x[2], x[3]), l1 = fmaxf(x[1], l2);
-        const float r9 = fmaxf(x[8], x[9]), r10 = fmaxf(r9, x[10]);
-        best[0] = fmaxf(core, l1);
-        best[1] = max3f(core, l2, x[8]);
-        best[2] = max3f(core, x[3], r9);
-        best[3] = fmaxf(core, r10);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float m = x[4 + i];
-#pragma unroll
-            for (int u = 1; u <= 4; ++u) if (u <= radius) m = fmaxf(m, fmaxf(x[4 + i - u], x[4 + i + u]));
-            best[i] = m;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) key[i] = order_key(best[i]);
-}
-
 // Order key of the largest of the 12 staged scores around quad `at`: an upper bound of the quad's four pooled keys
 // (every window lies inside those 12), so a quad whose bound is below a threshold holds nothing at or above it and
 // the passes that only look for such keys skip its pooling.
@@ -652,7 +613,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
             const int nval = q < qb ? min(4, L - 4 * q) : 0;
             uint32_t key[4];
             float best[4];
-            pooled_quad(bf, 32 * u + lane, radius, key, best);
+            pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
             if (pooled && nval && JQ_IN(soff + 4 * q + nval - 1, ext.scores, kDbgSelect, 25))
                 for (int i = 0; i < nval; ++i) pooled[4 * q + i] = best[i];
             // one addition per warp when all its positions share the digit (the usual case: 128 neighbouring
@@ -693,7 +654,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
                     if (nval == 0 || (quad_bound_key(bf, 32 * u + lane) >> 21) < pre) continue;
                     uint32_t key[4];
                     float best[4];
-                    pooled_quad(bf, 32 * u + lane, radius, key, best);
+                    pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
                     int nhit = 0;
                     for (int i = 0; i < 4; ++i) if (i < nval) { nhit += (key[i] >> 21) == pre; hi_cnt += (key[i] >> 21) > pre; }
                     if (nhit) {
@@ -731,7 +692,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
                         if (nval == 0 || (quad_bound_key(bf, 32 * u + lane) >> (sh + wd)) < pre) continue;
                         uint32_t key[4], dg[4];
                         float best[4];
-                        pooled_quad(bf, 32 * u + lane, radius, key, best);
+                        pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
                         for (int i = 0; i < 4; ++i) dg[i] = (key[i] >> (sh + wd)) == pre ? ((key[i] >> sh) & mask) : 0xffffffffu;
                         hist_add_runs(hist, dg, nval JQ_DBG_ARG_DEV);
                     }
@@ -765,7 +726,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
                     if (nval == 0 || quad_bound_key(bf, 32 * u + lane) < tau) continue;
                     uint32_t key[4];
                     float best[4];
-                    pooled_quad(bf, 32 * u + lane, radius, key, best);
+                    pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
                     for (int i = 0; i < 4; ++i) if (i < nval) { cgt += key[i] > tau; ceq += key[i] == tau; }
                 }
             }
@@ -788,7 +749,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
                 if (!__any_sync(0xffffffffu, may)) continue;         // nothing of these 128 quads is at or above tau
                 uint32_t key[4] = {0u, 0u, 0u, 0u};
                 float best[4];
-                if (may) pooled_quad(bf, 32 * u + lane, radius, key, best);
+                if (may) pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
                 int g = 0, e = 0;
                 for (int i = 0; i < 4; ++i) if (may && i < nval) { g += key[i] > tau; e += key[i] == tau; }
                 const int mine = g | (e << 16);

@@ -1,0 +1,127 @@
+"""The one-launch layer pass (a cluster per KV head, csrc/jq_fused.cu) and the clustered decoding step at the sizes where they
+can go wrong: tile and quad edges, parts whose lengths are no multiple of anything, every cluster size, budgets that make
+the in-place move take several steps, tied scores.  Against the fp64 oracle under the end-to-end rule of gpu_util."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import jq_workloads as W
+import paper_2509_10798_b200 as jq
+from gpu_util import assert_kept_sets_agree, dev_bf16, host_bits, shape_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__ as entry
+    entry.build()
+
+
+def wl_of(Hkv, g, w, L, budget, pool=7):
+    return W.Workload("t", 2, Hkv=Hkv, Hq=Hkv * g, L=L, w=w, budget=budget, pool=pool)
+
+
+def outputs(Hkv, rows, nidx):
+    return (torch.zeros((Hkv, rows, 128), dtype=torch.bfloat16, device="cuda"), torch.zeros((Hkv, rows, 128), dtype=torch.bfloat16, device="cuda"),
+            torch.full((Hkv, nidx), -1, dtype=torch.int32, device="cuda"))
+
+
+# Hkv, g, w, L, budget, pool: L around a tile, around 2 and 4 tiles per CTA, up to the longest the kernel takes; one head and more
+# heads than clusters fit at a time; one and two blocks of query rows, rows that are no multiple of 32; pools on both code paths
+CASES = [(1, 1, 1, 1, 1, 1), (1, 1, 3, 5, 2, 3), (2, 4, 16, 127, 40, 7), (2, 4, 16, 128, 128, 7), (2, 4, 32, 129, 128, 7),
+         (3, 4, 33, 257, 100, 9), (2, 4, 16, 2048, 256, 7), (1, 8, 32, 2049, 64, 7), (8, 4, 32, 1025, 1000, 5), (5, 7, 36, 1500, 333, 11),
+         (2, 4, 8, 4096, 4095, 63), (8, 4, 32, 4097, 512, 7), (8, 4, 64, 3001, 700, 7), (4, 4, 32, 12288, 2048, 7), (40, 2, 32, 513, 50, 7),
+         (2, 1, 5, 6001, 1, 7)]
+
+
+@pytest.mark.parametrize("Hkv,g,w,L,budget,pool", CASES)
+def test_layer_in_one_launch(Hkv, g, w, L, budget, pool):
+    wl = wl_of(Hkv, g, w, L, budget, pool)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    Ko, Vo, idx = outputs(Hkv, wl.nkeep, wl.nkeep)
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer(dev_bf16(K), dev_bf16(V), dev_bf16(Q), s, Ko, Vo, idx, ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK
+    assert jq.launch_count() - n0 == 1
+    pooled = oracle.pool(oracle.score(K, Q), pool)
+    gi = idx.cpu().numpy()
+    assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
+    gK, gV = host_bits(Ko), host_bits(Vo)
+    for kv in range(Hkv):
+        assert np.array_equal(gK[kv], K[kv][gi[kv]]) and np.array_equal(gV[kv], V[kv][gi[kv]])
+
+
+@pytest.mark.parametrize("L,budget", [(700, 100), (4096, 513), (9000, 2048)])
+def test_tied_scores_keep_the_lowest_positions(L, budget):
+    """Equal keys give equal scores: with Q = 0 every pooled score is the same number, and the first `budget` positions stay."""
+    wl = wl_of(2, 4, 16, L, budget)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    Ko, Vo, idx = outputs(2, budget, budget)
+    jq.evict_layer(dev_bf16(K), dev_bf16(V), dev_bf16(np.zeros_like(Q)), s, Ko, Vo, idx, jq.new_workspace(s))
+    assert np.array_equal(idx.cpu().numpy(), np.tile(np.arange(budget), (2, 1)))
+
+
+@pytest.mark.parametrize("Hkv,g,w,L,budget", [(2, 4, 32, 128, 64), (8, 4, 32, 1000, 300), (2, 2, 128, 2500, 700), (3, 4, 64, 5001, 900)])
+def test_window_kept_in_one_launch(Hkv, g, w, L, budget):
+    wl = wl_of(Hkv, g, w, L, budget)
+    if budget <= w:
+        wl = wl.with_budget(w + 5)
+    K, V, Q, _ = W.make_layer(wl)
+    Kw = W.make_window_keys(wl, Q)
+    Vw = W.make_v(wl_of(Hkv, g, w, w, 1), 77)
+    s = shape_of(wl)
+    np_ = min(wl.budget - w, L)
+    Ko, Vo, _ = outputs(Hkv, np_ + w, 1)
+    idx = torch.full((Hkv, np_), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_workspace(s)
+    jq.evict_layer_window_kept(dev_bf16(K), dev_bf16(V), dev_bf16(Q), dev_bf16(Kw), dev_bf16(Vw), s, Ko, Vo, idx, ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK
+    gi, gK, gV = idx.cpu().numpy(), host_bits(Ko), host_bits(Vo)
+    pooled = oracle.pool(oracle.score_windowed(K, Q, Kw), wl.pool)
+    assert_kept_sets_agree(gi, oracle.select(pooled, np_), pooled, np_)
+    for kv in range(Hkv):
+        assert np.array_equal(gK[kv, :np_], K[kv][gi[kv]]) and np.array_equal(gV[kv, :np_], V[kv][gi[kv]])
+        assert np.array_equal(gK[kv, np_:], Kw[kv]) and np.array_equal(gV[kv, np_:], Vw[kv])
+
+
+# n_old, n_new: parts that end inside a tile and inside a quad; everything kept; a move of several steps (many rows)
+@pytest.mark.parametrize("Hkv,g,w,n_old,n_new,budget,cap", [(2, 4, 32, 129, 127, 200, 256), (2, 4, 32, 130, 3, 133, 200), (8, 4, 32, 1021, 257, 1021, 1300),
+                                                             (1, 4, 64, 4096, 1000, 4096, 5200), (2, 2, 16, 3, 2000, 1500, 2003), (2, 4, 16, 0, 300, 100, 300),
+                                                             (1, 4, 32, 9000, 3000, 11000, 12000)])
+def test_append_in_one_launch(Hkv, g, w, n_old, n_new, budget, cap):
+    wl = wl_of(Hkv, g, w, n_old + n_new, budget)
+    K, V, Q, _ = W.make_layer(wl, layer=2)
+    s = shape_of(wl)
+    Kc = torch.zeros((Hkv, cap, 128), dtype=torch.bfloat16, device="cuda")
+    Vc = torch.zeros_like(Kc)
+    Kc[:, :n_old] = dev_bf16(K[:, :n_old]); Vc[:, :n_old] = dev_bf16(V[:, :n_old])
+    idx = torch.full((Hkv, wl.nkeep), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_append_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_append(Kc, Vc, n_old, dev_bf16(K[:, n_old:]), dev_bf16(V[:, n_old:]), dev_bf16(Q), s, idx, ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK
+    assert jq.launch_count() - n0 == 1
+    gi = idx.cpu().numpy()
+    pooled = oracle.pool(oracle.score(K, Q), wl.pool)
+    assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
+    gK, gV = host_bits(Kc), host_bits(Vc)
+    for kv in range(Hkv):
+        assert np.array_equal(gK[kv, :wl.nkeep], K[kv][gi[kv]]) and np.array_equal(gV[kv, :wl.nkeep], V[kv][gi[kv]])
+
+
+# keys around a unit of 16 and around what one, two and sixteen CTAs of eight warps take at a time; groups on both sides of 4
+@pytest.mark.parametrize("Hkv,group,n", [(1, 1, 1), (2, 4, 15), (2, 5, 16), (2, 8, 17), (3, 3, 129), (1, 4, 2049), (2, 7, 4100), (150, 2, 40), (40, 4, 700)])
+def test_decode_step_edges(Hkv, group, n):
+    rng = np.random.default_rng(n)
+    Kc, Vc = W.bf16_bits(rng.standard_normal((Hkv, n, 128))), W.bf16_bits(rng.standard_normal((Hkv, n, 128)))
+    q = W.bf16_bits(2.0 * rng.standard_normal((Hkv * group, 128)))
+    out = torch.full((Hkv * group, 128), -1.0, dtype=torch.float32, device="cuda")
+    ws = torch.empty(jq.decode_workspace_bytes(Hkv, Hkv * group, n), dtype=torch.uint8, device="cuda")
+    jq.decode_attention(dev_bf16(Kc), dev_bf16(Vc), dev_bf16(q), out, ws)
+    # fp32 sums of n <= 4100 terms whose weights add up to 1 (bounded by sqrt(n) 2^-24 of values of size 1) and ex2 (2 ulp)
+    np.testing.assert_allclose(out.cpu().numpy(), oracle.decode_attention(Kc, Vc, q), rtol=2e-5, atol=5e-6)
