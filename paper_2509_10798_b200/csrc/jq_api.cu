@@ -134,18 +134,14 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     // prefix rows: the window-inclusive pass with budget - w; then the w window rows behind them, head by head
     jq_shape sp = *s;
     sp.budget = s->budget - s->w;
-    const size_t row = (size_t)s->d * 2, np = (size_t)(sp.budget < s->L ? sp.budget : s->L), nt = np + (size_t)s->w;
+    const size_t np = (size_t)(sp.budget < s->L ? sp.budget : s->L), nt = np + (size_t)s->w;
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin; src.Vwin = Vwin;
     bool taken;
     if ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
     if ((rc = launch_score_tc(K, Qwin, sp, w.scores, w, st, Kwin)) != JQ_OK) return rc;
-    if ((rc = launch_select(w.scores, sp, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, 0, (int)nt)) != JQ_OK) return rc;
-    if (cudaMemcpy2DAsync((char *)Kout + np * row, nt * row, Kwin, (size_t)s->w * row, (size_t)s->w * row, (size_t)s->Hkv, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaMemcpy2DAsync((char *)Vout + np * row, nt * row, Vwin, (size_t)s->w * row, (size_t)s->w * row, (size_t)s->Hkv, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return JQ_ERR_CUDA;
-    return JQ_OK;
+    return launch_select(w.scores, sp, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, 0, (int)nt, Kwin, Vwin);
 }
 
 jq_status jq_score_fma(const void *K, const void *Qwin, const jq_shape *s, float *scores, void *ws,

@@ -44,7 +44,7 @@ constexpr int kFTile = 128;                         // keys per tile
 constexpr int kFWarps = 16;                         // epilogue warps
 constexpr int kFT = 32 * kFWarps;                   // threads that take part in the selection
 constexpr int kFThreads = kFT + 64;                 // plus the producer and the MMA warp
-constexpr int kFMaxCluster = 16;                   // (sizes the statistics' extent)
+[[maybe_unused]] constexpr int kFMaxCluster = 16; // (sizes the statistics' extent)
 constexpr int kFMaxStages = 6;
 constexpr int kFCand = 512;                         // keys of one bin that are ranked by comparison
 constexpr int kFMaxL = 12288;                       // what shared memory has room for, and about where the general path overtakes

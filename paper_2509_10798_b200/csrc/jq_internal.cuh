@@ -121,10 +121,11 @@ jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float
 // head has a length, a budget and offsets of its own (s.L, s.budget unused).
 // src_head_rows: rows between consecutive heads of K and V in memory when the heads are not packed (0: s.L);
 // out_head_rows: rows between consecutive heads of Kout and Vout when more than nkeep (0: nkeep).
+// Kwin, Vwin: with both given, the w window rows of every head follow its kept rows in Kout and Vout.
 jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, float *pooled,
                         const Workspace &w, cudaStream_t st, const void *K = nullptr, const void *V = nullptr,
                         void *Kout = nullptr, void *Vout = nullptr, const UnitTables *tables = nullptr,
-                        int src_head_rows = 0, int out_head_rows = 0);
+                        int src_head_rows = 0, int out_head_rows = 0, const void *Kwin = nullptr, const void *Vwin = nullptr);
 // The keys and values of a one-launch layer call: rows [0, LA) of every head in KA, VA (a_rows rows apart; 0: packed), rows
 // [LA, LA + LB) in KB, VB (packed), and the window's (Kwin: one more tile of the denominator; Vwin too: its rows are kept).
 struct FusedSource {

@@ -1,42 +1,48 @@
-// Max-pool + exact top-k selection per KV head.  Two kernels share the arithmetic: select_cluster, one
-// thread-block cluster per head (8 CTAs when the call has few heads, 4 or 2 when it has more heads than
-// clusters fit on the GPU at a time, see choose_plan), and, for calls over 128 heads or more, select_stream
-// further down, one CTA per head.  The cluster kernel:
+// Max-pool + exact top-k selection per KV head.  Two kernels share the arithmetic: select_cluster, one thread-block cluster
+// of 2 to 16 CTAs per head (choose_plan), and, for calls over 128 heads or more, select_stream further down, one CTA per
+// head.  The cluster kernel:
 //
-//   1. pool: pooled[j] = max of the centred window (edges clipped), turned into an order-preserving
-//      32-bit integer key (float order == unsigned order).  Each CTA owns a contiguous share of
-//      the positions and keeps its keys in shared memory (in the workspace for very long prefixes).
-//   2. radix select, 3 rounds of 11/11/10 bits, most significant first: local integer histograms
-//      are summed into the leading CTA through distributed shared memory, which finds the digit
-//      holding the nkeep-th largest key and broadcasts it.  After the first round the keys that
-//      share that digit are normally few: they are then copied into the leading CTA, which runs
-//      the two remaining rounds on them alone (no further pass over all keys, no further
-//      histogram traffic).  Result: the key tau of the nkeep-th largest element and how many
-//      elements equal to tau are kept.  Max-pooling copies every peak
-//      into up to `pool` neighbours, so ties at tau are the normal case: all keys > tau are kept,
-//      then the lowest-index keys == tau.
-//   3. ordered compaction: kept positions are written in ascending order (CTA rank, warp,
-//      iteration and lane order all follow the position order).
-//   4. (fused layer path only) the cluster copies the kept K and V rows of its head.
-// Everything is integer arithmetic on bit patterns, hence deterministic and exact.
+//   1. pool: pooled[j] = max of the centred window (edges clipped), turned into an order-preserving 32-bit integer key
+//      (float order == unsigned order).  Each CTA owns a contiguous share of the positions and keeps its keys in shared
+//      memory (in the workspace for very long prefixes).
+//   2. the threshold: 2048 equal bins over the range of the head's keys - not their leading bits, which are the same for
+//      most keys of a flat head and would need further rounds over all of them.  The histograms are summed through
+//      distributed shared memory, every CTA owning a share of the bins, and every CTA finds the bin of the nkeep-th
+//      largest key for itself.  Its keys, normally a few dozen, go to the leading CTA with their positions, and every CTA
+//      ranks them by comparison: the key tau of the nkeep-th largest element and how many elements equal to tau are
+//      kept.  (While the bin holds more than kCandMax keys it is split into 2048 bins again.)  Max-pooling copies every peak into up to `pool` neighbours, so ties at tau are
+//      the normal case: all keys > tau are kept, then the lowest-index keys == tau.
+//   3. ordered compaction: kept positions are written in ascending order (CTA rank, warp, iteration and lane order all
+//      follow the position order); the list also gives every warp its number of kept keys, so nothing is counted again.
+//   4. (fused layer path only) the cluster copies the kept K and V rows of its head, and the window rows behind them.
+// Everything is integer arithmetic on bit patterns, hence deterministic and exact.  The kernel is a chain of short phases
+// between cluster barriers (four; about 700 cycles each), so what bounds it is latency.  Measured (8 heads, us, against
+// leading-bit radix rounds of 11 bits, a counting pass, clusters of 8 and one row in flight per 16 lanes in the copy):
+// selection alone 12000 keys 10.6 -> 8.6, 30011 12.1 -> 10.8, 131072 21.3 -> 18.5; with the rows of a layer 131072 keys, budget
+// 4096, 73.6 k -> 42.9 k cycles; the windowed layer of 11999 keys (two strided copies before) 46.3 -> 36.9 us.
 #include "jq_internal.cuh"
 #include "jq_pool.cuh"
 #include "jq_debug.cuh"
 #include <cooperative_groups.h>
+#include <mutex>
 
 namespace cg = cooperative_groups;
 
 namespace jq {
 namespace {
 
-constexpr int kClMax = 8;          // most CTAs per cluster (= per KV head); the kernel also exists for 4 and 2
-constexpr int kSelThreads = 1024;
+constexpr int kClMax = 16;         // most CTAs per cluster (= per KV head)
+constexpr int kSelThreads = 512, kSelWarps = kSelThreads / 32;   // two CTAs to an SM (a cluster of 16 then fits for 8 heads at a time)
 constexpr int kBins = 2048;
-constexpr int kRawTile = 20480;    // most scores staged per pooling step (a CTA's whole share unless the prefix is very long)
+constexpr int kOwnBins = 3 * kBins / 2;   // select_cluster: a CTA's share of the bins in each of three rounds, with two CTAs per cluster
+constexpr int kRawTile = 8192;     // most scores staged per pooling step
 constexpr int kHalo = 32;          // >= pool radius
 constexpr int kKeysSmemMax = 24576; // keys a CTA can keep in shared memory
-constexpr int kCandMax = 8192;     // candidates the leading CTA finishes alone (they live in its staging buffer)
-static_assert(kCandMax <= kRawTile, "candidates are kept in the staging buffer");
+constexpr size_t kSelTwoPerSm = 100 * 1024;   // shared memory per CTA up to which two CTAs fit on an SM
+constexpr double kSelChain = 7.5, kSelChain16 = 10.0, kSelPerKey = 0.0007;   // choose_plan's estimate, us
+constexpr int kCandMax = 512;      // keys of one bin that are ranked by comparison (one per thread)
+static_assert(kCandMax <= kSelThreads, "a thread ranks one candidate");
+static_assert(kBins == 4 * kSelThreads, "a thread takes four bins");
 
 // Extents of what the kernel indexes (read by the bounds-checked build only).
 struct SelExtents {
@@ -45,39 +51,45 @@ struct SelExtents {
     long long src_heads;  // heads in one source buffer of K / V
 };
 
+// The window rows that follow every head's kept rows: K, V [Hkv][w] rows (w = 0: none).
+struct WindowRows { const uint4 *K, *V; int w; };
+
 struct SelCtl {
-    uint32_t prefix;
-    int krem;
-    int found_prefix_digit, found_krem, found_count;
-    int cand_total;      // keys sharing the first-round digit (broadcast by the leading CTA)
-    int cand_count;      // leading CTA only: candidates appended so far
-    int counts_gt[kClMax], counts_eq[kClMax];
-    int warp_gt[32], warp_eq[32];
-    int tot_gt, tot_eq;
-    int scan[33];
+    int digit, krem, count;              // find_digit: the bin of the krem-th key, the rank within it, its population
+    uint32_t tau;
+    int need_eq;
+    int cand_count;                      // leading CTA only: candidates appended so far
+    int base_gt, base_eq;                // kept-or-tied keys of the CTAs before this one
+    uint32_t mn[kClMax], mx[kClMax];     // range of every CTA's keys
+    int gt_of[kClMax], eq_of[kClMax];    // every CTA's keys above the bin (above tau, equal to tau)
+    int warp_gt[kSelWarps], warp_eq[kSelWarps];
+    uint32_t wmn[kSelWarps], wmx[kSelWarps];
+    int scan[kSelWarps];
+    uint32_t cand_key[kCandMax], my_key[kCandMax];   // leading CTA: the list; everybody's copy of it
+    int cand_pos[kCandMax], my_pos[kCandMax];
 };
 
-// Block-wide exclusive scan of one int per thread (1024 threads).
-__device__ __forceinline__ int block_excl_scan(int v, int *warp_sums)
+// Block-wide exclusive scan of one int per thread, any number of whole warps.
+__device__ __forceinline__ int cta_excl_scan(int v, int *warp_sums)
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     int inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int n = __shfl_up_sync(0xffffffffu, inc, o);
+        const int n = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += n;
     }
     if (lane == 31) warp_sums[wid] = inc;
     __syncthreads();
     if (wid == 0) {
-        int ws = warp_sums[lane];
+        const int ws = lane < nw ? warp_sums[lane] : 0;
         int winc = ws;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            int n = __shfl_up_sync(0xffffffffu, winc, o);
+            const int n = __shfl_up_sync(0xffffffffu, winc, o);
             if (lane >= o) winc += n;
         }
-        warp_sums[lane] = winc - ws;       // exclusive warp offsets
+        if (lane < nw) warp_sums[lane] = winc - ws;
     }
     __syncthreads();
     const int excl = warp_sums[wid] + inc - v;
@@ -85,72 +97,91 @@ __device__ __forceinline__ int block_excl_scan(int v, int *warp_sums)
     return excl;
 }
 
-// All 1024 threads of a CTA: in a histogram of kBins bins find, walking the bins from the top, the bin
-// that holds the krem-th element; leaves the bin, the rank within it and its population in ctl.
-__device__ __forceinline__ void find_digit(const uint32_t *g, int krem, SelCtl &ctl)
+// All threads of a CTA of 512 or 1024: the bin of h[kBins] that holds the krem-th key counted from the top.
+template <typename Ctl>
+__device__ __forceinline__ void find_digit_cta(const uint32_t *h, int krem, Ctl &ctl)
 {
-    // bins in descending order: thread t looks at bins 2047-2t and 2046-2t
-    const int hi = kBins - 1 - 2 * (int)threadIdx.x, lo = hi - 1;
-    const int h_hi = (int)g[hi], h_lo = (int)g[lo];
-    const int above = block_excl_scan(h_hi + h_lo, ctl.scan);
-    if (above < krem && krem <= above + h_hi) {
-        ctl.found_prefix_digit = hi; ctl.found_krem = krem - above; ctl.found_count = h_hi;
-    } else if (above + h_hi < krem && krem <= above + h_hi + h_lo) {
-        ctl.found_prefix_digit = lo; ctl.found_krem = krem - above - h_hi; ctl.found_count = h_lo;
+    const int per = kBins / (int)blockDim.x;                  // 4 or 2 bins per thread, descending
+    const int hi = kBins - 1 - per * (int)threadIdx.x;
+    int tot = 0;
+    for (int i = 0; i < per; ++i) tot += (int)h[hi - i];
+    int above = cta_excl_scan(tot, ctl.scan);
+    for (int i = 0; i < per; ++i) {
+        const int c = (int)h[hi - i];
+        if (above < krem && krem <= above + c) { ctl.digit = hi - i; ctl.krem = krem - above; ctl.count = c; }
+        above += c;
     }
     __syncthreads();
 }
 
-// The cluster copies the kept K and V rows of its head (256 bytes each: 16 lanes x 16 bytes), CTA r the
-// r-th share of them, once every index of the head has been written.
+// Rows [r0, r1) of a head's kept rows (256 bytes each: 16 lanes x 16 bytes), four rows of K and V in flight per 16 lanes.
 // kv_in: the head's index within the buffer the rows come from; orow: the head's first row in the outputs.
-template <int CL>
-__device__ __forceinline__ void copy_kept_rows(cg::cluster_group &cluster, const int32_t *out, int kv_in, long long orow, int L, int nkeep,
-                                               const uint4 *Kin, const uint4 *Vin, uint4 *Kout, uint4 *Vout, int src_rows,
-                                               const SelExtents &ext JQ_DBG_PARAM)
+__device__ __forceinline__ void copy_rows(const int32_t *out, int r0, int r1, int kv_in, long long orow, int L, const uint4 *__restrict__ Kin,
+                                          const uint4 *__restrict__ Vin, uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, int src_rows,
+                                          const SelExtents &ext JQ_DBG_PARAM)
 {
-    __threadfence();
-    cluster.sync();
-    const int rank = (int)cluster.block_rank();
-    const int r0 = (int)((long long)rank * nkeep / CL), r1 = (int)((long long)(rank + 1) * nkeep / CL);
-    const int lane16 = threadIdx.x & 15;
-    for (int t = r0 + (int)(threadIdx.x >> 4); t < r1; t += kSelThreads / 16) {
-        const int j = min(max(__ldcg(out + t), 0), L - 1);
-        const size_t src = ((size_t)kv_in * src_rows + j) * 16 + lane16, dst = (size_t)(orow + t) * 16 + lane16;
-        if (JQ_IN((long long)kv_in * src_rows + j, ext.src_heads * src_rows, kDbgSelect, 1) && JQ_IN(orow + t, ext.out_rows, kDbgSelect, 2)) {
-            Kout[dst] = Kin[src];
-            Vout[dst] = Vin[src];
+    (void)ext;
+    const int lane16 = threadIdx.x & 15, grp = threadIdx.x >> 4, ngrp = blockDim.x >> 4;
+    for (int t0 = r0 + 4 * grp; t0 < r1; t0 += 4 * ngrp) {
+        int j[4];
+        uint4 a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) j[r] = t0 + r < r1 ? min(max(__ldcg(out + t0 + r), 0), L - 1) : 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const size_t src = ((size_t)kv_in * src_rows + j[r]) * 16 + lane16;
+            const bool in = t0 + r < r1 && JQ_IN((long long)kv_in * src_rows + j[r], ext.src_heads * src_rows, kDbgSelect, 1);
+            a[r] = in ? Kin[src] : make_uint4(0u, 0u, 0u, 0u);
+            b[r] = in ? Vin[src] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const size_t dst = (size_t)(orow + t0 + r) * 16 + lane16;
+            if (t0 + r < r1 && JQ_IN(orow + t0 + r, ext.out_rows, kDbgSelect, 2)) { Kout[dst] = a[r]; Vout[dst] = b[r]; }
         }
     }
 }
 
-// grid (Hkv * CL), cluster CL, block 1024.  With htab (ragged calls) every head has a length, a budget, offsets
+// Window rows [i0, w), every `step`-th group's share, behind the kept rows of head kv (row `row0` of the outputs on).
+__device__ __forceinline__ void copy_window(const WindowRows &win, int kv, long long row0, int first, int step, uint4 *__restrict__ Kout,
+                                            uint4 *__restrict__ Vout, const SelExtents &ext JQ_DBG_PARAM)
+{
+    (void)ext;
+    const int lane16 = threadIdx.x & 15;
+    for (int i = first; i < win.w; i += step) {
+        const size_t src = ((size_t)kv * win.w + i) * 16 + lane16, dst = (size_t)(row0 + i) * 16 + lane16;
+        if (JQ_IN(row0 + i, ext.out_rows, kDbgSelect, 32)) { Kout[dst] = win.K[src]; Vout[dst] = win.V[src]; }
+    }
+}
+
+// grid (Hkv * CL), cluster CL, block 512.  With htab (ragged calls) every head has a length, a budget, offsets
 // into the scores, the keys and the outputs, and a source buffer of its own; L, nkeep, chunk, keys_in_smem are
 // then those of the longest head and only size the shared memory.
-template <int CL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kSelThreads, 2)
+__global__ void __launch_bounds__(kSelThreads, 2)
 select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, int32_t *__restrict__ idx,
                float *__restrict__ pooled, uint32_t *__restrict__ gkeys, int chunk, int keys_in_smem, int raw_tile,
                const uint4 *__restrict__ Kin, const uint4 *__restrict__ Vin, uint4 *__restrict__ Kout,
                uint4 *__restrict__ Vout, const HeadRec *__restrict__ htab, const uint4 *const *__restrict__ Ktab,
-               const uint4 *const *__restrict__ Vtab, int src_rows, int out_rows, const SelExtents ext JQ_DBG_PARAM)
+               const uint4 *const *__restrict__ Vtab, int src_rows, int out_rows, const WindowRows win, const SelExtents ext JQ_DBG_PARAM)
 {
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
-    const int kv = blockIdx.x / CL;
+    const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
+    const int kv = (int)blockIdx.x / CL;
     int kv_in = kv;                                  // the head's index within the buffer its rows come from
     long long soff = (long long)kv * L, orow = (long long)kv * nkeep;   // offsets of the head's scores and of its kept indices
     long long krow = (long long)kv * out_rows;                          // first row of the head in the compacted outputs
     extern __shared__ __align__(16) uint8_t sm[];
-    uint32_t *ghist = (uint32_t *)sm;                       // [kBins]; the leading CTA's copy accumulates the cluster's histogram of a round
-    uint32_t *hist = ghist + kBins;                         // [kBins]
-    float *raw = (float *)(hist + kBins);                   // [raw_tile + 2*kHalo]; later the candidate keys
+    uint32_t *ghist = (uint32_t *)sm;                       // [3][kBins / CL]: the cluster's counts of the bins this CTA owns, one set per round
+    uint32_t *hist = ghist + kOwnBins;                      // [kBins]
+    float *raw = (float *)(hist + kBins);                   // [raw_tile + 2*kHalo]
     uint32_t *keys_s = (uint32_t *)(raw + raw_tile + 2 * kHalo);
     __shared__ SelCtl ctl;
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int raw_cap = raw_tile + 2 * kHalo, keys_cap = keys_in_smem ? chunk : 0;   // shared-memory extents (those of the launch)
     (void)raw_cap; (void)keys_cap;
+    for (int i = tid; i < kOwnBins + kBins; i += kSelThreads) ghist[i] = 0;
+    if (tid == 0) ctl.cand_count = 0;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
     if (htab) {
         const HeadRec r = htab[kv];
@@ -164,76 +195,43 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     int32_t *out = idx + orow;
     if (pooled) pooled += soff;
 
-    // ---- 1. max-pool -> keys
-    // With the keys in shared memory and a window of at most 9, a thread pools four neighbouring
-    // positions from three 16-byte reads and the first-round histogram is built on the way.
+    // ---- 1. max-pool -> keys, and their range
+    // With the keys in shared memory and a window of at most 9, a thread pools four neighbouring positions from three
+    // 16-byte reads.
     const bool fast_pool = keys_in_smem && radius <= 4;
-    for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
+    const int left = fast_pool ? 4 : radius;                // staged values before the first position
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
     for (int t0 = 0; t0 < n; t0 += raw_tile) {
-        const int tile = min(raw_tile, n - t0);
+        const int tile = min(raw_tile, n - t0), staged = fast_pool ? ((tile + 3) & ~3) + 8 : tile + 2 * radius;
         __syncthreads();
         // eight loads in flight per thread: the scores come from L2, one round trip each
-        for (int i0 = tid; i0 < tile + 2 * radius; i0 += 8 * kSelThreads) {
+        for (int i0 = tid; i0 < staged; i0 += 8 * kSelThreads) {
             float vals[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int j = j0 + t0 - radius + i0 + q * kSelThreads;
-                vals[q] = (i0 + q * kSelThreads < tile + 2 * radius && j >= 0 && j < L && JQ_IN(soff + j, ext.scores, kDbgSelect, 3)) ? __ldcg(s + j) : -INFINITY;
+                const int i = i0 + q * kSelThreads, j = j0 + t0 - left + i;
+                vals[q] = (i < staged && j >= 0 && j < L && JQ_IN(soff + j, ext.scores, kDbgSelect, 3)) ? __ldcg(s + j) : -INFINITY;
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (i0 + q * kSelThreads < tile + 2 * radius && JQ_IN(i0 + q * kSelThreads, raw_cap, kDbgSelect, 4)) raw[i0 + q * kSelThreads] = vals[q];
+                if (i0 + q * kSelThreads < staged && JQ_IN(i0 + q * kSelThreads, raw_cap, kDbgSelect, 4)) raw[i0 + q * kSelThreads] = vals[q];
         }
-        if (fast_pool) for (int i = tid; i < 8; i += kSelThreads) if (JQ_IN(tile + 2 * radius + i, raw_cap, kDbgSelect, 5)) raw[tile + 2 * radius + i] = -INFINITY;   // its 16-byte reads run a little past the window
         __syncthreads();
         if (fast_pool) {
             const int nquads = (tile + 3) / 4;
             const float4 *raw4 = (const float4 *)raw;
-            for (int base = 0; base < nquads; base += kSelThreads) {      // uniform trip count: whole warps reach the votes
-                const int g4 = base + tid;
-                const bool act = g4 < nquads;
-                float x[12];
-                {
-                    const bool rd = act && JQ_IN(4 * (g4 + 2) + 3, raw_cap, kDbgSelect, 6);
-                    const float4 a = rd ? raw4[g4] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 b = rd ? raw4[g4 + 1] : a, c = rd ? raw4[g4 + 2] : a;
-                    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-                    x[8] = c.x; x[9] = c.y; x[10] = c.z; x[11] = c.w;
-                }
+            for (int g4 = tid; g4 < nquads; g4 += kSelThreads) {
+                const int nval = min(4, tile - 4 * g4);              // positions of this quad inside the tile
+                if (!JQ_IN(4 * (g4 + 2) + 3, raw_cap, kDbgSelect, 6) || !JQ_IN(t0 + 4 * g4 + nval - 1, keys_cap, kDbgSelect, 7)) continue;
                 uint32_t key[4];
                 float best[4];
+                pooled_quad(raw4[g4], raw4[g4 + 1], raw4[g4 + 2], radius, key, best);
+                if (nval == 4) *(uint4 *)(mykeys + t0 + 4 * g4) = make_uint4(key[0], key[1], key[2], key[3]);
+                else for (int i = 0; i < nval; ++i) mykeys[t0 + 4 * g4 + i] = key[i];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float m = x[i];
-#pragma unroll
-                    for (int u = 1; u <= 8; ++u) if (u <= 2 * radius) m = fmaxf(m, x[i + u]);
-                    best[i] = m;
-                    key[i] = order_key(m);
-                }
-                const int nval = act ? min(4, tile - 4 * g4) : 0;          // positions of this quad inside the tile
-                if (act && JQ_IN(t0 + 4 * g4 + nval - 1, keys_cap, kDbgSelect, 7) && (!pooled || JQ_IN(soff + j0 + t0 + 4 * g4 + nval - 1, ext.scores, kDbgSelect, 8))) {
-                    if (nval == 4) *(uint4 *)(mykeys + t0 + 4 * g4) = make_uint4(key[0], key[1], key[2], key[3]);
-                    else for (int i = 0; i < nval; ++i) mykeys[t0 + 4 * g4 + i] = key[i];
-                    if (pooled) for (int i = 0; i < nval; ++i) pooled[j0 + t0 + 4 * g4 + i] = best[i];
-                }
-                // first-round histogram: one addition per warp when all its positions share the digit (the usual
-                // case: 128 neighbouring positions of similar size), else runs of equal digits per thread
-                const uint32_t d0 = key[0] >> 21;
-                bool same = true;
-                for (int i = 1; i < 4; ++i) if (i < nval && (key[i] >> 21) != d0) same = false;
-                const uint32_t lead = __shfl_sync(0xffffffffu, d0, 0);
-                if (__all_sync(0xffffffffu, nval == 0 || (same && d0 == lead))) {
-                    const int tot = __reduce_add_sync(0xffffffffu, nval);
-                    if (lane == 0 && tot && JQ_IN(lead, kBins, kDbgSelect, 9)) atomicAdd(&hist[lead], (uint32_t)tot);
-                } else {
-                    uint32_t cur = 0, cnt = 0;
-                    for (int i = 0; i < nval; ++i) {
-                        const uint32_t d = key[i] >> 21;
-                        if (cnt && d != cur) { atomicAdd(&hist[cur], cnt); cnt = 0; }
-                        cur = d; ++cnt;
-                    }
-                    if (cnt) atomicAdd(&hist[cur], cnt);
-                }
+                for (int i = 0; i < 4; ++i) if (i < nval) { kmin = min(kmin, key[i]); kmax = max(kmax, key[i]); }
+                if (pooled && JQ_IN(soff + j0 + t0 + 4 * g4 + nval - 1, ext.scores, kDbgSelect, 8))
+                    for (int i = 0; i < nval; ++i) pooled[j0 + t0 + 4 * g4 + i] = best[i];
             }
             continue;
         }
@@ -242,169 +240,200 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
             if (!JQ_IN(e + 2 * radius, raw_cap, kDbgSelect, 10)) continue;
             float best = raw[e];
             for (int u = 1; u <= 2 * radius; ++u) best = fmaxf(best, raw[e + u]);
-            if (JQ_IN(keys_in_smem ? t0 + e : soff + j0 + t0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 11)) mykeys[t0 + e] = order_key(best);
+            const uint32_t k = order_key(best);
+            kmin = min(kmin, k); kmax = max(kmax, k);
+            if (JQ_IN(keys_in_smem ? t0 + e : soff + j0 + t0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 11)) mykeys[t0 + e] = k;
             if (pooled && JQ_IN(soff + j0 + t0 + e, ext.scores, kDbgSelect, 12)) pooled[j0 + t0 + e] = best;
         }
     }
+    const int ngrp = kSelThreads / 16;
+    const int r0 = (int)((long long)rank * nkeep / CL), r1 = (int)((long long)(rank + 1) * nkeep / CL);   // the rows this CTA copies
     if (nkeep >= L) {   // everything is kept (uniform over the cluster; no cluster traffic yet)
         for (int e = tid; e < n; e += kSelThreads) if (JQ_IN(orow + j0 + e, ext.out_rows, kDbgSelect, 13)) out[j0 + e] = j0 + e;
-        if (Kin) copy_kept_rows<CL>(cluster, out, kv_in, krow, L, nkeep, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+        if (Kin) {
+            cluster.sync();
+            copy_rows(out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+            if (win.w) copy_window(win, kv, krow + nkeep, rank * ngrp + (tid >> 4), CL * ngrp, Kout, Vout, ext JQ_DBG_ARG_DEV);
+        }
         return;
     }
-    for (int i = tid; i < kBins; i += kSelThreads) ghist[i] = 0;
-    if (tid == 0) { ctl.prefix = 0; ctl.krem = nkeep; ctl.cand_count = 0; ctl.cand_total = 0; }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) { ctl.wmn[wid] = kmin; ctl.wmx[wid] = kmax; }
+    __syncthreads();
+    if (wid == 0) {
+        kmin = __reduce_min_sync(0xffffffffu, ctl.wmn[lane % kSelWarps]);
+        kmax = __reduce_max_sync(0xffffffffu, ctl.wmx[lane % kSelWarps]);
+        if (lane < CL) {
+            SelCtl *rc = cluster.map_shared_rank(&ctl, lane);
+            rc->mn[rank] = kmin; rc->mx[rank] = kmax;
+        }
+    }
     cluster.sync();
 
-    // ---- 2. radix select
-    const int n_up = (n + kSelThreads - 1) / kSelThreads * kSelThreads;
-    for (int round = 0; round < 3; ++round) {
-        const int shift = (round == 0) ? 21 : (round == 1 ? 10 : 0);
-        const int width = (round == 2) ? 10 : 11;
-        const uint32_t mask = (1u << width) - 1u;
-        const bool have_hist = round == 0 && fast_pool;          // built while pooling
-        if (!have_hist) for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
-        __syncthreads();
-        const uint32_t prefix = ctl.prefix;
-        // A thread takes a run of consecutive keys and adds equal neighbouring digits as one count: the
-        // max-pool leaves plateaus, so a few additions per thread replace one per key.
-        if (!have_hist) {
-            const int per = (n + kSelThreads - 1) / kSelThreads;
+    // ---- 2. the threshold
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    for (int q = 0; q < CL; ++q) { lo = min(lo, ctl.mn[q]); hi = max(hi, ctl.mx[q]); }
+    uint32_t lim = hi - lo;                      // the keys in [lo, lo + lim] are the ones the threshold is among,
+    int need = nkeep;                            // the need-th largest of them
+    bool listed = false;
+    const int own = kBins / CL;
+    const int per = (n + kSelThreads - 1) / kSelThreads;
+    for (int round = 0;; ++round) {
+        const int sh = lim >> 11 ? 21 - __clz(lim) : 0;            // lim >> sh < 2048
+        // A thread takes a run of consecutive keys and adds equal neighbouring bins as one count: the max-pool leaves
+        // plateaus, so a few additions per thread replace one per key.
+        {
             const int e0 = min(tid * per, n), e1 = min(e0 + per, n);
-            uint32_t cur = 0xffffffffu, cnt = 0;
-            int pos = per ? tid % per : 0;                      // rotated start: neighbouring threads hit different banks
+            uint32_t cur = 0u, cnt = 0u;
+            int pos = per ? tid % per : 0;                          // rotated start: neighbouring threads hit different banks
             for (int i = 0; i < per; ++i) {
                 const int e = e0 + pos;
                 if (++pos == per) pos = 0;
-                if (e >= e1) continue;
-                if (!JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 14)) continue;
-                const uint32_t k = mykeys[e];
-                const bool live = (round == 0) || ((k >> (shift + width)) == prefix);
-                const uint32_t digit = live ? ((k >> shift) & mask) : 0xffffffffu;
-                if (digit != cur) {
-                    if (cnt && cur != 0xffffffffu) atomicAdd(&hist[cur], cnt);
-                    cur = digit; cnt = 0;
-                }
+                if (e >= e1 || !JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 14)) continue;
+                const uint32_t k = mykeys[e] - lo;
+                if (k > lim) continue;
+                if (k >> sh != cur) { if (cnt && JQ_IN(cur, kBins, kDbgSelect, 9)) atomicAdd(&hist[cur], cnt); cur = k >> sh; cnt = 0; }
                 ++cnt;
             }
-            if (cnt && cur != 0xffffffffu) atomicAdd(&hist[cur], cnt);
+            if (cnt && JQ_IN(cur, kBins, kDbgSelect, 9)) atomicAdd(&hist[cur], cnt);
         }
         __syncthreads();
-        uint32_t *g0 = cluster.map_shared_rank(ghist, 0);
-        for (int i = tid; i < kBins; i += kSelThreads) {
-            const uint32_t v = hist[i];
-            if (v) atomicAdd(&g0[i], v);
+        // CTA q owns the bins [q * own, (q + 1) * own): every CTA adds its counts there (starting at its own, so that they do
+        // not all meet at one), then everybody reads the sums back and finds the bin for itself.
+        // (At most three rounds: 32 bits of range, 11 bits each.)
+        uint32_t *const sums = ghist + round * own;
+        {
+            const int at = (4 * tid + rank * own) & (kBins - 1);     // this thread's four bins
+            const uint4 v = *(const uint4 *)(hist + at);
+            *(uint4 *)(hist + at) = make_uint4(0u, 0u, 0u, 0u);     // for the next round
+            // (two bins per 64-bit addition: a bin's sum stays below 2^32, so nothing carries from one to the other)
+            unsigned long long *const g = (unsigned long long *)(cluster.map_shared_rank(sums, at / own) + at % own);
+            if (v.x | v.y) atomicAdd(g, (unsigned long long)v.y << 32 | v.x);
+            if (v.z | v.w) atomicAdd(g + 1, (unsigned long long)v.w << 32 | v.z);
         }
         cluster.sync();
-        if (rank == 0) {
-            find_digit(ghist, ctl.krem, ctl);
-            if (tid < CL) {
-                SelCtl *rc = cluster.map_shared_rank(&ctl, tid);
-                rc->prefix = (prefix << width) | (uint32_t)ctl.found_prefix_digit;
-                rc->krem = ctl.found_krem;
-                rc->cand_total = ctl.found_count;
-            }
-            for (int i = tid; i < kBins; i += kSelThreads) ghist[i] = 0;   // for the next round, before anybody adds to it
-        }
-        cluster.sync();
-        if (round == 0 && ctl.cand_total <= kCandMax) {
-            // The keys with the winning first digit go to the leading CTA (order does not matter: only
-            // their values decide the threshold), which finishes the selection on them alone.
-            const uint32_t d0 = ctl.prefix;
-            uint32_t *cand = (uint32_t *)cluster.map_shared_rank(raw, 0);
-            int *cand_count = &cluster.map_shared_rank(&ctl, 0)->cand_count;
-            for (int base = 0; base < n_up; base += kSelThreads) {
-                const int e = base + tid;
-                const uint32_t k = (e < n && JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 19)) ? mykeys[e] : 0u;
-                const bool hit = e < n && (k >> 21) == d0;
-                const uint32_t votes = __ballot_sync(0xffffffffu, hit);
-                if (votes) {
-                    int at = 0;
-                    if (lane == 0) at = atomicAdd(cand_count, __popc(votes));
-                    at = __shfl_sync(0xffffffffu, at, 0);
-                    if (hit && JQ_IN(at + __popc(votes & ((1u << lane) - 1u)), raw_cap, kDbgSelect, 15)) cand[at + __popc(votes & ((1u << lane) - 1u))] = k;
-                }
-            }
-            cluster.sync();
-            if (rank == 0) {
-                const int nc = ctl.cand_total;
-                const uint32_t *mine = (const uint32_t *)raw;
-                uint32_t pre = d0;
-                for (int r2 = 1; r2 < 3; ++r2) {
-                    const int sh = (r2 == 1) ? 10 : 0, wd = (r2 == 2) ? 10 : 11;
-                    for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
-                    __syncthreads();
-                    for (int e = tid; e < nc; e += kSelThreads) {
-                        const uint32_t k = mine[e];
-                        if ((k >> (sh + wd)) == pre && JQ_IN((k >> sh) & ((1u << wd) - 1u), kBins, kDbgSelect, 16)) atomicAdd(&hist[(k >> sh) & ((1u << wd) - 1u)], 1u);
-                    }
-                    __syncthreads();
-                    find_digit(hist, ctl.krem, ctl);
-                    pre = (pre << wd) | (uint32_t)ctl.found_prefix_digit;
-                    if (tid == 0) ctl.krem = ctl.found_krem;
-                    __syncthreads();
-                }
-                if (tid < CL) {
-                    SelCtl *rc = cluster.map_shared_rank(&ctl, tid);
-                    rc->prefix = pre;
-                    rc->krem = ctl.found_krem;
-                }
-            }
-            cluster.sync();
-            break;
-        }
-    }
-    const uint32_t tau = ctl.prefix;
-    const int need_eq = ctl.krem;   // how many of the keys == tau are kept (lowest positions first)
-
-    // ---- 3. ordered compaction; warp w owns the contiguous elements [w*seg, (w+1)*seg)
-    const int seg = ((n + 31) / 32 + 31) / 32 * 32;
-    const int w0 = min(wid * seg, n), w1 = min(w0 + seg, n);
-    int cgt = 0, ceq = 0;
-    for (int base = w0; base < w1; base += 32) {
-        const int e = base + lane;
-        const uint32_t k = (e < w1 && JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 20)) ? mykeys[e] : 0u;
-        const bool in = e < w1;
-        cgt += __popc(__ballot_sync(0xffffffffu, in && k > tau));
-        ceq += __popc(__ballot_sync(0xffffffffu, in && k == tau));
-    }
-    if (lane == 0) { ctl.warp_gt[wid] = cgt; ctl.warp_eq[wid] = ceq; }
-    __syncthreads();
-    if (wid == 0) {
-        const int g = ctl.warp_gt[lane], q = ctl.warp_eq[lane];
-        int gi = g, qi = q;
+        {
+            const int at = kBins - 4 - 4 * tid;                      // from the top
+            const uint4 v = *(const uint4 *)(cluster.map_shared_rank(sums, at / own) + at % own);
+            const int c[4] = {(int)v.w, (int)v.z, (int)v.y, (int)v.x};
+            int inc = c[0] + c[1] + c[2] + c[3];
+            const int mine = inc;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int a = __shfl_up_sync(0xffffffffu, gi, o), b = __shfl_up_sync(0xffffffffu, qi, o);
-            if (lane >= o) { gi += a; qi += b; }
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += x;
+            }
+            if (lane == 31) ctl.scan[wid] = inc;
+            __syncthreads();
+            int above = __reduce_add_sync(0xffffffffu, lane < wid ? ctl.scan[lane] : 0) + inc - mine;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (above < need && need <= above + c[i]) { ctl.digit = at + 3 - i; ctl.krem = need - above; ctl.count = c[i]; }
+                above += c[i];
+            }
+            __syncthreads();
         }
-        ctl.warp_gt[lane] = gi - g; ctl.warp_eq[lane] = qi - q;   // exclusive
-        if (lane == 31) { ctl.tot_gt = gi; ctl.tot_eq = qi; }
+        lo += (uint32_t)ctl.digit << sh;
+        need = ctl.krem;
+        lim = (1u << sh) - 1u;
+        listed = ctl.count <= kCandMax;
+        if (listed || sh == 0) break;
     }
-    __syncthreads();
-    if (tid < CL) {
-        SelCtl *rc = cluster.map_shared_rank(&ctl, tid);
-        rc->counts_gt[rank] = ctl.tot_gt;
-        rc->counts_eq[rank] = ctl.tot_eq;
+    // Warp w owns the contiguous elements [w0, w1).  Keys above the bin (listed) or above / equal to the threshold are
+    // counted per warp; the bin's own keys go to the leading CTA's list.
+    const int nc = listed ? ctl.count : 0;
+    const int seg = ((n + kSelWarps - 1) / kSelWarps + 31) / 32 * 32;
+    const int w0 = min(wid * seg, n), w1 = min(w0 + seg, n);
+    const uint32_t top = lo + lim;
+    SelCtl *lead = cluster.map_shared_rank(&ctl, 0);
+    {
+        int cgt = 0, ceq = 0;
+        for (int base = w0; base < w1; base += 32) {
+            const int e = base + lane;
+            const bool in = e < w1 && JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 19);
+            const uint32_t k = in ? mykeys[e] : 0u;
+            cgt += in && k > top;
+            const bool hit = in && k >= lo && k <= top;
+            ceq += hit;
+            if (!listed) continue;
+            const uint32_t votes = __ballot_sync(0xffffffffu, hit);
+            if (votes) {
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&lead->cand_count, __popc(votes));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(votes & ((1u << lane) - 1u));
+                if (hit && JQ_IN(at, kCandMax, kDbgSelect, 15)) { lead->cand_key[at] = k; lead->cand_pos[at] = j0 + e; }
+            }
+        }
+        cgt = __reduce_add_sync(0xffffffffu, cgt);
+        ceq = __reduce_add_sync(0xffffffffu, ceq);
+        if (lane == 0) { ctl.warp_gt[wid] = cgt; ctl.warp_eq[wid] = listed ? 0 : ceq; }
+        __syncthreads();
+        if (wid == 0) {
+            const int g = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? ctl.warp_gt[lane] : 0), q = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? ctl.warp_eq[lane] : 0);
+            if (lane < CL) {
+                SelCtl *rc = cluster.map_shared_rank(&ctl, lane);
+                rc->gt_of[rank] = g; rc->eq_of[rank] = q;
+            }
+        }
+        if (tid == 0) { ctl.base_gt = ctl.base_eq = 0; }
+        cluster.sync();
     }
-    cluster.sync();
-    int gt_before = ctl.warp_gt[wid], eq_before = ctl.warp_eq[wid];
-    for (int q = 0; q < rank; ++q) { gt_before += ctl.counts_gt[q]; eq_before += ctl.counts_eq[q]; }
+    uint32_t tau = lo;
+    int need_eq = need;             // how many of the keys == tau are kept (lowest positions first)
+    if (listed) {
+        if (tid < nc) { ctl.my_key[tid] = lead->cand_key[tid]; ctl.my_pos[tid] = lead->cand_pos[tid]; }
+        __syncthreads();
+        if (tid < nc) {
+            const uint32_t k = ctl.my_key[tid];
+            int gt = 0, eq = 0;
+#pragma unroll 4
+            for (int i = 0; i < nc; ++i) { const uint32_t x = ctl.my_key[i]; gt += x > k; eq += x == k; }
+            if (gt < need && need <= gt + eq) { ctl.tau = k; ctl.need_eq = need - gt; }   // (equal keys write the same)
+        }
+        __syncthreads();
+        tau = ctl.tau;
+        need_eq = ctl.need_eq;
+        if (tid < nc) {
+            const uint32_t k = ctl.my_key[tid];
+            const int at = ctl.my_pos[tid];
+            if (k >= tau && at < j0) atomicAdd(k > tau ? &ctl.base_gt : &ctl.base_eq, 1);
+            else if (k >= tau && at < j1) {
+                const int w = (at - j0) / seg;
+                if (JQ_IN(w, kSelWarps, kDbgSelect, 16)) atomicAdd(k > tau ? &ctl.warp_gt[w] : &ctl.warp_eq[w], 1);
+            }
+        }
+        __syncthreads();
+    }
+    int gt_before = ctl.base_gt, eq_before = ctl.base_eq;
+    for (int q = 0; q < rank; ++q) { gt_before += ctl.gt_of[q]; eq_before += ctl.eq_of[q]; }
+    gt_before += __reduce_add_sync(0xffffffffu, lane < wid ? ctl.warp_gt[lane] : 0);
+    eq_before += __reduce_add_sync(0xffffffffu, lane < wid ? ctl.warp_eq[lane] : 0);
+
+    // ---- 3. ordered compaction
     const uint32_t lt_mask = (1u << lane) - 1u;
-    for (int base = w0; base < w1; base += 32) {
-        const int e = base + lane;
-        const bool in = e < w1;
-        const uint32_t k = (in && JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 21)) ? mykeys[e] : 0u;
-        const uint32_t bg = __ballot_sync(0xffffffffu, in && k > tau);
-        const uint32_t be = __ballot_sync(0xffffffffu, in && k == tau);
-        const int g_here = gt_before + __popc(bg & lt_mask), e_here = eq_before + __popc(be & lt_mask);
-        if (in) {
-            if (k > tau) { if (JQ_IN(g_here + min(e_here, need_eq), nkeep, kDbgSelect, 17)) out[g_here + min(e_here, need_eq)] = j0 + e; }
-            else if (k == tau && e_here < need_eq) { if (JQ_IN(g_here + e_here, nkeep, kDbgSelect, 18)) out[g_here + e_here] = j0 + e; }
+    if (ctl.warp_gt[wid] | ctl.warp_eq[wid])
+        for (int base = w0; base < w1; base += 32) {
+            const int e = base + lane;
+            const bool in = e < w1 && JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 21);
+            const uint32_t k = in ? mykeys[e] : 0u;
+            const uint32_t bg = __ballot_sync(0xffffffffu, in && k > tau);
+            const uint32_t be = __ballot_sync(0xffffffffu, in && k == tau);
+            if (!(bg | be)) continue;
+            const int g_here = gt_before + __popc(bg & lt_mask), e_here = eq_before + __popc(be & lt_mask);
+            if (in) {
+                if (k > tau) { if (JQ_IN(g_here + min(e_here, need_eq), nkeep, kDbgSelect, 17)) out[g_here + min(e_here, need_eq)] = j0 + e; }
+                else if (k == tau && e_here < need_eq) { if (JQ_IN(g_here + e_here, nkeep, kDbgSelect, 18)) out[g_here + e_here] = j0 + e; }
+            }
+            gt_before += __popc(bg);
+            eq_before += __popc(be);
         }
-        gt_before += __popc(bg);
-        eq_before += __popc(be);
-    }
-    if (Kin) copy_kept_rows<CL>(cluster, out, kv_in, krow, L, nkeep, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+    // ---- 4. the rows, once every index of the head has been written.  (Without rows the cluster still leaves together: the
+    // leading CTA's list may be being read.)
+    cluster.sync();                 // (release and acquire at cluster scope: the readers are in the cluster)
+    if (!Kin) return;
+    copy_rows(out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+    if (win.w) copy_window(win, kv, krow + nkeep, rank * ngrp + (tid >> 4), CL * ngrp, Kout, Vout, ext JQ_DBG_ARG_DEV);
 }
 
 // ------------------------------------------------------------------ many heads: one CTA per head, no cluster
@@ -502,50 +531,6 @@ __device__ __forceinline__ uint32_t quad_bound_key(const float4 *buf, int at)
     return order_key(m);
 }
 
-// Block-wide exclusive scan of one int per thread, any number of whole warps.
-__device__ __forceinline__ int cta_excl_scan(int v, int *warp_sums)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += n;
-    }
-    if (lane == 31) warp_sums[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        const int ws = lane < nw ? warp_sums[lane] : 0;
-        int winc = ws;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int n = __shfl_up_sync(0xffffffffu, winc, o);
-            if (lane >= o) winc += n;
-        }
-        if (lane < nw) warp_sums[lane] = winc - ws;
-    }
-    __syncthreads();
-    const int excl = warp_sums[wid] + inc - v;
-    __syncthreads();
-    return excl;
-}
-
-// All threads of a CTA of 512 or 1024: the bin of h[kBins] that holds the krem-th key counted from the top.
-__device__ __forceinline__ void find_digit_cta(const uint32_t *h, int krem, StrCtl &ctl)
-{
-    const int per = kBins / (int)blockDim.x;                  // 4 or 2 bins per thread, descending
-    const int hi = kBins - 1 - per * (int)threadIdx.x;
-    int tot = 0;
-    for (int i = 0; i < per; ++i) tot += (int)h[hi - i];
-    int above = cta_excl_scan(tot, ctl.scan);
-    for (int i = 0; i < per; ++i) {
-        const int c = (int)h[hi - i];
-        if (above < krem && krem <= above + c) { ctl.digit = hi - i; ctl.krem = krem - above; ctl.count = c; }
-        above += c;
-    }
-    __syncthreads();
-}
-
 // Adds the digits of a thread's (up to) four neighbouring keys to the histogram: runs of equal digits as one count (the
 // max-pool leaves plateaus); digit 0xffffffff marks a key that does not take part.
 __device__ __forceinline__ void hist_add_runs(uint32_t *hist, const uint32_t (&digit)[4], int nval JQ_DBG_PARAM)
@@ -573,7 +558,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
               float *__restrict__ pooled, const uint4 *__restrict__ Kin, const uint4 *__restrict__ Vin,
               uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, const HeadRec *__restrict__ htab,
               const uint4 *const *__restrict__ Ktab, const uint4 *const *__restrict__ Vtab, int src_rows, int out_rows,
-              const SelExtents ext JQ_DBG_PARAM)
+              const WindowRows win, const SelExtents ext JQ_DBG_PARAM)
 {
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ uint32_t hist[kBins];
@@ -778,101 +763,103 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     }
     if (!Kin) return;
 
-    // ---- the kept rows (256 bytes each: 16 lanes x 16 bytes), four rows in flight per 16 lanes
+    // ---- the kept rows
     __syncthreads();
-    const int lane16 = tid & 15, grp = tid >> 4, ngrp = T >> 4;
-    for (int t0 = 4 * grp; t0 < nkeep; t0 += 4 * ngrp) {
-        int j[4];
-        uint4 a[4], b[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) j[r] = t0 + r < nkeep ? min(max(__ldcg(out + t0 + r), 0), L - 1) : 0;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const size_t src = ((size_t)kv_in * src_rows + j[r]) * 16 + lane16;
-            const bool in = t0 + r < nkeep && JQ_IN((long long)kv_in * src_rows + j[r], ext.src_heads * src_rows, kDbgSelect, 30);
-            a[r] = in ? Kin[src] : make_uint4(0u, 0u, 0u, 0u);
-            b[r] = in ? Vin[src] : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const size_t dst = (size_t)(krow + t0 + r) * 16 + lane16;
-            if (t0 + r < nkeep && JQ_IN(krow + t0 + r, ext.out_rows, kDbgSelect, 31)) { Kout[dst] = a[r]; Vout[dst] = b[r]; }
-        }
-    }
+    copy_rows(out, 0, nkeep, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+    if (win.w) copy_window(win, kv, krow + nkeep, tid >> 4, T >> 4, Kout, Vout, ext JQ_DBG_ARG_DEV);
 }
 
 // Shared memory of a CTA whose cluster has `cl` CTAs, the share of the head it holds, and whether its keys stay on chip.
 struct SelPlan { int cl, chunk, in_smem, raw_tile; size_t smem; };
 
-// small_stage: stage the scores in pieces of kCandMax (the least the buffer must hold) instead of a CTA's whole
-// share, so that two CTAs fit on an SM; worth it when the call has more heads than clusters fit at a time.
-SelPlan plan_for(int L, int cl, bool small_stage)
+SelPlan plan_for(int L, int cl)
 {
     SelPlan p;
     p.cl = cl;
     p.chunk = ((L + cl - 1) / cl + 31) / 32 * 32;
     p.in_smem = p.chunk <= kKeysSmemMax;
-    // the staging buffer holds a CTA's share of the scores (at most kRawTile) and later up to kCandMax candidates
     p.raw_tile = p.chunk < kRawTile ? p.chunk : kRawTile;
-    if (small_stage && p.in_smem) p.raw_tile = kCandMax;
-    if (p.raw_tile < kCandMax) p.raw_tile = kCandMax;
-    p.smem = (size_t)(2 * kBins + p.raw_tile + 2 * kHalo) * 4 + (p.in_smem ? (size_t)p.chunk * 4 : 0);
+    p.smem = (size_t)(kOwnBins + kBins + p.raw_tile + 2 * kHalo) * 4 + (p.in_smem ? (size_t)p.chunk * 4 : 0);
     return p;
 }
 
-// Cluster size for Hkv heads of L keys.  The kernel is a chain of short phases between cluster barriers
-// (about 20 k cycles of them) plus work in proportion to a CTA's share (about 1.7 cycles per key); few heads
-// want the largest cluster (shortest chain per head), many heads want smaller ones (more heads at a time,
-// and the chain is paid once per head either way).  Estimated as rounds of resident clusters times the
-// time of one.
-SelPlan choose_plan(int Hkv, int L, int sms)
+cudaLaunchConfig_t sel_config(const SelPlan &p, int heads, cudaLaunchAttribute (&attr)[2], cudaStream_t st)
 {
-    const bool many = Hkv > sms / kClMax;        // more heads than 8-CTA clusters fit at one CTA per SM
-    SelPlan best = plan_for(L, kClMax, many);
-    double best_cost = 0;
-    for (int cl = kClMax; cl >= 2; cl >>= 1) {
-        const SelPlan p = plan_for(L, cl, many);
-        if (cl != kClMax && !p.in_smem) break;
-        const int per_sm = p.smem <= 112 * 1024 + 512 ? 2 : 1;
-        const int resident = sms * per_sm / cl > 0 ? sms * per_sm / cl : 1;
-        const double cost = (double)((Hkv + resident - 1) / resident) * (20000.0 + 1.7 * p.chunk);
-        if (cl == kClMax || cost < best_cost) { best = p; best_cost = cost; }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(heads * p.cl));
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)p.cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    // Launched with programmatic stream serialisation: the CTAs may be set up while the kernel before it in the stream (the
+    // scoring kernel) drains; the kernel waits for that kernel's memory before reading anything.
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// Clusters of 2, 4, 8, 16 CTAs resident at a time, with two CTAs per SM (up to 100 KB of shared memory each) and with one.
+struct SelDevice { int resident[4][2] = {}; bool ready = false; };
+bool sel_device(SelDevice *out)
+{
+    static SelDevice devs[64];
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    SelDevice &d = devs[dev];
+    if (!d.ready) {
+        const int max_smem = (kOwnBins + kBins + kRawTile + 2 * kHalo + kKeysSmemMax) * 4;
+        if (cudaFuncSetAttribute(select_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) return false;
+        if (cudaFuncSetAttribute(select_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+        for (int i = 0; i < 4; ++i)
+            for (int x = 0; x < 2; ++x) {
+                SelPlan p = plan_for(1, 2 << i);
+                p.smem = x == 0 ? kSelTwoPerSm : (size_t)max_smem;
+                cudaLaunchAttribute attr[2];
+                const cudaLaunchConfig_t cfg = sel_config(p, 1, attr, nullptr);
+                if (cudaOccupancyMaxActiveClusters(&d.resident[i][x], select_cluster, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[i][x] = 0; }
+            }
+        if (d.resident[0][0] < 1 || d.resident[0][1] < 1) return false;
+        d.ready = true;
+    }
+    *out = d;
+    return true;
+}
+
+// Cluster size for Hkv heads of L keys: the least estimated time, rounds of resident clusters times the time of one.  That is
+// a chain of phases between cluster barriers, longer in a cluster of 16, plus work in proportion to a CTA's share.  Measured
+// for 8 heads with 2, 4, 8, 16 CTAs: 12.3, 9.8, 8.8, 10.3 us for 12000 keys, -, -, 19.8, 16.8 for 131072.
+SelPlan choose_plan(int Hkv, int L, const SelDevice &dev)
+{
+    SelPlan best = plan_for(L, 8);
+    double best_cost = 1e300;
+    for (int i = 3; i >= 0; --i) {
+        const SelPlan p = plan_for(L, 2 << i);
+        const int resident = dev.resident[i][p.smem <= kSelTwoPerSm ? 0 : 1];
+        if (resident < 1 || (!p.in_smem && best_cost < 1e300)) continue;
+        const double cost = (double)((Hkv + resident - 1) / resident) * ((p.cl == 16 ? kSelChain16 : kSelChain) + kSelPerKey * p.chunk);
+        if (cost < best_cost) { best = p; best_cost = cost; }
     }
     return best;
 }
 
-template <int CL>
-jq_status launch_select_cl(const SelPlan &p, const float *scores, const jq_shape &s, int nkeep, int32_t *idx, float *pooled,
-                           const Workspace &w, cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout, int dev,
-                           const UnitTables *tables, int src_rows, int out_rows)
+jq_status launch_select_cluster(const float *scores, const jq_shape &s, int nkeep, int Lmax, int32_t *idx, float *pooled,
+                                const Workspace &w, cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout,
+                                const UnitTables *tables, int src_rows, int out_rows, const WindowRows &win, const SelExtents &ext)
 {
-    static bool attr_done[64] = {};
-    if (!attr_done[dev]) {
-        const int max_smem = (2 * kBins + kRawTile + 2 * kHalo + kKeysSmemMax) * 4;
-        if (cudaFuncSetAttribute(select_cluster<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess)
-            return JQ_ERR_CUDA;
-        attr_done[dev] = true;
-    }
-    SelExtents ext;
-    ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
-    ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * out_rows;
-    ext.src_heads = tables ? tables->hpu : s.Hkv;
-    // Launched with programmatic stream serialisation: the CTAs may be set up while the kernel before it in
-    // the stream (the scoring kernel) drains; the kernel waits for that kernel's memory before reading anything.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(s.Hkv * CL));
-    cfg.blockDim = dim3(kSelThreads);
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, select_cluster<CL>, scores, s.L, nkeep, (s.pool - 1) / 2, idx, pooled, w.keys, p.chunk,
+    SelDevice dev;
+    if (!sel_device(&dev)) return JQ_ERR_CUDA;
+    const SelPlan p = choose_plan(s.Hkv, Lmax, dev);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = sel_config(p, s.Hkv, attr, st);
+    if (cudaLaunchKernelEx(&cfg, select_cluster, scores, s.L, nkeep, (s.pool - 1) / 2, idx, pooled, w.keys, p.chunk,
                            p.in_smem, p.raw_tile, (const uint4 *)K, (const uint4 *)V, (uint4 *)Kout, (uint4 *)Vout,
                            tables ? tables->heads : nullptr, (const uint4 *const *)(tables && Kout ? tables->K : nullptr),
-                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, ext JQ_DBG_ARG) != cudaSuccess) {
+                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, win, ext JQ_DBG_ARG) != cudaSuccess) {
         cudaGetLastError();
         return JQ_ERR_CUDA;
     }
@@ -884,7 +871,7 @@ jq_status launch_select_cl(const SelPlan &p, const float *scores, const jq_shape
 // when the scores of the heads that 512 would hold in flight (a head is read three times) are far more than the L2.
 jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep, int Lmax, int32_t *idx, float *pooled,
                                cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout, int sms, int dev,
-                               const UnitTables *tables, int src_rows, int out_rows)
+                               const UnitTables *tables, int src_rows, int out_rows, const WindowRows &win, const SelExtents &ext)
 {
     const long long resident = (long long)sms * stream_ctas_per_sm(512), inflight = s.Hkv < resident ? s.Hkv : resident;
     const int threads = inflight * Lmax * 4 <= (96ll << 20) ? 512 : 1024;
@@ -897,10 +884,6 @@ jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return JQ_ERR_CUDA;
         attr_done[dev][which] = true;
     }
-    SelExtents ext;
-    ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
-    ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * out_rows;
-    ext.src_heads = tables ? tables->hpu : s.Hkv;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)s.Hkv);
     cfg.blockDim = dim3((unsigned)threads);
@@ -914,7 +897,7 @@ jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep
     if (cudaLaunchKernelEx(&cfg, kernel, scores, s.L, nkeep, (s.pool - 1) / 2, idx, pooled, (const uint4 *)K,
                            (const uint4 *)V, (uint4 *)Kout, (uint4 *)Vout, tables ? tables->heads : nullptr,
                            (const uint4 *const *)(tables && Kout ? tables->K : nullptr),
-                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, ext JQ_DBG_ARG) != cudaSuccess) {
+                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, win, ext JQ_DBG_ARG) != cudaSuccess) {
         cudaGetLastError();
         return JQ_ERR_CUDA;
     }
@@ -926,26 +909,26 @@ jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep
 
 jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, float *pooled,
                         const Workspace &w, cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout,
-                        const UnitTables *tables, int src_head_rows, int out_head_rows)
+                        const UnitTables *tables, int src_head_rows, int out_head_rows, const void *Kwin, const void *Vwin)
 {
     const int src_rows = src_head_rows > s.L ? src_head_rows : s.L;
     // with tables: the plan and the shared memory follow the longest head; every head reads its own record
     const int Lmax = tables ? tables->max_L : s.L;
     const int nkeep = s.budget < Lmax ? s.budget : Lmax;
-    static int sms[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return JQ_ERR_CUDA;
-    if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return JQ_ERR_CUDA;
+    const int out_rows = out_head_rows > nkeep ? out_head_rows : nkeep;
+    const WindowRows win = {(const uint4 *)Kwin, (const uint4 *)Vwin, Vwin ? s.w : 0};
+    SelExtents ext;
+    ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
+    ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * out_rows;
+    ext.src_heads = tables ? tables->hpu : s.Hkv;
     // many heads and a window the quad pooling covers: one CTA per head
-    if (s.Hkv >= kStreamMinHeads && (s.pool - 1) / 2 <= 4)
-        return launch_select_stream(scores, s, nkeep, Lmax, idx, pooled, st, K, V, Kout, Vout, sms[dev], dev, tables, src_rows,
-                                    out_head_rows > nkeep ? out_head_rows : nkeep);
-    const SelPlan p = choose_plan(s.Hkv, Lmax, sms[dev]);
-    switch (p.cl) {
-    case 2: return launch_select_cl<2>(p, scores, s, nkeep, idx, pooled, w, st, K, V, Kout, Vout, dev, tables, src_rows, out_head_rows > nkeep ? out_head_rows : nkeep);
-    case 4: return launch_select_cl<4>(p, scores, s, nkeep, idx, pooled, w, st, K, V, Kout, Vout, dev, tables, src_rows, out_head_rows > nkeep ? out_head_rows : nkeep);
-    default: return launch_select_cl<8>(p, scores, s, nkeep, idx, pooled, w, st, K, V, Kout, Vout, dev, tables, src_rows, out_head_rows > nkeep ? out_head_rows : nkeep);
+    if (s.Hkv >= kStreamMinHeads && (s.pool - 1) / 2 <= 4) {
+        const int sms = device_sms();
+        int dev = 0;
+        if (sms < 1 || cudaGetDevice(&dev) != cudaSuccess) return JQ_ERR_CUDA;
+        return launch_select_stream(scores, s, nkeep, Lmax, idx, pooled, st, K, V, Kout, Vout, sms, dev, tables, src_rows, out_rows, win, ext);
     }
+    return launch_select_cluster(scores, s, nkeep, Lmax, idx, pooled, w, st, K, V, Kout, Vout, tables, src_rows, out_rows, win, ext);
 }
 
 }  // namespace jq
