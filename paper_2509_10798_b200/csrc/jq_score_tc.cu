@@ -375,7 +375,7 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
             for (int g = 0; g < P.ngroups; ++g) {
                 int ok = 1;
                 // this CTA's epilogue warps first (their partial stores happen-before the arrival), then the grid
-                ok = mbar_wait(&ctl->p1_done[g & 3], (g >> 2) & 1, ctl, P.status, kSleepLong) ? 1 : 0;
+                ok = mbar_wait(&ctl->p1_done[g & 3], (g >> 2) & 1, ctl, P.status, P.ngroups <= 2 ? kSleepShort : kSleepLong) ? 1 : 0;   // (with one group nothing hides the merge)
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lane == 0) {
@@ -411,21 +411,23 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
 #pragma unroll 1
                     for (int i0 = sub; i0 < nsl; i0 += lpr * kMergeLoads) {
                         float2 p[kMergeLoads];
+                        const float2 *at = src + (size_t)i0 * R;
 #pragma unroll
                         for (int k = 0; k < kMergeLoads; ++k) {
                             const int i = i0 + lpr * k;
                             p[k] = make_float2(-INFINITY, 0.f);
                             // (a CTA between b_lo and b_hi always has a tile of this head unless the group has fewer tiles than CTAs)
                             if (i < nsl && (T >= Gu || cta_has_tile(b_lo + i / kGroups, T, Gu)))
-                                if (JQ_IN(((long long)kv * kSlots + kGroups * b_lo + i) * P.R + r, n_part, kDbgScore, 5)) p[k] = __ldcg(src + (size_t)i * P.R);
+                                if (JQ_IN(((long long)kv * kSlots + kGroups * b_lo + i) * P.R + r, n_part, kDbgScore, 5)) p[k] = __ldcg(at + lpr * k * R);
                         }
+                        // (an empty partial is (-inf, 0) and adds nothing; the reference is finite once any key has been seen)
                         float mn = m;
 #pragma unroll
-                        for (int k = 0; k < kMergeLoads; ++k) if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
+                        for (int k = 0; k < kMergeLoads; ++k) mn = fmaxf(mn, p[k].x);
                         if (mn > -INFINITY) {
-                            float acc = (l > 0.f) ? l * ex2(c * (m - mn)) : 0.f;
+                            float acc = l * ex2(c * (m - mn));
 #pragma unroll
-                            for (int k = 0; k < kMergeLoads; ++k) if (p[k].y > 0.f) acc += p[k].y * ex2(c * (p[k].x - mn));
+                            for (int k = 0; k < kMergeLoads; ++k) acc = fmaf(p[k].y, ex2(c * (p[k].x - mn)), acc);
                             m = mn; l = acc;
                         }
                     }
@@ -480,8 +482,14 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
                     ok = mbar_wait(&ctl->ms_empty[buf], ((hs >> 1) & 1) ^ 1, ctl, status, kSleepLong) ? 1 : 0;
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
-                    for (int r = lane; r < kMaxR; r += 32)   // stored negated: x = c s + (-M_r); -inf silences a padding column
-                        ctl->Ms[buf][r] = (r < P.R && JQ_IN((long long)kv * P.R + r, (long long)P.Hkv * P.R, kDbgScore, 8)) ? -__ldcg(&P.Mrow[(size_t)kv * P.R + r]) : -INFINITY;
+                    float M[kMaxR / 32];                     // all loads in flight at once
+#pragma unroll
+                    for (int x = 0; x < kMaxR / 32; ++x) {
+                        const int r = 32 * x + lane;
+                        M[x] = r < R && JQ_IN((long long)kv * R + r, (long long)P.Hkv * R, kDbgScore, 8) ? __ldcg(&P.Mrow[(size_t)kv * R + r]) : INFINITY;
+                    }
+#pragma unroll
+                    for (int x = 0; x < kMaxR / 32; ++x) ctl->Ms[buf][32 * x + lane] = -M[x];   // stored negated: x = c s + (-M_r); -inf silences a padding column
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->ms_full[buf], 1);
                     ++hs;
