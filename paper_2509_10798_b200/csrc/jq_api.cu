@@ -391,6 +391,44 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     return JQ_OK;
 }
 
+namespace {
+
+constexpr int kHostChunks = 4;                 // most chunks of a call
+constexpr size_t kHostChunkBytes = 8u << 20;   // least keys of a chunk of heads
+constexpr size_t kHostIdxPad = 256;
+static_assert(kHostChunks * 4 * sizeof(int32_t) + 16 <= kHostIdxPad, "room for the chunks' alignment");
+
+// The stream beside the caller's and the events between the two: one set per host thread and device, made at the first call
+// that uses it and released with the thread.  Calls of one thread on several streams share it (their side work then runs in
+// the order of the calls).
+struct HostPipe {
+    cudaStream_t side = nullptr;
+    cudaEvent_t in = nullptr, out = nullptr;
+    ~HostPipe()
+    {
+        if (in) cudaEventDestroy(in);
+        if (out) cudaEventDestroy(out);
+        if (side) cudaStreamDestroy(side);
+    }
+};
+
+HostPipe *host_pipe()
+{
+    static thread_local HostPipe pipes[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    HostPipe &p = pipes[dev];
+    if ((!p.side && cudaStreamCreateWithFlags(&p.side, cudaStreamNonBlocking) != cudaSuccess) ||
+        (!p.in && cudaEventCreateWithFlags(&p.in, cudaEventDisableTiming) != cudaSuccess) ||
+        (!p.out && cudaEventCreateWithFlags(&p.out, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaGetLastError();
+        return nullptr;   // the call then runs on the caller's stream alone
+    }
+    return &p;
+}
+
+}  // namespace
+
 size_t jq_host_call_bytes(const jq_shape *s)
 {
     if (check_shape(s) != JQ_OK) return 0;
@@ -400,7 +438,7 @@ size_t jq_host_call_bytes(const jq_shape *s)
     b += 2 * align_up((size_t)s->Hkv * s->L * row, 256);      // K, V
     b += align_up((size_t)s->Hq * s->w * row, 256);           // Qwin
     b += 2 * align_up((size_t)s->Hkv * nkeep * row, 256);     // Kout, Vout
-    b += align_up((size_t)s->Hkv * nkeep * 4, 256);           // kept_idx
+    b += align_up((size_t)s->Hkv * nkeep * 4, 256) + kHostIdxPad;   // kept_idx, with room to align every chunk's
     b += carve(nullptr, *s).bytes;
     return b;
 }
@@ -425,29 +463,63 @@ jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin,
     char *dQ = p;          p += align_up(qb, 256);
     char *dKo = p;         p += align_up(ob, 256);
     char *dVo = p;         p += align_up(ob, 256);
-    char *dI = p;          p += align_up(ib, 256);
+    char *dI = p;          p += align_up(ib, 256) + kHostIdxPad;
     char *ws = p;
     const size_t wsb = carve(nullptr, *s).bytes;
     if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return JQ_ERR_CUDA;
     if (cudaMemcpyAsync(dQ, hQwin, qb, cudaMemcpyHostToDevice, st) != cudaSuccess) return JQ_ERR_CUDA;
-    if (cudaMemcpyAsync(dK, hK, kvb, cudaMemcpyHostToDevice, st) != cudaSuccess) return JQ_ERR_CUDA;
     // V is read at the kept rows only.  A page-locked host buffer is mapped into the device's address space: the
     // selection kernel then fetches those rows from it directly and the copy of all of V is skipped.
-    const void *v_src = dV;
+    const char *v_src = dV;
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, hV) == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer &&
         !((uintptr_t)pa.devicePointer & 15u)) {
-        v_src = pa.devicePointer;
+        v_src = (const char *)pa.devicePointer;
     } else {
         cudaGetLastError();
-        if (cudaMemcpyAsync(dV, hV, kvb, cudaMemcpyHostToDevice, st) != cudaSuccess) return JQ_ERR_CUDA;
     }
-    rc = jq_evict_layer(dK, v_src, dQ, s, dKo, dVo, (int32_t *)dI, ws, wsb, stream);
-    if (rc != JQ_OK) return rc;
-    if (cudaMemcpyAsync(hkept_idx, dI, ib, cudaMemcpyDeviceToHost, st) != cudaSuccess) return JQ_ERR_CUDA;
-    if (cudaMemcpyAsync(hKout, dKo, ob, cudaMemcpyDeviceToHost, st) != cudaSuccess) return JQ_ERR_CUDA;
-    if (cudaMemcpyAsync(hVout, dVo, ob, cudaMemcpyDeviceToHost, st) != cudaSuccess) return JQ_ERR_CUDA;
-    return JQ_OK;
+    // The heads are taken in chunks: while one chunk's keys cross to the device on `stream`, the one before is evicted and
+    // its results cross back on a stream beside it (the link carries both directions at once).  The copy of K, about 19 us
+    // per MB, is what bounds the call; in one piece the pass and the copies back came on top of it.  Measured (us, one
+    // piece, 2, 3, 4, 8 chunks): 8 heads x 32768 keys 1412, 1371, 1353, 1357, 1370; 4 x 65000, budget 4000, 1513, 1436,
+    // 1443, 1409, 1435; 8 x 8000 480, 474, 483, 483, 483: each chunk's small copies back slow the keys down, so calls below
+    // 32 MB stay in one piece.
+    HostPipe *pipe = nullptr;
+    int chunk = s->Hkv;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return JQ_ERR_CUDA;
+    const size_t head_bytes = (size_t)s->L * row;
+    if (s->Hkv > 1 && kvb >= kHostChunks * kHostChunkBytes && cap == cudaStreamCaptureStatusNone && (pipe = host_pipe()) != nullptr) {
+        chunk = (int)((kHostChunkBytes + head_bytes - 1) / head_bytes);
+        const int least = (s->Hkv + kHostChunks - 1) / kHostChunks;
+        if (chunk < least) chunk = least;
+    }
+    cudaStream_t side = pipe ? pipe->side : st;
+    for (int h = 0, n = 0; h < s->Hkv; h += chunk, ++n) {
+        jq_shape sc = *s;
+        sc.Hkv = s->Hkv - h < chunk ? s->Hkv - h : chunk;
+        sc.Hq = sc.Hkv * s->group;
+        const size_t koff = (size_t)h * head_bytes, kb = (size_t)sc.Hkv * head_bytes, rows = (size_t)h * nkeep;
+        const size_t cob = (size_t)sc.Hkv * nkeep * row;
+        int32_t *const idx = (int32_t *)dI + align_up(rows, 4) + 4 * (size_t)n;   // 16-byte aligned, chunks apart
+        if (cudaMemcpyAsync(dK + koff, (const char *)hK + koff, kb, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+            (v_src == dV && cudaMemcpyAsync(dV + koff, (const char *)hV + koff, kb, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
+            (pipe && (cudaEventRecord(pipe->in, st) != cudaSuccess || cudaStreamWaitEvent(side, pipe->in, 0) != cudaSuccess))) {
+            rc = JQ_ERR_CUDA;
+            break;
+        }
+        rc = jq_evict_layer(dK + koff, v_src + koff, dQ + (size_t)h * s->group * s->w * row, &sc, dKo + rows * row, dVo + rows * row, idx,
+                            ws, wsb, (jq_stream_t)side);
+        if (rc == JQ_OK &&
+            (cudaMemcpyAsync(hkept_idx + rows, idx, (size_t)sc.Hkv * nkeep * 4, cudaMemcpyDeviceToHost, side) != cudaSuccess ||
+             cudaMemcpyAsync((char *)hKout + rows * row, dKo + rows * row, cob, cudaMemcpyDeviceToHost, side) != cudaSuccess ||
+             cudaMemcpyAsync((char *)hVout + rows * row, dVo + rows * row, cob, cudaMemcpyDeviceToHost, side) != cudaSuccess))
+            rc = JQ_ERR_CUDA;
+        if (rc != JQ_OK) break;
+    }
+    // whatever has been issued beside the stream belongs to the call (after an error too)
+    if (pipe && (cudaEventRecord(pipe->out, side) != cudaSuccess || cudaStreamWaitEvent(st, pipe->out, 0) != cudaSuccess)) return JQ_ERR_CUDA;
+    return rc;
 }
 
 jq_status jq_last_device_status(const void *ws, jq_stream_t stream)

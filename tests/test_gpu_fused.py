@@ -125,3 +125,25 @@ def test_decode_step_edges(Hkv, group, n):
     jq.decode_attention(dev_bf16(Kc), dev_bf16(Vc), dev_bf16(q), out, ws)
     # fp32 sums of n <= 4100 terms whose weights add up to 1 (bounded by sqrt(n) 2^-24 of values of size 1) and ex2 (2 ulp)
     np.testing.assert_allclose(out.cpu().numpy(), oracle.decode_attention(Kc, Vc, q), rtol=2e-5, atol=5e-6)
+
+
+# heads that go over the link in several chunks: odd kept counts (every chunk's indices start at an alignment of their own),
+# a last chunk that is shorter, pageable values
+@pytest.mark.parametrize("Hkv,g,w,L,budget,pageable", [(3, 2, 4, 44001, 333, False), (8, 1, 8, 16411, 1001, False), (5, 1, 4, 26301, 77, True)])
+def test_host_call_in_chunks(Hkv, g, w, L, budget, pageable):
+    wl = wl_of(Hkv, g, w, L, budget)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    pin = lambda a: torch.from_numpy(a.view(np.int16)).pin_memory()
+    hKo = torch.zeros((Hkv, wl.nkeep, 128), dtype=torch.int16).pin_memory()
+    hVo, hidx = torch.zeros_like(hKo).pin_memory(), torch.zeros((Hkv, wl.nkeep), dtype=torch.int32).pin_memory()
+    buf = torch.empty(jq.host_call_bytes(s), dtype=torch.uint8, device="cuda")
+    hK, hQ, hV = pin(K), pin(Q), torch.from_numpy(V.view(np.int16).copy()) if pageable else pin(V)
+    for _ in range(2):                      # the second call finds the buffers in use by the first
+        jq.evict_layer_host(hK, hV, hQ, s, hKo, hVo, hidx, buf)
+    torch.cuda.current_stream().synchronize()
+    pooled = oracle.pool(oracle.score(K, Q), wl.pool)
+    gi = hidx.numpy()
+    assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
+    for kv in range(Hkv):
+        assert np.array_equal(hKo.numpy().view(np.uint16)[kv], K[kv][gi[kv]]) and np.array_equal(hVo.numpy().view(np.uint16)[kv], V[kv][gi[kv]])
