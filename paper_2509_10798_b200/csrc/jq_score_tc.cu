@@ -17,8 +17,6 @@
 //           and adds exp2(c s - M_r) over the rows, M_r = c m_r + log2(l_r) merged from the partials.
 //           With more than 128 query rows a key gets two blocks, added into the scores with red.add
 //           (two commutative additions onto zero: the result does not depend on their order).
-// A share of the exponentials is evaluated on the FMA pipe (round, degree-4 polynomial on
-// [-1/2, 1/2], exponent insertion) because the ex2 unit, at 16 results per clock per SM, is the binding unit.
 //
 // An epilogue warp is the only source of work for the ex2 unit of its scheduler, and it has two or three
 // peers there: whatever it does between two exponentials leaves the unit idle unless a peer happens to be

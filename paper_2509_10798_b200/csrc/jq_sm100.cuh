@@ -8,7 +8,6 @@ namespace jq {
 namespace {
 
 constexpr long long kWaitCycles = 4000000000ll;  // about 2 s of SM clock per wait
-constexpr int kPolyOf8 = 2;                      // of every 8 pairs of exponentials, this many go to the FMA pipe
 constexpr int kWStatus = 0;                      // the status word of the workspace's status block
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -174,65 +173,35 @@ __device__ __forceinline__ void tc_mma_block(uint32_t d_tmem, uint32_t a_lo, uin
 
 // ------------------------------------------------------------------ exponentials
 
-// exp2 of a pair on the FMA pipe, for x < 100 (pass 1 asks for at most +64, see p1_half; pass 2 for
-// x <= 0: a logit minus the row's log-sum-exp).  x is clamped to >= -126 (so that the exponent
-// insertion cannot wrap; 2^-126 stands in for anything smaller), split into n = round(x) and
-// r = x - n in [-1/2, 1/2] by the add-a-large-constant trick, 2^r comes from a degree-4 polynomial
-// (relative error < 3e-6, a least-maximum fit of 2^r on that interval) and n is added into the
-// exponent field.
-__device__ __forceinline__ float2 exp2_fma_pair(float2 x)
-{
-    const float kMagic = 12582912.f;   // 1.5 * 2^23: x + kMagic holds round(x) in its low mantissa bits
-    x.x = fmaxf(x.x, -126.f);
-    x.y = fmaxf(x.y, -126.f);
-    const float2 t = __fadd2_rn(x, make_float2(kMagic, kMagic));
-    const float2 nn = __ffma2_rn(t, make_float2(-1.f, -1.f), make_float2(kMagic, kMagic));   // -round(x)
-    const float2 r = __fadd2_rn(x, nn);
-    float2 p = __ffma2_rn(make_float2(0.009570101276040077f, 0.009570101276040077f), r,
-                          make_float2(0.05591785907745361f, 0.05591785907745361f));
-    p = __ffma2_rn(p, r, make_float2(0.240247443318367f, 0.240247443318367f));
-    p = __ffma2_rn(p, r, make_float2(0.6931217908859253f, 0.6931217908859253f));
-    p = __ffma2_rn(p, r, make_float2(0.9999992847442627f, 0.9999992847442627f));
-    return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
-                       __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
-}
-
-// acc += exp2(v * c + b) for two values; POLY picks the pipe.
-template <bool POLY>
+// acc += exp2(v * c + b) for two values.  All of them on the ex2 unit: a share on the FMA pipe (round, polynomial, exponent
+// insertion) shortened the stream by itself, but sustained scoring runs at the GPU's power limit (1000 W), and the ten
+// instructions of a polynomial pair cost more energy than they saved time: with 2 of 8 pairs on the FMA pipe 32 layers of
+// 32768 keys took 1071 us, with 1 of 8 1055, with none 1037 (128K keys, 256 rows: 6292, 6230, 6258).
 __device__ __forceinline__ void exp_acc2(float2 &acc, uint32_t v0, uint32_t v1, float2 cc, float2 b)
 {
     const float2 x = __ffma2_rn(make_float2(__uint_as_float(v0), __uint_as_float(v1)), cc, b);
-    acc = __fadd2_rn(acc, POLY ? exp2_fma_pair(x) : make_float2(ex2(x.x), ex2(x.y)));
+    acc = __fadd2_rn(acc, make_float2(ex2(x.x), ex2(x.y)));
 }
-
-// Pair i of the 8 pairs of a 16-column read goes to the FMA pipe when this says so: kPolyOf8 of them, spread evenly.
-__host__ __device__ constexpr bool poly_pair(int i) { return ((i + 1) * kPolyOf8) / 8 != (i * kPolyOf8) / 8; }
 
 // 16 values against 16 biases (pass 2: the negated row normalisers, from shared memory).
 __device__ __forceinline__ void exp_acc16(float2 &a0, float2 &a1, const uint32_t (&v)[16], float2 cc, const float4 *bias)
 {
-    const float4 b0 = bias[0], b1 = bias[1], b2 = bias[2], b3 = bias[3];
-    exp_acc2<poly_pair(0)>(a0, v[0], v[1], cc, make_float2(b0.x, b0.y));
-    exp_acc2<poly_pair(1)>(a1, v[2], v[3], cc, make_float2(b0.z, b0.w));
-    exp_acc2<poly_pair(2)>(a0, v[4], v[5], cc, make_float2(b1.x, b1.y));
-    exp_acc2<poly_pair(3)>(a1, v[6], v[7], cc, make_float2(b1.z, b1.w));
-    exp_acc2<poly_pair(4)>(a0, v[8], v[9], cc, make_float2(b2.x, b2.y));
-    exp_acc2<poly_pair(5)>(a1, v[10], v[11], cc, make_float2(b2.z, b2.w));
-    exp_acc2<poly_pair(6)>(a0, v[12], v[13], cc, make_float2(b3.x, b3.y));
-    exp_acc2<poly_pair(7)>(a1, v[14], v[15], cc, make_float2(b3.z, b3.w));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 b = bias[i];
+        exp_acc2(a0, v[4 * i], v[4 * i + 1], cc, make_float2(b.x, b.y));
+        exp_acc2(a1, v[4 * i + 2], v[4 * i + 3], cc, make_float2(b.z, b.w));
+    }
 }
 
-// 16 values against one bias (pass 1: minus the running maximum of the row).
+// 16 values against one bias (pass 1: minus the reference of the row).
 __device__ __forceinline__ void exp_acc16(float2 &a0, float2 &a1, const uint32_t (&v)[16], float2 cc, float2 b)
 {
-    exp_acc2<poly_pair(0)>(a0, v[0], v[1], cc, b);
-    exp_acc2<poly_pair(1)>(a1, v[2], v[3], cc, b);
-    exp_acc2<poly_pair(2)>(a0, v[4], v[5], cc, b);
-    exp_acc2<poly_pair(3)>(a1, v[6], v[7], cc, b);
-    exp_acc2<poly_pair(4)>(a0, v[8], v[9], cc, b);
-    exp_acc2<poly_pair(5)>(a1, v[10], v[11], cc, b);
-    exp_acc2<poly_pair(6)>(a0, v[12], v[13], cc, b);
-    exp_acc2<poly_pair(7)>(a1, v[14], v[15], cc, b);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        exp_acc2(a0, v[4 * i], v[4 * i + 1], cc, b);
+        exp_acc2(a1, v[4 * i + 2], v[4 * i + 3], cc, b);
+    }
 }
 
 __device__ __forceinline__ float max_of16(const uint32_t (&v)[16])
