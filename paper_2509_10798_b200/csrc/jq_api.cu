@@ -306,12 +306,12 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         ooff += (long long)hpu * nkeep;
     }
     // head groups of the scoring kernel: every run of consecutive units of one length is cut into groups of
-    // about 32 MiB of keys (short prefixes share a group across units, so that a group still has tiles for every CTA)
+    // at most 56 MiB of keys (short prefixes share a group across units, so that a group still has tiles for every CTA)
     for (int u0 = 0; u0 < nunits;) {
         const int Lu = L ? L[u0] : common->L, tph = (Lu + 127) / 128;
         int u1 = u0 + 1;
         while (u1 < nunits && (L ? L[u1] : common->L) == Lu) ++u1;
-        const int heads = (u1 - u0) * hpu, hpg = heads_per_group(Lu, heads, tph, sms);
+        const int heads = (u1 - u0) * hpu, hpg = heads_per_group(Lu, heads, tph, sms, R > 128);
         for (int h0 = 0; h0 < heads; h0 += hpg) {
             GroupRec &g = h_grp[ngroups++];
             g.h0 = u0 * hpu + h0; g.nh = h0 + hpg <= heads ? hpg : heads - h0;

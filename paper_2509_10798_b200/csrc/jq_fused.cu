@@ -742,17 +742,18 @@ bool fused_layout(int L, int nkeep, int C, int nt, FParams *P, size_t *smem)
 }  // namespace
 
 // Whether this kernel takes the call, and with which cluster size (0: no): the cheaper of the two ways by what was measured
-// (us per call, back to back).  This kernel: 10.1, 12.2, 17.8, 29.6 us with 1, 2, 4, 8 tiles per CTA and 128 query rows,
-// 24.4, 40.3 us with 4, 8 tiles and 256; clusters that do not fit at a time take turns (8 heads in clusters of 16: 2 turns).
-// The two kernels of the general path: 30.8, 35.7, 39.9 us for 256, 512, 752 tiles in all and 128 rows, 36.7, 45.1, 51.8
-// with 256.  They meet at about 12000 keys for 8 heads.
+// (us per call, back to back).  This kernel: a chain of exchanges, the tiles of a CTA one after the other, and the selection,
+// which every CTA runs over the whole head; clusters that do not fit at a time take turns (8 heads in clusters of 16: 2).
+// 8 heads x 1024, 2048, 4096, 8192, 12000 keys in clusters of 8: 10.1, 11.9, 17.9, 28.8, 37.6; in clusters of 4: 11.4,
+// 14.8, 24.4, 39.9, 53.8; with 256 rows 4096 and 8192 keys 24.7, 40.0 and 35.0, 61.4.  The two kernels of the general path,
+// by tiles in all: 64, 256, 512, 752, 1024: 22.6, 26.7, 32.3, 35.6, 41; with 256 rows 128, 256, 512: 27.0, 30.8, 39.2.
 static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FParams *P, size_t *smem)
 {
     FusedDevice dev;
     if (s.L > kFMaxL || !fused_device(&dev)) return 0;
     const int TT = (src.LA + kFTile - 1) / kFTile + (src.LB + kFTile - 1) / kFTile, win = src.Kwin ? 1 : 0;
     const bool wide = P->Rbox == 256;
-    const double per_tile = wide ? 4.0 : 2.7;
+    const double chain = wide ? 9.3 : 7.4, per_tile = wide ? 2.6 : 1.0 + 0.4 * P->Rpad / 128;
     int best = 0;
     double best_cost = 1e30;
     for (int i = 0; i < 5 && (1 << i) <= TT; ++i) {
@@ -762,10 +763,11 @@ static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FPar
         FParams T = *P;
         size_t sm;
         if (!fused_layout(s.L, nkeep, C, nt, &T, &sm)) continue;
-        const double cost = (double)((s.Hkv + dev.resident[i] - 1) / dev.resident[i]) * (7.6 + per_tile * nt);
+        const double cost = (double)((s.Hkv + dev.resident[i] - 1) / dev.resident[i]) * (chain + per_tile * nt + (C == 16 ? 1.04e-3 : 1.24e-3) * s.L);
         if (cost < best_cost) { best_cost = cost; best = C; *P = T; *smem = sm; }
     }
-    const double other = (wide ? 29.0 : 26.3) + (wide ? 0.031 : 0.018) * s.Hkv * TT;
+    // (the general path appends and moves back with strided copies, two of each, about 4.5 us a piece)
+    const double other = (wide ? 23.5 : 22.5) + (wide ? 0.03 : 0.0185) * s.Hkv * TT + (src.LB > 0 ? 9.0 : 0.0) + (src.inplace ? 9.0 : 0.0);
     return best_cost <= other ? best : 0;
 }
 

@@ -99,7 +99,7 @@ static inline size_t unit_tables_bytes(int nunits, int hpu)
 // (head_rows: rows between consecutive heads in memory when they are not packed).
 bool make_tensor_map(void *map, const void *ptr, int rows, int heads, int box_rows, int head_rows = 0);
 // Most KV heads of L keys that the scoring kernel takes as one group (tiles of a group are split over `sms` CTAs).
-int heads_per_group(int L, int heads, int tiles_per_head, int sms);
+int heads_per_group(int L, int heads, int tiles_per_head, int sms, bool wide);   // wide: more than 128 query rows
 int score_sms();   // CTAs of the scoring kernel on the current device; 0 on error
 
 // Host-side bookkeeping.

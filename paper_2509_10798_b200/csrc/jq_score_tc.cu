@@ -791,25 +791,28 @@ int score_sms()
     return device_info(&dev) ? dev.sms : 0;
 }
 
-// KV heads are scored in groups whose keys fit in a share of the L2 (32 MiB), so that pass 2 finds them there.
-// Among the admissible group sizes, the one that wastes the fewest CTA-tile slots.
-int heads_per_group(int L, int heads, int tiles_per_head, int sms)
+// KV heads are scored in groups whose keys fit in a share of the L2 (56 MiB: pass 1 of the next group runs in between), so
+// that pass 2 finds them there.  Among the admissible group sizes, the one with the fewest waves of tiles over the CTAs, a
+// group costing about half a wave of its own; a single group has nothing to hide its merge behind and, from 32 MiB (256
+// rows) or 40 MiB (128) on, loses more by the L2 than it saves.  At equal cost the fewer groups, the more even ones.
+// Measured with at most 16, 24, 32, 48, 64 MiB (us): a ragged batch of 128 units 3215, 2746, 2515, 2389, 2398; 32 layers of
+// 32768 keys 1292, 1135, 1008, 1008, 1017, of 131072 keys (a head is 32 MiB) 6140, 6134, 6130, 6143, 6450; one layer of 4 x
+// 100000 keys in groups of 1, 2 heads 49.2, 41.0, of 8 x 32768 in 2, 1 groups 36.8, 38.9, of 8 x 13000 26.5, 24.6.
+int heads_per_group(int L, int heads, int tiles_per_head, int sms, bool wide)
 {
     const long long head_bytes = (long long)L * kD * 2;
-    long long hmax = (32ll << 20) / head_bytes;
+    long long hmax = (56ll << 20) / head_bytes;
     if (hmax < 1) hmax = 1;
     if (hmax > heads) hmax = heads;
     int best_hpg = 1;
-    double best_eff = -1.0;
+    double best = 1e300;
     for (int hpg = 1; hpg <= (int)hmax; ++hpg) {
-        long long work = 0, slots = 0;
-        for (int h0 = 0; h0 < heads; h0 += hpg) {
-            const long long T = (long long)(h0 + hpg <= heads ? hpg : heads - h0) * tiles_per_head;
-            work += T;
-            slots += (T + sms - 1) / sms;
-        }
-        const double eff = (double)work / ((double)slots * sms);
-        if (eff >= best_eff - 1e-9) { best_eff = eff > best_eff ? eff : best_eff; best_hpg = hpg; }
+        const int groups = (heads + hpg - 1) / hpg;
+        const bool alone = groups == 1 && heads > 1 && head_bytes * heads > ((wide ? 32ll : 40ll) << 20);
+        double cost = 0.5 * groups + (alone ? 1.6 : 0.0);
+        for (int h0 = 0; h0 < heads; h0 += hpg)
+            cost += (double)(((long long)(h0 + hpg <= heads ? hpg : heads - h0) * tiles_per_head + sms - 1) / sms);
+        if (cost < best - 1e-9 || (cost < best + 1e-9 && groups < (heads + best_hpg - 1) / best_hpg)) { best = cost < best ? cost : best; best_hpg = hpg; }
         if (hmax > 64 && hpg >= 64) break;   // the scan is only worth it over a small range
     }
     return best_hpg;
@@ -848,7 +851,7 @@ jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float
         P.gtab = nullptr; P.maps = nullptr; P.hpu = s.Hkv;
         if (!make_map(&mapK, K, s.L, s.Hkv, kTile, k_head_rows) || !make_map(&mapQ, Q, R, s.Hkv, P.Rbox)) return JQ_ERR_CUDA;
         if (Kwin) { if (!make_map(&mapW, Kwin, s.w, s.Hkv, kTile)) return JQ_ERR_CUDA; } else mapW = mapK;
-        P.hpg = heads_per_group(s.L, s.Hkv, P.tph, sms);
+        P.hpg = heads_per_group(s.L, s.Hkv, P.tph, sms, R > 128);
         P.ngroups = (s.Hkv + P.hpg - 1) / P.hpg;
         tmax = (long long)(P.hpg < s.Hkv ? P.hpg : s.Hkv) * P.tph;
     }
