@@ -12,6 +12,8 @@ __global__ void __launch_bounds__(256)
 gather_rows(const uint4 *__restrict__ K, const uint4 *__restrict__ V, const int32_t *__restrict__ idx,
             int L, int nkeep, long long nrows, uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, int Hkv JQ_DBG_PARAM)
 {
+    cudaGridDependencySynchronize();             // set up while the kernel before it in the stream was finishing
+    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
     const int lane16 = threadIdx.x & 15;
     long long row = (long long)blockIdx.x * (blockDim.x / 16) + (threadIdx.x >> 4);
     const long long stride = (long long)gridDim.x * (blockDim.x / 16);
@@ -37,8 +39,20 @@ jq_status launch_gather(const void *K, const void *V, const int32_t *idx, const 
     const long long nrows = (long long)s.Hkv * nkeep;
     long long blocks = (2 * nrows + 15) / 16;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    gather_rows<<<(unsigned)blocks, 256, 0, st>>>((const uint4 *)K, (const uint4 *)V, idx, s.L, nkeep, nrows,
-                                                  (uint4 *)Kout, (uint4 *)Vout, s.Hkv JQ_DBG_ARG);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, gather_rows, (const uint4 *)K, (const uint4 *)V, idx, s.L, nkeep, nrows, (uint4 *)Kout, (uint4 *)Vout,
+                           s.Hkv JQ_DBG_ARG) != cudaSuccess) {
+        cudaGetLastError();
+        return JQ_ERR_CUDA;
+    }
     count_launch(1);
     return check_launch();
 }

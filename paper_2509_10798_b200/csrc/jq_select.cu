@@ -183,6 +183,7 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     for (int i = tid; i < kOwnBins + kBins; i += kSelThreads) ghist[i] = 0;
     if (tid == 0) ctl.cand_count = 0;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
+    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
     if (htab) {
         const HeadRec r = htab[kv];
         L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; orow = r.ooff; krow = r.ooff; src_rows = L;
@@ -571,6 +572,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     int kv_in = kv;
     long long soff = (long long)kv * L, orow = (long long)kv * nkeep, krow = (long long)kv * out_rows;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
+    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
     if (htab) {
         const HeadRec r = htab[kv];
         L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; orow = r.ooff; krow = r.ooff; src_rows = L;
