@@ -27,7 +27,7 @@
 // towards lower positions, so the cluster moves them a chunk at a time, reading a chunk completely before writing it.
 //
 // Measured (B200, back-to-back calls through the Python entry points, two launches -> this one): 2 heads x 2048 keys, 64 query
-// rows 24.8 -> 9.8 us; 8 x 4096, 128 rows 30.8 -> 17.8 us; 8 x 8192 34.8 -> 28.9 us; re-eviction of 8 x (1024 + 256) keys, in
+// rows 24.8 -> 9.8 us; 8 x 4096, 128 rows 30.8 -> 17.8 us; 8 x 8192 34.8 -> 27.0 us; re-eviction of 8 x (1024 + 256) keys, in
 // place, 45.6 -> 15.9 us (six strided copies and two launches before).
 #include "jq_sm100.cuh"
 #include "jq_tmem_ld.cuh"
@@ -189,9 +189,8 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     float *const scores = (float *)(smem_raw + P.o_scores) + kFHalo;   // [L], with a halo of -inf on either side
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank(), C = cluster_size();
-    const int lgC = 31 - __clz(C);                            // (cluster sizes and row boxes are powers of two: no divisions here)
-    const int kv = (int)(blockIdx.x >> lgC);
-    const int t0 = (int)(rank * (uint32_t)P.tT >> lgC), t1 = (int)((rank + 1) * (uint32_t)P.tT >> lgC), nt = t1 - t0;
+    const int kv = (int)(blockIdx.x / C);
+    const int t0 = (int)(rank * (uint32_t)P.tT / C), t1 = (int)((rank + 1) * (uint32_t)P.tT / C), nt = t1 - t0;
     const int nt1 = nt + (P.wtile && rank == 0 ? 1 : 0);      // tiles of pass 1
     const int nblk = P.Rbox / 128, L = P.L, R = P.R, Rpad = P.Rpad;
     const int nrw = (R + 31) / 32;                            // warps that push row statistics
@@ -676,7 +675,7 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 
 // ------------------------------------------------------------------ host side
 
-struct FusedDevice { int resident[5] = {}; bool ready = false; };   // clusters of 1, 2, 4, 8, 16 CTAs that fit at a time
+struct FusedDevice { int resident[kFMaxCluster + 1] = {}; bool ready = false; };   // [C]: clusters of C CTAs that fit at a time
 
 bool fused_device(FusedDevice *out)
 {
@@ -689,17 +688,17 @@ bool fused_device(FusedDevice *out)
     if (!d.ready) {
         if (cudaFuncSetAttribute(evict_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFMaxSmem) != cudaSuccess) return false;
         if (cudaFuncSetAttribute(evict_fused, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
-        for (int i = 0; i < 5; ++i) {
+        for (int C = 1; C <= kFMaxCluster; ++C) {
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(1u << i);
+            cfg.gridDim = dim3((unsigned)C);
             cfg.blockDim = dim3(kFThreads);
             cfg.dynamicSmemBytes = kFMaxSmem;
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1u << i; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&d.resident[i], evict_fused, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[i] = 0; }
+            if (cudaOccupancyMaxActiveClusters(&d.resident[C], evict_fused, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[C] = 0; }
         }
         d.ready = true;
     }
@@ -743,9 +742,9 @@ bool fused_layout(int L, int nkeep, int C, int nt, FParams *P, size_t *smem)
 
 // Whether this kernel takes the call, and with which cluster size (0: no): the cheaper of the two ways by what was measured
 // (us per call, back to back).  This kernel: a chain of exchanges, the tiles of a CTA one after the other, and the selection,
-// which every CTA runs over the whole head; clusters that do not fit at a time take turns (8 heads in clusters of 16: 2).
-// 8 heads x 1024, 2048, 4096, 8192, 12000 keys in clusters of 8: 10.1, 11.9, 17.9, 28.8, 37.6; in clusters of 4: 11.4,
-// 14.8, 24.4, 39.9, 53.8; with 256 rows 4096 and 8192 keys 24.7, 40.0 and 35.0, 61.4.  The two kernels of the general path,
+// which every CTA runs over the whole head; clusters that do not fit at a time take turns (of 16 CTAs 7 fit, of 10 11).
+// 8 heads x 1024, 2048, 4096, 8192, 12000 keys in clusters of 8: 10.1, 11.9, 17.9, 29.4, 38.1; of 10: -, 12.3, 17.9, 27.2,
+// 34.7; of 4: 11.4, 14.8, 24.4, 40.1, 54.3; with 256 rows 4096 and 8192 keys 24.9, 40.6; 24.9, 37.3; 35.2, 62.0.  The two kernels of the general path,
 // by tiles in all: 64, 256, 512, 752, 1024: 22.6, 26.7, 32.3, 35.6, 41; with 256 rows 128, 256, 512: 27.0, 30.8, 39.2.
 static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FParams *P, size_t *smem)
 {
@@ -756,14 +755,13 @@ static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FPar
     const double chain = wide ? 9.3 : 7.4, per_tile = wide ? 2.6 : 1.0 + 0.4 * P->Rpad / 128;
     int best = 0;
     double best_cost = 1e30;
-    for (int i = 0; i < 5 && (1 << i) <= TT; ++i) {
-        const int C = 1 << i;
-        if (dev.resident[i] < 1) continue;
+    for (int C = 1; C <= kFMaxCluster && C <= TT; ++C) {
+        if (dev.resident[C] < 1) continue;
         const int up = (TT + C - 1) / C, first = TT / C + win, nt = up > first ? up : first;   // (rank 0 has the window tile)
         FParams T = *P;
         size_t sm;
         if (!fused_layout(s.L, nkeep, C, nt, &T, &sm)) continue;
-        const double cost = (double)((s.Hkv + dev.resident[i] - 1) / dev.resident[i]) * (chain + per_tile * nt + (C == 16 ? 1.04e-3 : 1.24e-3) * s.L);
+        const double cost = (double)((s.Hkv + dev.resident[C] - 1) / dev.resident[C]) * (chain + per_tile * nt + (C > 8 ? 1.04e-3 : 1.24e-3) * s.L);
         if (cost < best_cost) { best_cost = cost; best = C; *P = T; *smem = sm; }
     }
     // (the general path appends and moves back with strided copies, two of each, about 4.5 us a piece)
