@@ -46,7 +46,7 @@ struct DecSmem {
     float m[kDecWarps][kDecMaxGroup], l[kDecWarps][kDecMaxGroup];
     // what the cluster's CTAs push here: rank r's statistics of every head, and its share of the outputs written here
     float rm[kDecMaxCluster][kDecMaxGroup], rl[kDecMaxCluster][kDecMaxGroup];
-    float rO[kDecMaxGroup * kD];    // [rank][share]: the shares of all ranks add up to the head's outputs
+    float rO[kDecMaxGroup * kD + kDecMaxCluster];   // [rank][share]: the shares of all ranks make up the head's outputs
 };
 
 __device__ __forceinline__ float dec_ex2(float x)
@@ -229,7 +229,7 @@ decode_step(const uint4 *__restrict__ Kc, const uint4 *__restrict__ Vc, const __
     }
     __syncthreads();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA of the cluster runs: its memory may be written
-    const int items = group * kD, share = items / (int)C;   // (group * 128 is a multiple of every cluster size)
+    const int items = group * kD, share = (items + (int)C - 1) / (int)C;
     for (int it = tid; it < items; it += kDecThreads) {
         const int h = it / kD, c = it - h * kD;
         float M = -INFINITY;
@@ -251,6 +251,7 @@ decode_step(const uint4 *__restrict__ Kc, const uint4 *__restrict__ Vc, const __
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     for (int i = tid; i < share; i += kDecThreads) {
         const int it = (int)rank * share + i, h = it / kD;
+        if (it >= items) break;
         float M = -INFINITY, O = 0.f, Ls = 0.f;
         for (int r = 0; r < (int)C; ++r) M = fmaxf(M, sm.rm[r][h]);
         for (int r = 0; r < (int)C; ++r) {
@@ -264,10 +265,12 @@ decode_step(const uint4 *__restrict__ Kc, const uint4 *__restrict__ Vc, const __
 
 // CTAs per KV head: the cluster size that the estimate below finds fastest.  A cluster takes about 3.3 us of launch,
 // merge and latency and 1 us for each unit its busiest warp walks through, and only so many clusters of a size are
-// resident at a time (a cluster stays within a GPC: 148, 33, 15, 7 of 1, 4, 8, 16 CTAs; asked for once per device).
+// resident at a time (a cluster stays within a GPC: 148, 45, 33, 22, 15, 11, 7 of 1, 3, 4, 6, 8, 10, 16 CTAs; asked for once
+// per device).
 // Measured against it: 8 heads x 1024 keys 11.3, 7.5, 5.6, 4.3 us with 1, 2, 4, 8 CTAs; 128 x 2048 27, 30, 37, 56;
-// 24 x 3000 30.5, 17.9, 11.8, 15.6; 7 x 4096 34, -, 11.7, 7.9 and 5.9 with 16.
-struct DecPlan { int resident[5] = {}; bool ready = false; };   // resident clusters of 1, 2, 4, 8, 16 CTAs
+// 24 x 3000 30.5, 17.9, 11.8, 15.6 and 11.1 with 5; 20 x 3000 11.5, 9.6 with 4, 6; 36 x 2000 14.8, 12.8 with 2, 3; 7 x 4096
+// 34, -, 11.7, 7.9 and 5.9 with 16.
+struct DecPlan { int resident[kDecMaxCluster + 1] = {}; bool ready = false; };   // [C]: resident clusters of C CTAs
 
 bool decode_plan(DecPlan *out)
 {
@@ -280,19 +283,19 @@ bool decode_plan(DecPlan *out)
     if (!p.ready) {
         for (auto k : {decode_step<true>, decode_step<false>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
-        for (int i = 0; i < 5; ++i) {
+        for (int C = 1; C <= kDecMaxCluster; ++C) {
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(1u << i);
+            cfg.gridDim = dim3((unsigned)C);
             cfg.blockDim = dim3(kDecThreads);
             cfg.dynamicSmemBytes = sizeof(DecSmem);
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1u << i; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&p.resident[i], decode_step<true>, &cfg) != cudaSuccess) { cudaGetLastError(); p.resident[i] = 0; }
+            if (cudaOccupancyMaxActiveClusters(&p.resident[C], decode_step<true>, &cfg) != cudaSuccess) { cudaGetLastError(); p.resident[C] = 0; }
         }
-        if (p.resident[0] < 1) return false;
+        if (p.resident[1] < 1) return false;
         p.ready = true;
     }
     *out = p;
@@ -304,11 +307,12 @@ int decode_cluster(int Hkv, int n, const DecPlan &p)
     const int nunits = (n + kDecUnit - 1) / kDecUnit;
     int best = 1;
     double best_cost = 0;
-    for (int i = 0; i < 5; ++i) {
-        if (p.resident[i] < 1) continue;
-        const int per = kDecWarps << i;
-        const double cost = (double)((Hkv + p.resident[i] - 1) / p.resident[i]) * (3.3 + (nunits + per - 1) / per);
-        if (i == 0 || cost < best_cost) { best = 1 << i; best_cost = cost; }
+    for (int C = 1; C <= kDecMaxCluster; ++C) {
+        if (p.resident[C] < 1) continue;
+        const int per = kDecWarps * C;
+        const double cost = (double)((Hkv + p.resident[C] - 1) / p.resident[C]) * (3.3 + (nunits + per - 1) / per);
+        // (at equal cost a power of two: the outputs then divide evenly over the CTAs)
+        if (C == 1 || cost < best_cost || (cost == best_cost && (C & (C - 1)) == 0 && (best & (best - 1)) != 0)) { best = C; best_cost = cost; }
     }
     return best;
 }
