@@ -180,6 +180,7 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int raw_cap = raw_tile + 2 * kHalo, keys_cap = keys_in_smem ? chunk : 0;   // shared-memory extents (those of the launch)
     (void)raw_cap; (void)keys_cap;
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // waited for before the first store to another CTA
     for (int i = tid; i < kOwnBins + kBins; i += kSelThreads) ghist[i] = 0;
     if (tid == 0) ctl.cand_count = 0;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
@@ -247,9 +248,12 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
             if (pooled && JQ_IN(soff + j0 + t0 + e, ext.scores, kDbgSelect, 12)) pooled[j0 + t0 + e] = best;
         }
     }
+    // Every CTA of the cluster runs from here on: its shared memory may be written.  (The arrival is as old as the kernel:
+    // with the pooling in between nobody is waited for.)
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     const int ngrp = kSelThreads / 16;
     const int r0 = (int)((long long)rank * nkeep / CL), r1 = (int)((long long)(rank + 1) * nkeep / CL);   // the rows this CTA copies
-    if (nkeep >= L) {   // everything is kept (uniform over the cluster; no cluster traffic yet)
+    if (nkeep >= L) {   // everything is kept (uniform over the cluster)
         for (int e = tid; e < n; e += kSelThreads) if (JQ_IN(orow + j0 + e, ext.out_rows, kDbgSelect, 13)) out[j0 + e] = j0 + e;
         if (Kin) {
             cluster.sync();
