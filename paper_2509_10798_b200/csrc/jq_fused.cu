@@ -580,7 +580,11 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             for (int i = tid; i < kFBins / 4; i += kFT) ((uint4 *)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
             group_sync();
         }
-        // ---- ordered compaction: need_eq of the keys == tau are kept, the lowest positions
+        // ---- ordered compaction: need_eq of the keys == tau are kept, the lowest positions.  (After a wait that ran out, scores
+        // and counts may be anything, copies in flight may land on them, and the warps may learn of it at different times: the
+        // selection then runs to its end like any other, within its arrays whatever it reads - a thread's first place in the
+        // list is brought into range, and its at most 28 entries from there reach at most into the keys, which have been
+        // read - and no row is copied.)
         uint32_t gtm = 0u, eqm = 0u;                                      // bit 4 i + e: position e of the thread's i-th quad
 #pragma unroll 1
         for (int q = q0, i = 0; q < q1; ++q, i += 4) {
@@ -590,7 +594,7 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         }
         const int before = scan512(__popc(gtm) | __popc(eqm) << 16, ctl->scan[1]);   // (at most 12288 positions: 14 bits each)
         const int eb = before >> 16, room = max(need_eq - eb, 0);
-        int t = (before & 0xffff) + min(eb, need_eq), j = 4 * q0;
+        int t = min(max((before & 0xffff) + min(eb, need_eq), 0), P.nkeep), j = 4 * q0;
         while (__popc(eqm) > room) eqm ^= 0x80000000u >> __clz(eqm);
 #pragma unroll 1
         for (uint32_t m = gtm | eqm; m; m >>= 1, ++j)
@@ -665,9 +669,13 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
     // ---------------------------------------------------------------- exit
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    bool gave_up = false;
+    if (warp == kFWarps + 1) gave_up = *(volatile int *)&ctl->abort_flag != 0;   // (there is nothing left to wait for)
     tc_fence_before();
     __syncthreads();
     if (warp == kFWarps + 1) {
+        if (gave_up) __nanosleep(200000);        // let copies, pushes and products still in flight land before the CTA goes
+        __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kFTmemCols) : "memory");
     }

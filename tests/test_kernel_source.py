@@ -42,3 +42,22 @@ def test_a_cluster_has_started_before_its_shared_memory_is_touched(name):
 
 def test_the_cluster_kernels_are_found():
     assert {k for k, v in KERNELS.items() if REMOTE.search(v[1])} == {"decode_step", "evict_fused", "select_cluster"}
+
+
+@pytest.mark.parametrize("name", sorted(k for k, v in KERNELS.items() if "tcgen05.dealloc" in v[1]))
+def test_a_kernel_that_gave_up_waits_for_its_copies(name):
+    """A kernel with bounded waits leaves only when what it has in flight has had time to land: tensor copies and products
+    are written into shared and tensor memory that is the next block's once this one has gone."""
+    body = KERNELS[name][1]
+    tail = body[:body.index("tcgen05.dealloc")]
+    assert re.search(r"\(\*\(volatile int \*\)&ctl->abort_flag\)\s*__nanosleep\(\d{6,}\)"
+                     r"|gave_up = \*\(volatile int \*\)&ctl->abort_flag != 0;.*if \(gave_up\)\s*__nanosleep\(\d{6,}\)", tail, re.S)
+
+
+def test_the_one_launch_pass_stays_in_bounds_after_a_wait_that_ran_out():
+    """The selection runs even when the CTA gave up a wait (its warps need not agree on that, and they share barriers),
+    with whatever scores and counts it then finds: the places it stores at are brought into range, whatever they are."""
+    body = KERNELS["evict_fused"][1]
+    assert "int t = min(max((before & 0xffff) + min(eb, need_eq), 0), P.nkeep)" in body
+    assert body.count("list[t] = ") == 2 and "for (int t = tid; t < P.nkeep; t += kFT) list[t] = t;" in body
+    assert body.count("min(max(list[t0r + i") == 2     # and so are the positions that rows are read at
