@@ -8,9 +8,10 @@
 //   2. the threshold: 2048 equal bins over the range of the head's keys - not their leading bits, which are the same for
 //      most keys of a flat head and would need further rounds over all of them.  The histograms are summed through
 //      distributed shared memory, every CTA owning a share of the bins, and every CTA finds the bin of the nkeep-th
-//      largest key for itself.  Its keys, normally a few dozen, go to the leading CTA with their positions, and every CTA
-//      ranks them by comparison: the key tau of the nkeep-th largest element and how many elements equal to tau are
-//      kept.  (While the bin holds more than kCandMax keys it is split into 2048 bins again.)  Max-pooling copies every peak into up to `pool` neighbours, so ties at tau are
+//      largest key for itself.  Every CTA lists its keys of that bin, brings the lists of all together and finishes on
+//      them - a few dozen by comparison, more by bins of its own: the key tau of the nkeep-th largest element and how many
+//      elements equal to tau are kept.  (While the bin holds more than kCandMax keys it is split into 2048 bins by the
+//      whole cluster again.)  Max-pooling copies every peak into up to `pool` neighbours, so ties at tau are
 //      the normal case: all keys > tau are kept, then the lowest-index keys == tau.
 //   3. ordered compaction: kept positions are written in ascending order (CTA rank, warp, iteration and lane order all
 //      follow the position order); the list also gives every warp its number of kept keys, so nothing is counted again.
@@ -18,8 +19,11 @@
 // Everything is integer arithmetic on bit patterns, hence deterministic and exact.  The kernel is a chain of short phases
 // between cluster barriers (four; about 700 cycles each), so what bounds it is latency.  Measured (8 heads, us, against
 // leading-bit radix rounds of 11 bits, a counting pass, clusters of 8 and one row in flight per 16 lanes in the copy):
-// selection alone 12000 keys 10.6 -> 8.6, 30011 12.1 -> 10.8, 131072 21.3 -> 18.5; with the rows of a layer 131072 keys, budget
+// selection alone 12000 keys 10.6 -> 8.8, 30011 12.1 -> 11.0, 131072 21.3 -> 18.2; with the rows of a layer 131072 keys, budget
 // 4096, 73.6 k -> 42.9 k cycles; the windowed layer of 11999 keys (two strided copies before) 46.3 -> 36.9 us.
+// Several hundred keys in the threshold's bin (scores whose 24th roots are even; those kernels -> one list in the leading
+// CTA, ranked by comparison up to 512 keys -> now): 8 x 30011 12.7 -> 15.5 -> 12.0, 8 x 60000 15.6 -> 24.4 -> 15.4, 127 x
+// 60000 70 -> 116 -> 75; 8 x 500 with five different scores 9.7 -> 16.2 -> 8.4.
 #include "jq_internal.cuh"
 #include "jq_pool.cuh"
 #include "jq_debug.cuh"
@@ -38,10 +42,15 @@ constexpr int kOwnBins = 3 * kBins / 2;   // select_cluster: a CTA's share of th
 constexpr int kRawTile = 8192;     // most scores staged per pooling step
 constexpr int kHalo = 32;          // >= pool radius
 constexpr int kKeysSmemMax = 24576; // keys a CTA can keep in shared memory
-constexpr size_t kSelTwoPerSm = 100 * 1024;   // shared memory per CTA up to which two CTAs fit on an SM
+constexpr size_t kSelTwoPerSm = 110 * 1024;   // shared memory per CTA up to which two CTAs fit on an SM
 constexpr double kSelChain = 7.5, kSelChain16 = 10.0, kSelPerKey = 0.0007;   // choose_plan's estimate, us
-constexpr int kCandMax = 512;      // keys of one bin that are ranked by comparison (one per thread)
-static_assert(kCandMax <= kSelThreads, "a thread ranks one candidate");
+constexpr int kCandMax = 1024;     // keys of one bin that are finished on a list of them
+constexpr int kRankMax = 64;       // of which so many are sent to every CTA and ranked by comparison; more are fetched, and split into bins again
+static_assert(kClMax * kRankMax <= kCandMax, "a place for every CTA's list");
+// Lists of keys and of their positions, in the place of the staged scores: this CTA's keys of the bin, and those of all CTAs
+// (or the short lists that they sent).
+constexpr int kOwnKey = 0, kOwnPos = kCandMax, kAllKey = 2 * kCandMax, kAllPos = 3 * kCandMax, kListWords = 4 * kCandMax;
+__host__ __device__ constexpr int raw_words(int raw_tile) { return raw_tile + 2 * kHalo > kListWords ? raw_tile + 2 * kHalo : kListWords; }
 static_assert(kBins == 4 * kSelThreads, "a thread takes four bins");
 
 // Extents of what the kernel indexes (read by the bounds-checked build only).
@@ -58,15 +67,13 @@ struct SelCtl {
     int digit, krem, count;              // find_digit: the bin of the krem-th key, the rank within it, its population
     uint32_t tau;
     int need_eq;
-    int cand_count;                      // leading CTA only: candidates appended so far
+    int cand_count;                      // this CTA's keys of the bin
     int base_gt, base_eq;                // kept-or-tied keys of the CTAs before this one
     uint32_t mn[kClMax], mx[kClMax];     // range of every CTA's keys
-    int gt_of[kClMax], eq_of[kClMax];    // every CTA's keys above the bin (above tau, equal to tau)
+    int gt_of[kClMax], eq_of[kClMax], cand_of[kClMax];   // every CTA's keys above the bin (above tau, equal to tau); its keys of the bin
     int warp_gt[kSelWarps], warp_eq[kSelWarps];
     uint32_t wmn[kSelWarps], wmx[kSelWarps];
     int scan[kSelWarps];
-    uint32_t cand_key[kCandMax], my_key[kCandMax];   // leading CTA: the list; everybody's copy of it
-    int cand_pos[kCandMax], my_pos[kCandMax];
 };
 
 // Block-wide exclusive scan of one int per thread, any number of whole warps.
@@ -110,6 +117,30 @@ __device__ __forceinline__ void find_digit_cta(const uint32_t *h, int krem, Ctl 
         const int c = (int)h[hi - i];
         if (above < krem && krem <= above + c) { ctl.digit = hi - i; ctl.krem = krem - above; ctl.count = c; }
         above += c;
+    }
+    __syncthreads();
+}
+
+// The bin that holds the need-th key counted from the top, from a thread's four bins (those at kBins - 4 - 4 tid) -> ctl: the
+// bin, the rank within it, its population.
+__device__ __forceinline__ void find_bin(const uint4 v, int need, SelCtl &ctl)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, at = kBins - 4 - 4 * (int)threadIdx.x;
+    const int c[4] = {(int)v.w, (int)v.z, (int)v.y, (int)v.x};
+    int inc = c[0] + c[1] + c[2] + c[3];
+    const int mine = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) ctl.scan[wid] = inc;
+    __syncthreads();
+    int above = __reduce_add_sync(0xffffffffu, lane < wid ? ctl.scan[lane] : 0) + inc - mine;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (above < need && need <= above + c[i]) { ctl.digit = at + 3 - i; ctl.krem = need - above; ctl.count = c[i]; }
+        above += c[i];
     }
     __syncthreads();
 }
@@ -173,8 +204,9 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     extern __shared__ __align__(16) uint8_t sm[];
     uint32_t *ghist = (uint32_t *)sm;                       // [3][kBins / CL]: the cluster's counts of the bins this CTA owns, one set per round
     uint32_t *hist = ghist + kOwnBins;                      // [kBins]
-    float *raw = (float *)(hist + kBins);                   // [raw_tile + 2*kHalo]
-    uint32_t *keys_s = (uint32_t *)(raw + raw_tile + 2 * kHalo);
+    float *raw = (float *)(hist + kBins);                   // [raw_tile + 2*kHalo]; when all is pooled,
+    uint32_t *const lists = (uint32_t *)raw;                // [kListWords]
+    uint32_t *keys_s = (uint32_t *)(raw + raw_words(raw_tile));
     __shared__ SelCtl ctl;
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -283,7 +315,7 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     int need = nkeep;                            // the need-th largest of them
     bool listed = false;
     const int own = kBins / CL;
-    const int per = (n + kSelThreads - 1) / kSelThreads;
+    const int per = (n + kSelThreads - 1) / kSelThreads | 1;   // odd: neighbouring threads hit different banks
     for (int round = 0;; ++round) {
         const int sh = lim >> 11 ? 21 - __clz(lim) : 0;            // lim >> sh < 2048
         // A thread takes a run of consecutive keys and adds equal neighbouring bins as one count: the max-pool leaves
@@ -291,11 +323,8 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
         {
             const int e0 = min(tid * per, n), e1 = min(e0 + per, n);
             uint32_t cur = 0u, cnt = 0u;
-            int pos = per ? tid % per : 0;                          // rotated start: neighbouring threads hit different banks
-            for (int i = 0; i < per; ++i) {
-                const int e = e0 + pos;
-                if (++pos == per) pos = 0;
-                if (e >= e1 || !JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 14)) continue;
+            for (int e = e0; e < e1; ++e) {
+                if (!JQ_IN(keys_in_smem ? e : soff + j0 + e, keys_in_smem ? keys_cap : ext.scores, kDbgSelect, 14)) continue;
                 const uint32_t k = mykeys[e] - lo;
                 if (k > lim) continue;
                 if (k >> sh != cur) { if (cnt && JQ_IN(cur, kBins, kDbgSelect, 9)) atomicAdd(&hist[cur], cnt); cur = k >> sh; cnt = 0; }
@@ -320,38 +349,20 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
         cluster.sync();
         {
             const int at = kBins - 4 - 4 * tid;                      // from the top
-            const uint4 v = *(const uint4 *)(cluster.map_shared_rank(sums, at / own) + at % own);
-            const int c[4] = {(int)v.w, (int)v.z, (int)v.y, (int)v.x};
-            int inc = c[0] + c[1] + c[2] + c[3];
-            const int mine = inc;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int x = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += x;
-            }
-            if (lane == 31) ctl.scan[wid] = inc;
-            __syncthreads();
-            int above = __reduce_add_sync(0xffffffffu, lane < wid ? ctl.scan[lane] : 0) + inc - mine;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (above < need && need <= above + c[i]) { ctl.digit = at + 3 - i; ctl.krem = need - above; ctl.count = c[i]; }
-                above += c[i];
-            }
-            __syncthreads();
+            find_bin(*(const uint4 *)(cluster.map_shared_rank(sums, at / own) + at % own), need, ctl);
         }
         lo += (uint32_t)ctl.digit << sh;
         need = ctl.krem;
         lim = (1u << sh) - 1u;
-        listed = ctl.count <= kCandMax;
+        listed = sh != 0 && ctl.count <= kCandMax;                   // (a bin of one key value needs no list)
         if (listed || sh == 0) break;
     }
     // Warp w owns the contiguous elements [w0, w1).  Keys above the bin (listed) or above / equal to the threshold are
-    // counted per warp; the bin's own keys go to the leading CTA's list.
+    // counted per warp; the bin's own keys are listed.
     const int nc = listed ? ctl.count : 0;
     const int seg = ((n + kSelWarps - 1) / kSelWarps + 31) / 32 * 32;
     const int w0 = min(wid * seg, n), w1 = min(w0 + seg, n);
     const uint32_t top = lo + lim;
-    SelCtl *lead = cluster.map_shared_rank(&ctl, 0);
     {
         int cgt = 0, ceq = 0;
         for (int base = w0; base < w1; base += 32) {
@@ -365,20 +376,25 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
             const uint32_t votes = __ballot_sync(0xffffffffu, hit);
             if (votes) {
                 int at = 0;
-                if (lane == 0) at = atomicAdd(&lead->cand_count, __popc(votes));
+                if (lane == 0) at = atomicAdd(&ctl.cand_count, __popc(votes));
                 at = __shfl_sync(0xffffffffu, at, 0) + __popc(votes & ((1u << lane) - 1u));
-                if (hit && JQ_IN(at, kCandMax, kDbgSelect, 15)) { lead->cand_key[at] = k; lead->cand_pos[at] = j0 + e; }
+                if (hit && JQ_IN(at, kCandMax, kDbgSelect, 15)) { lists[kOwnKey + at] = k; lists[kOwnPos + at] = (uint32_t)(j0 + e); }
             }
         }
         cgt = __reduce_add_sync(0xffffffffu, cgt);
         ceq = __reduce_add_sync(0xffffffffu, ceq);
         if (lane == 0) { ctl.warp_gt[wid] = cgt; ctl.warp_eq[wid] = listed ? 0 : ceq; }
         __syncthreads();
+        if (listed && nc <= kRankMax && wid < CL) {                  // warp q sends this CTA's list to CTA q
+            uint32_t *to = cluster.map_shared_rank(lists, wid) + rank * kRankMax;
+            for (int i = lane; i < ctl.cand_count; i += 32)
+                if (JQ_IN(i, kRankMax, kDbgSelect, 34)) { to[kAllKey + i] = lists[kOwnKey + i]; to[kAllPos + i] = lists[kOwnPos + i]; }
+        }
         if (wid == 0) {
             const int g = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? ctl.warp_gt[lane] : 0), q = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? ctl.warp_eq[lane] : 0);
             if (lane < CL) {
                 SelCtl *rc = cluster.map_shared_rank(&ctl, lane);
-                rc->gt_of[rank] = g; rc->eq_of[rank] = q;
+                rc->gt_of[rank] = g; rc->eq_of[rank] = q; rc->cand_of[rank] = ctl.cand_count;
             }
         }
         if (tid == 0) { ctl.base_gt = ctl.base_eq = 0; }
@@ -387,25 +403,72 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     uint32_t tau = lo;
     int need_eq = need;             // how many of the keys == tau are kept (lowest positions first)
     if (listed) {
-        if (tid < nc) { ctl.my_key[tid] = lead->cand_key[tid]; ctl.my_pos[tid] = lead->cand_pos[tid]; }
-        __syncthreads();
-        if (tid < nc) {
-            const uint32_t k = ctl.my_key[tid];
-            int gt = 0, eq = 0;
+        // Every CTA brings the lists together for itself, 16 / CL warps each.  (One list in the leading CTA, appended to by all,
+        // cost a round trip between the CTAs for every group of 32 keys that had one.)
+        const uint32_t *const list = lists + (nc <= kRankMax ? kOwnKey : kAllKey);
+        {
+            const int q = wid & (CL - 1), have = lane < CL ? ctl.cand_of[lane] : 0;
+            const int before = __reduce_add_sync(0xffffffffu, lane < q ? have : 0), mine = __shfl_sync(0xffffffffu, have, q);
+            const int i0 = wid / CL * 32 + lane, step = kSelWarps / CL * 32;
+            if (nc <= kRankMax) {
+                for (int i = i0; i < mine; i += step)
+                    if (JQ_IN(before + i, kCandMax, kDbgSelect, 16)) {
+                        lists[kOwnKey + before + i] = lists[kAllKey + q * kRankMax + i];
+                        lists[kOwnPos + before + i] = lists[kAllPos + q * kRankMax + i];
+                    }
+            } else {
+                const uint32_t *from = cluster.map_shared_rank(lists, q);
 #pragma unroll 4
-            for (int i = 0; i < nc; ++i) { const uint32_t x = ctl.my_key[i]; gt += x > k; eq += x == k; }
-            if (gt < need && need <= gt + eq) { ctl.tau = k; ctl.need_eq = need - gt; }   // (equal keys write the same)
+                for (int i = i0; i < mine; i += step)
+                    if (JQ_IN(before + i, kCandMax, kDbgSelect, 35)) {
+                        lists[kAllKey + before + i] = from[kOwnKey + i];
+                        lists[kAllPos + before + i] = from[kOwnPos + i];
+                    }
+            }
         }
         __syncthreads();
-        tau = ctl.tau;
-        need_eq = ctl.need_eq;
-        if (tid < nc) {
-            const uint32_t k = ctl.my_key[tid];
-            const int at = ctl.my_pos[tid];
-            if (k >= tau && at < j0) atomicAdd(k > tau ? &ctl.base_gt : &ctl.base_eq, 1);
-            else if (k >= tau && at < j1) {
+        if (nc <= kRankMax) {
+            if (tid < nc) {
+                const uint32_t k = list[tid];
+                int gt = 0, eq = 0;
+#pragma unroll 4
+                for (int i = 0; i < nc; ++i) { const uint32_t x = list[i]; gt += x > k; eq += x == k; }
+                if (gt < need && need <= gt + eq) { ctl.tau = k; ctl.need_eq = need - gt; }   // (equal keys write the same)
+            }
+            __syncthreads();
+            tau = ctl.tau;
+            need_eq = ctl.need_eq;
+        } else {
+            // at most two rounds of bins over the list (the bin spans 21 bits at most), in this CTA alone
+            for (;;) {
+                const int sh = lim >> 11 ? 21 - __clz(lim) : 0;
+                for (int i = tid; i < nc; i += kSelThreads) {
+                    const uint32_t k = list[i] - lo;
+                    if (k <= lim && JQ_IN(k >> sh, kBins, kDbgSelect, 33)) atomicAdd(&hist[k >> sh], 1u);
+                }
+                __syncthreads();
+                uint4 *const mine = (uint4 *)(hist + kBins - 4 - 4 * tid);
+                const uint4 v = *mine;
+                *mine = make_uint4(0u, 0u, 0u, 0u);
+                find_bin(v, need, ctl);
+                lo += (uint32_t)ctl.digit << sh;
+                need = ctl.krem;
+                if (sh == 0) break;
+                lim = (1u << sh) - 1u;
+            }
+            tau = lo;
+            need_eq = need;
+        }
+        // the kept and tied keys among them before this CTA's share, and of this CTA's warps
+        for (int i = tid; i - lane < nc; i += kSelThreads) {
+            const uint32_t k = i < nc ? list[i] : 0u;
+            const int at = i < nc ? (int)list[kCandMax + i] : L;
+            const uint32_t bg = __ballot_sync(0xffffffffu, at < j0 && k > tau), be = __ballot_sync(0xffffffffu, at < j0 && k == tau);
+            if (lane == 0 && bg) atomicAdd(&ctl.base_gt, __popc(bg));
+            if (lane == 0 && be) atomicAdd(&ctl.base_eq, __popc(be));
+            if (k >= tau && at >= j0 && at < j1) {
                 const int w = (at - j0) / seg;
-                if (JQ_IN(w, kSelWarps, kDbgSelect, 16)) atomicAdd(k > tau ? &ctl.warp_gt[w] : &ctl.warp_eq[w], 1);
+                if (JQ_IN(w, kSelWarps, kDbgSelect, 20)) atomicAdd(k > tau ? &ctl.warp_gt[w] : &ctl.warp_eq[w], 1);
             }
         }
         __syncthreads();
@@ -433,8 +496,8 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
             gt_before += __popc(bg);
             eq_before += __popc(be);
         }
-    // ---- 4. the rows, once every index of the head has been written.  (Without rows the cluster still leaves together: the
-    // leading CTA's list may be being read.)
+    // ---- 4. the rows, once every index of the head has been written.  (Without rows the cluster still leaves together: a
+    // CTA's list may be being read.)
     cluster.sync();                 // (release and acquire at cluster scope: the readers are in the cluster)
     if (!Kin) return;
     copy_rows(out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
@@ -785,7 +848,7 @@ SelPlan plan_for(int L, int cl)
     p.chunk = ((L + cl - 1) / cl + 31) / 32 * 32;
     p.in_smem = p.chunk <= kKeysSmemMax;
     p.raw_tile = p.chunk < kRawTile ? p.chunk : kRawTile;
-    p.smem = (size_t)(kOwnBins + kBins + p.raw_tile + 2 * kHalo) * 4 + (p.in_smem ? (size_t)p.chunk * 4 : 0);
+    p.smem = (size_t)(kOwnBins + kBins + raw_words(p.raw_tile)) * 4 + (p.in_smem ? (size_t)p.chunk * 4 : 0);
     return p;
 }
 
@@ -818,7 +881,7 @@ bool sel_device(SelDevice *out)
     std::lock_guard<std::mutex> lock(mu);
     SelDevice &d = devs[dev];
     if (!d.ready) {
-        const int max_smem = (kOwnBins + kBins + kRawTile + 2 * kHalo + kKeysSmemMax) * 4;
+        const int max_smem = (kOwnBins + kBins + raw_words(kRawTile) + kKeysSmemMax) * 4;
         if (cudaFuncSetAttribute(select_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) return false;
         if (cudaFuncSetAttribute(select_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
         for (int i = 0; i < 4; ++i)

@@ -134,6 +134,26 @@ def test_select_many_heads_bit_exact(Hkv, L, B, p, kind):
     assert np.array_equal(got_idx, want_idx)
 
 
+# Keys in the threshold's bin on either side of what is ranked by comparison (64), of what is listed (1024), and, with equal
+# keys, of what further bins can tell apart; clusters of 16, 8, 4 and 2 CTAs, and lists that come from one CTA alone.
+@pytest.mark.parametrize("Hkv,L,p", [(2, 20000, 1), (8, 60000, 1), (60, 9001, 5), (127, 30011, 1)])
+@pytest.mark.parametrize("near", [63, 64, 65, 1023, 1024, 1025, 3000])
+@pytest.mark.parametrize("kind", ["spread", "together", "equal"])
+def test_select_with_many_keys_in_the_bin(Hkv, L, p, near, kind):
+    rng = np.random.default_rng(L + near)
+    s32 = rng.random((Hkv, L), dtype=np.float32) * 1e-6
+    for h in range(Hkv):
+        at = np.arange(100, 100 + near) if kind == "together" else rng.choice(L, near, replace=False)
+        # within 2^-12 of one another, when the bins of the range [1e-13, 1) are 2^-6 wide
+        s32[h, at] = 0.5 if kind == "equal" else 0.5 + rng.random(near, dtype=np.float32) * 2.0 ** -12
+        s32[h, (L - 1 - h) // 2] = 0.9
+    B = near // 2
+    want_idx, want_pooled = oracle.select_f32(s32, B, p)
+    got_idx, got_pooled = gpu_select(s32, jq.shape(Hkv, Hkv, L, 1, B, p))
+    assert np.array_equal(got_pooled.view(np.uint32), want_pooled.view(np.uint32))
+    assert np.array_equal(got_idx, want_idx)
+
+
 @pytest.mark.parametrize("Hkv", [2, 150])
 def test_select_all_equal_keeps_lowest_indices(Hkv):
     s32 = np.full((Hkv, 5000), 0.25, np.float32)
