@@ -502,12 +502,23 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 pooled_quad(a, b, nx, P.radius, k, best);
                 a = b; b = nx;
             } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) best[e] = scores[4 * q + e - P.radius];
+                // The four windows share the positions [4q + 3 - radius, 4q + radius], taken as whole quads and what is left of
+                // them on either side; each window then has three more of its own.  (The halo is at least as wide as the radius.)
+                const int from = 4 * q + 3 - P.radius, to = 4 * q + P.radius, qa = (from + 3) >> 2, qb = (to + 1) >> 2;
+                float4 c4 = s4[qa];
 #pragma unroll 1
-                for (int o = 1 - P.radius; o <= P.radius; ++o)            // (the halo is at least as wide as the radius)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) best[e] = fmaxf(best[e], scores[4 * q + e + o]);
+                for (int x = qa + 1; x < qb; ++x) {
+                    const float4 v = s4[x];
+                    c4 = make_float4(fmaxf(c4.x, v.x), fmaxf(c4.y, v.y), fmaxf(c4.z, v.z), fmaxf(c4.w, v.w));
+                }
+                float core = fmaxf(max3f(c4.x, c4.y, c4.z), c4.w);
+                for (int j = from; j < 4 * qa; ++j) core = fmaxf(core, scores[j]);
+                for (int j = 4 * qb; j <= to; ++j) core = fmaxf(core, scores[j]);
+                const float l2 = fmaxf(scores[from - 2], scores[from - 1]), r1 = scores[to + 1], r2 = fmaxf(r1, scores[to + 2]);
+                best[0] = max3f(core, l2, scores[from - 3]);
+                best[1] = max3f(core, l2, r1);
+                best[2] = max3f(core, scores[from - 1], r2);
+                best[3] = max3f(core, r2, scores[to + 3]);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) k[e] = order_key(best[e]);
             }
@@ -752,8 +763,10 @@ bool fused_layout(int L, int nkeep, int C, int nt, FParams *P, size_t *smem)
 // (us per call, back to back).  This kernel: a chain of exchanges, the tiles of a CTA one after the other, and the selection,
 // which every CTA runs over the whole head; clusters that do not fit at a time take turns (of 16 CTAs 7 fit, of 10 11).
 // 8 heads x 1024, 2048, 4096, 8192, 12000 keys in clusters of 8: 10.1, 11.9, 17.9, 29.4, 38.1; of 10: -, 12.3, 17.9, 27.2,
-// 34.7; of 4: 11.4, 14.8, 24.4, 40.1, 54.3; with 256 rows 4096 and 8192 keys 24.9, 40.6; 24.9, 37.3; 35.2, 62.0.  The two kernels of the general path,
-// by tiles in all: 64, 256, 512, 752, 1024: 22.6, 26.7, 32.3, 35.6, 41; with 256 rows 128, 256, 512: 27.0, 30.8, 39.2.
+// 34.7; of 4: 11.4, 14.8, 24.4, 40.1, 54.3; with 256 rows 4096 and 8192 keys 24.9, 40.6; 24.9, 37.3; 35.2, 62.0.  A window
+// wider than 9 adds 0.5 us per 1000 keys: 8 x 4096, 8192, 12000 keys, pool 63: 20.4, 31.3, 39.7.
+// The two kernels of the general path, by tiles in all: 64, 256, 512, 752, 1024: 22.6, 26.7, 32.3, 35.6, 41; with 256 rows
+// 128, 256, 512: 27.0, 30.8, 39.2.
 static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FParams *P, size_t *smem)
 {
     FusedDevice dev;
@@ -769,7 +782,8 @@ static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FPar
         FParams T = *P;
         size_t sm;
         if (!fused_layout(s.L, nkeep, C, nt, &T, &sm)) continue;
-        const double cost = (double)((s.Hkv + dev.resident[C] - 1) / dev.resident[C]) * (chain + per_tile * nt + (C > 8 ? 1.04e-3 : 1.24e-3) * s.L);
+        const double per_key = (C > 8 ? 1.04e-3 : 1.24e-3) + (s.pool > 9 ? 0.5e-3 : 0.0);
+        const double cost = (double)((s.Hkv + dev.resident[C] - 1) / dev.resident[C]) * (chain + per_tile * nt + per_key * s.L);
         if (cost < best_cost) { best_cost = cost; best = C; *P = T; *smem = sm; }
     }
     // (the general path appends and moves back with strided copies, two of each, about 4.5 us a piece)

@@ -55,6 +55,22 @@ def test_layer_in_one_launch(Hkv, g, w, L, budget, pool):
         assert np.array_equal(gK[kv], K[kv][gi[kv]]) and np.array_equal(gV[kv], V[kv][gi[kv]])
 
 
+# windows wider than nine: every remainder of the radius modulo the quad, windows wider than the prefix, prefixes that end
+# anywhere in a quad
+@pytest.mark.parametrize("pool", [11, 13, 15, 17, 19, 31, 61, 63])
+@pytest.mark.parametrize("L,budget", [(3, 2), (30, 7), (1027, 200), (4098, 999)])
+def test_wide_pools_in_one_launch(pool, L, budget):
+    wl = wl_of(2, 4, 8, L, budget, pool)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    Ko, Vo, idx = outputs(2, budget, budget)
+    n0 = jq.launch_count()
+    jq.evict_layer(dev_bf16(K), dev_bf16(V), dev_bf16(Q), s, Ko, Vo, idx, jq.new_workspace(s))
+    assert jq.launch_count() - n0 == 1
+    pooled = oracle.pool(oracle.score(K, Q), pool)
+    assert_kept_sets_agree(idx.cpu().numpy(), oracle.select(pooled, budget), pooled, budget)
+
+
 @pytest.mark.parametrize("L,budget", [(700, 100), (4096, 513), (9000, 2048)])
 def test_tied_scores_keep_the_lowest_positions(L, budget):
     """Equal keys give equal scores: with Q = 0 every pooled score is the same number, and the first `budget` positions stay."""
