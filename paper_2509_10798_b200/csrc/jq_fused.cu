@@ -765,8 +765,12 @@ bool fused_layout(int L, int nkeep, int C, int nt, FParams *P, size_t *smem)
 // 8 heads x 1024, 2048, 4096, 8192, 12000 keys in clusters of 8: 10.1, 11.9, 17.9, 29.4, 38.1; of 10: -, 12.3, 17.9, 27.2,
 // 34.7; of 4: 11.4, 14.8, 24.4, 40.1, 54.3; with 256 rows 4096 and 8192 keys 24.9, 40.6; 24.9, 37.3; 35.2, 62.0.  A window
 // wider than 9 adds 0.5 us per 1000 keys: 8 x 4096, 8192, 12000 keys, pool 63: 20.4, 31.3, 39.7.
-// The two kernels of the general path, by tiles in all: 64, 256, 512, 752, 1024: 22.6, 26.7, 32.3, 35.6, 41; with 256 rows
-// 128, 256, 512: 27.0, 30.8, 39.2.
+// The two kernels of the general path: launches and merge, the tiles of all SMs (past about ten each the next group of heads
+// hides the merge), a little per head and per 1000 keys of a head for the selection, and a step at 128 heads, where the other
+// selection kernel takes over.  32, 64, 128, 256 heads x 3000 keys: 37.0, 49.3, 88.4, 136.8 (this kernel 23.7, 36.6, 63.7,
+// 128.1); x 8192 51.3, 80.7, 150.2, 269.1 (43.5, 72.6, 135.5, 269.3); x 12000 60.9, 102, 204 (58.3, 98.6, 188); with 256 rows
+// x 8192 65.8, 110, 214, 400 (65.5, 116, 236, 489).  160 x 3000: 105 (112), 512 x 1000: 156 (111).  Over 412 calls of 1 to 512
+// heads, 100 to 12000 keys, 8 to 256 rows the rule's choice takes 0.2 % longer than the better one, at most 9 %.
 static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FParams *P, size_t *smem)
 {
     FusedDevice dev;
@@ -787,7 +791,10 @@ static int fused_plan(const jq_shape &s, const FusedSource &src, int nkeep, FPar
         if (cost < best_cost) { best_cost = cost; best = C; *P = T; *smem = sm; }
     }
     // (the general path appends and moves back with strided copies, two of each, about 4.5 us a piece)
-    const double other = (wide ? 23.5 : 22.5) + (wide ? 0.03 : 0.0185) * s.Hkv * TT + (src.LB > 0 ? 9.0 : 0.0) + (src.inplace ? 9.0 : 0.0);
+    const double tiles = (double)s.Hkv * (TT + win), first = tiles < 1500.0 ? tiles : 1500.0, rest = tiles - first;
+    const double other = (wide ? 23.5 + 0.02 * first + 0.014 * rest + 0.06 * s.Hkv
+                               : 22.5 + (0.0115 * first + 0.0095 * rest) * (0.87 + 0.13 * P->Rpad / 128) + 0.04 * s.Hkv) +
+                         (s.Hkv >= 128 ? 8.0 : 0.0) + 0.25e-3 * s.L + (src.LB > 0 ? 9.0 : 0.0) + (src.inplace ? 9.0 : 0.0);
     return best_cost <= other ? best : 0;
 }
 

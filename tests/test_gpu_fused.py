@@ -163,3 +163,27 @@ def test_host_call_in_chunks(Hkv, g, w, L, budget, pageable):
     assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
     for kv in range(Hkv):
         assert np.array_equal(hKo.numpy().view(np.uint16)[kv], K[kv][gi[kv]]) and np.array_equal(hVo.numpy().view(np.uint16)[kv], V[kv][gi[kv]])
+
+
+# one launch where it is the faster way: few heads or short prefixes; two where the rows are many or the heads leave most of
+# the GPU's last round idle
+@pytest.mark.parametrize("Hkv,g,w,L,launches", [(8, 4, 32, 8192, 1), (128, 4, 32, 8192, 1), (512, 4, 32, 1000, 1), (128, 4, 64, 8192, 2), (160, 4, 32, 3000, 2),
+                                                (300, 4, 64, 5000, 2), (8, 4, 32, 12289, 2)])
+def test_calls_over_many_heads_take_the_faster_way(Hkv, g, w, L, launches):
+    """... and both give what the stages give one by one (here their scores stand in for the oracle's)."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(L)
+    K, V = (torch.randn((Hkv, L, 128), generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    Q = torch.randn((Hkv * g, w, 128), generator=gen, device="cuda", dtype=torch.bfloat16)
+    s = jq.shape(Hkv, Hkv * g, L, w, 300)
+    Ko, Vo, idx = outputs(Hkv, 300, 300)
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer(K, V, Q, s, Ko, Vo, idx, ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK and jq.launch_count() - n0 == launches
+    scores, pooled, want = torch.empty((Hkv, L), device="cuda"), torch.empty((Hkv, L), device="cuda"), torch.empty_like(idx)
+    jq.score(K, Q, s, scores, ws)
+    jq.select_topk(scores, s, want, ws, pooled=pooled)
+    assert_kept_sets_agree(idx.cpu().numpy(), want.cpu().numpy(), pooled.cpu().numpy().astype(np.float64), 300)
+    at = idx.long()[:, :, None].expand(-1, -1, 128)
+    assert torch.equal(Ko.view(torch.int16), K.gather(1, at).view(torch.int16)) and torch.equal(Vo.view(torch.int16), V.gather(1, at).view(torch.int16))
