@@ -639,7 +639,6 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     int kv_in = kv;
     long long soff = (long long)kv * L, orow = (long long)kv * nkeep, krow = (long long)kv * out_rows;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
-    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
     if (htab) {
         const HeadRec r = htab[kv];
         L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; orow = r.ooff; krow = r.ooff; src_rows = L;
