@@ -175,6 +175,26 @@ __device__ __forceinline__ void find_bin(const uint32_t *h, int krem, FCtl *ctl)
     group_sync();
 }
 
+// Pooled values of quad q for a radius above 4 (out of line: the loop around it is fetched faster without).  The four windows
+// share the positions [4q + 3 - radius, 4q + radius], taken as whole quads and what is left of them on either side; each
+// window then has three more of its own.  (The halo is at least as wide as the radius.)
+__device__ __noinline__ float4 pool_wide(const float *scores, int q, int radius)
+{
+    const float4 *s4 = (const float4 *)scores;
+    const int from = 4 * q + 3 - radius, to = 4 * q + radius, qa = (from + 3) >> 2, qb = (to + 1) >> 2;
+    float4 c = s4[qa];
+#pragma unroll 1
+    for (int x = qa + 1; x < qb; ++x) {
+        const float4 v = s4[x];
+        c = make_float4(fmaxf(c.x, v.x), fmaxf(c.y, v.y), fmaxf(c.z, v.z), fmaxf(c.w, v.w));
+    }
+    float core = fmaxf(max3f(c.x, c.y, c.z), c.w);
+    for (int j = from; j < 4 * qa; ++j) core = fmaxf(core, scores[j]);
+    for (int j = 4 * qb; j <= to; ++j) core = fmaxf(core, scores[j]);
+    const float l2 = fmaxf(scores[from - 2], scores[from - 1]), r1 = scores[to + 1], r2 = fmaxf(r1, scores[to + 2]);
+    return make_float4(max3f(core, l2, scores[from - 3]), max3f(core, l2, r1), max3f(core, scores[from - 1], r2), max3f(core, r2, scores[to + 3]));
+}
+
 __global__ void __launch_bounds__(kFThreads, 1)
 evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
             const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapW, const __grid_constant__ FParams P)
@@ -502,23 +522,8 @@ evict_fused(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 pooled_quad(a, b, nx, P.radius, k, best);
                 a = b; b = nx;
             } else {
-                // The four windows share the positions [4q + 3 - radius, 4q + radius], taken as whole quads and what is left of
-                // them on either side; each window then has three more of its own.  (The halo is at least as wide as the radius.)
-                const int from = 4 * q + 3 - P.radius, to = 4 * q + P.radius, qa = (from + 3) >> 2, qb = (to + 1) >> 2;
-                float4 c4 = s4[qa];
-#pragma unroll 1
-                for (int x = qa + 1; x < qb; ++x) {
-                    const float4 v = s4[x];
-                    c4 = make_float4(fmaxf(c4.x, v.x), fmaxf(c4.y, v.y), fmaxf(c4.z, v.z), fmaxf(c4.w, v.w));
-                }
-                float core = fmaxf(max3f(c4.x, c4.y, c4.z), c4.w);
-                for (int j = from; j < 4 * qa; ++j) core = fmaxf(core, scores[j]);
-                for (int j = 4 * qb; j <= to; ++j) core = fmaxf(core, scores[j]);
-                const float l2 = fmaxf(scores[from - 2], scores[from - 1]), r1 = scores[to + 1], r2 = fmaxf(r1, scores[to + 2]);
-                best[0] = max3f(core, l2, scores[from - 3]);
-                best[1] = max3f(core, l2, r1);
-                best[2] = max3f(core, scores[from - 1], r2);
-                best[3] = max3f(core, r2, scores[to + 3]);
+                const float4 w = pool_wide(scores, q, P.radius);
+                best[0] = w.x; best[1] = w.y; best[2] = w.z; best[3] = w.w;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) k[e] = order_key(best[e]);
             }
