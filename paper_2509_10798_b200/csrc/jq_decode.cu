@@ -60,10 +60,12 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p)   // read once: not kept in the L1
+// Read once: not kept in the L1.  (Not through the read-only path, which is for data that nobody writes during the kernel's
+// life: the kernel may be set up while the one that writes the cache still runs.)
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)   // lo in the low half
@@ -91,7 +93,7 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t v)   // 8 x 8 matrix o
 // carries two of the three parts of P.
 template <bool DUP>
 __global__ void __launch_bounds__(kDecThreads, kDecResident)
-decode_step(const uint4 *__restrict__ Kc, const uint4 *__restrict__ Vc, const __nv_bfloat16 *__restrict__ q, int n,
+decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
             int group, float scale_log2, float *__restrict__ out JQ_DBG_PARAM)
 {
     extern __shared__ __align__(16) uint8_t dec_raw[];

@@ -8,8 +8,10 @@ namespace {
 
 constexpr int kVecPerRow = kD * 2 / 16;  // 16 uint4 per bf16 row of 128
 
+// (The inputs are not __restrict__: the kernel may be set up while the one that writes them still runs, and the read-only
+// path is for data that nobody writes during the kernel's life.)
 __global__ void __launch_bounds__(256)
-gather_rows(const uint4 *__restrict__ K, const uint4 *__restrict__ V, const int32_t *__restrict__ idx,
+gather_rows(const uint4 *K, const uint4 *V, const int32_t *idx,
             int L, int nkeep, long long nrows, uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, int Hkv JQ_DBG_PARAM)
 {
     cudaGridDependencySynchronize();             // set up while the kernel before it in the stream was finishing

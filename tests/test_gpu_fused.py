@@ -165,6 +165,44 @@ def test_host_call_in_chunks(Hkv, g, w, L, budget, pageable):
         assert np.array_equal(hKo.numpy().view(np.uint16)[kv], K[kv][gi[kv]]) and np.array_equal(hVo.numpy().view(np.uint16)[kv], V[kv][gi[kv]])
 
 
+def test_each_kernel_sees_what_the_one_before_it_wrote():
+    """Re-eviction in place, decoding over the cache, selection, and a copy by the positions it kept, queued back to back
+    round after round: every result is what the same calls give one at a time."""
+    Hkv, g, w, n, new = 8, 4, 16, 512, 96
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    rnd = lambda *sh: torch.randn(sh, generator=gen, device="cuda", dtype=torch.bfloat16)
+    s = jq.shape(Hkv, Hkv * g, n + new, w, n)
+    s2 = jq.shape(Hkv, Hkv * g, n, w, 100)
+    rounds = [(rnd(Hkv, new, 128), rnd(Hkv, new, 128), rnd(Hkv * g, w, 128), rnd(Hkv * g, 128), torch.rand((Hkv, n), generator=gen, device="cuda")) for _ in range(40)]
+    K0, V0 = rnd(Hkv, n + new, 128), rnd(Hkv, n + new, 128)
+    ws, ws2 = jq.new_append_workspace(s), jq.new_workspace(s2)
+    wsd = torch.empty(jq.decode_workspace_bytes(Hkv, Hkv * g, n), dtype=torch.uint8, device="cuda")
+
+    def run(step_by_step):
+        Kc, Vc = K0.clone(), V0.clone()
+        outs = [tuple(torch.zeros(sh, dtype=t, device="cuda") for sh, t in (((Hkv, n), torch.int32), ((Hkv * g, 128), torch.float32),
+                ((Hkv, 100), torch.int32), ((Hkv, 100, 128), torch.bfloat16), ((Hkv, 100, 128), torch.bfloat16))) for _ in rounds]
+        packed = torch.empty((2, Hkv, n, 128), dtype=torch.bfloat16, device="cuda")
+        torch.cuda.synchronize()
+        for (Kn, Vn, Q, q, sc), (idx, out, idx2, Ko, Vo) in zip(rounds, outs):
+            for call in (lambda: jq.evict_append(Kc, Vc, n, Kn, Vn, Q, s, idx, ws), lambda: jq.compact_kv(Kc, Vc, first, s, packed[0], packed[1]),
+                         lambda: jq.decode_attention(packed[0], packed[1], q, out, wsd), lambda: jq.select_topk(sc, s2, idx2, ws2),
+                         lambda: jq.compact_kv(packed[0], packed[1], idx2, s2, Ko, Vo)):
+                call()
+                if step_by_step:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert jq.last_device_status(ws) == jq.JQ_OK
+        return [t for o in outs for t in o]
+
+    first = torch.arange(n, dtype=torch.int32, device="cuda")[None].expand(Hkv, n).contiguous()
+    want = run(True)
+    for _ in range(3):
+        for a, b in zip(run(False), want):
+            assert torch.equal(a, b)
+
+
 # one launch where it is the faster way: few heads or short prefixes; two where the rows are many or the heads leave most of
 # the GPU's last round idle
 @pytest.mark.parametrize("Hkv,g,w,L,launches", [(8, 4, 32, 8192, 1), (128, 4, 32, 8192, 1), (512, 4, 32, 1000, 1), (128, 4, 64, 8192, 2), (160, 4, 32, 3000, 2),

@@ -61,3 +61,15 @@ def test_the_one_launch_pass_stays_in_bounds_after_a_wait_that_ran_out():
     assert "int t = min(max((before & 0xffff) + min(eb, need_eq), 0), P.nkeep)" in body
     assert body.count("list[t] = ") == 2 and "for (int t = tid; t < P.nkeep; t += kFT) list[t] = t;" in body
     assert body.count("min(max(list[t0r + i") == 2     # and so are the positions that rows are read at
+
+
+@pytest.mark.parametrize("name", ["decode_step", "gather_rows"])
+def test_what_the_kernel_before_may_still_write_is_not_read_as_read_only(name):
+    """These two read what the kernel right before them in the stream has written (the pruned cache, the kept positions) and
+    may be set up while it runs: their inputs do not go through the read-only path, which is for data that nobody writes
+    during a kernel's life."""
+    params, body = KERNELS[name]
+    assert "cudaGridDependencySynchronize" in body
+    assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", params) and "__ldg" not in body
+    with open(os.path.join(CSRC, {"decode_step": "jq_decode.cu", "gather_rows": "jq_gather.cu"}[name])) as f:
+        assert "ld.global.nc" not in f.read()
