@@ -166,15 +166,17 @@ def _calls():
             from . import _jqcall
         except ImportError as e:
             raise RuntimeError("_jqcall is not built: run `python -m paper_2509_10798_b200.build` (%s)" % e) from e
-        _jqcall.bind({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in EXPORTS}, _stream_lookup())
+        _jqcall.bind({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in EXPORTS}, _stream_lookup(), JqShape)
         _fast = _jqcall
     return _fast
 
 
 def _stream_lookup():
-    """A callable that gives the current stream of the current device as an integer."""
-    C = _torch()._C
-    device, raw = C._cuda_getDevice, C._cuda_getCurrentRawStream
+    """A callable that gives the current stream of the current device as an integer (without a device it raises)."""
+    import torch
+    if not torch.cuda.is_available():
+        return _torch
+    device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
     return lambda: raw(device())
 
 

@@ -28,6 +28,7 @@ static struct {
 
 static PyObject *s_data_ptr, *s_numel, *s_element_size, *s_shape, *s_cuda_stream;
 static PyObject *raw_stream;   /* callable: the current CUDA stream of the current device, as an integer */
+static PyObject *shape_type;   /* JqShape */
 
 static const struct { const char *name; void **slot; } slots[] = {
     {"jq_score", (void **)&jq.score}, {"jq_score_fma", (void **)&jq.score_fma}, {"jq_select_topk", (void **)&jq.select_topk},
@@ -37,11 +38,11 @@ static const struct { const char *name; void **slot; } slots[] = {
     {"jq_evict_append", (void **)&jq.evict_append}, {"jq_decode_attention", (void **)&jq.decode_attention},
 };
 
-/* bind(addresses, raw_stream): the entry points' addresses by name, and the stream lookup. */
+/* bind(addresses, raw_stream, shape_type): the entry points' addresses by name, the stream lookup, the class of a shape. */
 static PyObject *bind(PyObject *self, PyObject *args)
 {
-    PyObject *d, *fn;
-    if (!PyArg_ParseTuple(args, "O!O", &PyDict_Type, &d, &fn)) return NULL;
+    PyObject *d, *fn, *cls;
+    if (!PyArg_ParseTuple(args, "O!OO!", &PyDict_Type, &d, &fn, &PyType_Type, &cls)) return NULL;
     for (size_t i = 0; i < sizeof slots / sizeof *slots; ++i) {
         PyObject *a = PyDict_GetItemString(d, slots[i].name);
         if (!a) { PyErr_Format(PyExc_KeyError, "%s", slots[i].name); return NULL; }
@@ -51,9 +52,20 @@ static PyObject *bind(PyObject *self, PyObject *args)
     }
     Py_INCREF(fn);
     Py_XSETREF(raw_stream, fn);
+    Py_INCREF(cls);
+    Py_XSETREF(shape_type, cls);
     Py_RETURN_NONE;
 }
 
+/* What int(o) gives, as a C int (as ctypes takes it: the low bits). */
+static int to_int(PyObject *o, int *out)
+{
+    PyObject *v = PyNumber_Long(o);
+    if (!v) return -1;
+    *out = (int)PyLong_AsUnsignedLongMask(v);
+    Py_DECREF(v);
+    return 0;
+}
 /* Integer result of a method without arguments; -1 with an exception set on failure. */
 static long long ask(PyObject *o, PyObject *method)
 {
@@ -63,22 +75,35 @@ static long long ask(PyObject *o, PyObject *method)
     Py_DECREF(r);
     return v;
 }
-/* A tensor's address; None is a null pointer. */
+/* A tensor's address. */
+static int address(PyObject *o, void **p)
+{
+    PyObject *r = PyObject_CallMethodNoArgs(o, s_data_ptr);
+    if (!r) return -1;
+    *p = PyLong_AsVoidPtr(r);
+    Py_DECREF(r);
+    return !*p && PyErr_Occurred() ? -1 : 0;
+}
+/* The same; None is a null pointer. */
 static int ptr(PyObject *o, void **p)
 {
     *p = NULL;
-    if (o == Py_None) return 0;
-    PyObject *r = PyObject_CallMethodNoArgs(o, s_data_ptr);
-    if (!r) return -1;
-    *p = (void *)(uintptr_t)PyLong_AsUnsignedLongLong(r);
-    Py_DECREF(r);
-    return PyErr_Occurred() ? -1 : 0;
+    return o == Py_None ? 0 : address(o, p);
 }
+/* Bytes of a workspace: its elements (a workspace is made of bytes; of another type it has to hold as many elements). */
 static int bytes_of(PyObject *ws, size_t *n)
 {
-    const long long e = ask(ws, s_numel), k = e < 0 && PyErr_Occurred() ? -1 : ask(ws, s_element_size);
-    if (PyErr_Occurred()) return -1;
-    *n = (size_t)(e * k);
+    const long long e = ask(ws, s_numel);
+    if (e == -1 && PyErr_Occurred()) return -1;
+    *n = (size_t)e;
+    return 0;
+}
+/* Bytes of a decoding workspace, of any type. */
+static int size_of(PyObject *ws, size_t *n)
+{
+    const long long k = ask(ws, s_element_size);
+    if ((k == -1 && PyErr_Occurred()) || bytes_of(ws, n)) return -1;
+    *n *= (size_t)k;
     return 0;
 }
 static int dim(PyObject *t, Py_ssize_t i, int *out)
@@ -88,15 +113,17 @@ static int dim(PyObject *t, Py_ssize_t i, int *out)
     PyObject *v = PySequence_GetItem(sh, i);
     Py_DECREF(sh);
     if (!v) return -1;
-    const long x = PyLong_AsLong(v);
+    const int bad = to_int(v, out);
     Py_DECREF(v);
-    if (x == -1 && PyErr_Occurred()) return -1;
-    *out = (int)x;
-    return 0;
+    return bad;
 }
 static int shape_of(PyObject *s, jq_shape *out)
 {
     Py_buffer b;
+    if (!PyObject_TypeCheck(s, (PyTypeObject *)shape_type)) {
+        PyErr_Format(PyExc_TypeError, "expected a JqShape, got %.100s", Py_TYPE(s)->tp_name);
+        return -1;
+    }
     if (PyObject_GetBuffer(s, &b, PyBUF_SIMPLE)) return -1;
     const int ok = b.len == (Py_ssize_t)sizeof *out;
     if (ok) *out = *(const jq_shape *)b.buf;
@@ -108,7 +135,7 @@ static int stream_of(PyObject *o, jq_stream_t *out)
 {
     PyObject *r = o == Py_None ? PyObject_CallNoArgs(raw_stream) : PyObject_GetAttr(o, s_cuda_stream);
     if (!r) return -1;
-    *out = (jq_stream_t)(uintptr_t)PyLong_AsUnsignedLongLong(r);
+    *out = (jq_stream_t)PyLong_AsVoidPtr(r);
     Py_DECREF(r);
     return PyErr_Occurred() ? -1 : 0;
 }
@@ -182,46 +209,43 @@ FN(evict_layer_window_kept)
 /* Kc, Vc, n_old, Knew, Vnew, Qrecent, shape, idx, ws, stream */
 FN(evict_append)
 {
-    void *p[2], *q[3], *o[2]; size_t wb; jq_shape s; jq_stream_t st; int cap, n_new = 0;
-    if (want(n, 10) || ptrs(a, 2, p) || dim(a[0], 1, &cap) || ptrs(a + 3, 3, q) || (a[3] != Py_None && dim(a[3], 1, &n_new)) ||
+    void *p[2], *q[3], *o[2]; size_t wb; jq_shape s; jq_stream_t st; int cap, n_old, n_new = 0;
+    if (want(n, 10) || ptrs(a, 2, p) || dim(a[0], 1, &cap) || to_int(a[2], &n_old) || ptrs(a + 3, 3, q) || (a[3] != Py_None && dim(a[3], 1, &n_new)) ||
         shape_of(a[6], &s) || ptrs(a + 7, 2, o) || bytes_of(a[8], &wb) || stream_of(a[9], &st)) return NULL;
-    const long n_old = PyLong_AsLong(a[2]);
-    if (n_old == -1 && PyErr_Occurred()) return NULL;
-    CALL(jq.evict_append(p[0], p[1], cap, (int)n_old, q[0], q[1], n_new, q[2], &s, o[0], o[1], wb, st));
+    CALL(jq.evict_append(p[0], p[1], cap, n_old, q[0], q[1], n_new, q[2], &s, o[0], o[1], wb, st));
 }
 /* Kc, Vc, q, out, ws, stream */
 FN(decode_attention)
 {
     void *p[5]; size_t wb; jq_stream_t st; int Hkv, Hq, rows;
-    if (want(n, 6) || ptrs(a, 5, p) || dim(a[0], 0, &Hkv) || dim(a[2], 0, &Hq) || dim(a[0], 1, &rows) || bytes_of(a[4], &wb) || stream_of(a[5], &st)) return NULL;
+    if (want(n, 6) || ptrs(a, 5, p) || dim(a[0], 0, &Hkv) || dim(a[2], 0, &Hq) || dim(a[0], 1, &rows) || size_of(a[4], &wb) || stream_of(a[5], &st)) return NULL;
     CALL(jq.decode_attention(p[0], p[1], p[2], Hkv, Hq, rows, p[3], p[4], wb, st));
 }
 
-/* The units' addresses of a list of tensors. */
+/* The addresses of a sequence of tensors, one per unit; units beyond its end get null pointers, which the call rejects. */
 static int list_ptrs(PyObject *l, Py_ssize_t n, void **p)
 {
     PyObject *f = PySequence_Fast(l, "expected a sequence of tensors");
     if (!f) return -1;
-    int bad = 0;
-    if (PySequence_Fast_GET_SIZE(f) != n) { PyErr_SetString(PyExc_ValueError, "lists of different lengths"); bad = 1; }
-    for (Py_ssize_t i = 0; i < n && !bad; ++i) bad = ptr(PySequence_Fast_GET_ITEM(f, i), p + i) != 0;
+    const Py_ssize_t have = PySequence_Fast_GET_SIZE(f);
+    int bad = have > n;
+    if (bad) PyErr_Format(PyExc_IndexError, "%zd tensors for %zd units", have, n);
+    for (Py_ssize_t i = 0; i < n && !bad; ++i) {
+        p[i] = NULL;
+        if (i < have) bad = address(PySequence_Fast_GET_ITEM(f, i), p + i) != 0;
+    }
     Py_DECREF(f);
     return bad ? -1 : 0;
 }
+/* The first n of a list of numbers. */
 static int list_ints(PyObject *l, Py_ssize_t n, int *p)
 {
+    if (PyObject_Size(l) < 0) return -1;   /* (an iterator is no list) */
     PyObject *f = PySequence_Fast(l, "expected a sequence of integers");
     if (!f) return -1;
-    int bad = 0;
-    if (PySequence_Fast_GET_SIZE(f) != n) { PyErr_SetString(PyExc_ValueError, "lists of different lengths"); bad = 1; }
-    for (Py_ssize_t i = 0; i < n && !bad; ++i) {
-        PyObject *v = PyNumber_Long(PySequence_Fast_GET_ITEM(f, i));
-        if (!v) { bad = 1; break; }
-        const long x = PyLong_AsLong(v);
-        Py_DECREF(v);
-        if (x == -1 && PyErr_Occurred()) bad = 1;
-        p[i] = (int)x;
-    }
+    int bad = PySequence_Fast_GET_SIZE(f) < n;
+    if (bad) PyErr_Format(PyExc_ValueError, "%zd numbers for %zd units", PySequence_Fast_GET_SIZE(f), n);
+    for (Py_ssize_t i = 0; i < n && !bad; ++i) bad = to_int(PySequence_Fast_GET_ITEM(f, i), p + i) != 0;
     Py_DECREF(f);
     return bad ? -1 : 0;
 }
@@ -229,7 +253,7 @@ static int list_ints(PyObject *l, Py_ssize_t n, int *p)
 FN(evict_ragged)
 {
     if (want(n, 11)) return NULL;
-    const Py_ssize_t m = PySequence_Size(a[0]);
+    const Py_ssize_t m = PyObject_Size(a[0]);
     if (m < 0) return NULL;
     void **buf = malloc((3 * (size_t)m + 1) * sizeof *buf);
     int *ib = malloc((2 * (size_t)m + 1) * sizeof *ib);
