@@ -94,6 +94,36 @@ ws = jq.new_append_workspace(shape_of(wl))
 jq.evict_append(Kc, Vc, 512, dev_bf16(K[:, 512:]), dev_bf16(V[:, 512:]), dev_bf16(Q), shape_of(wl), idx, ws)
 assert jq.last_device_status(ws) == jq.JQ_OK
 
+# past the prefix that the one-launch pass takes: the window-retaining call and the re-eviction in two launches, with clusters
+# and with a CTA per head
+for Hkv, g, w, L, B, p in [(2, 4, 16, 12300, 400, 7), (2, 2, 8, 12289, 13000, 7), (129, 1, 2, 12291, 130, 7)]:
+    wl = wl_of(Hkv, g, w, L, B, p)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    np_ = min(B - w, L)
+    dK, dV, dQ, Kw = dev_bf16(K), dev_bf16(V), dev_bf16(Q), dev_bf16(W.make_window_keys(wl, Q))
+    Ko = torch.zeros((Hkv, np_ + w, 128), dtype=torch.bfloat16, device="cuda"); Vo = torch.zeros_like(Ko)
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer_window_kept(dK, dV, dQ, Kw, Kw, s, Ko, Vo, torch.zeros((Hkv, np_), dtype=torch.int32, device="cuda"), ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK
+    Kc = torch.zeros((Hkv, L + 5, 128), dtype=torch.bfloat16, device="cuda"); Vc = torch.zeros_like(Kc)
+    Kc[:, :L - 33] = dK[:, :L - 33]; Vc[:, :L - 33] = dV[:, :L - 33]
+    ws = jq.new_append_workspace(s)
+    jq.evict_append(Kc, Vc, L - 33, dK[:, L - 33:].contiguous(), dV[:, L - 33:].contiguous(), dQ, s, torch.zeros((Hkv, wl.nkeep), dtype=torch.int32, device="cuda"), ws)
+    assert jq.last_device_status(ws) == jq.JQ_OK and jq.launch_count() - n0 == 4
+
+# and the window-retaining call in one, with a threshold among many nearly equal scores
+wl = wl_of(2, 4, 16, 5000, 600)
+K, V, Q, _ = W.make_layer(wl)
+Q = W.bf16_bits(W.bf16_to_f32(Q) * 1e-3)
+s = shape_of(wl)
+Kw = dev_bf16(W.make_window_keys(wl, Q))
+Ko = torch.zeros((2, 600, 128), dtype=torch.bfloat16, device="cuda"); Vo = torch.zeros_like(Ko)
+ws = jq.new_workspace(s)
+jq.evict_layer_window_kept(dev_bf16(K), dev_bf16(V), dev_bf16(Q), Kw, Kw, s, Ko, Vo, torch.zeros((2, 584), dtype=torch.int32, device="cuda"), ws)
+assert jq.last_device_status(ws) == jq.JQ_OK
+
 assert lib.jq_debug_read(rec) == 0
 print("DEBUG-SWEEP violations=%%d kernel=%%d site=%%d index=%%d extent=%%d" %% tuple(rec))
 '''

@@ -82,6 +82,49 @@ def test_tied_scores_keep_the_lowest_positions(L, budget):
     assert np.array_equal(idx.cpu().numpy(), np.tile(np.arange(budget), (2, 1)))
 
 
+def in_the_first_bin(pooled, budget):
+    """Keys in the threshold's bin when the range of a head's pooled scores (as 32-bit patterns) is cut into 2048."""
+    k = np.sort(pooled.astype(np.float32).view(np.uint32).astype(np.int64))[::-1]
+    width = int(k[0] - k[-1])
+    sh = max(width.bit_length() - 11, 0)
+    return int(np.sum((k - k[-1]) >> sh == (k[budget - 1] - k[-1]) >> sh))
+
+
+# a flat head with a dominant key: most scores fall into one of 2048 bins, which has to be cut again.  With equal keys around
+# the threshold (a run of copies of one row, or copies all over) the third cut ends at a single value, kept by position.
+@pytest.mark.parametrize("L,budget,pool", [(4096, 1000, 1), (10000, 3000, 1), (9001, 4500, 3)])
+@pytest.mark.parametrize("copies", ["none", "run", "spread"])
+def test_a_threshold_among_nearly_equal_scores(L, budget, pool, copies):
+    wl = wl_of(1, 2, 8, L, budget, pool)
+    rng = np.random.default_rng(L)
+    Kf = rng.standard_normal((1, L, 128)).astype(np.float32)
+    Qf = 2e-3 * rng.standard_normal((2, 8, 128)).astype(np.float32)         # logits of about 2e-3: scores within a per mille or two
+    Kf[0, 5] = 10 * 11.3 * Qf[0, 0] / np.sum(Qf[0, 0] ** 2)                 # and a key with a logit of 10 for one query row
+    at = np.arange(0)
+    if copies != "none":
+        at = np.arange(100, 1600) if copies == "run" else np.sort(rng.choice(np.arange(6, L - 1), 1500, replace=False))
+        Kf[0, at] = 0.1 * Kf[0, L - 1]
+    K, Q, V = W.bf16_bits(Kf), W.bf16_bits(Qf), W.make_v(wl, 3)
+    pooled = oracle.pool(oracle.score(K, Q), pool)
+    if len(at):                                                             # the threshold in the middle of the copies
+        budget = int(np.sum(pooled[0] > pooled[0, at].min())) + int(np.sum(pooled[0] == pooled[0, at].min())) // 2
+    assert in_the_first_bin(pooled[0], budget) > 512
+    s = shape_of(wl.with_budget(budget))
+    Ko, Vo, idx = outputs(1, budget, budget)
+    n0 = jq.launch_count()
+    jq.evict_layer(dev_bf16(K), dev_bf16(V), dev_bf16(Q), s, Ko, Vo, idx, jq.new_workspace(s))
+    assert jq.launch_count() - n0 == 1
+    gi = idx.cpu().numpy()
+    # sums of 16 terms of equal size in 32 bits, against an exact normaliser: 16 x 2^-24 and the 2^-22 of an exponential
+    kth = np.sort(pooled[0])[L - budget]
+    diff = np.setxor1d(gi[0], oracle.select(pooled, budget)[0])
+    assert np.all(np.diff(gi[0]) > 0) and np.all(np.abs(pooled[0, diff] - kth) <= 2e-6 * kth)
+    assert np.array_equal(host_bits(Ko)[0], K[0][gi[0]]) and np.array_equal(host_bits(Vo)[0], V[0][gi[0]])
+    if len(at) and pool == 1:                                               # of equal rows the lowest positions stay
+        kept = np.isin(at, gi[0])
+        assert 0 < np.sum(kept) < len(at) and np.all(kept[:-1] >= kept[1:])
+
+
 @pytest.mark.parametrize("Hkv,g,w,L,budget", [(2, 4, 32, 128, 64), (8, 4, 32, 1000, 300), (2, 2, 128, 2500, 700), (3, 4, 64, 5001, 900)])
 def test_window_kept_in_one_launch(Hkv, g, w, L, budget):
     wl = wl_of(Hkv, g, w, L, budget)
@@ -155,14 +198,50 @@ def test_host_call_in_chunks(Hkv, g, w, L, budget, pageable):
     hVo, hidx = torch.zeros_like(hKo).pin_memory(), torch.zeros((Hkv, wl.nkeep), dtype=torch.int32).pin_memory()
     buf = torch.empty(jq.host_call_bytes(s), dtype=torch.uint8, device="cuda")
     hK, hQ, hV = pin(K), pin(Q), torch.from_numpy(V.view(np.int16).copy()) if pageable else pin(V)
-    for _ in range(2):                      # the second call finds the buffers in use by the first
-        jq.evict_layer_host(hK, hV, hQ, s, hKo, hVo, hidx, buf)
+    # a second layer right behind, through the same device buffer into outputs of its own; and what the stream does next
+    # finds the first call's results
+    K2, V2, Q2, _ = W.make_layer(wl, layer=1)
+    hK2, hQ2, hV2 = pin(K2), pin(Q2), torch.from_numpy(V2.view(np.int16).copy()) if pageable else pin(V2)
+    hKo2, hVo2, hidx2 = torch.zeros_like(hKo).pin_memory(), torch.zeros_like(hKo).pin_memory(), torch.zeros_like(hidx).pin_memory()
+    seen = [torch.empty(x.shape, dtype=x.dtype, device="cuda") for x in (hKo, hVo, hidx)]
+    jq.evict_layer_host(hK, hV, hQ, s, hKo, hVo, hidx, buf)
+    for d, h in zip(seen, (hKo, hVo, hidx)):
+        d.copy_(h, non_blocking=True)
+    jq.evict_layer_host(hK2, hV2, hQ2, s, hKo2, hVo2, hidx2, buf)
     torch.cuda.current_stream().synchronize()
-    pooled = oracle.pool(oracle.score(K, Q), wl.pool)
-    gi = hidx.numpy()
-    assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
-    for kv in range(Hkv):
-        assert np.array_equal(hKo.numpy().view(np.uint16)[kv], K[kv][gi[kv]]) and np.array_equal(hVo.numpy().view(np.uint16)[kv], V[kv][gi[kv]])
+    for (Ki, Vi, Qi), outs in (((K, V, Q), (hKo, hVo, hidx)), ((K, V, Q), [d.cpu() for d in seen]), ((K2, V2, Q2), (hKo2, hVo2, hidx2))):
+        pooled = oracle.pool(oracle.score(Ki, Qi), wl.pool)
+        gKo, gVo, gi = outs[0].numpy().view(np.uint16), outs[1].numpy().view(np.uint16), outs[2].numpy()
+        assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, wl.nkeep)
+        for kv in range(Hkv):
+            assert np.array_equal(gKo[kv], Ki[kv][gi[kv]]) and np.array_equal(gVo[kv], Vi[kv][gi[kv]])
+
+
+def test_host_calls_of_one_thread_on_two_streams():
+    """They share the stream that the library works on beside a caller's, and nothing else."""
+    wl = wl_of(4, 2, 8, 33001, 500)
+    s = shape_of(wl)
+    pin = lambda a: torch.from_numpy(a.view(np.int16)).pin_memory()
+    work = []
+    for i in range(4):
+        K, V, Q, _ = W.make_layer(wl, layer=i)
+        outs = (torch.zeros((4, 500, 128), dtype=torch.int16).pin_memory(), torch.zeros((4, 500, 128), dtype=torch.int16).pin_memory(),
+                torch.zeros((4, 500), dtype=torch.int32).pin_memory())
+        work.append(((K, V, Q), (pin(K), pin(V), pin(Q)), outs))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    bufs = [torch.empty(jq.host_call_bytes(s), dtype=torch.uint8, device="cuda") for _ in streams]
+    torch.cuda.synchronize()
+    for i, (_, (hK, hV, hQ), outs) in enumerate(work):
+        jq.evict_layer_host(hK, hV, hQ, s, *outs, bufs[i & 1], stream=streams[i & 1])
+    for st in streams:
+        st.synchronize()
+    for (K, V, Q), _, (gKo, gVo, gi) in work:
+        pooled = oracle.pool(oracle.score(K, Q), wl.pool)
+        gi = gi.numpy()
+        assert_kept_sets_agree(gi, oracle.select(pooled, 500), pooled, 500)
+        for kv in range(4):
+            assert np.array_equal(gKo.numpy().view(np.uint16)[kv], K[kv][gi[kv]]) and np.array_equal(gVo.numpy().view(np.uint16)[kv], V[kv][gi[kv]])
+
 
 
 def test_each_kernel_sees_what_the_one_before_it_wrote():
