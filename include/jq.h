@@ -14,7 +14,8 @@
  *
  * Conventions, for every entry point unless it says otherwise:
  *  - pointers named K, V, Qwin, scores, kept_idx, Kout, Vout, ws are DEVICE pointers owned by the
- *    caller, contiguous row-major, 16-byte aligned; the library allocates and frees nothing;
+ *    caller, contiguous row-major, 16-byte aligned; the library allocates and frees no device memory
+ *    (jq_evict_layer_host keeps a stream and two events of its own per host thread and device);
  *  - bf16 tensors are raw 16-bit patterns:  K, V [Hkv, L, d];  Qwin [Hq, w, d];
  *    Kout, Vout [Hkv, nkeep, d];  scores, pooled [Hkv, L] fp32;  kept_idx [Hkv, nkeep] int32,
  *    nkeep = jq_num_kept(shape) = min(budget, L);
@@ -23,6 +24,10 @@
  *  - outputs must not overlap inputs or the workspace; the same workspace may be reused by
  *    successive calls on ONE stream; calls on different streams need different workspaces;
  *  - inputs must be finite; NaN or Inf give unspecified kept sets (never a fault);
+ *  - every call is deterministic.  "The results of" another call below means: the copied rows are bit
+ *    for bit those that the returned indices name, and the indices are the other call's except among
+ *    positions whose pooled scores agree to fp32 rounding at the threshold (the calls may add the same
+ *    exponentials in another order; identical scores always give identical indices);
  *  - errors are return codes; argument errors are detected on the host before anything is
  *    launched and leave every output untouched.
  *
@@ -168,8 +173,8 @@ jq_status jq_compact_kv(const void *K, const void *V, const int32_t *kept_idx,
 
 /*
  * The whole pass for one layer, with the results of jq_score -> jq_select_topk -> jq_compact_kv, on one
- * stream in two launches (the selection kernel also copies the kept rows); the scores stay in the
- * workspace.  K may hold several layers of equal shape stacked along the KV-head axis (Hkv = layers x
+ * stream: in one launch for short prefixes (at most 12288 keys, where that is the faster way), else in two
+ * (the selection kernel also copies the kept rows).  Scores are not handed out.  K may hold several layers of equal shape stacked along the KV-head axis (Hkv = layers x
  * heads per layer, Qwin stacked alike): heads are independent, so one call evicts them all.
  */
 jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const jq_shape *shape,
@@ -182,8 +187,8 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
  * and a budget B_u of its own; all units share the head geometry of `common` (Hkv, Hq, group, d, w, pool).
  * (Every (unit, KV head) is an independent instance of the pass of the inference section; lengths that differ
  * are the 4K-32K contexts of the paper's length sweeps, budgets that differ per layer are the layer-wise
- * schedule its experimental-setting paragraph describes for one of the compared methods.)  The results are
- * those of one jq_evict_layer call per unit, bit for bit.
+ * schedule its experimental-setting paragraph describes for one of the compared methods.)  The results of
+ * one jq_evict_layer call per unit.
  *   K, V, Qwin: HOST arrays of nunits DEVICE pointers, each as jq_evict_layer takes it for unit u;
  *   L, budget:  HOST arrays of nunits ints, or NULL for "common->L / common->budget for every unit"
  *               (the corresponding field of `common` is ignored when the array is given);
@@ -244,8 +249,8 @@ jq_status jq_hit_rate(const int32_t *cur, const int32_t *ref, int Hkv, int ncur,
  * Kc, Vc: device, bf16 [Hkv, n, 128] (what jq_evict_layer wrote), 16-byte aligned.  q: device, bf16 [Hq, 128].
  * out: device, fp32 [Hq, 128], 16-byte aligned.  workspace: device, 16-byte aligned, at least
  * jq_decode_workspace_bytes(Hkv, Hq, n) bytes (0 for arguments the call would reject); no initialisation
- * needed, contents undefined afterwards.  Hq / Hkv <= 8.  Asynchronous on `stream`; one launch (and a memset
- * of Hkv counters in the workspace).
+ * needed, contents undefined afterwards (the present kernel keeps its partial results on chip and leaves it
+ * alone).  Hq / Hkv <= 8.  Asynchronous on `stream`; one launch.
  */
 size_t jq_decode_workspace_bytes(int Hkv, int Hq, int n);
 jq_status jq_decode_attention(const void *Kc, const void *Vc, const void *q, int Hkv, int Hq, int n, float *out,
@@ -262,10 +267,11 @@ jq_status jq_decode_attention(const void *Kc, const void *Vc, const void *q, int
  * The call appends the new rows behind the retained ones, runs the pass of jq_evict_layer over the
  * L rows of every head, and leaves the min(budget, L) kept rows, in ascending order of their position in
  * that concatenation, in rows [0, nkeep) of Kc and Vc; kept_idx [Hkv, nkeep] holds those positions (values
- * below n_old are old rows).  Rows [nkeep, cap) are unspecified afterwards.  Same results as jq_evict_layer on
+ * below n_old are old rows).  Rows [nkeep, cap) are unspecified afterwards.  The results of jq_evict_layer on
  * the concatenated tensors.  ws: at least jq_append_workspace_bytes(shape) bytes (it also holds the compacted
  * rows before they are moved to the head of the cache), first 256 bytes initialised by jq_workspace_init.
- * Two launches and up to six strided device copies, all on `stream`.
+ * One launch for short caches (as jq_evict_layer), else two launches and up to six strided device copies, all
+ * on `stream`.
  */
 size_t jq_append_workspace_bytes(const jq_shape *shape);
 jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Knew, const void *Vnew, int n_new,
