@@ -16,16 +16,12 @@ struct Workspace {
     int *status;        // [kStatusWords]
     float *Mrow;        // [Hkv][R]   log2-domain normaliser per query row: c*max + log2(sumexp)
     float2 *part;       // [Hkv][kSlots][R]   (raw max, sum of exp2(c*(s-max))) per contributing block
-    float *scores;      // [Hkv][L]   pre-pool scores (jq_evict_layer keeps them here)
-    uint32_t *keys;     // [Hkv][L]   order-preserving bit patterns of the pooled scores
-    uint32_t *sel;      // select scratch
+    float *scores;      // [Hkv][L]   pre-pool scores (of the two-launch path)
+    uint32_t *keys;     // [Hkv][L]   order-preserving bit patterns of the pooled scores (of heads whose keys do not fit on chip)
     size_t bytes;       // total
 };
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
-// Select scratch per KV head, in 32-bit words: histograms and counters (see jq_select.cu).
-constexpr int kSelWordsPerHead = 4096 + 64;
 
 // Carve-up of a workspace for `heads` KV heads with R query rows each and `keys` prefix positions in total
 // (heads x L for one shape; the sum over the units of a ragged call).
@@ -44,8 +40,6 @@ static inline Workspace carve(void *base, size_t heads, size_t R, size_t keys)
     off += align_up(keys * sizeof(float), 256);
     w.keys = (uint32_t *)(p + off);
     off += align_up(keys * sizeof(uint32_t), 256);
-    w.sel = (uint32_t *)(p + off);
-    off += align_up(heads * kSelWordsPerHead * sizeof(uint32_t), 256);
     w.bytes = off;
     return w;
 }

@@ -745,7 +745,6 @@ constexpr size_t smem_bytes(int Rbox, int stages)
 
 struct DeviceInfo {
     int sms = 0;        // CTAs of score_fused that can be resident at once (one per SM)
-    long long l2 = 0;
     bool ready = false;
 };
 
@@ -758,9 +757,8 @@ bool device_info(DeviceInfo *out)
     std::lock_guard<std::mutex> lock(mu);
     DeviceInfo &d = info[dev];
     if (!d.ready) {
-        int l2 = 0, sms = 0, coop = 0, per_sm = 0;
+        int sms = 0, coop = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-        if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) return false;
         if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return false;
         const size_t smem = smem_bytes(256, 3) > smem_bytes(128, 5) ? smem_bytes(256, 3) : smem_bytes(128, 5);
         if (cudaFuncSetAttribute(score_fused<kGroupsNarrow>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
@@ -770,7 +768,6 @@ bool device_info(DeviceInfo *out)
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_fused<kGroupsWide>, threads_for(kGroupsWide), smem) != cudaSuccess || per_sm < 1)
             return false;
         d.sms = sms;
-        d.l2 = l2;
         d.ready = true;
     }
     *out = d;
