@@ -1,6 +1,6 @@
 // Bounds-checked build of the kernels (-DJQ_DEBUG; build.build(debug=True) makes libjq_debug.so from the same
-// sources).  It stands in for a memory checker: every index that score_fused, select_cluster, gather_rows and
-// decode_step compute into global, shared or tensor memory goes through JQ_IN(index, extent, kernel, site) before
+// sources).  It stands in for a memory checker: every index that score_fused, evict_fused, select_cluster,
+// select_stream, gather_rows and decode_step compute into global, shared or tensor memory goes through JQ_IN(index, extent, kernel, site) before
 // the access.  An index outside [0, extent) is counted in a record in device memory, the first one is kept
 // (which kernel, which site, the index and the extent), and the access is skipped: the kernel never traps and
 // always runs to its end.  The host reads the record with jq_debug_read (exported by the debug library only).

@@ -49,6 +49,7 @@ constexpr int kFMaxStages = 6;
 constexpr int kFCand = 512;                         // keys of one bin that are ranked by comparison
 constexpr int kFMaxL = 12288;                       // what shared memory has room for, and about where the general path overtakes
 constexpr int kFRowPad = 8;                         // float2s between the CTAs' statistics: their rows fall into different banks
+static_assert(kFMaxL <= 4 * 7 * kFT, "the compaction's masks hold seven quads of a thread, four bits each");
 constexpr int kFHalo = 32;                          // >= pool radius, in floats
 constexpr uint32_t kFHalf = kFTile * 128;           // one 64-column half of a tile
 constexpr uint32_t kFStage = 2 * kFHalf;

@@ -284,8 +284,8 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
                 int head_c2 = 0;
                 // A key tile is read by pass 1, which brings it into the L2, and then once more by pass 2 of its group: after
                 // that it is the first to go, and the tiles that pass 1 of the next groups brings in meanwhile stay.  (With no
-                // hints a quarter more than one read of K came from HBM; 32 layers of 32768 keys 996 -> 962 us, of 131072 keys
-                // 6095 -> 5895 us.)
+                // hints a quarter more than one read of K came from HBM; 32 layers of 32768 keys 1049 -> 1008 us, of 131072 keys
+                // 6341 -> 6135 us.)
                 uint64_t stay, leave;
                 asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(stay));
                 asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(leave));
