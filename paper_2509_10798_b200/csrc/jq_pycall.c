@@ -1,8 +1,8 @@
 /* Argument marshalling between Python and the C ABI of include/jq.h: one C function per entry point that is called in
- * a loop.  A layer call costs the GPU 10 to 30 us and its two launches about 8 us of host time; marshalled by ctypes,
- * with the current stream asked for through torch.cuda, the same call took 18 us on the host, more than the GPU needs
- * for short prompts and for a decoding step.  Here a tensor costs its data_ptr(), the shape its buffer, the stream one
- * raw lookup: evict_layer 18.0 -> 9.7 us, decode_attention 10.1 -> 3.4 us per call.
+ * a loop.  A layer call costs the GPU 10 to 30 us; marshalled by ctypes, with the current stream asked for through
+ * torch.cuda, a call of two launches took 18 us on the host and a decoding step 10, more than the GPU needs for short
+ * prompts and for a decoding step.  Here a tensor costs its data_ptr(), the shape its buffer, the stream one raw lookup:
+ * evict_layer 6.3 us in two launches and 3.5 in one, decode_attention 3.2.
  * The library itself is reached through addresses that the package takes from the libjq it has loaded (bind), so the
  * bounds-checked build can stand in for it. */
 #define PY_SSIZE_T_CLEAN
