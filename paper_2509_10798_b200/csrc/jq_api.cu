@@ -46,6 +46,16 @@ static jq_status check_ws(const jq_shape *s, void *ws, size_t ws_bytes, Workspac
     return ws_bytes < out->bytes ? JQ_ERR_WORKSPACE : JQ_OK;
 }
 
+// The scores of one layer for a selection that follows, by the faster of the two ways.
+static jq_status score_layer(const void *K, const void *Qwin, const jq_shape &s, const Workspace &w, cudaStream_t st,
+                             const void *Kwin = nullptr, int k_head_rows = 0)
+{
+    const long long tiles = (long long)s.Hkv * ((s.L + 127) / 128), keys = (long long)s.Hkv * s.L;
+    const long long kept = (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L);
+    if (prune_taken(s, s.Hkv, tiles, keys, kept, s.L, device_sms())) return launch_score_pruned(K, Qwin, s, w.scores, w, st, Kwin, nullptr, k_head_rows);
+    return launch_score_tc(K, Qwin, s, w.scores, w, st, Kwin, nullptr, k_head_rows);
+}
+
 }  // namespace jq
 
 using namespace jq;
@@ -113,7 +123,7 @@ jq_status jq_evict_layer_windowed(const void *K, const void *V, const void *Qwin
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin;
     bool taken;
     if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    if ((rc = launch_score_tc(K, Qwin, *s, w.scores, w, st, Kwin)) != JQ_OK) return rc;
+    if ((rc = score_layer(K, Qwin, *s, w, st, Kwin)) != JQ_OK) return rc;
     return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);
 }
 
@@ -140,7 +150,7 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     bool taken;
     if ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
-    if ((rc = launch_score_tc(K, Qwin, sp, w.scores, w, st, Kwin)) != JQ_OK) return rc;
+    if ((rc = score_layer(K, Qwin, sp, w, st, Kwin)) != JQ_OK) return rc;
     return launch_select(w.scores, sp, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, 0, (int)nt, Kwin, Vwin);
 }
 
@@ -192,7 +202,7 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
     src.KA = K; src.VA = V; src.LA = s->L;
     bool taken;
     if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    if ((rc = launch_score_tc(K, Qwin, *s, w.scores, w, st)) != JQ_OK) return rc;
+    if ((rc = score_layer(K, Qwin, *s, w, st)) != JQ_OK) return rc;
     return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);   // selects, then copies the kept rows
 }
 
@@ -280,20 +290,23 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     static thread_local std::vector<unsigned char> staging;
     staging.assign(tab_bytes, 0);
     unsigned char *hb = staging.data();
-    const size_t maps_bytes = align_up((size_t)nunits * 2 * kTensorMapBytes, 256), ptr_bytes = align_up((size_t)nunits * sizeof(void *), 256);
+    const size_t maps_bytes = align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256), ptr_bytes = align_up((size_t)nunits * sizeof(void *), 256);
     const size_t head_bytes = align_up((size_t)nunits * hpu * sizeof(HeadRec), 256), grp_off = maps_bytes + 2 * ptr_bytes + head_bytes;
     unsigned char *h_maps = hb;
     const void **h_K = (const void **)(hb + maps_bytes), **h_V = (const void **)(hb + maps_bytes + ptr_bytes);
     HeadRec *h_head = (HeadRec *)(hb + maps_bytes + 2 * ptr_bytes);
     GroupRec *h_grp = (GroupRec *)(hb + grp_off);   // last: there are far fewer than there is room for
     UnitTables t;
-    long long soff = 0, ooff = 0;
+    for (int u = 0; u < nunits; ++u) t.total_tiles += (long long)hpu * (((L ? L[u] : common->L) + 127) / 128);
+    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L, sms);
+    long long soff = 0, ooff = 0, tbase = 0;
     int ngroups = 0;
     for (int u = 0; u < nunits; ++u) {
         const int Lu = L ? L[u] : common->L, Bu = budget ? budget[u] : common->budget;
         const int nkeep = Bu < Lu ? Bu : Lu;
-        if (!make_tensor_map(h_maps + (size_t)(2 * u) * kTensorMapBytes, K[u], Lu, hpu, 128) ||
-            !make_tensor_map(h_maps + (size_t)(2 * u + 1) * kTensorMapBytes, Qwin[u], R, hpu, R <= 128 ? 128 : 256))
+        unsigned char *const m = h_maps + (size_t)(kMapsPerUnit * u) * kTensorMapBytes;
+        if (!make_tensor_map(m, K[u], Lu, hpu, 128) || !make_tensor_map(m + kTensorMapBytes, Qwin[u], R, hpu, R <= 128 ? 128 : 256) ||
+            (pruned && !make_tensor_map(m + 2 * kTensorMapBytes, K[u], Lu, hpu, 16)))
             return JQ_ERR_CUDA;
         h_K[u] = K[u]; h_V[u] = V[u];
         for (int h = 0; h < hpu; ++h) {
@@ -301,13 +314,15 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
             r.L = Lu; r.nkeep = nkeep; r.unit = u; r.kv_in = h;
             r.soff = soff + (long long)h * Lu;
             r.ooff = ooff + (long long)h * nkeep;
+            r.tbase = tbase + (long long)h * ((Lu + 127) / 128);
         }
+        tbase += (long long)hpu * ((Lu + 127) / 128);
         soff += (long long)hpu * Lu;
         ooff += (long long)hpu * nkeep;
     }
     // head groups of the scoring kernel: every run of consecutive units of one length is cut into groups of
     // at most 56 MiB of keys (short prefixes share a group across units, so that a group still has tiles for every CTA)
-    for (int u0 = 0; u0 < nunits;) {
+    for (int u0 = 0; u0 < nunits && !pruned;) {
         const int Lu = L ? L[u0] : common->L, tph = (Lu + 127) / 128;
         int u1 = u0 + 1;
         while (u1 < nunits && (L ? L[u1] : common->L) == Lu) ++u1;
@@ -335,7 +350,8 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     t.heads = (const HeadRec *)(tab + maps_bytes + 2 * ptr_bytes);
     t.groups = (const GroupRec *)(tab + grp_off);
     t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows;
-    if ((rc = launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t)) != JQ_OK) return rc;
+    rc = pruned ? launch_score_pruned(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t) : launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t);
+    if (rc != JQ_OK) return rc;
     return launch_select(w.scores, pl.S, kept_idx, nullptr, w, st, nullptr, nullptr, Kout, Vout, &t);
 }
 
@@ -389,7 +405,7 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     }
     // 2. the pass over the L = n_old + n_new rows of every head, compacted into the workspace (a row may move
     //    onto a row that another thread still has to read, so the compaction cannot run in place)
-    if ((rc = launch_score_tc(Kc, Qrecent, *s, w.scores, w, st, nullptr, nullptr, cap)) != JQ_OK) return rc;
+    if ((rc = score_layer(Kc, Qrecent, *s, w, st, nullptr, cap)) != JQ_OK) return rc;
     if ((rc = launch_select(w.scores, *s, kept_idx, nullptr, w, st, Kc, Vc, Ktmp, Vtmp, nullptr, cap)) != JQ_OK) return rc;
     // 3. back to the head of the cache
     if (cudaMemcpy2DAsync(Kc, (size_t)cap * row, Ktmp, nkeep * row, nkeep * row, (size_t)s->Hkv, cudaMemcpyDeviceToDevice, st) != cudaSuccess)

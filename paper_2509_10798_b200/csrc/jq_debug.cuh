@@ -1,7 +1,7 @@
 // Bounds-checked build of the kernels (-DJQ_DEBUG; build.build(debug=True) makes libjq_debug.so from the same
-// sources).  It stands in for a memory checker: every index that score_fused, evict_fused, select_cluster,
-// select_stream, gather_rows and decode_step compute into global, shared or tensor memory goes through JQ_IN(index, extent, kernel, site) before
-// the access.  An index outside [0, extent) is counted in a record in device memory, the first one is kept
+// sources).  It stands in for a memory checker: every index that score_fused, row_stats, score_candidates, evict_fused,
+// select_cluster, select_stream, gather_rows and decode_step compute into global, shared or tensor memory goes through JQ_IN(index,
+// extent, kernel, site) before the access.  An index outside [0, extent) is counted in a record in device memory, the first one is kept
 // (which kernel, which site, the index and the extent), and the access is skipped: the kernel never traps and
 // always runs to its end.  The host reads the record with jq_debug_read (exported by the debug library only).
 // In the ordinary build JQ_IN is the constant true and the extra kernel parameter does not exist.
@@ -14,7 +14,7 @@ struct DebugRecord {
     int kernel, site;                // of the first one
     long long index, extent;
 };
-enum { kDbgScore = 1, kDbgSelect = 2, kDbgGather = 3, kDbgDecode = 4, kDbgFused = 5 };
+enum { kDbgScore = 1, kDbgSelect = 2, kDbgGather = 3, kDbgDecode = 4, kDbgFused = 5, kDbgPrune = 6 };
 
 #ifdef JQ_DEBUG
 DebugRecord *debug_record();   // host: device address of the record on the current device (nullptr on error)

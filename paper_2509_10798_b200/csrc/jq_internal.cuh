@@ -18,8 +18,11 @@ struct Workspace {
     float2 *part;       // [Hkv][kSlots][R]   (raw max, sum of exp2(c*(s-max))) per contributing block
     float *scores;      // [Hkv][L]   pre-pool scores (of the two-launch path)
     uint32_t *keys;     // [Hkv][L]   order-preserving bit patterns of the pooled scores (of heads whose keys do not fit on chip)
+    void *prune;        // scratch of the one-pass scoring, in the place of Mrow and part (a call uses one or the other)
     size_t bytes;       // total
 };
+// Bytes of that scratch for `tiles` tiles of keys in total (every head's rounded up, window tiles included).
+size_t prune_bytes(long long tiles, int heads, int R);
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -32,10 +35,12 @@ static inline Workspace carve(void *base, size_t heads, size_t R, size_t keys)
     size_t off = 0;
     w.status = (int *)(p + off);
     off += align_up(kStatusWords * sizeof(int), 256);
+    const size_t mrow = align_up(heads * R * sizeof(float), 256), part = align_up(heads * kSlots * R * sizeof(float2), 256);
+    const size_t prune = prune_bytes((long long)(keys / 128 + 2 * heads), (int)heads, (int)R);
+    w.prune = p + off;
     w.Mrow = (float *)(p + off);
-    off += align_up(heads * R * sizeof(float), 256);
-    w.part = (float2 *)(p + off);
-    off += align_up(heads * kSlots * R * sizeof(float2), 256);
+    w.part = (float2 *)(p + off + mrow);
+    off += mrow + part > prune ? mrow + part : prune;
     w.scores = (float *)(p + off);
     off += align_up(keys * sizeof(float), 256);
     w.keys = (uint32_t *)(p + off);
@@ -53,6 +58,7 @@ static inline Workspace carve(void *base, const jq_shape &s)
 // KV heads are numbered through all units; unit u owns heads [u * hpu, (u + 1) * hpu).
 constexpr int kMaxUnits = 4096;
 constexpr size_t kTensorMapBytes = 128;
+constexpr int kMapsPerUnit = 3;
 // A head group of the scoring kernel: consecutive KV heads of one prefix length whose keys fit a share of the
 // L2.  A group may run over consecutive units of equal length (their scores are consecutive too).
 struct GroupRec {
@@ -71,9 +77,10 @@ struct HeadRec {
     int unit, kv_in;     // the unit and the head's index within it
     long long soff;      // offset (floats / keys) of the head's scores and select keys
     long long ooff;      // offset (rows) of the head's kept indices and compacted rows in the stacked outputs
+    long long tbase;     // tiles of the heads before it
 };
 struct UnitTables {
-    const void *maps = nullptr;          // device: [nunits][2] TMA tensor maps (K, Qwin)
+    const void *maps = nullptr;          // device: [nunits][kMapsPerUnit] TMA tensor maps (K, Qwin, K in blocks of 16 keys)
     const void *const *K = nullptr;      // device: [nunits] base of K
     const void *const *V = nullptr;      // device: [nunits] base of V
     const GroupRec *groups = nullptr;    // device: [ngroups]
@@ -83,10 +90,11 @@ struct UnitTables {
     int max_L = 0;                       // longest prefix (sizes the selection kernel's shared memory)
     long long total_keys = 0;            // keys of all units (floats in the scores array)
     long long total_rows = 0;            // rows of the stacked outputs
+    long long total_tiles = 0;           // tiles of all heads
 };
 static inline size_t unit_tables_bytes(int nunits, int hpu)
 {
-    return align_up((size_t)nunits * 2 * kTensorMapBytes, 256) + 2 * align_up((size_t)nunits * sizeof(void *), 256) +
+    return align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256) + 2 * align_up((size_t)nunits * sizeof(void *), 256) +
            align_up((size_t)nunits * hpu * sizeof(GroupRec), 256) + align_up((size_t)nunits * hpu * sizeof(HeadRec), 256);
 }
 // One tensor map for a bf16 tensor [heads][rows][128], boxes of 64 columns x box_rows rows (host).
@@ -111,6 +119,12 @@ jq_status launch_score_fma(const void *K, const void *Q, const jq_shape &s, floa
 jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float *scores,
                           const Workspace &w, cudaStream_t st, const void *Kwin = nullptr,
                           const UnitTables *tables = nullptr, int k_head_rows = 0);
+// The scores that a selection of s.budget pairs per head needs (jq_prune.cu): those of launch_score_tc for every key that can be
+// kept or make a neighbour kept, zero elsewhere.  prune_taken: whether a call over `heads` heads (tiles, keys and kept pairs of all
+// of them, the longest max_L) is one that this is the faster way for.
+bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L, int sms);
+jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, float *scores, const Workspace &w, cudaStream_t st,
+                              const void *Kwin = nullptr, const UnitTables *tables = nullptr, int k_head_rows = 0);
 // With K, V, Kout, Vout given, the kernel also copies the kept rows (the fused layer path).  With tables, every
 // head has a length, a budget and offsets of its own (s.L, s.budget unused).
 // src_head_rows: rows between consecutive heads of K and V in memory when the heads are not packed (0: s.L);

@@ -1,0 +1,933 @@
+// Scoring for a small budget: Eq. 3 where it decides what is kept, in ONE streaming pass over K and a second look at the few
+// keys that can be among the kept ones.  The scores it hands to the selection are those of jq_score for every key that
+// could be kept or lift a neighbour (by the max-pool) to be kept, and zero elsewhere, so the selection's result is the same.
+//
+//   row_stats         pass 1 over all heads of the call: a CTA takes a contiguous run of key tiles, computes S = Q K^T on the
+//                     tensor cores and keeps, per query row, (reference m, l = sum of exponentials), as score_fused does.  Beside
+//                     them it leaves the largest logit of every row in every block of 16 keys, as a half (2 bytes per row and
+//                     block against the 4096 of the block's keys).
+//   score_candidates  a cluster of 1 to 16 CTAs per KV head.  From the merged normalisers M_r and those maxima follows a bound
+//                         score[j] <= UB[block of j] = sum_r exp2(c max_r - M_r)       for the price of one exponential per 16.
+//                     Round 1 scores the blocks with the largest bounds (S^T = K Q^T on the tensor cores, the blocks gathered
+//                     16 rows at a time by TMA into tiles of 128 keys) and counts, in a histogram, the pooled scores that they
+//                     alone guarantee: the nkeep-th largest of these, rounded down, is a value that the threshold of the
+//                     selection cannot lie below.  Round 2 scores the blocks whose bounds reach it and that round 1 left out.
+//                     A block whose bound does not reach it holds no kept key and no neighbour that makes one kept.
+//
+// Nothing is assumed about the data: where the bounds do not separate (flat scores), round 2 takes every block and the work is
+// that of the two-pass kernel.  prune_plan has the rule by which a call comes here, with what was measured.
+//
+// The bound holds for the scores as they are computed, not only on paper: the half is read as x + |x| / 1024 (its rounding is
+// at most 1 / 2048), the sum is raised by 1 / 64, and it is rounded up to 16 bits, far above the differences in rounding
+// between the two orders of the product.
+#include "jq_sm100.cuh"
+#include "jq_tmem_ld.cuh"
+#include "jq_debug.cuh"
+#include <cstddef>
+#include <cstring>
+#include <cuda_fp16.h>
+#include <mutex>
+
+namespace jq {
+namespace {
+
+constexpr int kPTile = 128;                      // keys per tile
+constexpr uint32_t kPHalf = kPTile * 128;        // one 64-column half of a tile
+constexpr uint32_t kPStage = 2 * kPHalf;
+constexpr int kPBlock = 16;                      // keys per block
+constexpr uint32_t kPBlockHalf = kPBlock * 128;  // one 64-column half of a block
+
+// ------------------------------------------------------------------ row statistics
+
+constexpr int kSGroupsNarrow = 3, kSGroupsWide = 4;   // epilogue groups for R <= 128 / R > 128
+constexpr int kSMaxStages = 5;
+constexpr uint32_t kSSlots = 4, kSSlotCols = 128, kSTmemCols = 512;
+__host__ __device__ constexpr int stats_threads(int groups) { return (4 * groups + 2) * 32; }
+static_assert(kSGroupsNarrow <= (int)kSSlots && kSGroupsWide <= (int)kSSlots, "no more epilogue groups than accumulator slots");
+// A role that waits while others work sleeps between polls (ns).
+constexpr uint32_t kSSleepLong = 256, kSSleepShort = 32;
+
+struct SCtl {
+    uint64_t full[kSMaxStages], empty[kSMaxStages];
+    uint64_t q_full[2], q_empty[2];
+    uint64_t t_full[kSSlots], t_empty[kSSlots];
+    uint32_t tmem_base;
+    int abort_flag;
+};
+constexpr uint32_t kSCtlBytes = 1024;
+static_assert(sizeof(SCtl) <= kSCtlBytes, "control block");
+
+struct SParams {
+    int L, tph;                // one shape: keys and tiles per head (the window tile included)
+    int R, Rbox, Rpad, w;
+    int wtile;                 // every head has one more tile, the last, holding the w window keys
+    int stages, hpu;           // hpu: heads per unit (ragged calls)
+    long long T;               // tiles of all heads
+    float c;
+    int heads;
+    float2 *part;              // [(CTA + head) * groups + group][R]: the statistics of one CTA's share of a head
+    uint32_t *bmax;            // [tile][4][Rpad]: maxima of two blocks of 16 keys each, as halves, times c
+    int *status;
+    const HeadRec *htab;       // units in buffers of their own: lengths and first tiles of the heads,
+    const CUtensorMap *maps;   // [units][kMapsPerUnit] tensor maps (K, Qwin, K in blocks)
+#ifdef JQ_DEBUG
+    DebugRecord *dbg_rec;
+    long long n_part, n_bmax;
+#endif
+};
+
+// Where a CTA's run of tiles starts, and how a role walks it.
+struct Walk {
+    int h, t, tph, L;
+    __device__ __forceinline__ void load(const SParams &P)
+    {
+        if (!P.htab) return;
+        L = P.htab[h].L;
+        tph = (L + kPTile - 1) / kPTile;
+    }
+    __device__ __forceinline__ void start(const SParams &P, long long tile)
+    {
+        tph = P.tph; L = P.L;
+        if (!P.htab) {
+            h = (int)(tile / P.tph);
+            t = (int)(tile - (long long)h * P.tph);
+            return;
+        }
+        int lo = 0, hi = P.heads - 1;                         // the last head whose first tile is not past `tile`
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (P.htab[mid].tbase <= tile) lo = mid; else hi = mid - 1;
+        }
+        h = lo;
+        t = (int)(tile - P.htab[lo].tbase);
+        load(P);
+    }
+    __device__ __forceinline__ void advance(const SParams &P, int n)   // (never past the last tile of the call)
+    {
+        t += n;
+        while (t >= tph) { t -= tph; ++h; load(P); }
+    }
+};
+
+// Two block maxima, times c, as halves: the first block in the low half.
+__device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
+{
+    uint32_t d;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+
+// As p1_half, with the largest of the 16 values handed back.
+__device__ __forceinline__ float p1_half_max(uint32_t (&v)[16], int c0, int valid, float c, float lazy, float2 cc, RowState &st)
+{
+    if (valid < c0 + 16) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) if (c0 + t >= valid) v[t] = 0xff800000u;
+    }
+    const float cm = max_of16(v);
+    if (cm > st.m + lazy) {
+        const float f = ex2(c * (st.m - cm));
+        st.l01 = make_float2(st.l01.x * f, st.l01.y * f);
+        st.l23 = make_float2(st.l23.x * f, st.l23.y * f);
+        st.m = cm;
+    }
+    const float nb = -st.m * c;
+    exp_acc16(st.l01, st.l23, v, cc, make_float2(nb, nb));
+    return cm;
+}
+
+// grid: one CTA per SM; CTA b takes tiles [b T / G, (b + 1) T / G) of the call.  Warps 0 .. 4 kGroups - 1 are the epilogue groups
+// (a thread owns a query row), then the TMA producer and the MMA issuer.
+template <int kGroups>
+__global__ void __launch_bounds__(stats_threads(kGroups), 1)
+row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ,
+          const __grid_constant__ CUtensorMap mapW, const __grid_constant__ SParams P)
+{
+    constexpr int kEpi = 4 * kGroups;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    if (smem_u32(smem_raw) & 1023u) {
+        if (threadIdx.x == 0) atomicMax(P.status + kWStatus, (int)JQ_ERR_CUDA);
+        return;
+    }
+    const uint32_t q_bytes = (uint32_t)P.Rbox * kD * 2;
+    uint8_t *const qbuf = smem_raw, *const kbuf = smem_raw + 2 * (size_t)q_bytes;
+    SCtl *const ctl = (SCtl *)(kbuf + (size_t)P.stages * kPStage);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int R = P.R, Rpad = P.Rpad, stages = P.stages, nblk = P.Rbox / 128;
+    int *const status = P.status;
+#ifdef JQ_DEBUG
+    DebugRecord *const dbg = P.dbg_rec;
+#endif
+    const long long G = gridDim.x, first = blockIdx.x * P.T / G;
+    const int ntiles = (int)((blockIdx.x + 1) * P.T / G - first);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kSMaxStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->q_full[s], 1); mbar_init(&ctl->q_empty[s], 1); }
+        for (uint32_t s = 0; s < kSSlots; ++s) { mbar_init(&ctl->t_full[s], 1); mbar_init(&ctl->t_empty[s], 4); }
+        ctl->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kEpi + 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(kSTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *(volatile uint32_t *)&ctl->tmem_base;
+    cudaGridDependencySynchronize();             // no global memory has been touched so far
+    cudaTriggerProgrammaticLaunchCompletion();   // the next kernel may be set up where there is room; it waits for this one's results
+
+    if (warp == kEpi) {
+        // ---------------------------------------------------------------- TMA producer
+        if (lane == 0) {
+            uint32_t st = 0, ph = 0, qn = 0;
+            int prev_h = -1, prev_unit = -1, c2 = 0;
+            const CUtensorMap *mk = &mapK, *mq = &mapQ;
+            Walk at;
+            at.start(P, first);
+#pragma unroll 1
+            for (int n = 0; n < ntiles; ++n) {
+                if (at.h != prev_h) {
+                    prev_h = c2 = at.h;
+                    if (P.maps) {
+                        const int unit = at.h / P.hpu;
+                        c2 = at.h - unit * P.hpu;
+                        if (unit != prev_unit) {
+                            mk = P.maps + kMapsPerUnit * (size_t)unit; mq = mk + 1;
+                            tensormap_acquire(mk); tensormap_acquire(mq);
+                            prev_unit = unit;
+                        }
+                    }
+                    const uint32_t qb = qn & 1;
+                    if (!mbar_wait(&ctl->q_empty[qb], ((qn >> 1) & 1) ^ 1, &ctl->abort_flag, status, kSSleepLong)) break;
+                    mbar_expect_tx(&ctl->q_full[qb], q_bytes);
+                    tma_load_3d(qbuf + (size_t)qb * q_bytes, mq, &ctl->q_full[qb], 0, 0, c2);
+                    tma_load_3d(qbuf + (size_t)qb * q_bytes + q_bytes / 2, mq, &ctl->q_full[qb], 64, 0, c2);
+                    ++qn;
+                }
+                if (!mbar_wait(&ctl->empty[st], ph ^ 1, &ctl->abort_flag, status, kSSleepLong)) break;
+                mbar_expect_tx(&ctl->full[st], kPStage);
+                const bool wt = P.wtile && at.t == at.tph - 1;   // the window keys of the head (rows past w read as zero)
+                const CUtensorMap *map = wt ? &mapW : mk;
+                const int j0 = wt ? 0 : at.t * kPTile;
+                if (JQ_IN(st, stages, kDbgPrune, 1)) {
+                    tma_load_3d(kbuf + (size_t)st * kPStage, map, &ctl->full[st], 0, j0, c2);
+                    tma_load_3d(kbuf + (size_t)st * kPStage + kPHalf, map, &ctl->full[st], 64, j0, c2);
+                }
+                if (++st == (uint32_t)stages) { st = 0; ph ^= 1; }
+                if (n + 1 < ntiles) at.advance(P, 1);
+            }
+        }
+        __syncwarp();
+    } else if (warp == kEpi + 1) {
+        // ---------------------------------------------------------------- MMA issuer (all 32 lanes walk the loop)
+        const uint32_t idesc = instr_desc(128, kPTile);
+        uint32_t st = 0, ph = 0, qn = 0, u = 0;
+        int prev_h = -1;
+        bool ok = true;
+        Walk at;
+        at.start(P, first);
+#pragma unroll 1
+        for (int n = 0; n < ntiles && ok; ++n) {
+            if (at.h != prev_h) {
+                if (qn > 0) tc_commit(&ctl->q_empty[(qn - 1) & 1]);   // the previous head's queries are free once its products retire
+                if (!mbar_wait(&ctl->q_full[qn & 1], (qn >> 1) & 1, &ctl->abort_flag, status, kSSleepShort)) { ok = false; break; }
+                prev_h = at.h; ++qn;
+            }
+            if (!mbar_wait(&ctl->full[st], ph, &ctl->abort_flag, status, kSSleepShort)) { ok = false; break; }
+            const uint32_t k_lo = desc_lo(smem_u32(kbuf) + st * kPStage), q_lo = desc_lo(smem_u32(qbuf) + ((qn - 1) & 1) * q_bytes);
+#pragma unroll 1
+            for (int blk = 0; blk < nblk; ++blk, ++u) {
+                const uint32_t slot = u % kSSlots;
+                if (!mbar_wait(&ctl->t_empty[slot], ((u / kSSlots) & 1) ^ 1, &ctl->abort_flag, status, kSSleepShort)) { ok = false; break; }
+                tc_fence_after();
+                if (!JQ_IN(st, stages, kDbgPrune, 2)) { ok = false; break; }
+                tc_mma_block(tmem + slot * kSSlotCols, q_lo + (uint32_t)blk * (kPHalf >> 4), k_lo, q_bytes / 2, kPHalf, idesc);
+                tc_commit(&ctl->t_full[slot]);
+            }
+            if (ok) tc_commit(&ctl->empty[st]);
+            if (++st == (uint32_t)stages) { st = 0; ph ^= 1; }
+            if (n + 1 < ntiles) at.advance(P, 1);
+        }
+    } else {
+        // ---------------------------------------------------------------- epilogue groups: accumulator block u is group u % kGroups'
+        const int grp = warp >> 2, quarter = warp & 3, row0 = quarter * 32 + lane;
+        const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int bs = nblk - 1, nunits = ntiles << bs;
+        const float c = P.c, lazy = 64.f / c;
+        const float2 cc = make_float2(c, c);
+        const int win_i0 = row0 % P.w, win_i1 = (row0 + 128) % P.w;   // soft-token index of this thread's row in block 0 / block 1
+        uint32_t va[16], vb[16];
+        bool ok = true, pre = false;
+        auto release = [&](uint32_t slot) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->t_empty[slot], 1);
+        };
+        // (with as many groups as slots a group's next block cannot be complete before it gives its slot back)
+        constexpr bool kLookAhead = kGroups < (int)kSSlots;
+        auto try_begin = [&](uint32_t u) -> bool {
+            const uint32_t slot = u % kSSlots;
+            if (!__all_sync(0xffffffffu, mbar_test(&ctl->t_full[slot], (u / kSSlots) & 1))) return false;
+            tc_fence_after();
+            JQ_TMEM_LD16(lane_addr + slot * kSSlotCols, va);
+            return true;
+        };
+        auto begin = [&](uint32_t u) -> bool {
+            const uint32_t slot = u % kSSlots;
+            if (!mbar_wait(&ctl->t_full[slot], (u / kSSlots) & 1, &ctl->abort_flag, status, kSSleepShort)) return false;
+            tc_fence_after();
+            JQ_TMEM_LD16(lane_addr + slot * kSSlotCols, va);
+            return true;
+        };
+        RowState st0 = {-INFINITY, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, st1 = st0;
+        Walk at;
+        if (ntiles > 0) at.start(P, first);
+        int pub = ntiles > 0 ? at.h : 0, tile = 0;            // next head whose statistics this warp has to publish; tile of the run
+        // Every group publishes for every head of the CTA's run, nothing seen as (-inf, 0).
+        auto publish_upto = [&](int head_end) {
+#pragma unroll 1
+            for (; pub < head_end; ++pub) {
+                const long long slot = ((long long)blockIdx.x + pub) * kGroups + grp;
+                float2 *dst = P.part + slot * R;
+                const bool in = JQ_IN(slot * R + R - 1, P.n_part, kDbgPrune, 3);
+                if (row0 < R && in) dst[row0] = make_float2(st0.m, (st0.l01.x + st0.l01.y) + (st0.l23.x + st0.l23.y));
+                if (nblk == 2 && row0 + 128 < R && in) dst[row0 + 128] = make_float2(st1.m, (st1.l01.x + st1.l01.y) + (st1.l23.x + st1.l23.y));
+                st0.m = st1.m = -INFINITY;
+                st0.l01 = st0.l23 = st1.l01 = st1.l23 = make_float2(0.f, 0.f);
+            }
+        };
+#pragma unroll 1
+        for (int k = grp; k < nunits; k += kGroups) {
+            const int n = k >> bs, blk = k & bs;
+            at.advance(P, n - tile);
+            tile = n;
+            if (at.h != pub) publish_upto(at.h);
+            const uint32_t u = (uint32_t)k, slot = u % kSSlots, taddr = lane_addr + slot * kSSlotCols;
+            if (!pre && !begin(u)) { ok = false; break; }
+            // keys of the tile that count for this thread's row: the prefix keys or, in the window tile, the window keys up to
+            // the row's own position (causal)
+            const bool wt = P.wtile && at.t == at.tph - 1;
+            const int valid = wt ? min(P.w, (blk ? win_i1 : win_i0) + 1) : min(kPTile, at.L - at.t * kPTile);
+            uint32_t *const bm = P.bmax + (first + n) * 4 * Rpad + blk * 128 + row0;
+            const bool store = blk * 128 + row0 < Rpad && JQ_IN((first + n + 1) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 4);   // warp-uniform
+            if (blk == 1) { const RowState x = st0; st0 = st1; st1 = x; }
+#pragma unroll 1
+            for (int c0 = 0; c0 < kPTile; c0 += 32) {
+                JQ_TMEM_WAIT16(va);
+                JQ_TMEM_LD16(taddr + c0 + 16, vb);
+                const float ma = p1_half_max(va, c0, valid, c, lazy, cc, st0);
+                JQ_TMEM_WAIT16(vb);
+                if (c0 + 32 < kPTile) JQ_TMEM_LD16(taddr + c0 + 32, va);
+                else {
+                    release(slot);
+                    if (kLookAhead) pre = k + kGroups < nunits && try_begin(u + kGroups);
+                }
+                const float mb = p1_half_max(vb, c0 + 16, valid, c, lazy, cc, st0);
+                if (store) bm[(c0 >> 5) * Rpad] = pack_half2(ma * c, mb * c);
+            }
+            if (blk == 1) { const RowState x = st0; st0 = st1; st1 = x; }
+        }
+        if (ok && ntiles > 0) {
+            at.advance(P, ntiles - 1 - tile);
+            publish_upto(at.h + 1);
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");   // (a read requested ahead on a path that gave up)
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (*(volatile int *)&ctl->abort_flag) __nanosleep(200000);   // let copies still in flight land before the CTA goes
+    if (warp == kEpi + 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSTmemCols) : "memory");
+    }
+}
+
+// ------------------------------------------------------------------ scores of the candidates
+
+constexpr int kCMaxCluster = 16;
+constexpr int kCBins = 1024;                     // bins of 1/16 octave: 64 octaves from 2^-54 up to 2^10
+constexpr int kCBase = (127 - 54) << 4;
+constexpr int kCMaxStages = 4;
+constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16 bits
+__host__ __device__ constexpr int cand_groups(bool wide) { return wide ? 4 : 2; }
+__host__ __device__ constexpr int cand_threads(bool wide) { return cand_groups(wide) * 128 + 64; }
+
+struct CCtl {
+    uint64_t full[kCMaxStages], empty[kCMaxStages], q_full, t_full[2], t_empty[2];
+    uint32_t tmem_base;
+    int abort_flag;
+    int bin, total;                              // find_bin's answer; candidates of the whole head in this round
+    int n;                                       // blocks on this CTA's list
+    int scan[16];
+    int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
+    alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads; before, pairs of statistics
+    alignas(16) float Ms[kMaxR];                 // minus the row normalisers
+};
+constexpr uint32_t kCCtlBytes = 4096;
+static_assert(sizeof(CCtl) <= kCCtlBytes && offsetof(CCtl, Ms) % 16 == 0 && offsetof(CCtl, xs) % 16 == 0, "control block");
+
+struct CParams {
+    int L, tph, nkeep;         // one shape (tph: tiles per head in row_stats' numbering, the window tile included)
+    int R, Rbox, Rpad, radius;
+    int stages, groups;        // K ring; row_stats' epilogue groups
+    int sms;                   // row_stats' grid
+    int share;                 // most tiles of a head that a CTA looks after
+    int hpu, first_pct;        // heads per unit; blocks of round 1 per 100 pairs kept
+    long long T;
+    float c;
+    const float2 *part;
+    const uint32_t *bmax;
+    float *scores;
+    int *status;
+    const HeadRec *htab;
+    const CUtensorMap *maps;
+#ifdef JQ_DEBUG
+    DebugRecord *dbg_rec;
+    long long n_part, n_bmax, n_scores;
+#endif
+};
+
+__device__ __forceinline__ uint32_t remote(const void *p, uint32_t rank)   // the same place in CTA `rank` of the cluster
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ uint4 remote_ld4(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+// The bin of a value >= 0 (given as the upper 16 bits of a float, rounded either way): its lower edge is not above the value.
+__device__ __forceinline__ int bin_of(uint32_t top16) { return min(max((int)(top16 >> 3) - kCBase, 0), kCBins - 1); }
+// The lower edge of a bin, as the upper 16 bits of a float; of the lowest bin 0.
+__device__ __forceinline__ uint32_t edge_of(int bin) { return bin > 0 ? (uint32_t)(bin + kCBase) << 3 : 0u; }
+
+template <bool kWide>
+__global__ void __launch_bounds__(cand_threads(kWide), kWide ? 1 : 2)
+score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CParams P)
+{
+    constexpr int kGroups = cand_groups(kWide), kEpi = 4 * kGroups, kTE = 32 * kEpi;
+    constexpr uint32_t kSlotCols = kWide ? 256 : 128, kCols = 2 * kSlotCols;   // two accumulators in tensor memory
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t q_bytes = (uint32_t)P.Rbox * kD * 2;
+    uint8_t *const qbuf = smem_raw, *const kbuf = smem_raw + q_bytes;
+    CCtl *const ctl = (CCtl *)(kbuf + (size_t)P.stages * kPStage);
+    uint32_t *const hist = (uint32_t *)((uint8_t *)ctl + kCCtlBytes);            // [kCBins]
+    uint16_t *const ub = (uint16_t *)(hist + kCBins);                            // [8 share]: bounds of this CTA's share, upper 16 bits
+    uint16_t *const list = ub + 8 * P.share;                                     // [8 share]: blocks that this CTA scores
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint32_t rank, C;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    const int head = (int)(blockIdx.x / C);
+    int *const status = P.status;
+    const int R = P.R, Rpad = P.Rpad;
+#ifdef JQ_DEBUG
+    DebugRecord *const dbg = P.dbg_rec;
+#endif
+    if (smem_u32(smem_raw) & 1023u) {   // uniform over the grid
+        if (tid == 0) atomicMax(status + kWStatus, (int)JQ_ERR_CUDA);
+        return;
+    }
+    if (tid == 0) {
+        for (int s = 0; s < kCMaxStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        mbar_init(&ctl->q_full, 1);
+        for (int s = 0; s < 2; ++s) { mbar_init(&ctl->t_full[s], 1); mbar_init(&ctl->t_empty[s], kWide ? 8 : 4); }
+        ctl->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kEpi + 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int i = tid; i < kCBins; i += blockDim.x) hist[i] = 0u;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *(volatile uint32_t *)&ctl->tmem_base;
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // waited for before another CTA's memory is touched
+    cudaGridDependencySynchronize();             // nothing in global memory has been touched so far
+    cudaTriggerProgrammaticLaunchCompletion();
+
+    int L = P.L, nkeep = P.nkeep, kv_in = head, tph1 = P.tph;
+    long long soff = (long long)head * L, tbase = (long long)head * P.tph;
+    const CUtensorMap *mb = &mapB, *mq = &mapQ;
+    if (P.htab) {
+        const HeadRec r = P.htab[head];
+        L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; tbase = r.tbase;
+        tph1 = (L + kPTile - 1) / kPTile;
+        mq = P.maps + kMapsPerUnit * (size_t)r.unit + 1; mb = mq + 1;
+    }
+    const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
+    const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
+    const int b0 = 8 * ts, nbs = min(8 * te, nb) - b0;                                          // and their blocks
+    auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kTE) : "memory"); };
+    // everybody: all CTAs of the head have got here, and what they wrote is seen
+    auto sync_all = [&]() {
+        if (C == 1) { __syncthreads(); return; }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
+    // epilogue threads: exclusive scan of one int per thread, and the sum
+    auto scan = [&](int v, int &total) -> int {
+        int inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
+        if (lane == 31) ctl->scan[warp] = inc;
+        epi_sync();
+        const int s = lane < kEpi ? ctl->scan[lane] : 0;
+        total = __reduce_add_sync(0xffffffffu, s);
+        const int before = __reduce_add_sync(0xffffffffu, lane < warp ? s : 0);
+        epi_sync();
+        return before + inc - v;
+    };
+    // epilogue threads: the highest bin with at least `target` entries in it and above it, over all CTAs of the head (0: there is none)
+    auto find_bin = [&](int target) -> int {
+        constexpr int per = kCBins / kTE;                     // 4 or 2 bins per thread, from the top
+        const int at = kCBins - per * (tid + 1);
+        int n[per] = {};
+#pragma unroll 4
+        for (uint32_t d = 0; d < C; ++d) {
+            if (per == 4) {
+                const uint4 v = remote_ld4(remote(hist + at, d));
+                n[0] += (int)v.x; n[1] += (int)v.y; n[per - 2] += (int)v.z; n[per - 1] += (int)v.w;
+            } else {
+                const uint4 v = remote_ld4(remote(hist + (at & ~3), d));
+                n[0] += (int)(at & 2 ? v.z : v.x); n[1] += (int)(at & 2 ? v.w : v.y);
+            }
+        }
+        int sum = 0, total;
+#pragma unroll
+        for (int i = 0; i < per; ++i) sum += n[i];
+        if (tid == 0) ctl->bin = 0;
+        int above = scan(sum, total);
+#pragma unroll
+        for (int i = per - 1; i >= 0; --i) {
+            if (above < target && target <= above + n[i]) ctl->bin = at + i;
+            above += n[i];
+        }
+        epi_sync();
+        return ctl->bin;
+    };
+
+    uint32_t st = 0, ph = 0, u = 0;                           // K ring and its phase; tiles so far (producer, MMA, epilogue alike)
+    uint32_t lo16 = 0u, hi16 = 0u;                            // the blocks of a round: bounds in [lo16, hi16)
+    uint32_t cut = 0u;                                        // in the end: blocks with bounds from here on have been scored
+
+    if (warp == kEpi) {
+        if (lane == 0) {
+            if (P.maps) { tensormap_acquire(mq); tensormap_acquire(mb); }
+            mbar_expect_tx(&ctl->q_full, q_bytes);
+            tma_load_3d(qbuf, mq, &ctl->q_full, 0, 0, kv_in);
+            tma_load_3d(qbuf + q_bytes / 2, mq, &ctl->q_full, 64, 0, kv_in);
+        }
+        __syncwarp();
+        if (P.maps) tensormap_acquire(mb);                    // (all lanes load)
+    } else if (warp < kEpi) {
+        // ---- the normalisers: the CTAs of row_stats that had tiles of this head, each with a pair per row and group
+        {
+            const long long T = P.T, G = P.sms;
+            const long long c_lo = ((tbase + 1) * G - 1) / T, c_hi = ((tbase + tph1) * G - 1) / T;   // owners of the first and last tile
+            const int nsl = (int)(c_hi - c_lo + 1) * P.groups;
+            const long long s0 = (c_lo + head) * P.groups;
+            const int row = tid & (kWide ? 255 : 127), sub = tid >> (kWide ? 8 : 7);          // two threads per row
+            const float2 *src = P.part + s0 * R + row;
+            float m = -INFINITY, l = 0.f;
+            if (row < R) {
+#pragma unroll 1
+                for (int i0 = sub; i0 < nsl; i0 += 16) {
+                    float2 p[8];
+                    float mn = m;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int i = i0 + 2 * k;
+                        p[k] = i < nsl && JQ_IN((s0 + i) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)i * R) : make_float2(-INFINITY, 0.f);
+                        if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
+                    }
+                    if (mn > -INFINITY) {
+                        l *= ex2(P.c * (m - mn));
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) if (p[k].y > 0.f) l = fmaf(p[k].y, ex2(P.c * (p[k].x - mn)), l);
+                        m = mn;
+                    }
+                }
+            }
+            float2 *const other = (float2 *)&ctl->xs[0][0][0];
+            static_assert(sizeof(ctl->xs) >= kMaxR * sizeof(float2), "room for a pair per row");
+            if (sub == 1) other[row] = make_float2(m, l);
+            epi_sync();
+            if (sub == 0) {
+                const float2 o = other[row];
+                float M = INFINITY;                           // silences a column that is not a query row
+                if (row < R) {
+                    const float mn = fmaxf(m, o.x);
+                    l = (l > 0.f ? l * ex2(P.c * (m - mn)) : 0.f) + (o.y > 0.f ? o.y * ex2(P.c * (o.x - mn)) : 0.f);
+                    M = fmaf(P.c, mn, log2f(l));
+                }
+                ctl->Ms[row] = -M;
+                if (!kWide) ctl->Ms[128 + row] = -INFINITY;
+            }
+            epi_sync();
+        }
+        // ---- the bounds.  A lane takes four neighbouring rows (eight with more than 128), of two blocks at a time.
+        {
+            constexpr int kV = kWide ? 2 : 1;
+            float nm[4 * kV];
+#pragma unroll
+            for (int i = 0; i < 4 * kV; ++i) nm[i] = ctl->Ms[(i >> 2) * 128 + 4 * lane + (i & 3)];
+#pragma unroll 1
+            for (int t = ts + warp; t < te; t += kEpi) {
+                uint4 v[4][kV];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int x = 0; x < kV; ++x) {
+                        const long long at = ((tbase + t) * 4 + q) * Rpad + x * 128 + 4 * lane;
+                        const bool in = x * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6);
+                        v[q][x] = in ? __ldcg((const uint4 *)(P.bmax + at)) : make_uint4(0u, 0u, 0u, 0u);   // (rows that are none have a normaliser of inf)
+                    }
+                float s[8];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    s[2 * q] = s[2 * q + 1] = 0.f;
+#pragma unroll
+                    for (int x = 0; x < kV; ++x) {
+                        const uint32_t e[4] = {v[q][x].x, v[q][x].y, v[q][x].z, v[q][x].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float2 f = __half22float2(*(const __half2 *)&e[i]);
+                            f.x = fmaxf(f.x, -65504.f); f.y = fmaxf(f.y, -65504.f);
+                            s[2 * q] += ex2(fmaf(fabsf(f.x), 1.f / 1024.f, f.x) + nm[4 * x + i]);
+                            s[2 * q + 1] += ex2(fmaf(fabsf(f.y), 1.f / 1024.f, f.y) + nm[4 * x + i]);
+                        }
+                    }
+                }
+                // eight sums over the 32 lanes: after three exchanges of halves a lane holds one block's part
+                const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+                float a[4], b[2], r;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i] = (h4 ? s[4 + i] : s[i]) + __shfl_xor_sync(0xffffffffu, h4 ? s[i] : s[4 + i], 16);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) b[i] = (h3 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[2 + i], 8);
+                r = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+                r += __shfl_xor_sync(0xffffffffu, r, 2);
+                r += __shfl_xor_sync(0xffffffffu, r, 1);
+                const int blk = 8 * (t - ts) + (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
+                if ((lane & 3) == 0 && blk < nbs && JQ_IN(blk, 8 * P.share, kDbgPrune, 7)) {
+                    const uint32_t x = (__float_as_uint(r * (1.f + 1.f / 64.f)) + 0xffffu) >> 16;
+                    ub[blk] = (uint16_t)x;
+                    atomicAdd(&hist[bin_of(x)], 1u);
+                }
+            }
+        }
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    sync_all();
+
+    const int wanted = max(1, min(nb, (int)((long long)nkeep * P.first_pct / 100) + 1));
+#pragma unroll 1
+    for (int round = 0; round < 2; ++round) {
+        // ---- the blocks of this round: [lo16, hi16) of the bounds
+        if (warp < kEpi) {
+            const int bin = find_bin(round == 0 ? wanted : nkeep);
+            if (round == 0) { lo16 = edge_of(bin); hi16 = 0x10000u; cut = lo16; }
+            else { hi16 = lo16; lo16 = min(edge_of(bin), lo16); cut = lo16; }
+            // this CTA's share of them, and their places in the head's list
+            const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
+            int mine = 0, total;
+            for (int i = i0; i < i1; ++i) mine += ub[i] >= lo16 && ub[i] < hi16;
+            int at = scan(mine, total);
+            if (C > 1 && warp == 0 && lane < (int)C)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(&ctl->cnt[rank], lane)), "r"(total) : "memory");
+            if (C == 1) {
+                for (int i = i0; i < i1; ++i)
+                    if (ub[i] >= lo16 && ub[i] < hi16) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 8)) list[at] = (uint16_t)i; ++at; }
+                if (tid == 0) ctl->n = total;
+                for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;   // (read by this CTA alone, before the scan)
+            }
+        }
+        sync_all();
+        if (C > 1) {
+            if (warp < kEpi) {
+                const int have = lane < (int)C ? ctl->cnt[lane] : 0;
+                const int all = __reduce_add_sync(0xffffffffu, have), before = __reduce_add_sync(0xffffffffu, lane < (int)rank ? have : 0);
+                const int per_cta = ((all + (int)C - 1) / (int)C + 7) & ~7;      // whole tiles
+                const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
+                int mine = 0, total;
+                for (int i = i0; i < i1; ++i) mine += ub[i] >= lo16 && ub[i] < hi16;
+                int at = before + scan(mine, total);
+                for (int i = i0; i < i1; ++i)
+                    if (ub[i] >= lo16 && ub[i] < hi16) {
+                        const int to = at / per_cta, x = at - to * per_cta;
+                        if (JQ_IN(x, 8 * P.share, kDbgPrune, 9) && JQ_IN(to, C, kDbgPrune, 10))
+                            asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(remote(list + x, (uint32_t)to)), "h"((uint16_t)(b0 + i)) : "memory");
+                        ++at;
+                    }
+                if (tid == 0) ctl->n = per_cta > 0 ? min(max(all - (int)rank * per_cta, 0), per_cta) : 0;
+                for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;            // (everybody has read it)
+            }
+            sync_all();
+        }
+        const int n = ctl->n, nt = (n + 7) >> 3;
+        if (warp == kEpi) {
+            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, a lane each
+#pragma unroll 1
+            for (int i = 0; i < nt; ++i) {
+                const int have = min(8, n - 8 * i);
+                if (!__all_sync(0xffffffffu, mbar_wait(&ctl->empty[st], ph ^ 1, &ctl->abort_flag, status, 64))) break;
+                if (lane == 0) mbar_expect_tx(&ctl->full[st], (uint32_t)have * 2u * kPBlockHalf);
+                __syncwarp();
+                if ((lane >> 1) < have) {
+                    const int x = lane >> 1, half = lane & 1, blk = list[8 * i + x];
+                    if (JQ_IN(blk, nb, kDbgPrune, 11) && JQ_IN(st, P.stages, kDbgPrune, 12))
+                        tma_load_3d(kbuf + (size_t)st * kPStage + half * kPHalf + x * kPBlockHalf, mb, &ctl->full[st], 64 * half, blk * kPBlock, kv_in);
+                }
+                __syncwarp();
+                if (++st == (uint32_t)P.stages) { st = 0; ph ^= 1; }
+            }
+        } else if (warp == kEpi + 1) {
+            // ------------------------------------------------------------ MMA issuer
+            const uint32_t ia = instr_desc(kPTile, min(128, Rpad)), ib = instr_desc(kPTile, max(32, Rpad - 128));
+            const uint32_t q_lo = desc_lo(smem_u32(qbuf));
+            bool ok = mbar_wait(&ctl->q_full, 0, &ctl->abort_flag, status, 32);   // (also without tiles: the copy must have landed when the CTA leaves)
+#pragma unroll 1
+            for (int i = 0; i < nt && ok; ++i, ++u) {
+                const uint32_t slot = u & 1;
+                if (!mbar_wait(&ctl->full[st], ph, &ctl->abort_flag, status, 32) ||
+                    !mbar_wait(&ctl->t_empty[slot], ((u >> 1) & 1) ^ 1, &ctl->abort_flag, status, 32)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t k_lo = desc_lo(smem_u32(kbuf) + st * kPStage), d = tmem + slot * kSlotCols;
+                tc_mma_block(d, k_lo, q_lo, kPHalf, q_bytes / 2, ia);
+                if (kWide) tc_mma_block(d + 128, k_lo, q_lo + (kPHalf >> 4), kPHalf, q_bytes / 2, ib);
+                tc_commit(&ctl->t_full[slot]);
+                tc_commit(&ctl->empty[st]);
+                if (++st == (uint32_t)P.stages) { st = 0; ph ^= 1; }
+            }
+        } else {
+            // ------------------------------------------------------------ epilogue: a thread owns a key and adds exp2(c s - M_r) over the rows
+            const int grp = warp >> 2, quarter = warp & 3, row0 = quarter * 32 + lane;
+            const uint32_t mine = kWide ? (uint32_t)grp >> 1 : (uint32_t)grp;     // which of the two accumulators: every other tile
+            const int half = kWide ? grp & 1 : 0;                                 // (R > 128) the first or the second 128 columns
+            const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + mine * kSlotCols + (uint32_t)half * 128;
+            const int np = (half ? Rpad - 128 : min(128, Rpad)) >> 5;
+            const float2 cc = make_float2(P.c, P.c);
+            const float4 *const bias = (const float4 *)(ctl->Ms + 128 * half);
+            uint32_t va[16], vb[16];
+#pragma unroll 1
+            for (int i = (int)((mine - u) & 1u); i < nt; i += 2) {
+                const uint32_t uu = u + (uint32_t)i;
+                // (after a wait that ran out the loop goes on without reading: the groups meet at a barrier below)
+                const bool ok = __all_sync(0xffffffffu, mbar_wait(&ctl->t_full[mine], (uu >> 1) & 1, &ctl->abort_flag, status, 32));
+                tc_fence_after();
+                if (ok) JQ_TMEM_LD16(lane_addr, va);
+                float2 a01 = make_float2(0.f, 0.f), a23 = a01;
+#pragma unroll 1
+                for (int p = 0; p < (ok ? np : 0); ++p) {
+                    JQ_TMEM_WAIT16(va);
+                    JQ_TMEM_LD16(lane_addr + 32 * p + 16, vb);
+                    exp_acc16(a01, a23, va, cc, bias + 8 * p);
+                    JQ_TMEM_WAIT16(vb);
+                    if (p + 1 < np) JQ_TMEM_LD16(lane_addr + 32 * p + 32, va);
+                    else {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&ctl->t_empty[mine], 1);
+                    }
+                    exp_acc16(a01, a23, vb, cc, bias + 8 * p + 4);
+                }
+                float sum = (a01.x + a01.y) + (a23.x + a23.y);
+                if (kWide) {                                  // the two halves of a key's sum meet in the first half's thread
+                    float *const xs = ctl->xs[mine][(uu >> 1) & 1];
+                    if (half) xs[row0] = sum;
+                    asm volatile("bar.sync %0, 256;" ::"r"(2 + mine) : "memory");
+                    if (half) continue;
+                    sum += xs[row0];
+                }
+                const int x = 8 * i + (row0 >> 4), blk = x < n ? list[x] : nb, key = blk * kPBlock + (row0 & 15);
+                const bool have = x < n && key < L;
+                if (have && JQ_IN(soff + key, P.n_scores, kDbgPrune, 13)) P.scores[soff + key] = sum;
+                if (round == 0) {
+                    // what this block alone guarantees of the pooled scores of its positions
+                    float m = have ? sum : 0.f;
+                    int w = 0;
+#pragma unroll 1
+                    while (w < min(P.radius, 15)) {
+                        const int s = min(2 * w + 1, min(P.radius, 15) - w);
+                        m = fmaxf(m, fmaxf(__shfl_up_sync(0xffffffffu, m, s, 16), __shfl_down_sync(0xffffffffu, m, s, 16)));
+                        w += s;
+                    }
+                    if (have) atomicAdd(&hist[bin_of(__float_as_uint(m) >> 16)], 1u);
+                }
+            }
+        }
+        if (warp < kEpi) u += (uint32_t)nt;
+        sync_all();
+    }
+    // the blocks of this CTA's share that nothing needs
+    if (warp < kEpi && cut > 0u) {
+        float *const s = P.scores + soff + (long long)b0 * kPBlock;
+        const int m = min(nbs * kPBlock, L - b0 * kPBlock);
+        for (int i = tid; i < m; i += kTE)
+            if (ub[i >> 4] < cut && JQ_IN(soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
+    }
+    // ---------------------------------------------------------------- exit
+    tc_fence_before();
+    __syncthreads();
+    if (*(volatile int *)&ctl->abort_flag) __nanosleep(200000);   // let copies still in flight land before the CTA goes
+    if (warp == kEpi + 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+    }
+}
+
+// ------------------------------------------------------------------ host side
+
+constexpr size_t stats_smem(int Rbox, int stages) { return 2 * (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kSCtlBytes; }
+size_t cand_smem(int Rbox, int stages, int share) { return (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kCCtlBytes + kCBins * 4 + (size_t)share * 32; }
+constexpr size_t kCMaxSmem = 227 * 1024, kCTwoPerSm = 113 * 1024;
+
+struct PruneDevice {
+    int sms = 0;
+    int resident[2][kCMaxCluster + 1] = {};   // [R > 128][C]: clusters of C CTAs that fit at a time
+    bool ready = false;
+};
+
+bool prune_device(PruneDevice *out)
+{
+    static PruneDevice devs[64];
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    PruneDevice &d = devs[dev];
+    if (!d.ready) {
+        d.sms = device_sms();
+        if (d.sms < 1) return false;
+        for (auto k : {row_stats<kSGroupsNarrow>, row_stats<kSGroupsWide>})
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess) return false;
+        for (int wide = 0; wide < 2; ++wide) {
+            const auto k = wide ? score_candidates<true> : score_candidates<false>;
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess ||
+                cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+            for (int C = 1; C <= kCMaxCluster; ++C) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)C);
+                cfg.blockDim = dim3((unsigned)cand_threads(wide));
+                cfg.dynamicSmemBytes = wide ? kCMaxSmem : kCTwoPerSm;
+                cudaLaunchAttribute attr[1];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+                cfg.attrs = attr;
+                cfg.numAttrs = 1;
+                if (cudaOccupancyMaxActiveClusters(&d.resident[wide][C], k, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[wide][C] = 0; }
+            }
+        }
+        d.ready = true;
+    }
+    *out = d;
+    return true;
+}
+
+}  // namespace
+
+size_t prune_bytes(long long tiles, int heads, int R)
+{
+    const int Rpad = (R + 31) & ~31, groups = R > 128 ? kSGroupsWide : kSGroupsNarrow;
+    return align_up((size_t)tiles * 4 * Rpad * 4, 256) + align_up((size_t)(heads + 256) * groups * R * sizeof(float2), 256);
+}
+
+// Whether a call takes this way.  tiles: of all heads; keys: sum of the heads' lengths; kept: sum of what the heads keep.
+bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L, int sms)
+{
+    (void)heads; (void)sms;
+    const int R = s.group * s.w;
+    if (R <= 64 || tiles >= (1ll << 30) || max_L > kPBlock * kCMaxBlocks) return false;
+    const double per = s.pool >= 7 ? 6.0 : s.pool >= 3 ? 2.5 : 1.2;    // kept positions per block that holds one
+    return tiles * (R > 128 ? 2 : 1) >= 6000 && kept / per * 16.0 < 0.35 * keys;
+}
+
+jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, float *scores, const Workspace &w, cudaStream_t st,
+                              const void *Kwin, const UnitTables *tables, int k_head_rows)
+{
+    PruneDevice dev;
+    if (!prune_device(&dev)) return JQ_ERR_CUDA;
+    const int R = s.group * s.w, Rbox = R <= 128 ? 128 : 256, Rpad = (R + 31) & ~31, wide = R > 128;
+    const int wtile = Kwin ? 1 : 0, tph = (s.L + kPTile - 1) / kPTile + wtile;
+    const long long T = tables ? tables->total_tiles : (long long)s.Hkv * tph;
+    SParams S = {};
+    S.L = s.L; S.tph = tph; S.R = R; S.Rbox = Rbox; S.Rpad = Rpad; S.w = s.w; S.wtile = wtile;
+    S.stages = wide ? 3 : 5;
+    S.T = T; S.heads = s.Hkv; S.hpu = tables ? tables->hpu : s.Hkv;
+    S.c = 1.4426950408889634f / sqrtf((float)s.d);
+    const size_t bmax_bytes = align_up((size_t)T * 4 * Rpad * 4, 256);
+    S.bmax = (uint32_t *)w.prune;
+    S.part = (float2 *)((char *)w.prune + bmax_bytes);
+    S.status = w.status;
+    const int groups = wide ? kSGroupsWide : kSGroupsNarrow, grid = (int)(T < dev.sms ? T : dev.sms);
+    CParams Q2 = {};
+    CUtensorMap mapK, mapQ, mapW, mapB;
+    if (tables) {
+        memset(&mapK, 0, sizeof mapK);
+        mapQ = mapW = mapB = mapK;
+        S.htab = tables->heads; S.maps = (const CUtensorMap *)tables->maps;
+    } else {
+        if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, k_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
+            !make_tensor_map(&mapB, K, s.L, s.Hkv, kPBlock, k_head_rows))
+            return JQ_ERR_CUDA;
+        if (Kwin) { if (!make_tensor_map(&mapW, Kwin, s.w, s.Hkv, kPTile)) return JQ_ERR_CUDA; } else mapW = mapK;
+    }
+    const int max_tph = ((tables ? tables->max_L : s.L) + kPTile - 1) / kPTile;
+    // CTAs per head: as many as leave the heads resident at a time
+    int C = 1;
+    for (int x = 1; x <= kCMaxCluster && x <= max_tph; ++x)
+        if (dev.resident[wide][x] >= s.Hkv) C = x;
+    Q2.stages = wide ? 3 : 2;
+    while (C < kCMaxCluster && C < max_tph && cand_smem(Rbox, Q2.stages, (max_tph + C - 1) / C) > (wide ? kCMaxSmem : kCTwoPerSm)) ++C;
+    Q2.L = s.L; Q2.tph = tph; Q2.nkeep = s.budget < s.L ? s.budget : s.L;
+    Q2.R = R; Q2.Rbox = Rbox; Q2.Rpad = Rpad; Q2.radius = (s.pool - 1) / 2;
+    Q2.groups = groups; Q2.sms = grid; Q2.share = (max_tph + C - 1) / C; Q2.hpu = S.hpu;
+    Q2.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
+    Q2.T = T; Q2.c = S.c; Q2.part = S.part; Q2.bmax = S.bmax; Q2.scores = scores; Q2.status = w.status;
+    Q2.htab = S.htab; Q2.maps = S.maps;
+#ifdef JQ_DEBUG
+    S.dbg_rec = Q2.dbg_rec = debug_record();
+    if (!S.dbg_rec) return JQ_ERR_CUDA;
+    S.n_bmax = Q2.n_bmax = T * 4 * Rpad;
+    S.n_part = Q2.n_part = (long long)(s.Hkv + 256) * groups * R;
+    Q2.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
+#endif
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)stats_threads(groups));
+    cfg.dynamicSmemBytes = stats_smem(Rbox, S.stages);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, wide ? row_stats<kSGroupsWide> : row_stats<kSGroupsNarrow>, mapK, mapQ, mapW, S) != cudaSuccess) {
+        cudaGetLastError();
+        return JQ_ERR_CUDA;
+    }
+    cfg.gridDim = dim3((unsigned)(s.Hkv * C));
+    cfg.blockDim = dim3((unsigned)cand_threads(wide));
+    cfg.dynamicSmemBytes = cand_smem(Rbox, Q2.stages, Q2.share);
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+    if (cudaLaunchKernelEx(&cfg, wide ? score_candidates<true> : score_candidates<false>, mapB, mapQ, Q2) != cudaSuccess) {
+        cudaGetLastError();
+        return JQ_ERR_CUDA;
+    }
+    count_launch(2);
+    return check_launch();
+}
+
+}  // namespace jq

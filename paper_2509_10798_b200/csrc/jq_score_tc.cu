@@ -100,7 +100,7 @@ struct Params {
     int wtile;               // 1 in window-inclusive mode: every head has one more tile, the last, holding the w window keys
     int w;                   // soft-token queries per query head
     // Units in buffers of their own (ragged calls): the head groups, their lengths and score offsets come from
-    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps [units][2] (K, Qwin).
+    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps [units][kMapsPerUnit] (K, Qwin, ...).
     const GroupRec *gtab;
     const CUtensorMap *maps;
     int hpu;                 // KV heads per unit (a group may run over consecutive units of one length)
@@ -303,7 +303,7 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
                                 const int du = head_c2 / P.hpu, unit = sg.unit + du;
                                 head_c2 -= du * P.hpu;
                                 if (unit != prev_unit) {
-                                    head_mapK = P.maps + 2 * unit; head_mapQ = head_mapK + 1;
+                                    head_mapK = P.maps + kMapsPerUnit * (size_t)unit; head_mapQ = head_mapK + 1;
                                     tensormap_acquire(head_mapK); tensormap_acquire(head_mapQ);
                                     prev_unit = unit;
                                 }
