@@ -46,14 +46,19 @@ static jq_status check_ws(const jq_shape *s, void *ws, size_t ws_bytes, Workspac
     return ws_bytes < out->bytes ? JQ_ERR_WORKSPACE : JQ_OK;
 }
 
-// The scores of one layer for a selection that follows, by the faster of the two ways.
-static jq_status score_layer(const void *K, const void *Qwin, const jq_shape &s, const Workspace &w, cudaStream_t st,
-                             const void *Kwin = nullptr, int k_head_rows = 0)
+// One layer that the one-launch pass does not take, in two launches.  src_head_rows, out_head_rows: rows between consecutive heads
+// of K and V / of Kout and Vout when they are not packed; Vwin: the window rows follow the kept ones.
+static jq_status evict_in_two(const void *K, const void *V, const void *Qwin, const jq_shape &s, void *Kout, void *Vout, int32_t *kept_idx,
+                              const Workspace &w, cudaStream_t st, int src_head_rows = 0, int out_head_rows = 0,
+                              const void *Kwin = nullptr, const void *Vwin = nullptr)
 {
     const long long tiles = (long long)s.Hkv * ((s.L + 127) / 128), keys = (long long)s.Hkv * s.L;
     const long long kept = (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L);
-    if (prune_taken(s, s.Hkv, tiles, keys, kept, s.L, device_sms())) return launch_score_pruned(K, Qwin, s, w.scores, w, st, Kwin, nullptr, k_head_rows);
-    return launch_score_tc(K, Qwin, s, w.scores, w, st, Kwin, nullptr, k_head_rows);
+    if (prune_taken(s, s.Hkv, tiles, keys, kept, s.L))
+        return launch_evict_pruned(K, V, Qwin, s, Kout, Vout, kept_idx, w, st, nullptr, src_head_rows, out_head_rows, Kwin, Vwin);
+    const jq_status rc = launch_score_tc(K, Qwin, s, w.scores, w, st, Kwin, nullptr, src_head_rows);
+    if (rc != JQ_OK) return rc;
+    return launch_select(w.scores, s, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
 }
 
 }  // namespace jq
@@ -123,8 +128,7 @@ jq_status jq_evict_layer_windowed(const void *K, const void *V, const void *Qwin
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin;
     bool taken;
     if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    if ((rc = score_layer(K, Qwin, *s, w, st, Kwin)) != JQ_OK) return rc;
-    return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);
+    return evict_in_two(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st, 0, 0, Kwin);
 }
 
 jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Qwin, const void *Kwin, const void *Vwin,
@@ -150,8 +154,7 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     bool taken;
     if ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
-    if ((rc = score_layer(K, Qwin, sp, w, st, Kwin)) != JQ_OK) return rc;
-    return launch_select(w.scores, sp, kept_idx, nullptr, w, st, K, V, Kout, Vout, nullptr, 0, (int)nt, Kwin, Vwin);
+    return evict_in_two(K, V, Qwin, sp, Kout, Vout, kept_idx, w, st, 0, (int)nt, Kwin, Vwin);
 }
 
 jq_status jq_score_fma(const void *K, const void *Qwin, const jq_shape *s, float *scores, void *ws,
@@ -202,8 +205,7 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
     src.KA = K; src.VA = V; src.LA = s->L;
     bool taken;
     if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    if ((rc = score_layer(K, Qwin, *s, w, st)) != JQ_OK) return rc;
-    return launch_select(w.scores, *s, kept_idx, nullptr, w, st, K, V, Kout, Vout);   // selects, then copies the kept rows
+    return evict_in_two(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st);
 }
 
 // ---- units of one head geometry in buffers of their own: lengths, budgets and offsets per unit
@@ -298,7 +300,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     GroupRec *h_grp = (GroupRec *)(hb + grp_off);   // last: there are far fewer than there is room for
     UnitTables t;
     for (int u = 0; u < nunits; ++u) t.total_tiles += (long long)hpu * (((L ? L[u] : common->L) + 127) / 128);
-    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L, sms);
+    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L);
     long long soff = 0, ooff = 0, tbase = 0;
     int ngroups = 0;
     for (int u = 0; u < nunits; ++u) {
@@ -350,8 +352,8 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     t.heads = (const HeadRec *)(tab + maps_bytes + 2 * ptr_bytes);
     t.groups = (const GroupRec *)(tab + grp_off);
     t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows;
-    rc = pruned ? launch_score_pruned(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t) : launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t);
-    if (rc != JQ_OK) return rc;
+    if (pruned) return launch_evict_pruned(nullptr, nullptr, nullptr, pl.S, Kout, Vout, kept_idx, w, st, &t);
+    if ((rc = launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t)) != JQ_OK) return rc;
     return launch_select(w.scores, pl.S, kept_idx, nullptr, w, st, nullptr, nullptr, Kout, Vout, &t);
 }
 
@@ -405,8 +407,7 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     }
     // 2. the pass over the L = n_old + n_new rows of every head, compacted into the workspace (a row may move
     //    onto a row that another thread still has to read, so the compaction cannot run in place)
-    if ((rc = score_layer(Kc, Qrecent, *s, w, st, nullptr, cap)) != JQ_OK) return rc;
-    if ((rc = launch_select(w.scores, *s, kept_idx, nullptr, w, st, Kc, Vc, Ktmp, Vtmp, nullptr, cap)) != JQ_OK) return rc;
+    if ((rc = evict_in_two(Kc, Vc, Qrecent, *s, Ktmp, Vtmp, kept_idx, w, st, cap)) != JQ_OK) return rc;
     // 3. back to the head of the cache
     if (cudaMemcpy2DAsync(Kc, (size_t)cap * row, Ktmp, nkeep * row, nkeep * row, (size_t)s->Hkv, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return JQ_ERR_CUDA;

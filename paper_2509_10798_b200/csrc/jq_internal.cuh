@@ -119,12 +119,6 @@ jq_status launch_score_fma(const void *K, const void *Q, const jq_shape &s, floa
 jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float *scores,
                           const Workspace &w, cudaStream_t st, const void *Kwin = nullptr,
                           const UnitTables *tables = nullptr, int k_head_rows = 0);
-// The scores that a selection of s.budget pairs per head needs (jq_prune.cu): those of launch_score_tc for every key that can be
-// kept or make a neighbour kept, zero elsewhere.  prune_taken: whether a call over `heads` heads (tiles, keys and kept pairs of all
-// of them, the longest max_L) is one that this is the faster way for.
-bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L, int sms);
-jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, float *scores, const Workspace &w, cudaStream_t st,
-                              const void *Kwin = nullptr, const UnitTables *tables = nullptr, int k_head_rows = 0);
 // With K, V, Kout, Vout given, the kernel also copies the kept rows (the fused layer path).  With tables, every
 // head has a length, a budget and offsets of its own (s.L, s.budget unused).
 // src_head_rows: rows between consecutive heads of K and V in memory when the heads are not packed (0: s.L);
@@ -134,6 +128,13 @@ jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, fl
                         const Workspace &w, cudaStream_t st, const void *K = nullptr, const void *V = nullptr,
                         void *Kout = nullptr, void *Vout = nullptr, const UnitTables *tables = nullptr,
                         int src_head_rows = 0, int out_head_rows = 0, const void *Kwin = nullptr, const void *Vwin = nullptr);
+// Scoring, selection and rows in one pass over K and a look at the keys that can be kept (jq_prune.cu), arguments as launch_score_tc
+// and launch_select take them.  prune_taken: whether a call over `heads` heads (tiles, keys and kept pairs of all of them, the
+// longest max_L) is one that this is the faster way for.
+bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L);
+jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const jq_shape &s, void *Kout, void *Vout, int32_t *idx,
+                              const Workspace &w, cudaStream_t st, const UnitTables *tables = nullptr, int src_head_rows = 0,
+                              int out_head_rows = 0, const void *Kwin = nullptr, const void *Vwin = nullptr);
 // The keys and values of a one-launch layer call: rows [0, LA) of every head in KA, VA (a_rows rows apart; 0: packed), rows
 // [LA, LA + LB) in KB, VB (packed), and the window's (Kwin: one more tile of the denominator; Vwin too: its rows are kept).
 struct FusedSource {

@@ -22,7 +22,7 @@
 // between the two orders of the product.
 #include "jq_sm100.cuh"
 #include "jq_tmem_ld.cuh"
-#include "jq_debug.cuh"
+#include "jq_rows.cuh"
 #include <cstddef>
 #include <cstring>
 #include <cuda_fp16.h>
@@ -345,11 +345,12 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
     }
 }
 
-// ------------------------------------------------------------------ scores of the candidates
+// ------------------------------------------------------------------ candidates: scores, selection, rows
 
 constexpr int kCMaxCluster = 16;
 constexpr int kCBins = 1024;                     // bins of 1/16 octave: 64 octaves from 2^-54 up to 2^10
 constexpr int kCBase = (127 - 54) << 4;
+constexpr int kCDigits = 2048;                   // the selection's bins: 11, 11 and 10 bits of a key
 constexpr int kCMaxStages = 4;
 constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16 bits
 __host__ __device__ constexpr int cand_groups(bool wide) { return wide ? 4 : 2; }
@@ -357,12 +358,19 @@ __host__ __device__ constexpr int cand_threads(bool wide) { return cand_groups(w
 
 struct CCtl {
     uint64_t full[kCMaxStages], empty[kCMaxStages], q_full, t_full[2], t_empty[2];
+    uint64_t b_full[kCMaxStages], b_empty[kCMaxStages];
     uint32_t tmem_base;
     int abort_flag;
-    int bin, total;                              // find_bin's answer; candidates of the whole head in this round
+    int bin, rank;                               // find_bin's answer
     int n;                                       // blocks on this CTA's list
+    int huge;                                    // a normaliser is out of a half's range
     int scan[16];
+    int warp_gt[16], warp_eq[16];
     int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
+    int gt_of[kCMaxCluster], eq_of[kCMaxCluster];            // keys above / equal to the threshold in every CTA's share
+    uint16_t edge[kCMaxCluster][4];              // bounds of the first two and the last two blocks of every CTA's share,
+    int edge_n[kCMaxCluster];                    // and how many blocks it has
+    uint16_t halo[4];                            // bounds of the two blocks before this CTA's share and of the two behind it
     alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads; before, pairs of statistics
     alignas(16) float Ms[kMaxR];                 // minus the row normalisers
 };
@@ -375,18 +383,26 @@ struct CParams {
     int stages, groups;        // K ring; row_stats' epilogue groups
     int sms;                   // row_stats' grid
     int share;                 // most tiles of a head that a CTA looks after
-    int hpu, first_pct;        // heads per unit; blocks of round 1 per 100 pairs kept
+    int first_pct;             // blocks of round 1 per 100 pairs kept
     long long T;
     float c;
     const float2 *part;
     const uint32_t *bmax;
     float *scores;
+    uint32_t *gkeys;           // [keys of all heads]: the selection's keys where shared memory has no room for them
     int *status;
     const HeadRec *htab;
     const CUtensorMap *maps;
+    int32_t *idx;
+    const uint4 *K, *V;        // rows of 16 x 16 bytes
+    const uint4 *const *Ktab, *const *Vtab;
+    uint4 *Kout, *Vout;
+    int src_rows, out_rows;
+    WindowRows win;
+    SelExtents ext;
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
-    long long n_part, n_bmax, n_scores;
+    long long n_part, n_bmax;
 #endif
 };
 
@@ -396,11 +412,18 @@ __device__ __forceinline__ uint32_t remote(const void *p, uint32_t rank)   // th
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
-__device__ __forceinline__ uint4 remote_ld4(uint32_t a)
+__device__ __forceinline__ uint2 remote_ld2(uint32_t a)
 {
-    uint4 v;
-    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    uint2 v;
+    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
     return v;
+}
+__device__ __forceinline__ void remote_st(uint32_t a, int v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void remote_st16(uint32_t a, uint16_t v) { asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)   // all of it 16-byte aligned
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 // The bin of a value >= 0 (given as the upper 16 bits of a float, rounded either way): its lower edge is not above the value.
 __device__ __forceinline__ int bin_of(uint32_t top16) { return min(max((int)(top16 >> 3) - kCBase, 0), kCBins - 1); }
@@ -409,7 +432,7 @@ __device__ __forceinline__ uint32_t edge_of(int bin) { return bin > 0 ? (uint32_
 
 template <bool kWide>
 __global__ void __launch_bounds__(cand_threads(kWide), kWide ? 1 : 2)
-score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CParams P)
+evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CParams P)
 {
     constexpr int kGroups = cand_groups(kWide), kEpi = 4 * kGroups, kTE = 32 * kEpi;
     constexpr uint32_t kSlotCols = kWide ? 256 : 128, kCols = 2 * kSlotCols;   // two accumulators in tensor memory
@@ -420,6 +443,12 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     uint32_t *const hist = (uint32_t *)((uint8_t *)ctl + kCCtlBytes);            // [kCBins]
     uint16_t *const ub = (uint16_t *)(hist + kCBins);                            // [8 share]: bounds of this CTA's share, upper 16 bits
     uint16_t *const list = ub + 8 * P.share;                                     // [8 share]: blocks that this CTA scores
+    // when all is scored, in the place of queries and stages:
+    uint32_t *const digits = (uint32_t *)smem_raw;                               // [kCDigits]
+    float *const scratch = (float *)(digits + kCDigits);                         // [kEpi][2][80]
+    uint16_t *const act = (uint16_t *)(scratch + kEpi * 160);                    // [8 share]: blocks with positions that may be kept
+    uint32_t *const keys_s = (uint32_t *)(act + 8 * P.share);                    // their keys, 16 each
+    const int keys_room = (int)(((uint8_t *)ctl - (uint8_t *)keys_s) / 64);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t rank, C;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -435,10 +464,14 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kCMaxStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        for (int s = 0; s < kCMaxStages; ++s) {
+            mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1);
+            mbar_init(&ctl->b_full[s], 1); mbar_init(&ctl->b_empty[s], kEpi);
+        }
         mbar_init(&ctl->q_full, 1);
         for (int s = 0; s < 2; ++s) { mbar_init(&ctl->t_full[s], 1); mbar_init(&ctl->t_empty[s], kWide ? 8 : 4); }
         ctl->abort_flag = 0;
+        ctl->huge = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kEpi + 1) {
@@ -452,27 +485,31 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     const uint32_t tmem = *(volatile uint32_t *)&ctl->tmem_base;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // waited for before another CTA's memory is touched
     cudaGridDependencySynchronize();             // nothing in global memory has been touched so far
-    cudaTriggerProgrammaticLaunchCompletion();
+    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
 
-    int L = P.L, nkeep = P.nkeep, kv_in = head, tph1 = P.tph;
+    int L = P.L, nkeep = P.nkeep, kv_in = head, tph1 = P.tph, src_rows = P.src_rows;
     long long soff = (long long)head * L, tbase = (long long)head * P.tph;
+    long long orow = (long long)head * nkeep, krow = (long long)head * P.out_rows;      // first rows of the head's indices and of its compacted rows
+    const uint4 *Kin = P.K, *Vin = P.V;
     const CUtensorMap *mb = &mapB, *mq = &mapQ;
     if (P.htab) {
         const HeadRec r = P.htab[head];
-        L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; tbase = r.tbase;
+        L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; tbase = r.tbase; orow = krow = r.ooff; src_rows = L;
         tph1 = (L + kPTile - 1) / kPTile;
         mq = P.maps + kMapsPerUnit * (size_t)r.unit + 1; mb = mq + 1;
+        Kin = P.Ktab[r.unit]; Vin = P.Vtab[r.unit];
     }
     const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
     const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
     const int b0 = 8 * ts, nbs = min(8 * te, nb) - b0;                                          // and their blocks
     auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kTE) : "memory"); };
-    // everybody: all CTAs of the head have got here, and what they wrote is seen
-    auto sync_all = [&]() {
-        if (C == 1) { __syncthreads(); return; }
+    auto cluster_sync = [&]() {
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
+    // all warps of the head's CTAs; the epilogue warps of them (once the other two have left)
+    auto sync_all = [&]() { if (C == 1) __syncthreads(); else cluster_sync(); };
+    auto sync_epi = [&]() { if (C == 1) epi_sync(); else cluster_sync(); };
     // epilogue threads: exclusive scan of one int per thread, and the sum
     auto scan = [&](int v, int &total) -> int {
         int inc = v;
@@ -486,38 +523,40 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         epi_sync();
         return before + inc - v;
     };
-    // epilogue threads: the highest bin with at least `target` entries in it and above it, over all CTAs of the head (0: there is none)
-    auto find_bin = [&](int target) -> int {
-        constexpr int per = kCBins / kTE;                     // 4 or 2 bins per thread, from the top
-        const int at = kCBins - per * (tid + 1);
+    // epilogue threads: the bin that holds the target-th entry from the top, over all CTAs of the head -> ctl->bin, and the
+    // entry's rank in it -> ctl->rank (without so many entries: bin 0)
+    auto find_bin = [&](const uint32_t *h, auto bins, int target) {
+        constexpr int per = decltype(bins)::value / kTE;      // consecutive bins of a thread, from the top
+        const int at = decltype(bins)::value - per * (tid + 1);
         int n[per] = {};
-#pragma unroll 4
-        for (uint32_t d = 0; d < C; ++d) {
-            if (per == 4) {
-                const uint4 v = remote_ld4(remote(hist + at, d));
-                n[0] += (int)v.x; n[1] += (int)v.y; n[per - 2] += (int)v.z; n[per - 1] += (int)v.w;
-            } else {
-                const uint4 v = remote_ld4(remote(hist + (at & ~3), d));
-                n[0] += (int)(at & 2 ? v.z : v.x); n[1] += (int)(at & 2 ? v.w : v.y);
+#pragma unroll 2
+        for (uint32_t d = 0; d < C; ++d)
+#pragma unroll
+            for (int i = 0; i < per; i += 2) {
+                const uint2 v = remote_ld2(remote(h + at + i, d));
+                n[i] += (int)v.x; n[i + 1] += (int)v.y;
             }
-        }
         int sum = 0, total;
 #pragma unroll
         for (int i = 0; i < per; ++i) sum += n[i];
-        if (tid == 0) ctl->bin = 0;
+        if (tid == 0) { ctl->bin = 0; ctl->rank = 1; }
         int above = scan(sum, total);
 #pragma unroll
         for (int i = per - 1; i >= 0; --i) {
-            if (above < target && target <= above + n[i]) ctl->bin = at + i;
+            if (above < target && target <= above + n[i]) { ctl->bin = at + i; ctl->rank = target - above; }
             above += n[i];
         }
         epi_sync();
-        return ctl->bin;
     };
+    struct Bins { enum { value = kCBins }; };
+    struct Digits { enum { value = kCDigits }; };
 
-    uint32_t st = 0, ph = 0, u = 0;                           // K ring and its phase; tiles so far (producer, MMA, epilogue alike)
+    uint32_t st = 0, ph = 0, u = 0;                           // K ring and its phase; tiles so far
     uint32_t lo16 = 0u, hi16 = 0u;                            // the blocks of a round: bounds in [lo16, hi16)
     uint32_t cut = 0u;                                        // in the end: blocks with bounds from here on have been scored
+    // the maxima of the CTA's tiles go through the stages of the ring, as many tiles as fit
+    const uint32_t tile_bytes = (uint32_t)Rpad * 16;
+    const int per_stage = (int)(kPStage / tile_bytes), nchunks = (te - ts + per_stage - 1) / per_stage;
 
     if (warp == kEpi) {
         if (lane == 0) {
@@ -525,6 +564,16 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
             mbar_expect_tx(&ctl->q_full, q_bytes);
             tma_load_3d(qbuf, mq, &ctl->q_full, 0, 0, kv_in);
             tma_load_3d(qbuf + q_bytes / 2, mq, &ctl->q_full, 64, 0, kv_in);
+            int s = 0, round = 0;
+#pragma unroll 1
+            for (int j = 0; j < nchunks; ++j) {
+                if (round > 0 && !mbar_wait(&ctl->b_empty[s], (round - 1) & 1, &ctl->abort_flag, status, 64)) break;
+                const int t = ts + j * per_stage, cnt = min(per_stage, te - t);
+                mbar_expect_tx(&ctl->b_full[s], (uint32_t)cnt * tile_bytes);
+                if (JQ_IN((tbase + t + cnt) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 6))
+                    bulk_load(kbuf + (size_t)s * kPStage, P.bmax + (tbase + t) * 4 * Rpad, (uint32_t)cnt * tile_bytes, &ctl->b_full[s]);
+                if (++s == P.stages) { s = 0; ++round; }
+            }
         }
         __syncwarp();
         if (P.maps) tensormap_acquire(mb);                    // (all lanes load)
@@ -568,61 +617,71 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
                     const float mn = fmaxf(m, o.x);
                     l = (l > 0.f ? l * ex2(P.c * (m - mn)) : 0.f) + (o.y > 0.f ? o.y * ex2(P.c * (o.x - mn)) : 0.f);
                     M = fmaf(P.c, mn, log2f(l));
+                    if (!(fabsf(M) < 60000.f)) ctl->huge = 1;
                 }
                 ctl->Ms[row] = -M;
                 if (!kWide) ctl->Ms[128 + row] = -INFINITY;
             }
             epi_sync();
         }
-        // ---- the bounds.  A lane takes four neighbouring rows (eight with more than 128), of two blocks at a time.
+        // ---- the bounds.  A lane takes four neighbouring rows (eight with more than 128) of four blocks.  A maximum x within 64 of
+        // its row's normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60
+        // each, which is added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
         {
             constexpr int kV = kWide ? 2 : 1;
-            float nm[4 * kV];
+            float2 nm[4 * kV];
 #pragma unroll
-            for (int i = 0; i < 4 * kV; ++i) nm[i] = ctl->Ms[(i >> 2) * 128 + 4 * lane + (i & 3)];
+            for (int i = 0; i < 4 * kV; ++i) {
+                const float x = ctl->Ms[(i >> 2) * 128 + 4 * lane + (i & 3)], y = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;
+                nm[i] = make_float2(y, y);
+            }
+            const float floor_ = ctl->huge ? INFINITY : 3e-16f;
+            int s = 0, round = 0;
 #pragma unroll 1
-            for (int t = ts + warp; t < te; t += kEpi) {
-                uint4 v[4][kV];
+            for (int j = 0; j < nchunks; ++j) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&ctl->b_full[s], round & 1, &ctl->abort_flag, status, 32))) break;
+                const int t = j * per_stage, cnt = min(per_stage, te - ts - t);
+#pragma unroll 1
+                for (int x = warp; x < 2 * cnt; x += kEpi) {
+                    const uint4 *const src = (const uint4 *)(kbuf + (size_t)s * kPStage + (size_t)x * (tile_bytes / 2));
+                    uint4 v[2][kV];
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
+                    for (int q = 0; q < 2; ++q)
 #pragma unroll
-                    for (int x = 0; x < kV; ++x) {
-                        const long long at = ((tbase + t) * 4 + q) * Rpad + x * 128 + 4 * lane;
-                        const bool in = x * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6);
-                        v[q][x] = in ? __ldcg((const uint4 *)(P.bmax + at)) : make_uint4(0u, 0u, 0u, 0u);   // (rows that are none have a normaliser of inf)
-                    }
-                float s[8];
+                        for (int y = 0; y < kV; ++y)          // (a row that is none has a normaliser of inf)
+                            v[q][y] = y * 128 + 4 * lane < Rpad ? src[(q * Rpad + y * 128) / 4 + lane] : make_uint4(0u, 0u, 0u, 0u);
+                    float2 sum[2];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    s[2 * q] = s[2 * q + 1] = 0.f;
+                    for (int q = 0; q < 2; ++q) {
+                        sum[q] = make_float2(0.f, 0.f);
 #pragma unroll
-                    for (int x = 0; x < kV; ++x) {
-                        const uint32_t e[4] = {v[q][x].x, v[q][x].y, v[q][x].z, v[q][x].w};
+                        for (int y = 0; y < kV; ++y) {
+                            const uint32_t e[4] = {v[q][y].x, v[q][y].y, v[q][y].z, v[q][y].w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float2 f = __half22float2(*(const __half2 *)&e[i]);
-                            f.x = fmaxf(f.x, -65504.f); f.y = fmaxf(f.y, -65504.f);
-                            s[2 * q] += ex2(fmaf(fabsf(f.x), 1.f / 1024.f, f.x) + nm[4 * x + i]);
-                            s[2 * q + 1] += ex2(fmaf(fabsf(f.y), 1.f / 1024.f, f.y) + nm[4 * x + i]);
+                            for (int i = 0; i < 4; ++i) {
+                                const float2 f = __fadd2_rn(__half22float2(*(const __half2 *)&e[i]), nm[4 * y + i]);
+                                sum[q] = __fadd2_rn(sum[q], make_float2(ex2(f.x), ex2(f.y)));
+                            }
                         }
                     }
+                    // four sums over the 32 lanes: after two exchanges of halves a lane holds one block's part
+                    const bool h4 = lane & 16, h3 = lane & 8;
+                    const float p0 = (h4 ? sum[1].x : sum[0].x) + __shfl_xor_sync(0xffffffffu, h4 ? sum[0].x : sum[1].x, 16);
+                    const float p1 = (h4 ? sum[1].y : sum[0].y) + __shfl_xor_sync(0xffffffffu, h4 ? sum[0].y : sum[1].y, 16);
+                    float r = (h3 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h3 ? p0 : p1, 8);
+                    r += __shfl_xor_sync(0xffffffffu, r, 4);
+                    r += __shfl_xor_sync(0xffffffffu, r, 2);
+                    r += __shfl_xor_sync(0xffffffffu, r, 1);
+                    const int blk = 8 * t + 4 * x + (h4 ? 2 : 0) + (h3 ? 1 : 0);
+                    if ((lane & 7) == 0 && blk < nbs && JQ_IN(blk, 8 * P.share, kDbgPrune, 7)) {
+                        const uint32_t y = (__float_as_uint((r + floor_) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16;
+                        ub[blk] = (uint16_t)y;
+                        atomicAdd(&hist[bin_of(y)], 1u);
+                    }
                 }
-                // eight sums over the 32 lanes: after three exchanges of halves a lane holds one block's part
-                const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-                float a[4], b[2], r;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = (h4 ? s[4 + i] : s[i]) + __shfl_xor_sync(0xffffffffu, h4 ? s[i] : s[4 + i], 16);
-#pragma unroll
-                for (int i = 0; i < 2; ++i) b[i] = (h3 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[2 + i], 8);
-                r = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
-                r += __shfl_xor_sync(0xffffffffu, r, 2);
-                r += __shfl_xor_sync(0xffffffffu, r, 1);
-                const int blk = 8 * (t - ts) + (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
-                if ((lane & 3) == 0 && blk < nbs && JQ_IN(blk, 8 * P.share, kDbgPrune, 7)) {
-                    const uint32_t x = (__float_as_uint(r * (1.f + 1.f / 64.f)) + 0xffffu) >> 16;
-                    ub[blk] = (uint16_t)x;
-                    atomicAdd(&hist[bin_of(x)], 1u);
-                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->b_empty[s], 1);
+                if (++s == P.stages) { s = 0; ++round; }
             }
         }
     }
@@ -634,48 +693,41 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     for (int round = 0; round < 2; ++round) {
         // ---- the blocks of this round: [lo16, hi16) of the bounds
         if (warp < kEpi) {
-            const int bin = find_bin(round == 0 ? wanted : nkeep);
-            if (round == 0) { lo16 = edge_of(bin); hi16 = 0x10000u; cut = lo16; }
-            else { hi16 = lo16; lo16 = min(edge_of(bin), lo16); cut = lo16; }
+            find_bin(hist, Bins(), round == 0 ? wanted : nkeep);
+            const uint32_t edge = edge_of(ctl->bin);
+            if (round == 0) { lo16 = edge; hi16 = 0x10000u; }
+            else { hi16 = lo16; lo16 = min(edge, lo16); }
+            cut = lo16;
             // this CTA's share of them, and their places in the head's list
             const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
             int mine = 0, total;
             for (int i = i0; i < i1; ++i) mine += ub[i] >= lo16 && ub[i] < hi16;
             int at = scan(mine, total);
-            if (C > 1 && warp == 0 && lane < (int)C)
-                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(&ctl->cnt[rank], lane)), "r"(total) : "memory");
-            if (C == 1) {
-                for (int i = i0; i < i1; ++i)
-                    if (ub[i] >= lo16 && ub[i] < hi16) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 8)) list[at] = (uint16_t)i; ++at; }
-                if (tid == 0) ctl->n = total;
-                for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;   // (read by this CTA alone, before the scan)
-            }
-        }
-        sync_all();
-        if (C > 1) {
-            if (warp < kEpi) {
+            if (C > 1) {
+                if (warp == 0 && lane < (int)C) remote_st(remote(&ctl->cnt[rank], lane), total);
+                cluster_sync();
                 const int have = lane < (int)C ? ctl->cnt[lane] : 0;
-                const int all = __reduce_add_sync(0xffffffffu, have), before = __reduce_add_sync(0xffffffffu, lane < (int)rank ? have : 0);
-                const int per_cta = ((all + (int)C - 1) / (int)C + 7) & ~7;      // whole tiles
-                const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
-                int mine = 0, total;
-                for (int i = i0; i < i1; ++i) mine += ub[i] >= lo16 && ub[i] < hi16;
-                int at = before + scan(mine, total);
+                const int all = __reduce_add_sync(0xffffffffu, have);
+                at += __reduce_add_sync(0xffffffffu, lane < (int)rank ? have : 0);
+                const int per_cta = max(8, ((all + (int)C - 1) / (int)C + 7) & ~7);      // whole tiles
                 for (int i = i0; i < i1; ++i)
                     if (ub[i] >= lo16 && ub[i] < hi16) {
                         const int to = at / per_cta, x = at - to * per_cta;
-                        if (JQ_IN(x, 8 * P.share, kDbgPrune, 9) && JQ_IN(to, C, kDbgPrune, 10))
-                            asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(remote(list + x, (uint32_t)to)), "h"((uint16_t)(b0 + i)) : "memory");
+                        if (JQ_IN(x, 8 * P.share, kDbgPrune, 9) && JQ_IN(to, C, kDbgPrune, 10)) remote_st16(remote(list + x, (uint32_t)to), (uint16_t)(b0 + i));
                         ++at;
                     }
-                if (tid == 0) ctl->n = per_cta > 0 ? min(max(all - (int)rank * per_cta, 0), per_cta) : 0;
-                for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;            // (everybody has read it)
+                if (tid == 0) ctl->n = min(max(all - (int)rank * per_cta, 0), per_cta);
+            } else {
+                for (int i = i0; i < i1; ++i)
+                    if (ub[i] >= lo16 && ub[i] < hi16) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 8)) list[at] = (uint16_t)i; ++at; }
+                if (tid == 0) ctl->n = total;
             }
-            sync_all();
-        }
+            for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;   // (everybody has read it)
+        } else if (C > 1) cluster_sync();
+        sync_all();
         const int n = ctl->n, nt = (n + 7) >> 3;
         if (warp == kEpi) {
-            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, a lane each
+            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, two lanes each
 #pragma unroll 1
             for (int i = 0; i < nt; ++i) {
                 const int have = min(8, n - 8 * i);
@@ -750,7 +802,7 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
                 }
                 const int x = 8 * i + (row0 >> 4), blk = x < n ? list[x] : nb, key = blk * kPBlock + (row0 & 15);
                 const bool have = x < n && key < L;
-                if (have && JQ_IN(soff + key, P.n_scores, kDbgPrune, 13)) P.scores[soff + key] = sum;
+                if (have && JQ_IN(soff + key, P.ext.scores, kDbgPrune, 13)) P.scores[soff + key] = sum;
                 if (round == 0) {
                     // what this block alone guarantees of the pooled scores of its positions
                     float m = have ? sum : 0.f;
@@ -768,22 +820,168 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         if (warp < kEpi) u += (uint32_t)nt;
         sync_all();
     }
-    // the blocks of this CTA's share that nothing needs
-    if (warp < kEpi && cut > 0u) {
-        float *const s = P.scores + soff + (long long)b0 * kPBlock;
-        const int m = min(nbs * kPBlock, L - b0 * kPBlock);
-        for (int i = tid; i < m; i += kTE)
-            if (ub[i >> 4] < cut && JQ_IN(soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
+    if (warp >= kEpi) {
+        // all products have been read: the two warps are through
+        if (warp == kEpi + 1) {
+            if (*(volatile int *)&ctl->abort_flag) __nanosleep(200000);   // let copies still in flight land before the CTA goes
+            __syncwarp();
+            tc_fence_after();
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+        }
+        return;
     }
-    // ---------------------------------------------------------------- exit
-    tc_fence_before();
-    __syncthreads();
-    if (*(volatile int *)&ctl->abort_flag) __nanosleep(200000);   // let copies still in flight land before the CTA goes
-    if (warp == kEpi + 1) {
-        __syncwarp();
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+
+    // ---------------------------------------------------------------- selection (the epilogue warps).  What is not scored counts as zero: its
+    // scores lie below the threshold, and so does every pooled score that they alone would make.  (Whatever the scores are,
+    // after a wait that ran out too, every place that follows is brought into range.)
+    const int half = lane >> 4, i16 = lane & 15, reach = (P.radius + kPBlock - 1) / kPBlock;   // blocks that a window reaches into on either side
+    if (C > 1 && reach > 0) {
+        if (warp == 0 && lane < (int)C) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int i = x < 2 ? x : nbs - 4 + x;
+                remote_st16(remote(&ctl->edge[rank][x], lane), i >= 0 && i < nbs ? ub[i] : (uint16_t)0);
+            }
+            remote_st(remote(&ctl->edge_n[rank], lane), nbs);
+        }
+        cluster_sync();
+        if (tid < 4) {                                        // (a share may be shorter than two blocks, or empty)
+            int d = tid < 2 ? 2 - tid : tid - 1, q = (int)rank;   // the d-th block before / behind this CTA's share
+            uint16_t v = 0;
+            for (;;) {
+                q += tid < 2 ? -1 : 1;
+                if (q < 0 || q >= (int)C) break;
+                const int n = ctl->edge_n[q];
+                if (d <= n) { v = ctl->edge[q][tid < 2 ? 4 - d : d - 1]; break; }
+                d -= n;
+            }
+            ctl->halo[tid] = v;
+        }
+    } else if (tid < 4) ctl->halo[tid] = 0;
+    for (int i = tid; i < kCDigits; i += kTE) digits[i] = 0u;
+    epi_sync();
+    const bool out_of_share = C > 1 && cut > 0u;
+    auto scored = [&](int i) -> bool {                        // block b0 + i, for i up to two blocks outside of the share
+        if (i >= 0 && i < nbs) return ub[i] >= cut;
+        const int x = i < 0 ? i + 2 : i - nbs + 2;
+        return out_of_share ? ctl->halo[x] >= cut : (C > 1 && b0 + i >= 0 && b0 + i < nb);
+    };
+    int n_act;
+    {
+        const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
+        auto active = [&](int i) -> bool {
+            bool on = false;
+            for (int d = -reach; d <= reach; ++d) on |= scored(i + d);
+            return on;
+        };
+        int mine = 0;
+        for (int i = i0; i < i1; ++i) mine += active(i);
+        int at = scan(mine, n_act);
+        for (int i = i0; i < i1; ++i) if (active(i)) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 14)) act[at] = (uint16_t)i; ++at; }
+        epi_sync();
     }
+    // Warp w owns the active blocks [a0, a1), half a warp to a block; a thread reads the keys that it wrote itself.
+    const int seg = ((n_act + kEpi - 1) / kEpi + 1) & ~1, a0 = min(warp * seg, n_act), a1 = min(a0 + seg, n_act);
+    uint32_t *const keys = n_act <= keys_room ? keys_s : P.gkeys + soff + (long long)b0 * kPBlock;
+    auto block_of = [&](int a) -> int { return min((int)act[a], nbs - 1); };
+    {
+        float *const mine = scratch + (warp * 2 + half) * 80;
+#pragma unroll 1
+        for (int a = a0; a < a1; a += 8) {
+            float v[4][5];
+            int blk[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int x = a + 2 * e + half;
+                blk[e] = x < a1 ? block_of(x) : -4;
+#pragma unroll
+                for (int d = -2; d <= 2; ++d) {
+                    const int pos = (b0 + blk[e] + d) * kPBlock + i16;
+                    const bool in = blk[e] >= 0 && abs(d) <= reach && pos >= 0 && pos < L && scored(blk[e] + d);
+                    v[e][d + 2] = in && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 15) ? __ldcg(P.scores + soff + pos) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                __syncwarp();
+#pragma unroll
+                for (int d = 0; d < 5; ++d) if (abs(d - 2) <= reach) mine[16 * d + i16] = v[e][d];
+                __syncwarp();
+                float m = mine[32 + i16];
+#pragma unroll 1
+                for (int r = 1; r <= P.radius; ++r) m = max3(m, mine[32 + i16 - r], mine[32 + i16 + r]);
+                const int x = a + 2 * e + half;
+                if (x < a1 && (b0 + blk[e]) * kPBlock + i16 < L) {
+                    // (one above the bits of a value that is not negative: order and ties as the values have them)
+                    if (JQ_IN(x * 16 + i16, n_act <= keys_room ? keys_room * 16 : (long long)nbs * 16, kDbgPrune, 16)) keys[x * 16 + i16] = __float_as_uint(m) + 1u;
+                }
+            }
+        }
+    }
+    auto key_at = [&](int x) -> uint32_t {                    // of active block x (0: there is no such position)
+        return x < a1 && (b0 + block_of(x)) * kPBlock + i16 < L ? keys[x * 16 + i16] : 0u;
+    };
+    // The threshold: 11, 11 and 10 bits of it at a time, over the keys that agree with it so far.
+    uint32_t tau = 0u;
+    int krem = nkeep;
+#pragma unroll 1
+    for (int level = 0; level < 3; ++level) {
+        const int shift = level == 0 ? 21 : level == 1 ? 10 : 0, done = level == 0 ? 32 : level == 1 ? 21 : 10;
+#pragma unroll 1
+        for (int a = a0; a < a1; a += 2) {
+            const uint32_t k = key_at(a + half);
+            const bool in = k != 0u && (level == 0 || (k ^ tau) >> done == 0u);
+            const uint32_t d = in ? (k >> shift) & (kCDigits - 1) : 0xffffffffu;
+            const uint32_t same = __match_any_sync(0xffffffffu, d);   // (the max-pool's plateaus as one count)
+            if (in && lane == __ffs(same) - 1) atomicAdd(&digits[d], (uint32_t)__popc(same));
+        }
+        sync_epi();
+        find_bin(digits, Digits(), krem);
+        tau |= (uint32_t)ctl->bin << shift;
+        krem = ctl->rank;
+        if (level < 2) {
+            sync_epi();                                       // (everybody has read the counts)
+            for (int i = tid; i < kCDigits; i += kTE) digits[i] = 0u;
+            epi_sync();
+        }
+    }
+    // Kept: all keys above tau and, of those equal to it, the first krem.
+    int gt = 0, eq = 0;
+#pragma unroll 1
+    for (int a = a0; a < a1; a += 2) {
+        const uint32_t k = key_at(a + half);
+        gt += __popc(__ballot_sync(0xffffffffu, k > tau));
+        eq += __popc(__ballot_sync(0xffffffffu, k == tau && k != 0u));
+    }
+    if (lane == 0) { ctl->warp_gt[warp] = gt; ctl->warp_eq[warp] = eq; }
+    epi_sync();
+    {
+        const int g = lane < kEpi ? ctl->warp_gt[lane] : 0, e = lane < kEpi ? ctl->warp_eq[lane] : 0;
+        if (C > 1) {
+            const int tg = __reduce_add_sync(0xffffffffu, g), tq = __reduce_add_sync(0xffffffffu, e);
+            if (warp == 0 && lane < (int)C) { remote_st(remote(&ctl->gt_of[rank], lane), tg); remote_st(remote(&ctl->eq_of[rank], lane), tq); }
+            cluster_sync();
+        }
+        gt = __reduce_add_sync(0xffffffffu, (lane < warp ? g : 0) + (C > 1 && lane < (int)rank ? ctl->gt_of[lane] : 0));
+        eq = __reduce_add_sync(0xffffffffu, (lane < warp ? e : 0) + (C > 1 && lane < (int)rank ? ctl->eq_of[lane] : 0));
+    }
+    int32_t *const out = P.idx + orow;
+#pragma unroll 1
+    for (int a = a0; a < a1; a += 2) {
+        const uint32_t k = key_at(a + half), below = (1u << lane) - 1u;
+        const uint32_t bg = __ballot_sync(0xffffffffu, k > tau), be = __ballot_sync(0xffffffffu, k == tau && k != 0u);
+        if (!(bg | be)) continue;
+        const int g = gt + __popc(bg & below), e = eq + __popc(be & below), t = g + min(e, krem);
+        if ((k > tau || (k == tau && k != 0u && e < krem)) && t >= 0 && t < nkeep && JQ_IN(orow + t, P.ext.out_rows, kDbgPrune, 17))
+            out[t] = (b0 + block_of(a + half)) * kPBlock + i16;
+        gt += __popc(bg);
+        eq += __popc(be);
+    }
+    // ---------------------------------------------------------------- the rows, once every index of the head has been written
+    sync_epi();
+    copy_rows(tid, kTE, out, (int)((long long)rank * nkeep / C), (int)((long long)(rank + 1) * nkeep / C), kv_in, krow, L, Kin, Vin, P.Kout, P.Vout,
+              src_rows, P.ext JQ_DBG_ARG_DEV);
+    if (P.win.w) copy_window(P.win, head, krow + nkeep, (int)rank * (kTE / 16) + (tid >> 4), (int)C * (kTE / 16), P.Kout, P.Vout, P.ext JQ_DBG_ARG_DEV);
 }
 
 // ------------------------------------------------------------------ host side
@@ -812,7 +1010,7 @@ bool prune_device(PruneDevice *out)
         for (auto k : {row_stats<kSGroupsNarrow>, row_stats<kSGroupsWide>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess) return false;
         for (int wide = 0; wide < 2; ++wide) {
-            const auto k = wide ? score_candidates<true> : score_candidates<false>;
+            const auto k = wide ? evict_candidates<true> : evict_candidates<false>;
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess ||
                 cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
             for (int C = 1; C <= kCMaxCluster; ++C) {
@@ -843,17 +1041,18 @@ size_t prune_bytes(long long tiles, int heads, int R)
 }
 
 // Whether a call takes this way.  tiles: of all heads; keys: sum of the heads' lengths; kept: sum of what the heads keep.
-bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L, int sms)
+bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L)
 {
-    (void)heads; (void)sms;
+    (void)heads;
     const int R = s.group * s.w;
     if (R <= 64 || tiles >= (1ll << 30) || max_L > kPBlock * kCMaxBlocks) return false;
     const double per = s.pool >= 7 ? 6.0 : s.pool >= 3 ? 2.5 : 1.2;    // kept positions per block that holds one
     return tiles * (R > 128 ? 2 : 1) >= 6000 && kept / per * 16.0 < 0.35 * keys;
 }
 
-jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, float *scores, const Workspace &w, cudaStream_t st,
-                              const void *Kwin, const UnitTables *tables, int k_head_rows)
+jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const jq_shape &s, void *Kout, void *Vout, int32_t *idx,
+                              const Workspace &w, cudaStream_t st, const UnitTables *tables, int src_head_rows, int out_head_rows,
+                              const void *Kwin, const void *Vwin)
 {
     PruneDevice dev;
     if (!prune_device(&dev)) return JQ_ERR_CUDA;
@@ -865,20 +1064,19 @@ jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, f
     S.stages = wide ? 3 : 5;
     S.T = T; S.heads = s.Hkv; S.hpu = tables ? tables->hpu : s.Hkv;
     S.c = 1.4426950408889634f / sqrtf((float)s.d);
-    const size_t bmax_bytes = align_up((size_t)T * 4 * Rpad * 4, 256);
     S.bmax = (uint32_t *)w.prune;
-    S.part = (float2 *)((char *)w.prune + bmax_bytes);
+    S.part = (float2 *)((char *)w.prune + align_up((size_t)T * 4 * Rpad * 4, 256));
     S.status = w.status;
     const int groups = wide ? kSGroupsWide : kSGroupsNarrow, grid = (int)(T < dev.sms ? T : dev.sms);
-    CParams Q2 = {};
+    CParams P = {};
     CUtensorMap mapK, mapQ, mapW, mapB;
     if (tables) {
         memset(&mapK, 0, sizeof mapK);
         mapQ = mapW = mapB = mapK;
         S.htab = tables->heads; S.maps = (const CUtensorMap *)tables->maps;
     } else {
-        if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, k_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
-            !make_tensor_map(&mapB, K, s.L, s.Hkv, kPBlock, k_head_rows))
+        if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, src_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
+            !make_tensor_map(&mapB, K, s.L, s.Hkv, kPBlock, src_head_rows))
             return JQ_ERR_CUDA;
         if (Kwin) { if (!make_tensor_map(&mapW, Kwin, s.w, s.Hkv, kPTile)) return JQ_ERR_CUDA; } else mapW = mapK;
     }
@@ -887,20 +1085,30 @@ jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, f
     int C = 1;
     for (int x = 1; x <= kCMaxCluster && x <= max_tph; ++x)
         if (dev.resident[wide][x] >= s.Hkv) C = x;
-    Q2.stages = wide ? 3 : 2;
-    while (C < kCMaxCluster && C < max_tph && cand_smem(Rbox, Q2.stages, (max_tph + C - 1) / C) > (wide ? kCMaxSmem : kCTwoPerSm)) ++C;
-    Q2.L = s.L; Q2.tph = tph; Q2.nkeep = s.budget < s.L ? s.budget : s.L;
-    Q2.R = R; Q2.Rbox = Rbox; Q2.Rpad = Rpad; Q2.radius = (s.pool - 1) / 2;
-    Q2.groups = groups; Q2.sms = grid; Q2.share = (max_tph + C - 1) / C; Q2.hpu = S.hpu;
-    Q2.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
-    Q2.T = T; Q2.c = S.c; Q2.part = S.part; Q2.bmax = S.bmax; Q2.scores = scores; Q2.status = w.status;
-    Q2.htab = S.htab; Q2.maps = S.maps;
+    P.stages = wide ? 3 : 2;
+    while (C < kCMaxCluster && C < max_tph && cand_smem(Rbox, P.stages, (max_tph + C - 1) / C) > (wide ? kCMaxSmem : kCTwoPerSm)) ++C;
+    P.share = (max_tph + C - 1) / C;
+    const size_t smem = cand_smem(Rbox, P.stages, P.share);
+    if (smem > kCMaxSmem) return JQ_ERR_CUDA;   // (prune_taken's limit on the length keeps every call below)
+    P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
+    P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
+    P.groups = groups; P.sms = grid;
+    P.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
+    P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.gkeys = w.keys; P.status = w.status;
+    P.htab = S.htab; P.maps = S.maps;
+    P.idx = idx; P.K = (const uint4 *)K; P.V = (const uint4 *)V; P.Kout = (uint4 *)Kout; P.Vout = (uint4 *)Vout;
+    if (tables) { P.Ktab = (const uint4 *const *)tables->K; P.Vtab = (const uint4 *const *)tables->V; }
+    P.src_rows = src_head_rows > s.L ? src_head_rows : s.L;
+    P.out_rows = out_head_rows > P.nkeep ? out_head_rows : P.nkeep;
+    P.win.K = (const uint4 *)Kwin; P.win.V = (const uint4 *)Vwin; P.win.w = Vwin ? s.w : 0;
+    P.ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
+    P.ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * P.out_rows;
+    P.ext.src_heads = tables ? tables->hpu : s.Hkv;
 #ifdef JQ_DEBUG
-    S.dbg_rec = Q2.dbg_rec = debug_record();
+    S.dbg_rec = P.dbg_rec = debug_record();
     if (!S.dbg_rec) return JQ_ERR_CUDA;
-    S.n_bmax = Q2.n_bmax = T * 4 * Rpad;
-    S.n_part = Q2.n_part = (long long)(s.Hkv + 256) * groups * R;
-    Q2.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
+    S.n_bmax = P.n_bmax = T * 4 * Rpad;
+    S.n_part = P.n_part = (long long)(s.Hkv + 256) * groups * R;
 #endif
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -918,11 +1126,11 @@ jq_status launch_score_pruned(const void *K, const void *Q, const jq_shape &s, f
     }
     cfg.gridDim = dim3((unsigned)(s.Hkv * C));
     cfg.blockDim = dim3((unsigned)cand_threads(wide));
-    cfg.dynamicSmemBytes = cand_smem(Rbox, Q2.stages, Q2.share);
+    cfg.dynamicSmemBytes = smem;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, wide ? score_candidates<true> : score_candidates<false>, mapB, mapQ, Q2) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, wide ? evict_candidates<true> : evict_candidates<false>, mapB, mapQ, P) != cudaSuccess) {
         cudaGetLastError();
         return JQ_ERR_CUDA;
     }
