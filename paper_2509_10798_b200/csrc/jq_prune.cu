@@ -22,6 +22,7 @@
 // between the two orders of the product.
 #include "jq_sm100.cuh"
 #include "jq_tmem_ld.cuh"
+#include "jq_pool.cuh"
 #include "jq_rows.cuh"
 #include <cstddef>
 #include <cstring>
@@ -350,8 +351,10 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
 constexpr int kCMaxCluster = 16;
 constexpr int kCBins = 1024;                     // bins of 1/16 octave: 64 octaves from 2^-54 up to 2^10
 constexpr int kCBase = (127 - 54) << 4;
-constexpr int kCDigits = 2048;                   // the selection's bins: 11, 11 and 10 bits of a key
+constexpr int kCSelBins = 2048;                  // the selection's bins, equal parts of a range of keys
+constexpr int kCRank = 512;                      // keys of one bin that are ranked by comparison
 constexpr int kCMaxStages = 4;
+constexpr int kCAhead = 128;                     // blocks that are on their way into the L2 ahead of the ring
 constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16 bits
 __host__ __device__ constexpr int cand_groups(bool wide) { return wide ? 4 : 2; }
 __host__ __device__ constexpr int cand_threads(bool wide) { return cand_groups(wide) * 128 + 64; }
@@ -361,16 +364,14 @@ struct CCtl {
     uint64_t b_full[kCMaxStages], b_empty[kCMaxStages];
     uint32_t tmem_base;
     int abort_flag;
-    int bin, rank;                               // find_bin's answer
+    int bin, rank, count;                        // find_bin's answer
     int n;                                       // blocks on this CTA's list
     int huge;                                    // a normaliser is out of a half's range
+    int ncand, need;
+    uint32_t tau;
     int scan[16];
-    int warp_gt[16], warp_eq[16];
+    uint32_t wmin[16], wmax[16];
     int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
-    int gt_of[kCMaxCluster], eq_of[kCMaxCluster];            // keys above / equal to the threshold in every CTA's share
-    uint16_t edge[kCMaxCluster][4];              // bounds of the first two and the last two blocks of every CTA's share,
-    int edge_n[kCMaxCluster];                    // and how many blocks it has
-    uint16_t halo[4];                            // bounds of the two blocks before this CTA's share and of the two behind it
     alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads; before, pairs of statistics
     alignas(16) float Ms[kMaxR];                 // minus the row normalisers
 };
@@ -425,6 +426,10 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void prefetch_3d(const CUtensorMap *map, int c0, int c1, int c2)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
 // The bin of a value >= 0 (given as the upper 16 bits of a float, rounded either way): its lower edge is not above the value.
 __device__ __forceinline__ int bin_of(uint32_t top16) { return min(max((int)(top16 >> 3) - kCBase, 0), kCBins - 1); }
 // The lower edge of a bin, as the upper 16 bits of a float; of the lowest bin 0.
@@ -443,12 +448,8 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     uint32_t *const hist = (uint32_t *)((uint8_t *)ctl + kCCtlBytes);            // [kCBins]
     uint16_t *const ub = (uint16_t *)(hist + kCBins);                            // [8 share]: bounds of this CTA's share, upper 16 bits
     uint16_t *const list = ub + 8 * P.share;                                     // [8 share]: blocks that this CTA scores
-    // when all is scored, in the place of queries and stages:
-    uint32_t *const digits = (uint32_t *)smem_raw;                               // [kCDigits]
-    float *const scratch = (float *)(digits + kCDigits);                         // [kEpi][2][80]
-    uint16_t *const act = (uint16_t *)(scratch + kEpi * 160);                    // [8 share]: blocks with positions that may be kept
-    uint32_t *const keys_s = (uint32_t *)(act + 8 * P.share);                    // their keys, 16 each
-    const int keys_room = (int)(((uint8_t *)ctl - (uint8_t *)keys_s) / 64);
+    uint32_t *const words = (uint32_t *)(list + 8 * P.share);                    // [share / 4 + 1]: blocks as bits,
+    int *const wbase = (int *)(words + P.share / 4 + 1);                         // and how many come before each word
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t rank, C;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -507,9 +508,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
-    // all warps of the head's CTAs; the epilogue warps of them (once the other two have left)
-    auto sync_all = [&]() { if (C == 1) __syncthreads(); else cluster_sync(); };
-    auto sync_epi = [&]() { if (C == 1) epi_sync(); else cluster_sync(); };
+    auto sync_all = [&]() { if (C == 1) __syncthreads(); else cluster_sync(); };   // all warps of the head's CTAs
     // epilogue threads: exclusive scan of one int per thread, and the sum
     auto scan = [&](int v, int &total) -> int {
         int inc = v;
@@ -523,33 +522,47 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         epi_sync();
         return before + inc - v;
     };
-    // epilogue threads: the bin that holds the target-th entry from the top, over all CTAs of the head -> ctl->bin, and the
-    // entry's rank in it -> ctl->rank (without so many entries: bin 0)
-    auto find_bin = [&](const uint32_t *h, auto bins, int target) {
+    // epilogue threads: the bin that holds the target-th entry from the top, over the histograms of `ctas` CTAs of the head
+    // -> ctl->bin, with the entry's rank in it and its population (without so many entries: bin 0)
+    auto find_bin = [&](const uint32_t *h, auto bins, uint32_t ctas, int target) {
         constexpr int per = decltype(bins)::value / kTE;      // consecutive bins of a thread, from the top
         const int at = decltype(bins)::value - per * (tid + 1);
         int n[per] = {};
-#pragma unroll 2
-        for (uint32_t d = 0; d < C; ++d)
+        if (ctas == 1) {
 #pragma unroll
-            for (int i = 0; i < per; i += 2) {
-                const uint2 v = remote_ld2(remote(h + at + i, d));
-                n[i] += (int)v.x; n[i + 1] += (int)v.y;
-            }
+            for (int i = 0; i < per; i += 2) { const uint2 v = *(const uint2 *)(h + at + i); n[i] = (int)v.x; n[i + 1] = (int)v.y; }
+        } else {
+#pragma unroll 4
+            for (uint32_t d = 0; d < ctas; ++d)
+#pragma unroll
+                for (int i = 0; i < per; i += 2) {
+                    const uint2 v = remote_ld2(remote(h + at + i, d));
+                    n[i] += (int)v.x; n[i + 1] += (int)v.y;
+                }
+        }
         int sum = 0, total;
 #pragma unroll
         for (int i = 0; i < per; ++i) sum += n[i];
-        if (tid == 0) { ctl->bin = 0; ctl->rank = 1; }
+        if (tid == 0) { ctl->bin = 0; ctl->rank = 1; ctl->count = 0; }
         int above = scan(sum, total);
 #pragma unroll
         for (int i = per - 1; i >= 0; --i) {
-            if (above < target && target <= above + n[i]) { ctl->bin = at + i; ctl->rank = target - above; }
+            if (above < target && target <= above + n[i]) { ctl->bin = at + i; ctl->rank = target - above; ctl->count = n[i]; }
             above += n[i];
         }
         epi_sync();
     };
+    // epilogue threads: the set bits of words[] counted per word and before each word; returns how many there are.  (A word a thread.)
+    const int nw = (nbs + 31) >> 5;
+    auto count_words = [&]() -> int {
+        int total;
+        const int base = scan(tid < nw ? __popc(words[tid]) : 0, total);
+        if (tid < nw) wbase[tid] = base;
+        epi_sync();
+        return total;
+    };
     struct Bins { enum { value = kCBins }; };
-    struct Digits { enum { value = kCDigits }; };
+    struct SelBins { enum { value = kCSelBins }; };
 
     uint32_t st = 0, ph = 0, u = 0;                           // K ring and its phase; tiles so far
     uint32_t lo16 = 0u, hi16 = 0u;                            // the blocks of a round: bounds in [lo16, hi16)
@@ -693,43 +706,52 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     for (int round = 0; round < 2; ++round) {
         // ---- the blocks of this round: [lo16, hi16) of the bounds
         if (warp < kEpi) {
-            find_bin(hist, Bins(), round == 0 ? wanted : nkeep);
+            find_bin(hist, Bins(), C, round == 0 ? wanted : nkeep);
             const uint32_t edge = edge_of(ctl->bin);
             if (round == 0) { lo16 = edge; hi16 = 0x10000u; }
             else { hi16 = lo16; lo16 = min(edge, lo16); }
             cut = lo16;
             // this CTA's share of them, and their places in the head's list
-            const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
-            int mine = 0, total;
-            for (int i = i0; i < i1; ++i) mine += ub[i] >= lo16 && ub[i] < hi16;
-            int at = scan(mine, total);
+            for (int w = warp; w < nw; w += kEpi) {
+                const int i = 32 * w + lane;
+                const uint32_t x = i < nbs ? ub[i] : 0x10000u, m = __ballot_sync(0xffffffffu, x >= lo16 && x < hi16);
+                if (lane == 0) words[w] = m;
+            }
+            epi_sync();
+            const int total = count_words();
+            int before = 0, per_cta = 0x40000000;
             if (C > 1) {
                 if (warp == 0 && lane < (int)C) remote_st(remote(&ctl->cnt[rank], lane), total);
                 cluster_sync();
                 const int have = lane < (int)C ? ctl->cnt[lane] : 0;
                 const int all = __reduce_add_sync(0xffffffffu, have);
-                at += __reduce_add_sync(0xffffffffu, lane < (int)rank ? have : 0);
-                const int per_cta = max(8, ((all + (int)C - 1) / (int)C + 7) & ~7);      // whole tiles
-                for (int i = i0; i < i1; ++i)
-                    if (ub[i] >= lo16 && ub[i] < hi16) {
-                        const int to = at / per_cta, x = at - to * per_cta;
-                        if (JQ_IN(x, 8 * P.share, kDbgPrune, 9) && JQ_IN(to, C, kDbgPrune, 10)) remote_st16(remote(list + x, (uint32_t)to), (uint16_t)(b0 + i));
-                        ++at;
-                    }
+                before = __reduce_add_sync(0xffffffffu, lane < (int)rank ? have : 0);
+                per_cta = max(8, ((all + (int)C - 1) / (int)C + 7) & ~7);        // whole tiles
                 if (tid == 0) ctl->n = min(max(all - (int)rank * per_cta, 0), per_cta);
-            } else {
-                for (int i = i0; i < i1; ++i)
-                    if (ub[i] >= lo16 && ub[i] < hi16) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 8)) list[at] = (uint16_t)i; ++at; }
-                if (tid == 0) ctl->n = total;
+            } else if (tid == 0) ctl->n = total;
+            for (int w = warp; w < nw; w += kEpi) {
+                const uint32_t m = words[w];
+                if ((m >> lane & 1u) == 0u) continue;
+                const int at = before + wbase[w] + __popc(m & ((1u << lane) - 1u)), to = C > 1 ? at / per_cta : 0, x = at - to * per_cta;
+                if (!JQ_IN(x, 8 * P.share, kDbgPrune, 8) || !JQ_IN(to, C, kDbgPrune, 9)) continue;
+                if (C > 1) remote_st16(remote(list + x, (uint32_t)to), (uint16_t)(b0 + 32 * w + lane));
+                else list[x] = (uint16_t)(32 * w + lane);
             }
             for (int i = tid; i < kCBins; i += kTE) hist[i] = 0u;   // (everybody has read it)
         } else if (C > 1) cluster_sync();
         sync_all();
         const int n = ctl->n, nt = (n + 7) >> 3;
         if (warp == kEpi) {
-            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, two lanes each
+            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, two lanes each.  The ring
+            // holds two or three tiles, too few for a read from HBM: the blocks are asked for ahead, into the L2.
+            int ahead = 0;
 #pragma unroll 1
             for (int i = 0; i < nt; ++i) {
+                for (; ahead < min(n, 8 * i + kCAhead); ahead += 16) {
+                    const int x = ahead + (lane >> 1);
+                    if (x < n) prefetch_3d(mb, 64 * (lane & 1), list[x] * kPBlock, kv_in);
+                }
+                __syncwarp();
                 const int have = min(8, n - 8 * i);
                 if (!__all_sync(0xffffffffu, mbar_wait(&ctl->empty[st], ph ^ 1, &ctl->abort_flag, status, 64))) break;
                 if (lane == 0) mbar_expect_tx(&ctl->full[st], (uint32_t)have * 2u * kPBlockHalf);
@@ -831,163 +853,235 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
 
-    // ---------------------------------------------------------------- selection (the epilogue warps).  What is not scored counts as zero: its
-    // scores lie below the threshold, and so does every pooled score that they alone would make.  (Whatever the scores are,
-    // after a wait that ran out too, every place that follows is brought into range.)
-    const int half = lane >> 4, i16 = lane & 15, reach = (P.radius + kPBlock - 1) / kPBlock;   // blocks that a window reaches into on either side
-    if (C > 1 && reach > 0) {
-        if (warp == 0 && lane < (int)C) {
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int i = x < 2 ? x : nbs - 4 + x;
-                remote_st16(remote(&ctl->edge[rank][x], lane), i >= 0 && i < nbs ? ub[i] : (uint16_t)0);
-            }
-            remote_st(remote(&ctl->edge_n[rank], lane), nbs);
-        }
-        cluster_sync();
-        if (tid < 4) {                                        // (a share may be shorter than two blocks, or empty)
-            int d = tid < 2 ? 2 - tid : tid - 1, q = (int)rank;   // the d-th block before / behind this CTA's share
-            uint16_t v = 0;
-            for (;;) {
-                q += tid < 2 ? -1 : 1;
-                if (q < 0 || q >= (int)C) break;
-                const int n = ctl->edge_n[q];
-                if (d <= n) { v = ctl->edge[q][tid < 2 ? 4 - d : d - 1]; break; }
-                d -= n;
-            }
-            ctl->halo[tid] = v;
-        }
-    } else if (tid < 4) ctl->halo[tid] = 0;
-    for (int i = tid; i < kCDigits; i += kTE) digits[i] = 0u;
+    if (C > 1) {
+        // the selection is a kernel of its own, over all positions of the head: what has not been scored counts as zero
+        float *const s = P.scores + soff + (long long)b0 * kPBlock;
+        const int m = min(nbs * kPBlock, L - b0 * kPBlock);
+        for (int i = tid; i < m; i += kTE)
+            if (ub[i >> 4] < cut && JQ_IN(soff + (long long)b0 * kPBlock + i, P.ext.scores, kDbgPrune, 14)) s[i] = 0.f;
+        return;
+    }
+    // ---------------------------------------------------------------- selection (one CTA, the epilogue warps), among the positions of the
+    // active blocks: those that are scored and those that a window reaches from there.  What is not scored counts as zero: its
+    // scores lie below the threshold, and so does every pooled score that they alone would make.  Laid one after the other, the
+    // active blocks can be pooled as if they were neighbours: between two of them that are not lies a whole reach of zeros.
+    // (Whatever the scores are, after a wait that ran out too, every place that follows is brought into range.)
+    const int reach = (P.radius + kPBlock - 1) / kPBlock;    // blocks that a window reaches into on either side: 0, 1 or 2
+    uint32_t *const bins = (uint32_t *)smem_raw;             // in the place of queries and stages: [kCSelBins],
+    uint32_t *const cand = bins + kCSelBins;                 // [kCRank],
+    float *const sc = (float *)(cand + kCRank) + 32;         // [16 room] scores, then keys, with 32 zeros on either side
+    const int room = (int)(((uint8_t *)ctl - (uint8_t *)(sc + 32)) / 64);
+    uint16_t *const act = list;                              // the active blocks, in order
+    for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
+    if (tid == 0) ctl->ncand = 0;
+    for (int w = warp; w < nw; w += kEpi) {
+        const int i = 32 * w + lane;
+        const uint32_t m = __ballot_sync(0xffffffffu, i < nbs && ub[i] >= cut);
+        if (lane == 0) words[w] = m;
+    }
     epi_sync();
-    const bool out_of_share = C > 1 && cut > 0u;
-    auto scored = [&](int i) -> bool {                        // block b0 + i, for i up to two blocks outside of the share
-        if (i >= 0 && i < nbs) return ub[i] >= cut;
-        const int x = i < 0 ? i + 2 : i - nbs + 2;
-        return out_of_share ? ctl->halo[x] >= cut : (C > 1 && b0 + i >= 0 && b0 + i < nb);
-    };
-    int n_act;
     {
-        const int per = (nbs + kTE - 1) / kTE, i0 = min(tid * per, nbs), i1 = min(i0 + per, nbs);
-        auto active = [&](int i) -> bool {
-            bool on = false;
-            for (int d = -reach; d <= reach; ++d) on |= scored(i + d);
-            return on;
-        };
-        int mine = 0;
-        for (int i = i0; i < i1; ++i) mine += active(i);
-        int at = scan(mine, n_act);
-        for (int i = i0; i < i1; ++i) if (active(i)) { if (JQ_IN(at, 8 * P.share, kDbgPrune, 14)) act[at] = (uint16_t)i; ++at; }
+        uint32_t m = 0u;
+        if (tid < nw) {
+            const uint32_t p = tid > 0 ? words[tid - 1] : 0u, q = words[tid], r = tid + 1 < nw ? words[tid + 1] : 0u;
+            m = q;
+            for (int d = 1; d <= reach; ++d) m |= q << d | q >> d | p >> (32 - d) | r << (32 - d);
+            if (tid == nw - 1 && (nbs & 31)) m &= (1u << (nbs & 31)) - 1u;
+        }
+        epi_sync();
+        if (tid < nw) words[tid] = m;
+    }
+    const int n_act = count_words();
+    for (int w = warp; w < nw; w += kEpi) {
+        const uint32_t m = words[w];
+        const int at = wbase[w] + __popc(m & ((1u << lane) - 1u));
+        if ((m >> lane & 1u) && JQ_IN(at, 8 * P.share, kDbgPrune, 15)) act[at] = (uint16_t)(32 * w + lane);
+    }
+    epi_sync();
+    auto block_of = [&](int a) -> int { return min((int)act[a], nbs - 1); };
+    // The keys stay on chip, in the place of the scores that they are made of, or (more than there is room for, or a window
+    // that reaches past the next quad) go to memory a chunk at a time.  A key is one above the bits of a pooled score, which is
+    // not negative: order and ties are those of the values.  Positions that do not exist have the key 0.
+    const bool on_chip = n_act <= room && P.radius <= 4;
+    uint32_t *const gk = P.gkeys + soff;
+    const int chunk = on_chip ? n_act : room - 4;
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll 1
+    for (int c0 = 0; c0 < n_act; c0 += chunk) {
+        const int c1 = min(c0 + chunk, n_act), f0 = max(c0 - 2, 0), f1 = min(c1 + 2, n_act);   // (with two blocks of halo)
+        const int i16 = tid & 15;
+#pragma unroll 1
+        for (int a = f0 + (tid >> 4); a < f1; a += kTE / 2) {          // eight loads in flight per thread
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = a + e * (kTE / 16), blk = x < f1 ? block_of(x) : 0, pos = blk * kPBlock + i16;
+                v[e] = x < f1 && pos < L && ub[blk] >= cut && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 16) ? __ldcg(P.scores + soff + pos) : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = a + e * (kTE / 16);
+                if (x < f1 && JQ_IN(x - f0, room, kDbgPrune, 10)) sc[(x - f0) * 16 + i16] = v[e];
+            }
+        }
+        if (tid < 32) sc[tid - 32] = 0.f;
+        else if (tid < 64) sc[(f1 - f0) * 16 + tid - 32] = 0.f;
+        epi_sync();
+        const int nq = 4 * (c1 - c0), NQ = ((nq + kTE - 1) / kTE) | 1, q0 = min(tid * NQ, nq), q1 = min(q0 + NQ, nq), shift = 4 * (c0 - f0);
+        float4 *const s4 = (float4 *)sc + shift;
+        float4 before = s4[q0 - 1], last = s4[q1], here = s4[q0];
+        if (on_chip) epi_sync();                                     // (everybody has the quads next to his own)
+#pragma unroll 1
+        for (int q = q0; q < q1; ++q) {
+            float best[4];
+            if (P.radius <= 4) {
+                uint32_t unused[4];
+                const float4 next = q + 1 < q1 ? s4[q + 1] : last;
+                pooled_quad(before, here, next, P.radius, unused, best);
+                before = here; here = next;
+            } else {
+                const float *const x = (const float *)(s4 + q);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float m = x[e];
+#pragma unroll 1
+                    for (int r = 1; r <= P.radius; ++r) m = max3(m, x[e - r], x[e + r]);
+                    best[e] = m;
+                }
+            }
+            uint32_t k[4];
+            const int pos = block_of(c0 + (q >> 2)) * kPBlock + 4 * (q & 3);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                k[e] = pos + e < L ? __float_as_uint(best[e]) + 1u : 0u;
+                if (k[e]) { kmin = min(kmin, k[e]); kmax = max(kmax, k[e]); }
+            }
+            if (on_chip) ((uint4 *)s4)[q] = make_uint4(k[0], k[1], k[2], k[3]);
+            else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (k[e] && JQ_IN(soff + 16 * c0 + 4 * q + e, P.ext.scores, kDbgPrune, 18)) gk[16 * c0 + 4 * q + e] = k[e];
+            }
+        }
         epi_sync();
     }
-    // Warp w owns the active blocks [a0, a1), half a warp to a block; a thread reads the keys that it wrote itself.
-    const int seg = ((n_act + kEpi - 1) / kEpi + 1) & ~1, a0 = min(warp * seg, n_act), a1 = min(a0 + seg, n_act);
-    uint32_t *const keys = n_act <= keys_room ? keys_s : P.gkeys + soff + (long long)b0 * kPBlock;
-    auto block_of = [&](int a) -> int { return min((int)act[a], nbs - 1); };
-    {
-        float *const mine = scratch + (warp * 2 + half) * 80;
-#pragma unroll 1
-        for (int a = a0; a < a1; a += 8) {
-            float v[4][5];
-            int blk[4];
+    // A thread owns NQ consecutive quads from here on: the max-pool's plateaus then mostly fall within a thread, and thread order is
+    // position order.
+    const int nq = 4 * n_act, NQ = ((nq + kTE - 1) / kTE) | 1, q0 = min(tid * NQ, nq), q1 = min(q0 + NQ, nq);
+    auto keys_of = [&](int q, uint32_t (&k)[4]) {
+        if (on_chip) {
+            const uint4 v = ((const uint4 *)sc)[q];
+            k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+        } else {
+            const int pos = block_of(q >> 2) * kPBlock + 4 * (q & 3);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int x = a + 2 * e + half;
-                blk[e] = x < a1 ? block_of(x) : -4;
-#pragma unroll
-                for (int d = -2; d <= 2; ++d) {
-                    const int pos = (b0 + blk[e] + d) * kPBlock + i16;
-                    const bool in = blk[e] >= 0 && abs(d) <= reach && pos >= 0 && pos < L && scored(blk[e] + d);
-                    v[e][d + 2] = in && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 15) ? __ldcg(P.scores + soff + pos) : 0.f;
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                __syncwarp();
-#pragma unroll
-                for (int d = 0; d < 5; ++d) if (abs(d - 2) <= reach) mine[16 * d + i16] = v[e][d];
-                __syncwarp();
-                float m = mine[32 + i16];
-#pragma unroll 1
-                for (int r = 1; r <= P.radius; ++r) m = max3(m, mine[32 + i16 - r], mine[32 + i16 + r]);
-                const int x = a + 2 * e + half;
-                if (x < a1 && (b0 + blk[e]) * kPBlock + i16 < L) {
-                    // (one above the bits of a value that is not negative: order and ties as the values have them)
-                    if (JQ_IN(x * 16 + i16, n_act <= keys_room ? keys_room * 16 : (long long)nbs * 16, kDbgPrune, 16)) keys[x * 16 + i16] = __float_as_uint(m) + 1u;
-                }
-            }
+            for (int e = 0; e < 4; ++e) k[e] = pos + e < L && JQ_IN(soff + 4 * q + e, P.ext.scores, kDbgPrune, 19) ? __ldcg(gk + 4 * q + e) : 0u;
         }
-    }
-    auto key_at = [&](int x) -> uint32_t {                    // of active block x (0: there is no such position)
-        return x < a1 && (b0 + block_of(x)) * kPBlock + i16 < L ? keys[x * 16 + i16] : 0u;
     };
-    // The threshold: 11, 11 and 10 bits of it at a time, over the keys that agree with it so far.
-    uint32_t tau = 0u;
-    int krem = nkeep;
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) { ctl->wmin[warp] = kmin; ctl->wmax[warp] = kmax; }
+    epi_sync();
+    kmin = __reduce_min_sync(0xffffffffu, ctl->wmin[lane % kEpi]);
+    kmax = __reduce_max_sync(0xffffffffu, ctl->wmax[lane % kEpi]);
+    // The threshold key: 2048 equal bins over the keys' own range, then the bin's few keys ranked by comparison, or binned again
+    // while they are many.
+    uint32_t lo = kmin, lim = kmax - kmin, tau;
+    int need = nkeep;
 #pragma unroll 1
-    for (int level = 0; level < 3; ++level) {
-        const int shift = level == 0 ? 21 : level == 1 ? 10 : 0, done = level == 0 ? 32 : level == 1 ? 21 : 10;
+    for (;;) {
+        const int sh = lim >> 11 ? 21 - __clz(lim) : 0;               // lim >> sh < 2048
+        uint32_t cur = 0u, cnt = 0u;
 #pragma unroll 1
-        for (int a = a0; a < a1; a += 2) {
-            const uint32_t k = key_at(a + half);
-            const bool in = k != 0u && (level == 0 || (k ^ tau) >> done == 0u);
-            const uint32_t d = in ? (k >> shift) & (kCDigits - 1) : 0xffffffffu;
-            const uint32_t same = __match_any_sync(0xffffffffu, d);   // (the max-pool's plateaus as one count)
-            if (in && lane == __ffs(same) - 1) atomicAdd(&digits[d], (uint32_t)__popc(same));
+        for (int q = q0; q < q1; ++q) {
+            uint32_t k[4];
+            keys_of(q, k);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {                             // neighbours often share the bin: runs as one count
+                const uint32_t d = k[e] - lo;
+                const bool in = k[e] != 0u && d <= lim, other = in && d >> sh != cur;
+                if (other && cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
+                cnt = other ? 1u : cnt + in;
+                cur = other ? d >> sh : cur;
+            }
         }
-        sync_epi();
-        find_bin(digits, Digits(), krem);
-        tau |= (uint32_t)ctl->bin << shift;
-        krem = ctl->rank;
-        if (level < 2) {
-            sync_epi();                                       // (everybody has read the counts)
-            for (int i = tid; i < kCDigits; i += kTE) digits[i] = 0u;
+        if (cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
+        epi_sync();
+        find_bin(bins, SelBins(), 1, need);
+        lo += (uint32_t)ctl->bin << sh;
+        need = ctl->rank;
+        const int count = ctl->count;
+        tau = lo;
+        if (sh == 0) break;
+        lim = (1u << sh) - 1u;
+        if (count <= kCRank) {
+#pragma unroll 1
+            for (int q = q0; q < q1; ++q) {
+                uint32_t k[4];
+                keys_of(q, k);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (k[e] != 0u && k[e] - lo <= lim) {
+                        const int at = atomicAdd(&ctl->ncand, 1);
+                        if (at < kCRank) cand[at] = k[e];
+                    }
+            }
             epi_sync();
+            if (tid == 0) { ctl->tau = lo; ctl->need = need; }
+            epi_sync();
+            for (int i = tid; i < count; i += kTE) {
+                const uint32_t k = cand[i];
+                int gt = 0, eq = 0;
+#pragma unroll 4
+                for (int x = 0; x < count; ++x) { const uint32_t y = cand[x]; gt += y > k; eq += y == k; }
+                if (gt < need && need <= gt + eq) { ctl->tau = k; ctl->need = need - gt; }   // (equal keys write the same)
+            }
+            epi_sync();
+            tau = ctl->tau;
+            need = ctl->need;
+            break;
         }
+        for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
+        epi_sync();
     }
-    // Kept: all keys above tau and, of those equal to it, the first krem.
+    // Kept: all keys above tau and, of those equal to it, the first `need`.
     int gt = 0, eq = 0;
 #pragma unroll 1
-    for (int a = a0; a < a1; a += 2) {
-        const uint32_t k = key_at(a + half);
-        gt += __popc(__ballot_sync(0xffffffffu, k > tau));
-        eq += __popc(__ballot_sync(0xffffffffu, k == tau && k != 0u));
+    for (int q = q0; q < q1; ++q) {
+        uint32_t k[4];
+        keys_of(q, k);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { gt += k[e] > tau; eq += k[e] == tau && k[e] != 0u; }
     }
-    if (lane == 0) { ctl->warp_gt[warp] = gt; ctl->warp_eq[warp] = eq; }
-    epi_sync();
-    {
-        const int g = lane < kEpi ? ctl->warp_gt[lane] : 0, e = lane < kEpi ? ctl->warp_eq[lane] : 0;
-        if (C > 1) {
-            const int tg = __reduce_add_sync(0xffffffffu, g), tq = __reduce_add_sync(0xffffffffu, e);
-            if (warp == 0 && lane < (int)C) { remote_st(remote(&ctl->gt_of[rank], lane), tg); remote_st(remote(&ctl->eq_of[rank], lane), tq); }
-            cluster_sync();
-        }
-        gt = __reduce_add_sync(0xffffffffu, (lane < warp ? g : 0) + (C > 1 && lane < (int)rank ? ctl->gt_of[lane] : 0));
-        eq = __reduce_add_sync(0xffffffffu, (lane < warp ? e : 0) + (C > 1 && lane < (int)rank ? ctl->eq_of[lane] : 0));
-    }
+    int all;
+    gt = scan(gt, all);
+    eq = scan(eq, all);
     int32_t *const out = P.idx + orow;
 #pragma unroll 1
-    for (int a = a0; a < a1; a += 2) {
-        const uint32_t k = key_at(a + half), below = (1u << lane) - 1u;
-        const uint32_t bg = __ballot_sync(0xffffffffu, k > tau), be = __ballot_sync(0xffffffffu, k == tau && k != 0u);
-        if (!(bg | be)) continue;
-        const int g = gt + __popc(bg & below), e = eq + __popc(be & below), t = g + min(e, krem);
-        if ((k > tau || (k == tau && k != 0u && e < krem)) && t >= 0 && t < nkeep && JQ_IN(orow + t, P.ext.out_rows, kDbgPrune, 17))
-            out[t] = (b0 + block_of(a + half)) * kPBlock + i16;
-        gt += __popc(bg);
-        eq += __popc(be);
+    for (int q = q0; q < q1; ++q) {
+        uint32_t k[4];
+        keys_of(q, k);
+        if (k[0] < tau && k[1] < tau && k[2] < tau && k[3] < tau) continue;
+        const int pos = block_of(q >> 2) * kPBlock + 4 * (q & 3);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool same = k[e] == tau && k[e] != 0u;
+            const int t = gt + min(eq, need);
+            if ((k[e] > tau || (same && eq < need)) && t < nkeep && JQ_IN(orow + t, P.ext.out_rows, kDbgPrune, 17)) out[t] = pos + e;
+            gt += k[e] > tau;
+            eq += same;
+        }
     }
     // ---------------------------------------------------------------- the rows, once every index of the head has been written
-    sync_epi();
-    copy_rows(tid, kTE, out, (int)((long long)rank * nkeep / C), (int)((long long)(rank + 1) * nkeep / C), kv_in, krow, L, Kin, Vin, P.Kout, P.Vout,
-              src_rows, P.ext JQ_DBG_ARG_DEV);
-    if (P.win.w) copy_window(P.win, head, krow + nkeep, (int)rank * (kTE / 16) + (tid >> 4), (int)C * (kTE / 16), P.Kout, P.Vout, P.ext JQ_DBG_ARG_DEV);
+    epi_sync();
+    copy_rows(tid, kTE, out, 0, nkeep, kv_in, krow, L, Kin, Vin, P.Kout, P.Vout, src_rows, P.ext JQ_DBG_ARG_DEV);
+    if (P.win.w) copy_window(P.win, head, krow + nkeep, tid >> 4, kTE / 16, P.Kout, P.Vout, P.ext JQ_DBG_ARG_DEV);
 }
 
 // ------------------------------------------------------------------ host side
 
 constexpr size_t stats_smem(int Rbox, int stages) { return 2 * (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kSCtlBytes; }
-size_t cand_smem(int Rbox, int stages, int share) { return (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kCCtlBytes + kCBins * 4 + (size_t)share * 32; }
+size_t cand_smem(int Rbox, int stages, int share) { return (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kCCtlBytes + kCBins * 4 + (size_t)share * 32 + (size_t)(share / 4 + 1) * 8; }
 constexpr size_t kCMaxSmem = 227 * 1024, kCTwoPerSm = 113 * 1024;
 
 struct PruneDevice {
@@ -1135,6 +1229,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
         return JQ_ERR_CUDA;
     }
     count_launch(2);
+    if (C > 1) return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
     return check_launch();
 }
 
