@@ -346,49 +346,30 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
     }
 }
 
-// ------------------------------------------------------------------ candidates: scores, selection, rows
+// ------------------------------------------------------------------ what the kernels behind row_stats share
 
 constexpr int kCMaxCluster = 16;
 constexpr int kCBins = 1024;                     // bins of 1/16 octave: 64 octaves from 2^-54 up to 2^10
 constexpr int kCBase = (127 - 54) << 4;
-constexpr int kCSelBins = 2048;                  // the selection's bins, equal parts of a range of keys
-constexpr int kCRank = 512;                      // keys of one bin that are ranked by comparison
 constexpr int kCMaxStages = 4;
-constexpr int kCAhead = 128;                     // blocks that are on their way into the L2 ahead of the ring
 constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16 bits
-__host__ __device__ constexpr int cand_groups(bool wide) { return wide ? 4 : 2; }
-__host__ __device__ constexpr int cand_threads(bool wide) { return cand_groups(wide) * 128 + 64; }
-
-struct CCtl {
-    uint64_t full[kCMaxStages], empty[kCMaxStages], q_full, t_full[2], t_empty[2];
-    uint64_t b_full[kCMaxStages], b_empty[kCMaxStages];
-    uint32_t tmem_base;
-    int abort_flag;
-    int bin, rank, count;                        // find_bin's answer
-    int n;                                       // blocks on this CTA's list
-    int huge;                                    // a normaliser is out of a half's range
-    int ncand, need;
-    uint32_t tau;
-    int scan[16];
-    uint32_t wmin[16], wmax[16];
-    int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
-    alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads; before, pairs of statistics
-    alignas(16) float Ms[kMaxR];                 // minus the row normalisers
-};
-constexpr uint32_t kCCtlBytes = 4096;
-static_assert(sizeof(CCtl) <= kCCtlBytes && offsetof(CCtl, Ms) % 16 == 0 && offsetof(CCtl, xs) % 16 == 0, "control block");
 
 struct CParams {
     int L, tph, nkeep;         // one shape (tph: tiles per head in row_stats' numbering, the window tile included)
-    int R, Rbox, Rpad, radius;
-    int stages, groups;        // K ring; row_stats' epilogue groups
-    int sms;                   // row_stats' grid
-    int share;                 // most tiles of a head that a CTA looks after
+    int heads, R, Rbox, Rpad, radius;
+    int groups, sms;           // row_stats' epilogue groups and its grid
+    int stages, share;         // score_candidates: K ring; most tiles of a head that a CTA looks after
     int first_pct;             // blocks of round 1 per 100 pairs kept
+    int fill;                  // score_candidates writes zeros where it does not score (the selection reads every score)
+    int room;                  // select_candidates: active blocks whose keys stay on chip
+    int max_words;             // select_candidates: words of 32 blocks of the longest head
     long long T;
     float c;
     const float2 *part;
     const uint32_t *bmax;
+    float *Ms;                 // [heads][kMaxR]: minus the row normalisers
+    uint16_t *ub;              // [tile][8]: bounds of the blocks, upper 16 bits of a float
+    uint32_t *cut;             // [heads]: the blocks with bounds from here on have been scored
     float *scores;
     uint32_t *gkeys;           // [keys of all heads]: the selection's keys where shared memory has no room for them
     int *status;
@@ -407,6 +388,234 @@ struct CParams {
 #endif
 };
 
+// A head as these kernels see it: its length and budget, its tiles (in row_stats' numbering: all, and the first one's number)
+// and its scores.
+struct HeadAt {
+    int L, nkeep, tph1;
+    long long soff, tbase;
+};
+__device__ __forceinline__ HeadAt head_at(const CParams &P, int h)
+{
+    HeadAt a;
+    if (P.htab) {
+        const HeadRec *r = P.htab + h;
+        a.L = r->L; a.nkeep = r->nkeep; a.soff = r->soff; a.tbase = r->tbase;
+        a.tph1 = (a.L + kPTile - 1) / kPTile;
+    } else {
+        a.L = P.L; a.nkeep = P.nkeep; a.soff = (long long)h * P.L; a.tbase = (long long)h * P.tph; a.tph1 = P.tph;
+    }
+    return a;
+}
+
+// The bin of a value >= 0 (given as the upper 16 bits of a float, rounded either way): its lower edge is not above the value.
+__device__ __forceinline__ int bin_of(uint32_t top16) { return min(max((int)(top16 >> 3) - kCBase, 0), kCBins - 1); }
+// The lower edge of a bin, as the upper 16 bits of a float; of the lowest bin 0.
+__device__ __forceinline__ uint32_t edge_of(int bin) { return bin > 0 ? (uint32_t)(bin + kCBase) << 3 : 0u; }
+
+template <int kThreads>
+__device__ __forceinline__ void named_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
+
+// Threads 0 .. kThreads - 1 of a CTA: exclusive scan of one int per thread, and the sum.  sums: an int per warp.
+template <int kThreads>
+__device__ __forceinline__ int scan_threads(int v, int &total, int *sums)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
+    if (lane == 31) sums[warp] = inc;
+    named_sync<kThreads>();
+    const int s = lane < kThreads / 32 ? sums[lane] : 0;
+    total = __reduce_add_sync(0xffffffffu, s);
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? s : 0);
+    named_sync<kThreads>();
+    return before + inc - v;
+}
+
+struct BinAt { int bin, rank, count; };   // a bin, the rank in it of what was looked for, its population
+
+// The same threads: the bin that holds the target-th entry from the top (without so many entries: bin 0).  get(i) gives the
+// counts of bins i, i + 1.
+template <int kThreads, int kN, typename Get>
+__device__ __forceinline__ BinAt find_bin(Get get, int target, BinAt *res, int *sums)
+{
+    constexpr int per = kN / kThreads;                        // consecutive bins of a thread, from the top
+    const int at = kN - per * ((int)threadIdx.x + 1);
+    int n[per], sum = 0, total;
+#pragma unroll
+    for (int i = 0; i < per; i += 2) { const uint2 v = get(at + i); n[i] = (int)v.x; n[i + 1] = (int)v.y; }
+#pragma unroll
+    for (int i = 0; i < per; ++i) sum += n[i];
+    if (threadIdx.x == 0) *res = {0, 1, 0};
+    int above = scan_threads<kThreads>(sum, total, sums);
+#pragma unroll
+    for (int i = per - 1; i >= 0; --i) {
+        if (above < target && target <= above + n[i]) *res = {at + i, target - above, n[i]};
+        above += n[i];
+    }
+    named_sync<kThreads>();
+    return *res;
+}
+
+// ------------------------------------------------------------------ bounds
+
+constexpr int kBThreads = 256, kBPerSm = 4;
+
+// grid: four CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
+// then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  A maximum x within 64 of its row's
+// normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60 each, which is
+// added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
+template <bool kWide>
+__global__ void __launch_bounds__(kBThreads, kBPerSm)
+block_bounds(const __grid_constant__ CParams P)
+{
+    __shared__ float Ms[kMaxR];
+    __shared__ float2 other[kMaxR];
+    __shared__ int huge;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int R = P.R, Rpad = P.Rpad;
+#ifdef JQ_DEBUG
+    DebugRecord *const dbg = P.dbg_rec;
+#endif
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
+    const long long G = gridDim.x;
+    long long f = blockIdx.x * P.T / G;
+    const long long end = (blockIdx.x + 1) * P.T / G;
+    int h;
+    if (P.htab) {
+        int lo = 0, hi = P.heads - 1;                         // the last head whose first tile is not past f
+        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (P.htab[mid].tbase <= f) lo = mid; else hi = mid - 1; }
+        h = lo;
+    } else h = (int)(f / P.tph);
+#pragma unroll 1
+    for (; f < end; ++h) {
+        const HeadAt a = head_at(P, h);
+        const int t0 = (int)(f - a.tbase), tph = (a.L + kPTile - 1) / kPTile, nb = (a.L + kPBlock - 1) / kPBlock;
+        const int t1 = (int)min((long long)tph, end - a.tbase);       // (the window tile has no bounds)
+        f = a.tbase + a.tph1;
+        if (tid == 0) huge = 0;
+        {   // the CTAs of row_stats that had tiles of this head, each with a pair per row and group: eight loads in flight
+            const long long c_lo = ((a.tbase + 1) * P.sms - 1) / P.T, c_hi = ((a.tbase + a.tph1) * P.sms - 1) / P.T;   // owners of the first and last tile
+            const int nsl = (int)(c_hi - c_lo + 1) * P.groups;
+            const long long s0 = (c_lo + h) * P.groups;
+            constexpr int kSub = kWide ? 1 : 2;                       // threads per row
+            const int row = tid & (kWide ? 255 : 127), sub = kWide ? 0 : tid >> 7;
+            const float2 *src = P.part + s0 * R + row;
+            float m = -INFINITY, l = 0.f;
+            if (row < R) {
+#pragma unroll 1
+                for (int i0 = sub; i0 < nsl; i0 += 8 * kSub) {
+                    float2 p[8];
+                    float mn = m;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int i = i0 + kSub * k;
+                        p[k] = i < nsl && JQ_IN((s0 + i) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)i * R) : make_float2(-INFINITY, 0.f);
+                        if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
+                    }
+                    if (mn > -INFINITY) {
+                        l *= ex2(P.c * (m - mn));
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) if (p[k].y > 0.f) l = fmaf(p[k].y, ex2(P.c * (p[k].x - mn)), l);
+                        m = mn;
+                    }
+                }
+            }
+            if (sub == 1) other[row] = make_float2(m, l);
+            __syncthreads();
+            if (sub == 0) {
+                float M = INFINITY;                                   // silences a column that is not a query row
+                if (row < R) {
+                    if (kSub == 2) {
+                        const float2 o = other[row];
+                        const float mn = fmaxf(m, o.x);
+                        l = (l > 0.f ? l * ex2(P.c * (m - mn)) : 0.f) + (o.y > 0.f ? o.y * ex2(P.c * (o.x - mn)) : 0.f);
+                        m = mn;
+                    }
+                    M = fmaf(P.c, m, log2f(l));
+                    if (!(fabsf(M) < 60000.f)) huge = 1;
+                }
+                Ms[row] = -M;
+                if (!kWide) Ms[128 + row] = -INFINITY;
+                if (t0 == 0) { P.Ms[(size_t)h * kMaxR + row] = -M; if (!kWide) P.Ms[(size_t)h * kMaxR + 128 + row] = -INFINITY; }
+            }
+            __syncthreads();
+        }
+        // a lane takes four neighbouring rows (eight with more than 128)
+        constexpr int kV = kWide ? 2 : 1;
+        float nm[4 * kV];
+#pragma unroll
+        for (int i = 0; i < 4 * kV; ++i) {
+            const float x = Ms[(i >> 2) * 128 + 4 * lane + (i & 3)];
+            nm[i] = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;
+        }
+        const float least = huge ? INFINITY : 3e-16f;
+#pragma unroll 1
+        for (int t = t0 + warp; t < t1; t += kBThreads / 32) {
+            uint4 v[4][kV];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int y = 0; y < kV; ++y) {                        // (a row that is none has a normaliser of inf)
+                    const long long at = ((a.tbase + t) * 4 + q) * Rpad + y * 128 + 4 * lane;
+                    const bool in = y * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6);
+                    v[q][y] = in ? __ldcs((const uint4 *)(P.bmax + at)) : make_uint4(0u, 0u, 0u, 0u);
+                }
+            float2 sum[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                sum[q] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int y = 0; y < kV; ++y) {
+                    const uint32_t e[4] = {v[q][y].x, v[q][y].y, v[q][y].z, v[q][y].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 g = __fadd2_rn(__half22float2(*(const __half2 *)&e[i]), make_float2(nm[4 * y + i], nm[4 * y + i]));
+                        sum[q] = __fadd2_rn(sum[q], make_float2(ex2(g.x), ex2(g.y)));
+                    }
+                }
+            }
+            // eight sums over the 32 lanes: after three exchanges of halves a lane holds one block's part
+            const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+            float2 p[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float2 keep = h4 ? sum[2 + i] : sum[i], give = h4 ? sum[i] : sum[2 + i];
+                p[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16), keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16));
+            }
+            const float2 keep = h3 ? p[1] : p[0], give = h3 ? p[0] : p[1];
+            const float2 r2 = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8), keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8));
+            float r = (h2 ? r2.y : r2.x) + __shfl_xor_sync(0xffffffffu, h2 ? r2.x : r2.y, 4);
+            r += __shfl_xor_sync(0xffffffffu, r, 2);
+            r += __shfl_xor_sync(0xffffffffu, r, 1);
+            const int blk = (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
+            if ((lane & 3) == 0)
+                P.ub[(size_t)(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16) : (uint16_t)0;
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ scores of the candidates
+
+__host__ __device__ constexpr int cand_groups(bool wide) { return wide ? 4 : 2; }
+__host__ __device__ constexpr int cand_threads(bool wide) { return cand_groups(wide) * 128 + 64; }
+
+struct CCtl {
+    uint64_t full[kCMaxStages], empty[kCMaxStages], q_full, t_full[2], t_empty[2];
+    uint32_t tmem_base;
+    int abort_flag;
+    int n;                                       // blocks on this CTA's list
+    BinAt found;
+    int sums[16];
+    int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
+    alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads
+    alignas(16) float Ms[kMaxR];                 // minus the row normalisers
+};
+constexpr uint32_t kCCtlBytes = 4096;
+static_assert(sizeof(CCtl) <= kCCtlBytes && offsetof(CCtl, Ms) % 16 == 0, "control block");
+
 __device__ __forceinline__ uint32_t remote(const void *p, uint32_t rank)   // the same place in CTA `rank` of the cluster
 {
     uint32_t a;
@@ -421,23 +630,10 @@ __device__ __forceinline__ uint2 remote_ld2(uint32_t a)
 }
 __device__ __forceinline__ void remote_st(uint32_t a, int v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void remote_st16(uint32_t a, uint16_t v) { asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)   // all of it 16-byte aligned
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void prefetch_3d(const CUtensorMap *map, int c0, int c1, int c2)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-// The bin of a value >= 0 (given as the upper 16 bits of a float, rounded either way): its lower edge is not above the value.
-__device__ __forceinline__ int bin_of(uint32_t top16) { return min(max((int)(top16 >> 3) - kCBase, 0), kCBins - 1); }
-// The lower edge of a bin, as the upper 16 bits of a float; of the lowest bin 0.
-__device__ __forceinline__ uint32_t edge_of(int bin) { return bin > 0 ? (uint32_t)(bin + kCBase) << 3 : 0u; }
 
 template <bool kWide>
 __global__ void __launch_bounds__(cand_threads(kWide), kWide ? 1 : 2)
-evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CParams P)
+score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CParams P)
 {
     constexpr int kGroups = cand_groups(kWide), kEpi = 4 * kGroups, kTE = 32 * kEpi;
     constexpr uint32_t kSlotCols = kWide ? 256 : 128, kCols = 2 * kSlotCols;   // two accumulators in tensor memory
@@ -446,7 +642,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     uint8_t *const qbuf = smem_raw, *const kbuf = smem_raw + q_bytes;
     CCtl *const ctl = (CCtl *)(kbuf + (size_t)P.stages * kPStage);
     uint32_t *const hist = (uint32_t *)((uint8_t *)ctl + kCCtlBytes);            // [kCBins]
-    uint16_t *const ub = (uint16_t *)(hist + kCBins);                            // [8 share]: bounds of this CTA's share, upper 16 bits
+    uint16_t *const ub = (uint16_t *)(hist + kCBins);                            // [8 share]: bounds of this CTA's share
     uint16_t *const list = ub + 8 * P.share;                                     // [8 share]: blocks that this CTA scores
     uint32_t *const words = (uint32_t *)(list + 8 * P.share);                    // [share / 4 + 1]: blocks as bits,
     int *const wbase = (int *)(words + P.share / 4 + 1);                         // and how many come before each word
@@ -456,7 +652,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
     const int head = (int)(blockIdx.x / C);
     int *const status = P.status;
-    const int R = P.R, Rpad = P.Rpad;
+    const int Rpad = P.Rpad;
 #ifdef JQ_DEBUG
     DebugRecord *const dbg = P.dbg_rec;
 #endif
@@ -465,14 +661,10 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kCMaxStages; ++s) {
-            mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1);
-            mbar_init(&ctl->b_full[s], 1); mbar_init(&ctl->b_empty[s], kEpi);
-        }
+        for (int s = 0; s < kCMaxStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         mbar_init(&ctl->q_full, 1);
         for (int s = 0; s < 2; ++s) { mbar_init(&ctl->t_full[s], 1); mbar_init(&ctl->t_empty[s], kWide ? 8 : 4); }
         ctl->abort_flag = 0;
-        ctl->huge = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kEpi + 1) {
@@ -488,214 +680,52 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     cudaGridDependencySynchronize();             // nothing in global memory has been touched so far
     cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up meanwhile; it waits for this one's results
 
-    int L = P.L, nkeep = P.nkeep, kv_in = head, tph1 = P.tph, src_rows = P.src_rows;
-    long long soff = (long long)head * L, tbase = (long long)head * P.tph;
-    long long orow = (long long)head * nkeep, krow = (long long)head * P.out_rows;      // first rows of the head's indices and of its compacted rows
-    const uint4 *Kin = P.K, *Vin = P.V;
+    const HeadAt at = head_at(P, head);
+    const int L = at.L, nkeep = at.nkeep;
+    int kv_in = head;
     const CUtensorMap *mb = &mapB, *mq = &mapQ;
     if (P.htab) {
-        const HeadRec r = P.htab[head];
-        L = r.L; nkeep = r.nkeep; kv_in = r.kv_in; soff = r.soff; tbase = r.tbase; orow = krow = r.ooff; src_rows = L;
-        tph1 = (L + kPTile - 1) / kPTile;
-        mq = P.maps + kMapsPerUnit * (size_t)r.unit + 1; mb = mq + 1;
-        Kin = P.Ktab[r.unit]; Vin = P.Vtab[r.unit];
+        kv_in = P.htab[head].kv_in;
+        mq = P.maps + kMapsPerUnit * (size_t)P.htab[head].unit + 1; mb = mq + 1;
     }
     const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
     const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
-    const int b0 = 8 * ts, nbs = min(8 * te, nb) - b0;                                          // and their blocks
-    auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kTE) : "memory"); };
+    const int b0 = 8 * ts, nbs = min(8 * te, nb) - b0, nw = (nbs + 31) >> 5;                    // their blocks, as words of 32
     auto cluster_sync = [&]() {
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
     auto sync_all = [&]() { if (C == 1) __syncthreads(); else cluster_sync(); };   // all warps of the head's CTAs
-    // epilogue threads: exclusive scan of one int per thread, and the sum
-    auto scan = [&](int v, int &total) -> int {
-        int inc = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
-        if (lane == 31) ctl->scan[warp] = inc;
-        epi_sync();
-        const int s = lane < kEpi ? ctl->scan[lane] : 0;
-        total = __reduce_add_sync(0xffffffffu, s);
-        const int before = __reduce_add_sync(0xffffffffu, lane < warp ? s : 0);
-        epi_sync();
-        return before + inc - v;
-    };
-    // epilogue threads: the bin that holds the target-th entry from the top, over the histograms of `ctas` CTAs of the head
-    // -> ctl->bin, with the entry's rank in it and its population (without so many entries: bin 0)
-    auto find_bin = [&](const uint32_t *h, auto bins, uint32_t ctas, int target) {
-        constexpr int per = decltype(bins)::value / kTE;      // consecutive bins of a thread, from the top
-        const int at = decltype(bins)::value - per * (tid + 1);
-        int n[per] = {};
-        if (ctas == 1) {
-#pragma unroll
-            for (int i = 0; i < per; i += 2) { const uint2 v = *(const uint2 *)(h + at + i); n[i] = (int)v.x; n[i + 1] = (int)v.y; }
-        } else {
+    // counts of two bins, over all CTAs of the head
+    auto counts = [&](int i) -> uint2 {
+        if (C == 1) return *(const uint2 *)(hist + i);
+        uint2 s = make_uint2(0u, 0u);
 #pragma unroll 4
-            for (uint32_t d = 0; d < ctas; ++d)
-#pragma unroll
-                for (int i = 0; i < per; i += 2) {
-                    const uint2 v = remote_ld2(remote(h + at + i, d));
-                    n[i] += (int)v.x; n[i + 1] += (int)v.y;
-                }
-        }
-        int sum = 0, total;
-#pragma unroll
-        for (int i = 0; i < per; ++i) sum += n[i];
-        if (tid == 0) { ctl->bin = 0; ctl->rank = 1; ctl->count = 0; }
-        int above = scan(sum, total);
-#pragma unroll
-        for (int i = per - 1; i >= 0; --i) {
-            if (above < target && target <= above + n[i]) { ctl->bin = at + i; ctl->rank = target - above; ctl->count = n[i]; }
-            above += n[i];
-        }
-        epi_sync();
+        for (uint32_t d = 0; d < C; ++d) { const uint2 v = remote_ld2(remote(hist + i, d)); s.x += v.x; s.y += v.y; }
+        return s;
     };
-    // epilogue threads: the set bits of words[] counted per word and before each word; returns how many there are.  (A word a thread.)
-    const int nw = (nbs + 31) >> 5;
-    auto count_words = [&]() -> int {
-        int total;
-        const int base = scan(tid < nw ? __popc(words[tid]) : 0, total);
-        if (tid < nw) wbase[tid] = base;
-        epi_sync();
-        return total;
-    };
-    struct Bins { enum { value = kCBins }; };
-    struct SelBins { enum { value = kCSelBins }; };
 
     uint32_t st = 0, ph = 0, u = 0;                           // K ring and its phase; tiles so far
     uint32_t lo16 = 0u, hi16 = 0u;                            // the blocks of a round: bounds in [lo16, hi16)
-    uint32_t cut = 0u;                                        // in the end: blocks with bounds from here on have been scored
-    // the maxima of the CTA's tiles go through the stages of the ring, as many tiles as fit
-    const uint32_t tile_bytes = (uint32_t)Rpad * 16;
-    const int per_stage = (int)(kPStage / tile_bytes), nchunks = (te - ts + per_stage - 1) / per_stage;
-
     if (warp == kEpi) {
         if (lane == 0) {
             if (P.maps) { tensormap_acquire(mq); tensormap_acquire(mb); }
             mbar_expect_tx(&ctl->q_full, q_bytes);
             tma_load_3d(qbuf, mq, &ctl->q_full, 0, 0, kv_in);
             tma_load_3d(qbuf + q_bytes / 2, mq, &ctl->q_full, 64, 0, kv_in);
-            int s = 0, round = 0;
-#pragma unroll 1
-            for (int j = 0; j < nchunks; ++j) {
-                if (round > 0 && !mbar_wait(&ctl->b_empty[s], (round - 1) & 1, &ctl->abort_flag, status, 64)) break;
-                const int t = ts + j * per_stage, cnt = min(per_stage, te - t);
-                mbar_expect_tx(&ctl->b_full[s], (uint32_t)cnt * tile_bytes);
-                if (JQ_IN((tbase + t + cnt) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 6))
-                    bulk_load(kbuf + (size_t)s * kPStage, P.bmax + (tbase + t) * 4 * Rpad, (uint32_t)cnt * tile_bytes, &ctl->b_full[s]);
-                if (++s == P.stages) { s = 0; ++round; }
-            }
         }
         __syncwarp();
         if (P.maps) tensormap_acquire(mb);                    // (all lanes load)
     } else if (warp < kEpi) {
-        // ---- the normalisers: the CTAs of row_stats that had tiles of this head, each with a pair per row and group
-        {
-            const long long T = P.T, G = P.sms;
-            const long long c_lo = ((tbase + 1) * G - 1) / T, c_hi = ((tbase + tph1) * G - 1) / T;   // owners of the first and last tile
-            const int nsl = (int)(c_hi - c_lo + 1) * P.groups;
-            const long long s0 = (c_lo + head) * P.groups;
-            const int row = tid & (kWide ? 255 : 127), sub = tid >> (kWide ? 8 : 7);          // two threads per row
-            const float2 *src = P.part + s0 * R + row;
-            float m = -INFINITY, l = 0.f;
-            if (row < R) {
-#pragma unroll 1
-                for (int i0 = sub; i0 < nsl; i0 += 16) {
-                    float2 p[8];
-                    float mn = m;
+        for (int i = tid; i < kMaxR; i += kTE) ctl->Ms[i] = __ldcg(P.Ms + (size_t)head * kMaxR + i);
+        const uint16_t *const src = P.ub + (size_t)(at.tbase + ts) * 8;
+        for (int t = tid; t < te - ts; t += kTE) {
+            const uint4 v = __ldcg((const uint4 *)src + t);
+            if (!JQ_IN(t, P.share, kDbgPrune, 7)) continue;
+            ((uint4 *)ub)[t] = v;
+            const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int i = i0 + 2 * k;
-                        p[k] = i < nsl && JQ_IN((s0 + i) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)i * R) : make_float2(-INFINITY, 0.f);
-                        if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
-                    }
-                    if (mn > -INFINITY) {
-                        l *= ex2(P.c * (m - mn));
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) if (p[k].y > 0.f) l = fmaf(p[k].y, ex2(P.c * (p[k].x - mn)), l);
-                        m = mn;
-                    }
-                }
-            }
-            float2 *const other = (float2 *)&ctl->xs[0][0][0];
-            static_assert(sizeof(ctl->xs) >= kMaxR * sizeof(float2), "room for a pair per row");
-            if (sub == 1) other[row] = make_float2(m, l);
-            epi_sync();
-            if (sub == 0) {
-                const float2 o = other[row];
-                float M = INFINITY;                           // silences a column that is not a query row
-                if (row < R) {
-                    const float mn = fmaxf(m, o.x);
-                    l = (l > 0.f ? l * ex2(P.c * (m - mn)) : 0.f) + (o.y > 0.f ? o.y * ex2(P.c * (o.x - mn)) : 0.f);
-                    M = fmaf(P.c, mn, log2f(l));
-                    if (!(fabsf(M) < 60000.f)) ctl->huge = 1;
-                }
-                ctl->Ms[row] = -M;
-                if (!kWide) ctl->Ms[128 + row] = -INFINITY;
-            }
-            epi_sync();
-        }
-        // ---- the bounds.  A lane takes four neighbouring rows (eight with more than 128) of four blocks.  A maximum x within 64 of
-        // its row's normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60
-        // each, which is added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
-        {
-            constexpr int kV = kWide ? 2 : 1;
-            float2 nm[4 * kV];
-#pragma unroll
-            for (int i = 0; i < 4 * kV; ++i) {
-                const float x = ctl->Ms[(i >> 2) * 128 + 4 * lane + (i & 3)], y = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;
-                nm[i] = make_float2(y, y);
-            }
-            const float floor_ = ctl->huge ? INFINITY : 3e-16f;
-            int s = 0, round = 0;
-#pragma unroll 1
-            for (int j = 0; j < nchunks; ++j) {
-                if (!__all_sync(0xffffffffu, mbar_wait(&ctl->b_full[s], round & 1, &ctl->abort_flag, status, 32))) break;
-                const int t = j * per_stage, cnt = min(per_stage, te - ts - t);
-#pragma unroll 1
-                for (int x = warp; x < 2 * cnt; x += kEpi) {
-                    const uint4 *const src = (const uint4 *)(kbuf + (size_t)s * kPStage + (size_t)x * (tile_bytes / 2));
-                    uint4 v[2][kV];
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-#pragma unroll
-                        for (int y = 0; y < kV; ++y)          // (a row that is none has a normaliser of inf)
-                            v[q][y] = y * 128 + 4 * lane < Rpad ? src[(q * Rpad + y * 128) / 4 + lane] : make_uint4(0u, 0u, 0u, 0u);
-                    float2 sum[2];
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        sum[q] = make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int y = 0; y < kV; ++y) {
-                            const uint32_t e[4] = {v[q][y].x, v[q][y].y, v[q][y].z, v[q][y].w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const float2 f = __fadd2_rn(__half22float2(*(const __half2 *)&e[i]), nm[4 * y + i]);
-                                sum[q] = __fadd2_rn(sum[q], make_float2(ex2(f.x), ex2(f.y)));
-                            }
-                        }
-                    }
-                    // four sums over the 32 lanes: after two exchanges of halves a lane holds one block's part
-                    const bool h4 = lane & 16, h3 = lane & 8;
-                    const float p0 = (h4 ? sum[1].x : sum[0].x) + __shfl_xor_sync(0xffffffffu, h4 ? sum[0].x : sum[1].x, 16);
-                    const float p1 = (h4 ? sum[1].y : sum[0].y) + __shfl_xor_sync(0xffffffffu, h4 ? sum[0].y : sum[1].y, 16);
-                    float r = (h3 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h3 ? p0 : p1, 8);
-                    r += __shfl_xor_sync(0xffffffffu, r, 4);
-                    r += __shfl_xor_sync(0xffffffffu, r, 2);
-                    r += __shfl_xor_sync(0xffffffffu, r, 1);
-                    const int blk = 8 * t + 4 * x + (h4 ? 2 : 0) + (h3 ? 1 : 0);
-                    if ((lane & 7) == 0 && blk < nbs && JQ_IN(blk, 8 * P.share, kDbgPrune, 7)) {
-                        const uint32_t y = (__float_as_uint((r + floor_) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16;
-                        ub[blk] = (uint16_t)y;
-                        atomicAdd(&hist[bin_of(y)], 1u);
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->b_empty[s], 1);
-                if (++s == P.stages) { s = 0; ++round; }
-            }
+            for (int e = 0; e < 8; ++e) if (8 * t + e < nbs) atomicAdd(&hist[bin_of(x[e >> 1] >> (16 * (e & 1)) & 0xffffu)], 1u);
         }
     }
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -706,19 +736,20 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     for (int round = 0; round < 2; ++round) {
         // ---- the blocks of this round: [lo16, hi16) of the bounds
         if (warp < kEpi) {
-            find_bin(hist, Bins(), C, round == 0 ? wanted : nkeep);
-            const uint32_t edge = edge_of(ctl->bin);
+            const uint32_t edge = edge_of(find_bin<kTE, kCBins>(counts, round == 0 ? wanted : nkeep, &ctl->found, ctl->sums).bin);
             if (round == 0) { lo16 = edge; hi16 = 0x10000u; }
             else { hi16 = lo16; lo16 = min(edge, lo16); }
-            cut = lo16;
             // this CTA's share of them, and their places in the head's list
             for (int w = warp; w < nw; w += kEpi) {
                 const int i = 32 * w + lane;
                 const uint32_t x = i < nbs ? ub[i] : 0x10000u, m = __ballot_sync(0xffffffffu, x >= lo16 && x < hi16);
                 if (lane == 0) words[w] = m;
             }
-            epi_sync();
-            const int total = count_words();
+            named_sync<kTE>();
+            int total;
+            const int base = scan_threads<kTE>(tid < nw ? __popc(words[tid]) : 0, total, ctl->sums);
+            if (tid < nw) wbase[tid] = base;
+            named_sync<kTE>();
             int before = 0, per_cta = 0x40000000;
             if (C > 1) {
                 if (warp == 0 && lane < (int)C) remote_st(remote(&ctl->cnt[rank], lane), total);
@@ -732,7 +763,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
             for (int w = warp; w < nw; w += kEpi) {
                 const uint32_t m = words[w];
                 if ((m >> lane & 1u) == 0u) continue;
-                const int at = before + wbase[w] + __popc(m & ((1u << lane) - 1u)), to = C > 1 ? at / per_cta : 0, x = at - to * per_cta;
+                const int i = before + wbase[w] + __popc(m & ((1u << lane) - 1u)), to = C > 1 ? i / per_cta : 0, x = i - to * per_cta;
                 if (!JQ_IN(x, 8 * P.share, kDbgPrune, 8) || !JQ_IN(to, C, kDbgPrune, 9)) continue;
                 if (C > 1) remote_st16(remote(list + x, (uint32_t)to), (uint16_t)(b0 + 32 * w + lane));
                 else list[x] = (uint16_t)(32 * w + lane);
@@ -742,16 +773,9 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         sync_all();
         const int n = ctl->n, nt = (n + 7) >> 3;
         if (warp == kEpi) {
-            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, two lanes each.  The ring
-            // holds two or three tiles, too few for a read from HBM: the blocks are asked for ahead, into the L2.
-            int ahead = 0;
+            // ------------------------------------------------------------ TMA producer: up to eight blocks to a tile, two lanes each
 #pragma unroll 1
             for (int i = 0; i < nt; ++i) {
-                for (; ahead < min(n, 8 * i + kCAhead); ahead += 16) {
-                    const int x = ahead + (lane >> 1);
-                    if (x < n) prefetch_3d(mb, 64 * (lane & 1), list[x] * kPBlock, kv_in);
-                }
-                __syncwarp();
                 const int have = min(8, n - 8 * i);
                 if (!__all_sync(0xffffffffu, mbar_wait(&ctl->empty[st], ph ^ 1, &ctl->abort_flag, status, 64))) break;
                 if (lane == 0) mbar_expect_tx(&ctl->full[st], (uint32_t)have * 2u * kPBlockHalf);
@@ -824,7 +848,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
                 }
                 const int x = 8 * i + (row0 >> 4), blk = x < n ? list[x] : nb, key = blk * kPBlock + (row0 & 15);
                 const bool have = x < n && key < L;
-                if (have && JQ_IN(soff + key, P.ext.scores, kDbgPrune, 13)) P.scores[soff + key] = sum;
+                if (have && JQ_IN(at.soff + key, P.ext.scores, kDbgPrune, 13)) P.scores[at.soff + key] = sum;
                 if (round == 0) {
                     // what this block alone guarantees of the pooled scores of its positions
                     float m = have ? sum : 0.f;
@@ -853,52 +877,112 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
 
-    if (C > 1) {
-        // the selection is a kernel of its own, over all positions of the head: what has not been scored counts as zero
-        float *const s = P.scores + soff + (long long)b0 * kPBlock;
+    if (tid == 0 && rank == 0) P.cut[head] = lo16;
+    if (P.fill) {                                             // what nothing needs counts as zero
+        float *const s = P.scores + at.soff + (long long)b0 * kPBlock;
         const int m = min(nbs * kPBlock, L - b0 * kPBlock);
         for (int i = tid; i < m; i += kTE)
-            if (ub[i >> 4] < cut && JQ_IN(soff + (long long)b0 * kPBlock + i, P.ext.scores, kDbgPrune, 14)) s[i] = 0.f;
-        return;
+            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.ext.scores, kDbgPrune, 14)) s[i] = 0.f;
     }
-    // ---------------------------------------------------------------- selection (one CTA, the epilogue warps), among the positions of the
-    // active blocks: those that are scored and those that a window reaches from there.  What is not scored counts as zero: its
-    // scores lie below the threshold, and so does every pooled score that they alone would make.  Laid one after the other, the
-    // active blocks can be pooled as if they were neighbours: between two of them that are not lies a whole reach of zeros.
-    // (Whatever the scores are, after a wait that ran out too, every place that follows is brought into range.)
-    const int reach = (P.radius + kPBlock - 1) / kPBlock;    // blocks that a window reaches into on either side: 0, 1 or 2
-    uint32_t *const bins = (uint32_t *)smem_raw;             // in the place of queries and stages: [kCSelBins],
-    uint32_t *const cand = bins + kCSelBins;                 // [kCRank],
-    float *const sc = (float *)(cand + kCRank) + 32;         // [16 room] scores, then keys, with 32 zeros on either side
-    const int room = (int)(((uint8_t *)ctl - (uint8_t *)(sc + 32)) / 64);
-    uint16_t *const act = list;                              // the active blocks, in order
+}
+
+// ------------------------------------------------------------------ selection among the candidates, many heads
+
+constexpr int kCSelBins = 2048;                  // bins, equal parts of a range of keys
+constexpr int kCList = 1024;                     // keys of one bin that are finished on a list of them
+constexpr int kCRank = 64;                       // of which so many are ranked by comparison
+constexpr int kCSelThreads = 256, kCSelWarps = kCSelThreads / 32;
+
+struct SCtl2 {
+    BinAt found;
+    int sums[kCSelWarps];
+    int ncand, need;
+    uint32_t tau;
+    uint32_t wmin[kCSelWarps], wmax[kCSelWarps];
+};
+// Shared memory behind the control block: bins, list, words of blocks and their counts, active blocks, scores (then keys).
+__host__ __device__ constexpr size_t sel_fixed(int words) { return (size_t)(kCSelBins + kCList) * 4 + ((size_t)words * 8 + 15) / 16 * 16 + (size_t)words * 64 + 256; }
+
+// grid: a CTA per head.  Only the positions of the active blocks take part: those of the blocks that are scored and of those that a
+// window reaches from there.  What is not scored counts as zero: its scores lie below the threshold, and so does every pooled
+// score that they alone would make.  Laid one after the other, the active blocks can be pooled as if they were neighbours:
+// between two of them that are not lies a whole reach of zeros.  (Whatever the scores are, after a wait that ran out too, every
+// place that follows is brought into range.)
+__global__ void __launch_bounds__(kCSelThreads, 3)
+select_candidates(const __grid_constant__ CParams P)
+{
+    constexpr int kTE = kCSelThreads;
+    extern __shared__ __align__(16) uint8_t sel_raw[];
+    __shared__ SCtl2 ctl;
+    const int head = (int)blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+#ifdef JQ_DEBUG
+    DebugRecord *const dbg = P.dbg_rec;
+#endif
+    uint32_t *const bins = (uint32_t *)sel_raw, *const cand = bins + kCSelBins, *const words = cand + kCList;
+    int *const wbase = (int *)(words + P.max_words);
+    uint16_t *const act = (uint16_t *)(sel_raw + (size_t)(kCSelBins + kCList) * 4 + ((size_t)P.max_words * 8 + 15) / 16 * 16);   // [32 max_words]
+    float *const sc = (float *)(act + 32 * P.max_words) + 32;                    // [16 room] with 32 zeros on either side
+    const int room = P.room;
     for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
-    if (tid == 0) ctl->ncand = 0;
-    for (int w = warp; w < nw; w += kEpi) {
+    if (tid == 0) ctl.ncand = 0;
+    cudaGridDependencySynchronize();             // nothing in global memory has been touched so far
+    cudaTriggerProgrammaticLaunchCompletion();
+    const HeadAt at = head_at(P, head);
+    const int L = at.L, nkeep = at.nkeep, nb = (L + kPBlock - 1) / kPBlock, nw = (nb + 31) >> 5;
+    const long long soff = at.soff;
+    int kv_in = head, src_rows = P.src_rows;
+    long long orow = (long long)head * nkeep, krow = (long long)head * P.out_rows;   // first rows of the head's indices and of its compacted rows
+    const uint4 *Kin = P.K, *Vin = P.V;
+    if (P.htab) {
+        const HeadRec r = P.htab[head];
+        kv_in = r.kv_in; orow = krow = r.ooff; src_rows = L;
+        Kin = P.Ktab[r.unit]; Vin = P.Vtab[r.unit];
+    }
+    auto sync = [&]() { named_sync<kTE>(); };
+    // ---- the scored blocks as bits, widened by the reach of a window, and the list of them
+    const uint32_t cut = __ldcg(P.cut + head);
+    const uint16_t *const ub = P.ub + (size_t)at.tbase * 8;
+    for (int w = warp; w < nw; w += kCSelWarps) {
         const int i = 32 * w + lane;
-        const uint32_t m = __ballot_sync(0xffffffffu, i < nbs && ub[i] >= cut);
+        const uint32_t m = __ballot_sync(0xffffffffu, i < nb && __ldcg(ub + i) >= cut);
         if (lane == 0) words[w] = m;
     }
-    epi_sync();
+    sync();
+    const int reach = (P.radius + kPBlock - 1) / kPBlock;    // blocks that a window reaches into on either side: 0, 1 or 2
+    int n_act;
     {
-        uint32_t m = 0u;
-        if (tid < nw) {
-            const uint32_t p = tid > 0 ? words[tid - 1] : 0u, q = words[tid], r = tid + 1 < nw ? words[tid + 1] : 0u;
-            m = q;
-            for (int d = 1; d <= reach; ++d) m |= q << d | q >> d | p >> (32 - d) | r << (32 - d);
-            if (tid == nw - 1 && (nbs & 31)) m &= (1u << (nbs & 31)) - 1u;
+        constexpr int kMost = (kCMaxBlocks / 32 + kTE) / kTE;         // words per thread, consecutive
+        const int per = (nw + kTE - 1) / kTE;
+        uint32_t m[kMost];
+        int mine = 0;
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            const int w = tid * per + k;
+            m[k] = 0u;
+            if (k >= per || w >= nw) continue;
+            const uint32_t p = w > 0 ? words[w - 1] : 0u, q = words[w], r = w + 1 < nw ? words[w + 1] : 0u;
+            m[k] = q;
+            for (int d = 1; d <= reach; ++d) m[k] |= q << d | q >> d | p >> (32 - d) | r << (32 - d);
+            if (w == nw - 1 && (nb & 31)) m[k] &= (1u << (nb & 31)) - 1u;
+            mine += __popc(m[k]);
         }
-        epi_sync();
-        if (tid < nw) words[tid] = m;
+        int base = scan_threads<kTE>(mine, n_act, ctl.sums);          // (its barriers part the reads of words[] from the writes)
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            const int w = tid * per + k;
+            if (k >= per || w >= nw) continue;
+            words[w] = m[k]; wbase[w] = base;
+            base += __popc(m[k]);
+        }
     }
-    const int n_act = count_words();
-    for (int w = warp; w < nw; w += kEpi) {
+    sync();
+    for (int w = warp; w < nw; w += kCSelWarps) {
         const uint32_t m = words[w];
-        const int at = wbase[w] + __popc(m & ((1u << lane) - 1u));
-        if ((m >> lane & 1u) && JQ_IN(at, 8 * P.share, kDbgPrune, 15)) act[at] = (uint16_t)(32 * w + lane);
+        const int x = wbase[w] + __popc(m & ((1u << lane) - 1u));
+        if ((m >> lane & 1u) && JQ_IN(x, 32 * P.max_words, kDbgPrune, 15)) act[x] = (uint16_t)(32 * w + lane);
     }
-    epi_sync();
-    auto block_of = [&](int a) -> int { return min((int)act[a], nbs - 1); };
+    sync();
+    auto block_of = [&](int a) -> int { return min((int)act[a], nb - 1); };
     // The keys stay on chip, in the place of the scores that they are made of, or (more than there is room for, or a window
     // that reaches past the next quad) go to memory a chunk at a time.  A key is one above the bits of a pooled score, which is
     // not negative: order and ties are those of the values.  Positions that do not exist have the key 0.
@@ -916,7 +1000,8 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int x = a + e * (kTE / 16), blk = x < f1 ? block_of(x) : 0, pos = blk * kPBlock + i16;
-                v[e] = x < f1 && pos < L && ub[blk] >= cut && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 16) ? __ldcg(P.scores + soff + pos) : 0.f;
+                const bool in = x < f1 && pos < L && __ldcg(ub + blk) >= cut;
+                v[e] = in && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 16) ? __ldcg(P.scores + soff + pos) : 0.f;
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -926,11 +1011,11 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         }
         if (tid < 32) sc[tid - 32] = 0.f;
         else if (tid < 64) sc[(f1 - f0) * 16 + tid - 32] = 0.f;
-        epi_sync();
+        sync();
         const int nq = 4 * (c1 - c0), NQ = ((nq + kTE - 1) / kTE) | 1, q0 = min(tid * NQ, nq), q1 = min(q0 + NQ, nq), shift = 4 * (c0 - f0);
         float4 *const s4 = (float4 *)sc + shift;
         float4 before = s4[q0 - 1], last = s4[q1], here = s4[q0];
-        if (on_chip) epi_sync();                                     // (everybody has the quads next to his own)
+        if (on_chip) sync();                                         // (everybody has the quads next to his own)
 #pragma unroll 1
         for (int q = q0; q < q1; ++q) {
             float best[4];
@@ -963,7 +1048,7 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
                     if (k[e] && JQ_IN(soff + 16 * c0 + 4 * q + e, P.ext.scores, kDbgPrune, 18)) gk[16 * c0 + 4 * q + e] = k[e];
             }
         }
-        epi_sync();
+        sync();
     }
     // A thread owns NQ consecutive quads from here on: the max-pool's plateaus then mostly fall within a thread, and thread order is
     // position order.
@@ -980,41 +1065,52 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     };
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
-    if (lane == 0) { ctl->wmin[warp] = kmin; ctl->wmax[warp] = kmax; }
-    epi_sync();
-    kmin = __reduce_min_sync(0xffffffffu, ctl->wmin[lane % kEpi]);
-    kmax = __reduce_max_sync(0xffffffffu, ctl->wmax[lane % kEpi]);
-    // The threshold key: 2048 equal bins over the keys' own range, then the bin's few keys ranked by comparison, or binned again
-    // while they are many.
-    uint32_t lo = kmin, lim = kmax - kmin, tau;
+    if (lane == 0) { ctl.wmin[warp] = kmin; ctl.wmax[warp] = kmax; }
+    sync();
+    kmin = __reduce_min_sync(0xffffffffu, ctl.wmin[lane % kCSelWarps]);
+    kmax = __reduce_max_sync(0xffffffffu, ctl.wmax[lane % kCSelWarps]);
+    // The threshold key: 2048 equal bins over the keys' own range; the bin's keys, once they fit a list, are ranked by comparison or
+    // binned again.
+    uint32_t lo = kmin, lim = kmax - kmin;
     int need = nkeep;
+    bool listed = false;
+    int count = 0;
+    auto bin_counts = [&](int i) -> uint2 { return *(const uint2 *)(bins + i); };
 #pragma unroll 1
     for (;;) {
         const int sh = lim >> 11 ? 21 - __clz(lim) : 0;               // lim >> sh < 2048
-        uint32_t cur = 0u, cnt = 0u;
-#pragma unroll 1
-        for (int q = q0; q < q1; ++q) {
-            uint32_t k[4];
-            keys_of(q, k);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {                             // neighbours often share the bin: runs as one count
-                const uint32_t d = k[e] - lo;
-                const bool in = k[e] != 0u && d <= lim, other = in && d >> sh != cur;
-                if (other && cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
-                cnt = other ? 1u : cnt + in;
-                cur = other ? d >> sh : cur;
+        if (listed) {
+            for (int i = tid; i < count; i += kTE) {
+                const uint32_t d = cand[i] - lo;
+                if (d <= lim) atomicAdd(&bins[(d >> sh) & (kCSelBins - 1)], 1u);
             }
+        } else {
+            uint32_t cur = 0u, cnt = 0u;
+#pragma unroll 1
+            for (int q = q0; q < q1; ++q) {
+                uint32_t k[4];
+                keys_of(q, k);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {                         // neighbours often share the bin: runs as one count
+                    const uint32_t d = k[e] - lo;
+                    const bool in = k[e] != 0u && d <= lim, other = in && d >> sh != cur;
+                    if (other && cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
+                    cnt = other ? 1u : cnt + in;
+                    cur = other ? d >> sh : cur;
+                }
+            }
+            if (cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
         }
-        if (cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
-        epi_sync();
-        find_bin(bins, SelBins(), 1, need);
-        lo += (uint32_t)ctl->bin << sh;
-        need = ctl->rank;
-        const int count = ctl->count;
-        tau = lo;
+        sync();
+        const BinAt b = find_bin<kTE, kCSelBins>(bin_counts, need, &ctl.found, ctl.sums);
+        lo += (uint32_t)b.bin << sh;
+        need = b.rank;
         if (sh == 0) break;
         lim = (1u << sh) - 1u;
-        if (count <= kCRank) {
+        for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
+        if (!listed && b.count <= kCList) {
+            listed = true;
+            count = b.count;
 #pragma unroll 1
             for (int q = q0; q < q1; ++q) {
                 uint32_t k[4];
@@ -1022,28 +1118,28 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (k[e] != 0u && k[e] - lo <= lim) {
-                        const int at = atomicAdd(&ctl->ncand, 1);
-                        if (at < kCRank) cand[at] = k[e];
+                        const int x = atomicAdd(&ctl.ncand, 1);
+                        if (x < kCList) cand[x] = k[e];
                     }
             }
-            epi_sync();
-            if (tid == 0) { ctl->tau = lo; ctl->need = need; }
-            epi_sync();
-            for (int i = tid; i < count; i += kTE) {
-                const uint32_t k = cand[i];
-                int gt = 0, eq = 0;
+            if (tid == 0) { ctl.tau = lo; ctl.need = need; }
+            sync();
+            if (count <= kCRank) {
+                if (tid < count) {
+                    const uint32_t k = cand[tid];
+                    int gt = 0, eq = 0;
 #pragma unroll 4
-                for (int x = 0; x < count; ++x) { const uint32_t y = cand[x]; gt += y > k; eq += y == k; }
-                if (gt < need && need <= gt + eq) { ctl->tau = k; ctl->need = need - gt; }   // (equal keys write the same)
+                    for (int x = 0; x < count; ++x) { const uint32_t y = cand[x]; gt += y > k; eq += y == k; }
+                    if (gt < need && need <= gt + eq) { ctl.tau = k; ctl.need = need - gt; }   // (equal keys write the same)
+                }
+                sync();
+                lo = ctl.tau;
+                need = ctl.need;
+                break;
             }
-            epi_sync();
-            tau = ctl->tau;
-            need = ctl->need;
-            break;
-        }
-        for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
-        epi_sync();
+        } else sync();
     }
+    const uint32_t tau = lo;
     // Kept: all keys above tau and, of those equal to it, the first `need`.
     int gt = 0, eq = 0;
 #pragma unroll 1
@@ -1054,8 +1150,8 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         for (int e = 0; e < 4; ++e) { gt += k[e] > tau; eq += k[e] == tau && k[e] != 0u; }
     }
     int all;
-    gt = scan(gt, all);
-    eq = scan(eq, all);
+    gt = scan_threads<kTE>(gt, all, ctl.sums);
+    eq = scan_threads<kTE>(eq, all, ctl.sums);
     int32_t *const out = P.idx + orow;
 #pragma unroll 1
     for (int q = q0; q < q1; ++q) {
@@ -1072,8 +1168,8 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
             eq += same;
         }
     }
-    // ---------------------------------------------------------------- the rows, once every index of the head has been written
-    epi_sync();
+    // ---- the rows, once every index of the head has been written
+    sync();
     copy_rows(tid, kTE, out, 0, nkeep, kv_in, krow, L, Kin, Vin, P.Kout, P.Vout, src_rows, P.ext JQ_DBG_ARG_DEV);
     if (P.win.w) copy_window(P.win, head, krow + nkeep, tid >> 4, kTE / 16, P.Kout, P.Vout, P.ext JQ_DBG_ARG_DEV);
 }
@@ -1083,6 +1179,8 @@ evict_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
 constexpr size_t stats_smem(int Rbox, int stages) { return 2 * (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kSCtlBytes; }
 size_t cand_smem(int Rbox, int stages, int share) { return (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kCCtlBytes + kCBins * 4 + (size_t)share * 32 + (size_t)(share / 4 + 1) * 8; }
 constexpr size_t kCMaxSmem = 227 * 1024, kCTwoPerSm = 113 * 1024;
+constexpr size_t kCSelSmem = 74 * 1024, kCSelMaxSmem = 200 * 1024;   // three CTAs of select_candidates to an SM, and the most that one is given
+constexpr int kCSelMinHeads = 128;                // from here on a CTA per head selects (fewer heads: a cluster each)
 
 struct PruneDevice {
     int sms = 0;
@@ -1104,7 +1202,7 @@ bool prune_device(PruneDevice *out)
         for (auto k : {row_stats<kSGroupsNarrow>, row_stats<kSGroupsWide>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess) return false;
         for (int wide = 0; wide < 2; ++wide) {
-            const auto k = wide ? evict_candidates<true> : evict_candidates<false>;
+            const auto k = wide ? score_candidates<true> : score_candidates<false>;
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess ||
                 cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
             for (int C = 1; C <= kCMaxCluster; ++C) {
@@ -1120,19 +1218,50 @@ bool prune_device(PruneDevice *out)
                 if (cudaOccupancyMaxActiveClusters(&d.resident[wide][C], k, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[wide][C] = 0; }
             }
         }
+        if (cudaFuncSetAttribute(select_candidates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCSelMaxSmem) != cudaSuccess) return false;
         d.ready = true;
     }
     *out = d;
     return true;
 }
 
-}  // namespace
-
-size_t prune_bytes(long long tiles, int heads, int R)
+// The scratch: maxima, partial statistics, normalisers, bounds, cuts.
+struct PruneScratch { size_t part, Ms, ub, cut, bytes; };
+PruneScratch prune_layout(long long tiles, int heads, int R)
 {
     const int Rpad = (R + 31) & ~31, groups = R > 128 ? kSGroupsWide : kSGroupsNarrow;
-    return align_up((size_t)tiles * 4 * Rpad * 4, 256) + align_up((size_t)(heads + 256) * groups * R * sizeof(float2), 256);
+    PruneScratch s;
+    s.part = align_up((size_t)tiles * 4 * Rpad * 4, 256);
+    s.Ms = s.part + align_up((size_t)(heads + 256) * groups * R * sizeof(float2), 256);
+    s.ub = s.Ms + align_up((size_t)heads * kMaxR * 4, 256);
+    s.cut = s.ub + align_up((size_t)tiles * 16, 256);
+    s.bytes = s.cut + align_up((size_t)heads * 4, 256);
+    return s;
 }
+
+template <typename... A>
+bool launch(void (*kernel)(A...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return false; }
+    count_launch(1);
+    return true;
+}
+
+}  // namespace
+
+size_t prune_bytes(long long tiles, int heads, int R) { return prune_layout(tiles, heads, R).bytes; }
 
 // Whether a call takes this way.  tiles: of all heads; keys: sum of the heads' lengths; kept: sum of what the heads keep.
 bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L)
@@ -1159,7 +1288,9 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     S.T = T; S.heads = s.Hkv; S.hpu = tables ? tables->hpu : s.Hkv;
     S.c = 1.4426950408889634f / sqrtf((float)s.d);
     S.bmax = (uint32_t *)w.prune;
-    S.part = (float2 *)((char *)w.prune + align_up((size_t)T * 4 * Rpad * 4, 256));
+    const PruneScratch lay = prune_layout(T, s.Hkv, R);
+    char *const scratch = (char *)w.prune;
+    S.part = (float2 *)(scratch + lay.part);
     S.status = w.status;
     const int groups = wide ? kSGroupsWide : kSGroupsNarrow, grid = (int)(T < dev.sms ? T : dev.sms);
     CParams P = {};
@@ -1185,10 +1316,11 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     const size_t smem = cand_smem(Rbox, P.stages, P.share);
     if (smem > kCMaxSmem) return JQ_ERR_CUDA;   // (prune_taken's limit on the length keeps every call below)
     P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
-    P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
+    P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
     P.groups = groups; P.sms = grid;
     P.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
     P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.gkeys = w.keys; P.status = w.status;
+    P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub); P.cut = (uint32_t *)(scratch + lay.cut);
     P.htab = S.htab; P.maps = S.maps;
     P.idx = idx; P.K = (const uint4 *)K; P.V = (const uint4 *)V; P.Kout = (uint4 *)Kout; P.Vout = (uint4 *)Vout;
     if (tables) { P.Ktab = (const uint4 *const *)tables->K; P.Vtab = (const uint4 *const *)tables->V; }
@@ -1198,38 +1330,25 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     P.ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
     P.ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * P.out_rows;
     P.ext.src_heads = tables ? tables->hpu : s.Hkv;
+    const bool many = s.Hkv >= kCSelMinHeads;
+    P.fill = many ? 0 : 1;
+    P.max_words = (max_tph * 8 + 31) / 32;
+    size_t sel_smem = kCSelSmem;
+    while (sel_fixed(P.max_words) + 64 * 64 > sel_smem) sel_smem += 8 * 1024;
+    P.room = (int)((sel_smem - sel_fixed(P.max_words)) / 64);
 #ifdef JQ_DEBUG
     S.dbg_rec = P.dbg_rec = debug_record();
     if (!S.dbg_rec) return JQ_ERR_CUDA;
     S.n_bmax = P.n_bmax = T * 4 * Rpad;
     S.n_part = P.n_part = (long long)(s.Hkv + 256) * groups * R;
 #endif
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)stats_threads(groups));
-    cfg.dynamicSmemBytes = stats_smem(Rbox, S.stages);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, wide ? row_stats<kSGroupsWide> : row_stats<kSGroupsNarrow>, mapK, mapQ, mapW, S) != cudaSuccess) {
-        cudaGetLastError();
+    const unsigned bgrid = (unsigned)(T < (long long)kBPerSm * dev.sms ? T : kBPerSm * dev.sms);
+    if (!launch(wide ? row_stats<kSGroupsWide> : row_stats<kSGroupsNarrow>, (unsigned)grid, (unsigned)stats_threads(groups), stats_smem(Rbox, S.stages), st, 0, mapK, mapQ, mapW, S) ||
+        !launch(wide ? block_bounds<true> : block_bounds<false>, bgrid, (unsigned)kBThreads, 0, st, 0, P) ||
+        !launch(wide ? score_candidates<true> : score_candidates<false>, (unsigned)(s.Hkv * C), (unsigned)cand_threads(wide), smem, st, C, mapB, mapQ, P))
         return JQ_ERR_CUDA;
-    }
-    cfg.gridDim = dim3((unsigned)(s.Hkv * C));
-    cfg.blockDim = dim3((unsigned)cand_threads(wide));
-    cfg.dynamicSmemBytes = smem;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, wide ? evict_candidates<true> : evict_candidates<false>, mapB, mapQ, P) != cudaSuccess) {
-        cudaGetLastError();
-        return JQ_ERR_CUDA;
-    }
-    count_launch(2);
-    if (C > 1) return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
+    if (!many) return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
+    if (!launch(select_candidates, (unsigned)s.Hkv, (unsigned)kCSelThreads, sel_smem, st, 0, P)) return JQ_ERR_CUDA;
     return check_launch();
 }
 
