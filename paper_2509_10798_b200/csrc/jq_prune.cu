@@ -22,8 +22,7 @@
 // between the two orders of the product.
 #include "jq_sm100.cuh"
 #include "jq_tmem_ld.cuh"
-#include "jq_pool.cuh"
-#include "jq_rows.cuh"
+#include "jq_debug.cuh"
 #include <cstddef>
 #include <cstring>
 #include <cuda_fp16.h>
@@ -360,28 +359,17 @@ struct CParams {
     int groups, sms;           // row_stats' epilogue groups and its grid
     int stages, share;         // score_candidates: K ring; most tiles of a head that a CTA looks after
     int first_pct;             // blocks of round 1 per 100 pairs kept
-    int fill;                  // score_candidates writes zeros where it does not score (the selection reads every score)
-    int room;                  // select_candidates: active blocks whose keys stay on chip
-    int max_words;             // select_candidates: words of 32 blocks of the longest head
     long long T;
     float c;
     const float2 *part;
     const uint32_t *bmax;
     float *Ms;                 // [heads][kMaxR]: minus the row normalisers
     uint16_t *ub;              // [tile][8]: bounds of the blocks, upper 16 bits of a float
-    uint32_t *cut;             // [heads]: the blocks with bounds from here on have been scored
     float *scores;
-    uint32_t *gkeys;           // [keys of all heads]: the selection's keys where shared memory has no room for them
     int *status;
     const HeadRec *htab;
     const CUtensorMap *maps;
-    int32_t *idx;
-    const uint4 *K, *V;        // rows of 16 x 16 bytes
-    const uint4 *const *Ktab, *const *Vtab;
-    uint4 *Kout, *Vout;
-    int src_rows, out_rows;
-    WindowRows win;
-    SelExtents ext;
+    long long n_scores;        // floats in the scores array
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
     long long n_part, n_bmax;
@@ -459,21 +447,29 @@ __device__ __forceinline__ BinAt find_bin(Get get, int target, BinAt *res, int *
 
 // ------------------------------------------------------------------ bounds
 
-constexpr int kBThreads = 256, kBPerSm = 4;
+constexpr int kBThreads = 256, kBStages = 3;     // stages: tiles of a warp, two on their way while one is worked on
+__host__ __device__ constexpr int bounds_per_sm(bool wide) { return wide ? 2 : 4; }
+__host__ __device__ constexpr int bounds_smem(bool wide) { return kBThreads / 32 * kBStages * (wide ? 4096 : 2048); }
 
-// grid: four CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
+// grid: two or four CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
 // then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  A maximum x within 64 of its row's
 // normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60 each, which is
 // added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
 template <bool kWide>
-__global__ void __launch_bounds__(kBThreads, kBPerSm)
+__global__ void __launch_bounds__(kBThreads, bounds_per_sm(kWide))
 block_bounds(const __grid_constant__ CParams P)
 {
     __shared__ float Ms[kMaxR];
     __shared__ float2 other[kMaxR];
     __shared__ int huge;
+    extern __shared__ __align__(16) uint8_t bounds_raw[];
+    constexpr int kV = kWide ? 2 : 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int R = P.R, Rpad = P.Rpad;
+    // the warp's stages; a lane reads what it has copied itself, 16 bytes of four neighbouring rows (eight with more than 128) of
+    // two blocks at a time
+    uint4 *const ring = (uint4 *)bounds_raw + warp * kBStages * 4 * kV * 32 + lane;
+    for (int i = 0; i < kBStages * 4 * kV; ++i) ring[32 * i] = make_uint4(0u, 0u, 0u, 0u);   // (what is not copied: rows that are none)
 #ifdef JQ_DEBUG
     DebugRecord *const dbg = P.dbg_rec;
 #endif
@@ -495,6 +491,19 @@ block_bounds(const __grid_constant__ CParams P)
         const int t1 = (int)min((long long)tph, end - a.tbase);       // (the window tile has no bounds)
         f = a.tbase + a.tph1;
         if (tid == 0) huge = 0;
+        auto request = [&](int t, int stage) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int y = 0; y < kV; ++y) {
+                    const long long at = ((a.tbase + t) * 4 + q) * Rpad + y * 128 + 4 * lane;
+                    if (t < t1 && y * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6))
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(ring + 32 * ((stage * 4 + q) * kV + y))), "l"(P.bmax + at) : "memory");
+                }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        request(t0 + warp, 0);
+        request(t0 + warp + kBThreads / 32, 1);
         {   // the CTAs of row_stats that had tiles of this head, each with a pair per row and group: eight loads in flight
             const long long c_lo = ((a.tbase + 1) * P.sms - 1) / P.T, c_hi = ((a.tbase + a.tph1) * P.sms - 1) / P.T;   // owners of the first and last tile
             const int nsl = (int)(c_hi - c_lo + 1) * P.groups;
@@ -542,8 +551,6 @@ block_bounds(const __grid_constant__ CParams P)
             }
             __syncthreads();
         }
-        // a lane takes four neighbouring rows (eight with more than 128)
-        constexpr int kV = kWide ? 2 : 1;
         float nm[4 * kV];
 #pragma unroll
         for (int i = 0; i < 4 * kV; ++i) {
@@ -551,24 +558,19 @@ block_bounds(const __grid_constant__ CParams P)
             nm[i] = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;
         }
         const float least = huge ? INFINITY : 3e-16f;
+        int stage = 0;
 #pragma unroll 1
         for (int t = t0 + warp; t < t1; t += kBThreads / 32) {
-            uint4 v[4][kV];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int y = 0; y < kV; ++y) {                        // (a row that is none has a normaliser of inf)
-                    const long long at = ((a.tbase + t) * 4 + q) * Rpad + y * 128 + 4 * lane;
-                    const bool in = y * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6);
-                    v[q][y] = in ? __ldcs((const uint4 *)(P.bmax + at)) : make_uint4(0u, 0u, 0u, 0u);
-                }
+            request(t + 2 * (kBThreads / 32), stage == 0 ? 2 : stage - 1);
+            asm volatile("cp.async.wait_group 2;" ::: "memory");
             float2 sum[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 sum[q] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int y = 0; y < kV; ++y) {
-                    const uint32_t e[4] = {v[q][y].x, v[q][y].y, v[q][y].z, v[q][y].w};
+                    const uint4 v = ring[32 * ((stage * 4 + q) * kV + y)];
+                    const uint32_t e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float2 g = __fadd2_rn(__half22float2(*(const __half2 *)&e[i]), make_float2(nm[4 * y + i], nm[4 * y + i]));
@@ -592,7 +594,9 @@ block_bounds(const __grid_constant__ CParams P)
             const int blk = (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
             if ((lane & 3) == 0)
                 P.ub[(size_t)(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16) : (uint16_t)0;
+            stage = stage == kBStages - 1 ? 0 : stage + 1;
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");          // (the next head starts with the first stage again)
         __syncthreads();
     }
 }
@@ -848,7 +852,7 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
                 }
                 const int x = 8 * i + (row0 >> 4), blk = x < n ? list[x] : nb, key = blk * kPBlock + (row0 & 15);
                 const bool have = x < n && key < L;
-                if (have && JQ_IN(at.soff + key, P.ext.scores, kDbgPrune, 13)) P.scores[at.soff + key] = sum;
+                if (have && JQ_IN(at.soff + key, P.n_scores, kDbgPrune, 13)) P.scores[at.soff + key] = sum;
                 if (round == 0) {
                     // what this block alone guarantees of the pooled scores of its positions
                     float m = have ? sum : 0.f;
@@ -877,301 +881,11 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
 
-    if (tid == 0 && rank == 0) P.cut[head] = lo16;
-    if (P.fill) {                                             // what nothing needs counts as zero
-        float *const s = P.scores + at.soff + (long long)b0 * kPBlock;
-        const int m = min(nbs * kPBlock, L - b0 * kPBlock);
-        for (int i = tid; i < m; i += kTE)
-            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.ext.scores, kDbgPrune, 14)) s[i] = 0.f;
-    }
-}
-
-// ------------------------------------------------------------------ selection among the candidates, many heads
-
-constexpr int kCSelBins = 2048;                  // bins, equal parts of a range of keys
-constexpr int kCList = 1024;                     // keys of one bin that are finished on a list of them
-constexpr int kCRank = 64;                       // of which so many are ranked by comparison
-constexpr int kCSelThreads = 256, kCSelWarps = kCSelThreads / 32;
-
-struct SCtl2 {
-    BinAt found;
-    int sums[kCSelWarps];
-    int ncand, need;
-    uint32_t tau;
-    uint32_t wmin[kCSelWarps], wmax[kCSelWarps];
-};
-// Shared memory behind the control block: bins, list, words of blocks and their counts, active blocks, scores (then keys).
-__host__ __device__ constexpr size_t sel_fixed(int words) { return (size_t)(kCSelBins + kCList) * 4 + ((size_t)words * 8 + 15) / 16 * 16 + (size_t)words * 64 + 256; }
-
-// grid: a CTA per head.  Only the positions of the active blocks take part: those of the blocks that are scored and of those that a
-// window reaches from there.  What is not scored counts as zero: its scores lie below the threshold, and so does every pooled
-// score that they alone would make.  Laid one after the other, the active blocks can be pooled as if they were neighbours:
-// between two of them that are not lies a whole reach of zeros.  (Whatever the scores are, after a wait that ran out too, every
-// place that follows is brought into range.)
-__global__ void __launch_bounds__(kCSelThreads, 3)
-select_candidates(const __grid_constant__ CParams P)
-{
-    constexpr int kTE = kCSelThreads;
-    extern __shared__ __align__(16) uint8_t sel_raw[];
-    __shared__ SCtl2 ctl;
-    const int head = (int)blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-#ifdef JQ_DEBUG
-    DebugRecord *const dbg = P.dbg_rec;
-#endif
-    uint32_t *const bins = (uint32_t *)sel_raw, *const cand = bins + kCSelBins, *const words = cand + kCList;
-    int *const wbase = (int *)(words + P.max_words);
-    uint16_t *const act = (uint16_t *)(sel_raw + (size_t)(kCSelBins + kCList) * 4 + ((size_t)P.max_words * 8 + 15) / 16 * 16);   // [32 max_words]
-    float *const sc = (float *)(act + 32 * P.max_words) + 32;                    // [16 room] with 32 zeros on either side
-    const int room = P.room;
-    for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
-    if (tid == 0) ctl.ncand = 0;
-    cudaGridDependencySynchronize();             // nothing in global memory has been touched so far
-    cudaTriggerProgrammaticLaunchCompletion();
-    const HeadAt at = head_at(P, head);
-    const int L = at.L, nkeep = at.nkeep, nb = (L + kPBlock - 1) / kPBlock, nw = (nb + 31) >> 5;
-    const long long soff = at.soff;
-    int kv_in = head, src_rows = P.src_rows;
-    long long orow = (long long)head * nkeep, krow = (long long)head * P.out_rows;   // first rows of the head's indices and of its compacted rows
-    const uint4 *Kin = P.K, *Vin = P.V;
-    if (P.htab) {
-        const HeadRec r = P.htab[head];
-        kv_in = r.kv_in; orow = krow = r.ooff; src_rows = L;
-        Kin = P.Ktab[r.unit]; Vin = P.Vtab[r.unit];
-    }
-    auto sync = [&]() { named_sync<kTE>(); };
-    // ---- the scored blocks as bits, widened by the reach of a window, and the list of them
-    const uint32_t cut = __ldcg(P.cut + head);
-    const uint16_t *const ub = P.ub + (size_t)at.tbase * 8;
-    for (int w = warp; w < nw; w += kCSelWarps) {
-        const int i = 32 * w + lane;
-        const uint32_t m = __ballot_sync(0xffffffffu, i < nb && __ldcg(ub + i) >= cut);
-        if (lane == 0) words[w] = m;
-    }
-    sync();
-    const int reach = (P.radius + kPBlock - 1) / kPBlock;    // blocks that a window reaches into on either side: 0, 1 or 2
-    int n_act;
-    {
-        constexpr int kMost = (kCMaxBlocks / 32 + kTE) / kTE;         // words per thread, consecutive
-        const int per = (nw + kTE - 1) / kTE;
-        uint32_t m[kMost];
-        int mine = 0;
-#pragma unroll
-        for (int k = 0; k < kMost; ++k) {
-            const int w = tid * per + k;
-            m[k] = 0u;
-            if (k >= per || w >= nw) continue;
-            const uint32_t p = w > 0 ? words[w - 1] : 0u, q = words[w], r = w + 1 < nw ? words[w + 1] : 0u;
-            m[k] = q;
-            for (int d = 1; d <= reach; ++d) m[k] |= q << d | q >> d | p >> (32 - d) | r << (32 - d);
-            if (w == nw - 1 && (nb & 31)) m[k] &= (1u << (nb & 31)) - 1u;
-            mine += __popc(m[k]);
-        }
-        int base = scan_threads<kTE>(mine, n_act, ctl.sums);          // (its barriers part the reads of words[] from the writes)
-#pragma unroll
-        for (int k = 0; k < kMost; ++k) {
-            const int w = tid * per + k;
-            if (k >= per || w >= nw) continue;
-            words[w] = m[k]; wbase[w] = base;
-            base += __popc(m[k]);
-        }
-    }
-    sync();
-    for (int w = warp; w < nw; w += kCSelWarps) {
-        const uint32_t m = words[w];
-        const int x = wbase[w] + __popc(m & ((1u << lane) - 1u));
-        if ((m >> lane & 1u) && JQ_IN(x, 32 * P.max_words, kDbgPrune, 15)) act[x] = (uint16_t)(32 * w + lane);
-    }
-    sync();
-    auto block_of = [&](int a) -> int { return min((int)act[a], nb - 1); };
-    // The keys stay on chip, in the place of the scores that they are made of, or (more than there is room for, or a window
-    // that reaches past the next quad) go to memory a chunk at a time.  A key is one above the bits of a pooled score, which is
-    // not negative: order and ties are those of the values.  Positions that do not exist have the key 0.
-    const bool on_chip = n_act <= room && P.radius <= 4;
-    uint32_t *const gk = P.gkeys + soff;
-    const int chunk = on_chip ? n_act : room - 4;
-    uint32_t kmin = 0xffffffffu, kmax = 0u;
-#pragma unroll 1
-    for (int c0 = 0; c0 < n_act; c0 += chunk) {
-        const int c1 = min(c0 + chunk, n_act), f0 = max(c0 - 2, 0), f1 = min(c1 + 2, n_act);   // (with two blocks of halo)
-        const int i16 = tid & 15;
-#pragma unroll 1
-        for (int a = f0 + (tid >> 4); a < f1; a += kTE / 2) {          // eight loads in flight per thread
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int x = a + e * (kTE / 16), blk = x < f1 ? block_of(x) : 0, pos = blk * kPBlock + i16;
-                const bool in = x < f1 && pos < L && __ldcg(ub + blk) >= cut;
-                v[e] = in && JQ_IN(soff + pos, P.ext.scores, kDbgPrune, 16) ? __ldcg(P.scores + soff + pos) : 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int x = a + e * (kTE / 16);
-                if (x < f1 && JQ_IN(x - f0, room, kDbgPrune, 10)) sc[(x - f0) * 16 + i16] = v[e];
-            }
-        }
-        if (tid < 32) sc[tid - 32] = 0.f;
-        else if (tid < 64) sc[(f1 - f0) * 16 + tid - 32] = 0.f;
-        sync();
-        const int nq = 4 * (c1 - c0), NQ = ((nq + kTE - 1) / kTE) | 1, q0 = min(tid * NQ, nq), q1 = min(q0 + NQ, nq), shift = 4 * (c0 - f0);
-        float4 *const s4 = (float4 *)sc + shift;
-        float4 before = s4[q0 - 1], last = s4[q1], here = s4[q0];
-        if (on_chip) sync();                                         // (everybody has the quads next to his own)
-#pragma unroll 1
-        for (int q = q0; q < q1; ++q) {
-            float best[4];
-            if (P.radius <= 4) {
-                uint32_t unused[4];
-                const float4 next = q + 1 < q1 ? s4[q + 1] : last;
-                pooled_quad(before, here, next, P.radius, unused, best);
-                before = here; here = next;
-            } else {
-                const float *const x = (const float *)(s4 + q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float m = x[e];
-#pragma unroll 1
-                    for (int r = 1; r <= P.radius; ++r) m = max3(m, x[e - r], x[e + r]);
-                    best[e] = m;
-                }
-            }
-            uint32_t k[4];
-            const int pos = block_of(c0 + (q >> 2)) * kPBlock + 4 * (q & 3);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                k[e] = pos + e < L ? __float_as_uint(best[e]) + 1u : 0u;
-                if (k[e]) { kmin = min(kmin, k[e]); kmax = max(kmax, k[e]); }
-            }
-            if (on_chip) ((uint4 *)s4)[q] = make_uint4(k[0], k[1], k[2], k[3]);
-            else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (k[e] && JQ_IN(soff + 16 * c0 + 4 * q + e, P.ext.scores, kDbgPrune, 18)) gk[16 * c0 + 4 * q + e] = k[e];
-            }
-        }
-        sync();
-    }
-    // A thread owns NQ consecutive quads from here on: the max-pool's plateaus then mostly fall within a thread, and thread order is
-    // position order.
-    const int nq = 4 * n_act, NQ = ((nq + kTE - 1) / kTE) | 1, q0 = min(tid * NQ, nq), q1 = min(q0 + NQ, nq);
-    auto keys_of = [&](int q, uint32_t (&k)[4]) {
-        if (on_chip) {
-            const uint4 v = ((const uint4 *)sc)[q];
-            k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
-        } else {
-            const int pos = block_of(q >> 2) * kPBlock + 4 * (q & 3);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) k[e] = pos + e < L && JQ_IN(soff + 4 * q + e, P.ext.scores, kDbgPrune, 19) ? __ldcg(gk + 4 * q + e) : 0u;
-        }
-    };
-    kmin = __reduce_min_sync(0xffffffffu, kmin);
-    kmax = __reduce_max_sync(0xffffffffu, kmax);
-    if (lane == 0) { ctl.wmin[warp] = kmin; ctl.wmax[warp] = kmax; }
-    sync();
-    kmin = __reduce_min_sync(0xffffffffu, ctl.wmin[lane % kCSelWarps]);
-    kmax = __reduce_max_sync(0xffffffffu, ctl.wmax[lane % kCSelWarps]);
-    // The threshold key: 2048 equal bins over the keys' own range; the bin's keys, once they fit a list, are ranked by comparison or
-    // binned again.
-    uint32_t lo = kmin, lim = kmax - kmin;
-    int need = nkeep;
-    bool listed = false;
-    int count = 0;
-    auto bin_counts = [&](int i) -> uint2 { return *(const uint2 *)(bins + i); };
-#pragma unroll 1
-    for (;;) {
-        const int sh = lim >> 11 ? 21 - __clz(lim) : 0;               // lim >> sh < 2048
-        if (listed) {
-            for (int i = tid; i < count; i += kTE) {
-                const uint32_t d = cand[i] - lo;
-                if (d <= lim) atomicAdd(&bins[(d >> sh) & (kCSelBins - 1)], 1u);
-            }
-        } else {
-            uint32_t cur = 0u, cnt = 0u;
-#pragma unroll 1
-            for (int q = q0; q < q1; ++q) {
-                uint32_t k[4];
-                keys_of(q, k);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {                         // neighbours often share the bin: runs as one count
-                    const uint32_t d = k[e] - lo;
-                    const bool in = k[e] != 0u && d <= lim, other = in && d >> sh != cur;
-                    if (other && cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
-                    cnt = other ? 1u : cnt + in;
-                    cur = other ? d >> sh : cur;
-                }
-            }
-            if (cnt) atomicAdd(&bins[cur & (kCSelBins - 1)], cnt);
-        }
-        sync();
-        const BinAt b = find_bin<kTE, kCSelBins>(bin_counts, need, &ctl.found, ctl.sums);
-        lo += (uint32_t)b.bin << sh;
-        need = b.rank;
-        if (sh == 0) break;
-        lim = (1u << sh) - 1u;
-        for (int i = tid; i < kCSelBins; i += kTE) bins[i] = 0u;
-        if (!listed && b.count <= kCList) {
-            listed = true;
-            count = b.count;
-#pragma unroll 1
-            for (int q = q0; q < q1; ++q) {
-                uint32_t k[4];
-                keys_of(q, k);
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (k[e] != 0u && k[e] - lo <= lim) {
-                        const int x = atomicAdd(&ctl.ncand, 1);
-                        if (x < kCList) cand[x] = k[e];
-                    }
-            }
-            if (tid == 0) { ctl.tau = lo; ctl.need = need; }
-            sync();
-            if (count <= kCRank) {
-                if (tid < count) {
-                    const uint32_t k = cand[tid];
-                    int gt = 0, eq = 0;
-#pragma unroll 4
-                    for (int x = 0; x < count; ++x) { const uint32_t y = cand[x]; gt += y > k; eq += y == k; }
-                    if (gt < need && need <= gt + eq) { ctl.tau = k; ctl.need = need - gt; }   // (equal keys write the same)
-                }
-                sync();
-                lo = ctl.tau;
-                need = ctl.need;
-                break;
-            }
-        } else sync();
-    }
-    const uint32_t tau = lo;
-    // Kept: all keys above tau and, of those equal to it, the first `need`.
-    int gt = 0, eq = 0;
-#pragma unroll 1
-    for (int q = q0; q < q1; ++q) {
-        uint32_t k[4];
-        keys_of(q, k);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { gt += k[e] > tau; eq += k[e] == tau && k[e] != 0u; }
-    }
-    int all;
-    gt = scan_threads<kTE>(gt, all, ctl.sums);
-    eq = scan_threads<kTE>(eq, all, ctl.sums);
-    int32_t *const out = P.idx + orow;
-#pragma unroll 1
-    for (int q = q0; q < q1; ++q) {
-        uint32_t k[4];
-        keys_of(q, k);
-        if (k[0] < tau && k[1] < tau && k[2] < tau && k[3] < tau) continue;
-        const int pos = block_of(q >> 2) * kPBlock + 4 * (q & 3);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const bool same = k[e] == tau && k[e] != 0u;
-            const int t = gt + min(eq, need);
-            if ((k[e] > tau || (same && eq < need)) && t < nkeep && JQ_IN(orow + t, P.ext.out_rows, kDbgPrune, 17)) out[t] = pos + e;
-            gt += k[e] > tau;
-            eq += same;
-        }
-    }
-    // ---- the rows, once every index of the head has been written
-    sync();
-    copy_rows(tid, kTE, out, 0, nkeep, kv_in, krow, L, Kin, Vin, P.Kout, P.Vout, src_rows, P.ext JQ_DBG_ARG_DEV);
-    if (P.win.w) copy_window(P.win, head, krow + nkeep, tid >> 4, kTE / 16, P.Kout, P.Vout, P.ext JQ_DBG_ARG_DEV);
+    // what nothing needs counts as zero
+    float *const s = P.scores + at.soff + (long long)b0 * kPBlock;
+    const int m = min(nbs * kPBlock, L - b0 * kPBlock);
+    for (int i = tid; i < m; i += kTE)
+        if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
 }
 
 // ------------------------------------------------------------------ host side
@@ -1179,8 +893,6 @@ select_candidates(const __grid_constant__ CParams P)
 constexpr size_t stats_smem(int Rbox, int stages) { return 2 * (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kSCtlBytes; }
 size_t cand_smem(int Rbox, int stages, int share) { return (size_t)Rbox * kD * 2 + (size_t)stages * kPStage + kCCtlBytes + kCBins * 4 + (size_t)share * 32 + (size_t)(share / 4 + 1) * 8; }
 constexpr size_t kCMaxSmem = 227 * 1024, kCTwoPerSm = 113 * 1024;
-constexpr size_t kCSelSmem = 74 * 1024, kCSelMaxSmem = 200 * 1024;   // three CTAs of select_candidates to an SM, and the most that one is given
-constexpr int kCSelMinHeads = 128;                // from here on a CTA per head selects (fewer heads: a cluster each)
 
 struct PruneDevice {
     int sms = 0;
@@ -1202,6 +914,7 @@ bool prune_device(PruneDevice *out)
         for (auto k : {row_stats<kSGroupsNarrow>, row_stats<kSGroupsWide>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess) return false;
         for (int wide = 0; wide < 2; ++wide) {
+            if (cudaFuncSetAttribute(wide ? block_bounds<true> : block_bounds<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bounds_smem(wide)) != cudaSuccess) return false;
             const auto k = wide ? score_candidates<true> : score_candidates<false>;
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess ||
                 cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
@@ -1218,15 +931,14 @@ bool prune_device(PruneDevice *out)
                 if (cudaOccupancyMaxActiveClusters(&d.resident[wide][C], k, &cfg) != cudaSuccess) { cudaGetLastError(); d.resident[wide][C] = 0; }
             }
         }
-        if (cudaFuncSetAttribute(select_candidates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCSelMaxSmem) != cudaSuccess) return false;
         d.ready = true;
     }
     *out = d;
     return true;
 }
 
-// The scratch: maxima, partial statistics, normalisers, bounds, cuts.
-struct PruneScratch { size_t part, Ms, ub, cut, bytes; };
+// The scratch: maxima, partial statistics, normalisers, bounds.
+struct PruneScratch { size_t part, Ms, ub, bytes; };
 PruneScratch prune_layout(long long tiles, int heads, int R)
 {
     const int Rpad = (R + 31) & ~31, groups = R > 128 ? kSGroupsWide : kSGroupsNarrow;
@@ -1234,8 +946,7 @@ PruneScratch prune_layout(long long tiles, int heads, int R)
     s.part = align_up((size_t)tiles * 4 * Rpad * 4, 256);
     s.Ms = s.part + align_up((size_t)(heads + 256) * groups * R * sizeof(float2), 256);
     s.ub = s.Ms + align_up((size_t)heads * kMaxR * 4, 256);
-    s.cut = s.ub + align_up((size_t)tiles * 16, 256);
-    s.bytes = s.cut + align_up((size_t)heads * 4, 256);
+    s.bytes = s.ub + align_up((size_t)tiles * 16, 256);
     return s;
 }
 
@@ -1319,37 +1030,22 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
     P.groups = groups; P.sms = grid;
     P.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
-    P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.gkeys = w.keys; P.status = w.status;
-    P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub); P.cut = (uint32_t *)(scratch + lay.cut);
+    P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.status = w.status;
+    P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub);
     P.htab = S.htab; P.maps = S.maps;
-    P.idx = idx; P.K = (const uint4 *)K; P.V = (const uint4 *)V; P.Kout = (uint4 *)Kout; P.Vout = (uint4 *)Vout;
-    if (tables) { P.Ktab = (const uint4 *const *)tables->K; P.Vtab = (const uint4 *const *)tables->V; }
-    P.src_rows = src_head_rows > s.L ? src_head_rows : s.L;
-    P.out_rows = out_head_rows > P.nkeep ? out_head_rows : P.nkeep;
-    P.win.K = (const uint4 *)Kwin; P.win.V = (const uint4 *)Vwin; P.win.w = Vwin ? s.w : 0;
-    P.ext.scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
-    P.ext.out_rows = tables ? tables->total_rows : (long long)s.Hkv * P.out_rows;
-    P.ext.src_heads = tables ? tables->hpu : s.Hkv;
-    const bool many = s.Hkv >= kCSelMinHeads;
-    P.fill = many ? 0 : 1;
-    P.max_words = (max_tph * 8 + 31) / 32;
-    size_t sel_smem = kCSelSmem;
-    while (sel_fixed(P.max_words) + 64 * 64 > sel_smem) sel_smem += 8 * 1024;
-    P.room = (int)((sel_smem - sel_fixed(P.max_words)) / 64);
+    P.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
 #ifdef JQ_DEBUG
     S.dbg_rec = P.dbg_rec = debug_record();
     if (!S.dbg_rec) return JQ_ERR_CUDA;
     S.n_bmax = P.n_bmax = T * 4 * Rpad;
     S.n_part = P.n_part = (long long)(s.Hkv + 256) * groups * R;
 #endif
-    const unsigned bgrid = (unsigned)(T < (long long)kBPerSm * dev.sms ? T : kBPerSm * dev.sms);
+    const int bounds_ctas = bounds_per_sm(wide) * dev.sms;
     if (!launch(wide ? row_stats<kSGroupsWide> : row_stats<kSGroupsNarrow>, (unsigned)grid, (unsigned)stats_threads(groups), stats_smem(Rbox, S.stages), st, 0, mapK, mapQ, mapW, S) ||
-        !launch(wide ? block_bounds<true> : block_bounds<false>, bgrid, (unsigned)kBThreads, 0, st, 0, P) ||
+        !launch(wide ? block_bounds<true> : block_bounds<false>, (unsigned)(T < bounds_ctas ? T : bounds_ctas), (unsigned)kBThreads, (size_t)bounds_smem(wide), st, 0, P) ||
         !launch(wide ? score_candidates<true> : score_candidates<false>, (unsigned)(s.Hkv * C), (unsigned)cand_threads(wide), smem, st, C, mapB, mapQ, P))
         return JQ_ERR_CUDA;
-    if (!many) return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
-    if (!launch(select_candidates, (unsigned)s.Hkv, (unsigned)kCSelThreads, sel_smem, st, 0, P)) return JQ_ERR_CUDA;
-    return check_launch();
+    return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
 }
 
 }  // namespace jq
