@@ -76,6 +76,22 @@ struct SParams {
 #endif
 };
 
+// The head that tile `tile` of T belongs to: the last one whose first tile is not past it.  Heads of one length, or nearly, are found
+// at once; the search through the others is a chain of reads from memory.
+__device__ __forceinline__ int head_of_tile(const HeadRec *htab, int heads, long long T, long long tile)
+{
+    int lo = 0, hi = heads - 1;
+    const int guess = min((int)(tile * heads / T), hi);
+    const long long here = htab[guess].tbase, next = guess < hi ? htab[guess + 1].tbase : T;
+    if (here <= tile && tile < next) return guess;
+    if (here <= tile) lo = guess + 1; else hi = guess - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (htab[mid].tbase <= tile) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
 // Where a CTA's run of tiles starts, and how a role walks it.
 struct Walk {
     int h, t, tph, L;
@@ -93,13 +109,8 @@ struct Walk {
             t = (int)(tile - (long long)h * P.tph);
             return;
         }
-        int lo = 0, hi = P.heads - 1;                         // the last head whose first tile is not past `tile`
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (P.htab[mid].tbase <= tile) lo = mid; else hi = mid - 1;
-        }
-        h = lo;
-        t = (int)(tile - P.htab[lo].tbase);
+        h = head_of_tile(P.htab, P.heads, P.T, tile);
+        t = (int)(tile - P.htab[h].tbase);
         load(P);
     }
     __device__ __forceinline__ void advance(const SParams &P, int n)   // (never past the last tile of the call)
@@ -114,6 +125,14 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 {
     uint32_t d;
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+
+// x + y, with x a half.
+__device__ __forceinline__ float add_half(uint32_t x, float y)
+{
+    float d;
+    asm("{\n\t.reg .b16 h;\n\tcvt.u16.u32 h, %1;\n\tadd.rn.f32.f16 %0, h, %2;\n\t}" : "=f"(d) : "r"(x), "f"(y));
     return d;
 }
 
@@ -448,10 +467,10 @@ __device__ __forceinline__ BinAt find_bin(Get get, int target, BinAt *res, int *
 // ------------------------------------------------------------------ bounds
 
 constexpr int kBThreads = 256, kBStages = 3;     // stages: tiles of a warp, two on their way while one is worked on
-__host__ __device__ constexpr int bounds_per_sm(bool wide) { return wide ? 2 : 4; }
+__host__ __device__ constexpr int bounds_per_sm(bool wide) { return wide ? 2 : 3; }
 __host__ __device__ constexpr int bounds_smem(bool wide) { return kBThreads / 32 * kBStages * (wide ? 4096 : 2048); }
 
-// grid: two or four CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
+// grid: two or three CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
 // then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  A maximum x within 64 of its row's
 // normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60 each, which is
 // added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
@@ -463,13 +482,12 @@ block_bounds(const __grid_constant__ CParams P)
     __shared__ float2 other[kMaxR];
     __shared__ int huge;
     extern __shared__ __align__(16) uint8_t bounds_raw[];
-    constexpr int kV = kWide ? 2 : 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int R = P.R, Rpad = P.Rpad;
-    // the warp's stages; a lane reads what it has copied itself, 16 bytes of four neighbouring rows (eight with more than 128) of
-    // two blocks at a time
-    uint4 *const ring = (uint4 *)bounds_raw + warp * kBStages * 4 * kV * 32 + lane;
-    for (int i = 0; i < kBStages * 4 * kV; ++i) ring[32 * i] = make_uint4(0u, 0u, 0u, 0u);   // (what is not copied: rows that are none)
+    constexpr int kJ = kWide ? 8 : 4;                         // most pieces of 32 rows
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pair = lane >> 3, g = lane & 7;
+    const int R = P.R, Rpad = P.Rpad, nj = Rpad >> 5;
+    // The warp's stages.  Lanes 8 q .. 8 q + 7 have the blocks 2 q and 2 q + 1 of a tile: lane 8 q + g, of every piece of 32 rows, the
+    // rows 4 g .. 4 g + 3, 16 bytes that it copies and reads itself.
+    uint4 *const ring = (uint4 *)bounds_raw + warp * kBStages * kJ * 32 + lane;
 #ifdef JQ_DEBUG
     DebugRecord *const dbg = P.dbg_rec;
 #endif
@@ -478,12 +496,7 @@ block_bounds(const __grid_constant__ CParams P)
     const long long G = gridDim.x;
     long long f = blockIdx.x * P.T / G;
     const long long end = (blockIdx.x + 1) * P.T / G;
-    int h;
-    if (P.htab) {
-        int lo = 0, hi = P.heads - 1;                         // the last head whose first tile is not past f
-        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (P.htab[mid].tbase <= f) lo = mid; else hi = mid - 1; }
-        h = lo;
-    } else h = (int)(f / P.tph);
+    int h = P.htab ? head_of_tile(P.htab, P.heads, P.T, f) : (int)(f / P.tph);
 #pragma unroll 1
     for (; f < end; ++h) {
         const HeadAt a = head_at(P, h);
@@ -491,15 +504,15 @@ block_bounds(const __grid_constant__ CParams P)
         const int t1 = (int)min((long long)tph, end - a.tbase);       // (the window tile has no bounds)
         f = a.tbase + a.tph1;
         if (tid == 0) huge = 0;
+        const uint32_t *const mine = P.bmax + a.tbase * 4 * Rpad + pair * Rpad + 4 * g;
         auto request = [&](int t, int stage) {
+            const uint32_t *const from = mine + (long long)t * 4 * Rpad;
+            const uint32_t to = smem_u32(ring + stage * kJ * 32);
+            if (t < t1 && JQ_IN((a.tbase + t + 1) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 6)) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int y = 0; y < kV; ++y) {
-                    const long long at = ((a.tbase + t) * 4 + q) * Rpad + y * 128 + 4 * lane;
-                    if (t < t1 && y * 128 + 4 * lane < Rpad && JQ_IN(at + 3, P.n_bmax, kDbgPrune, 6))
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(ring + 32 * ((stage * 4 + q) * kV + y))), "l"(P.bmax + at) : "memory");
-                }
+                for (int j = 0; j < kJ; ++j)
+                    if (j < nj) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + j * 512), "l"(from + 32 * j) : "memory");
+            }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         request(t0 + warp, 0);
@@ -551,49 +564,41 @@ block_bounds(const __grid_constant__ CParams P)
             }
             __syncthreads();
         }
-        float nm[4 * kV];
+        float nm[4 * kJ];
 #pragma unroll
-        for (int i = 0; i < 4 * kV; ++i) {
-            const float x = Ms[(i >> 2) * 128 + 4 * lane + (i & 3)];
-            nm[i] = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;
-        }
+        for (int j = 0; j < kJ; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float x = Ms[32 * j + 4 * g + i];
+                nm[4 * j + i] = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;   // (a row that is none stays at -inf)
+            }
         const float least = huge ? INFINITY : 3e-16f;
         int stage = 0;
 #pragma unroll 1
         for (int t = t0 + warp; t < t1; t += kBThreads / 32) {
             request(t + 2 * (kBThreads / 32), stage == 0 ? 2 : stage - 1);
             asm volatile("cp.async.wait_group 2;" ::: "memory");
-            float2 sum[4];
+            float2 sum = make_float2(0.f, 0.f), sum2 = sum;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                sum[q] = make_float2(0.f, 0.f);
+            for (int j = 0; j < kJ; ++j) {
+                if (j >= nj) break;
+                const uint4 v = ring[(stage * kJ + j) * 32];
+                const uint32_t e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int y = 0; y < kV; ++y) {
-                    const uint4 v = ring[32 * ((stage * 4 + q) * kV + y)];
-                    const uint32_t e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 g = __fadd2_rn(__half22float2(*(const __half2 *)&e[i]), make_float2(nm[4 * y + i], nm[4 * y + i]));
-                        sum[q] = __fadd2_rn(sum[q], make_float2(ex2(g.x), ex2(g.y)));
-                    }
+                for (int i = 0; i < 4; ++i) {
+                    const float2 x = make_float2(ex2(add_half(e[i] & 0xffffu, nm[4 * j + i])), ex2(add_half(e[i] >> 16, nm[4 * j + i])));
+                    if (i & 1) sum2 = __fadd2_rn(sum2, x); else sum = __fadd2_rn(sum, x);
                 }
             }
-            // eight sums over the 32 lanes: after three exchanges of halves a lane holds one block's part
-            const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-            float2 p[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float2 keep = h4 ? sum[2 + i] : sum[i], give = h4 ? sum[i] : sum[2 + i];
-                p[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16), keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16));
-            }
-            const float2 keep = h3 ? p[1] : p[0], give = h3 ? p[0] : p[1];
-            const float2 r2 = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8), keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8));
-            float r = (h2 ? r2.y : r2.x) + __shfl_xor_sync(0xffffffffu, h2 ? r2.x : r2.y, 4);
+            sum = __fadd2_rn(sum, sum2);
+            // two sums over eight lanes: after an exchange of halves a lane holds one block's part
+            const bool odd = lane & 4;
+            float r = (odd ? sum.y : sum.x) + __shfl_xor_sync(0xffffffffu, odd ? sum.x : sum.y, 4);
             r += __shfl_xor_sync(0xffffffffu, r, 2);
             r += __shfl_xor_sync(0xffffffffu, r, 1);
-            const int blk = (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
+            const int blk = 2 * pair + (odd ? 1 : 0);
             if ((lane & 3) == 0)
-                P.ub[(size_t)(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16) : (uint16_t)0;
+                P.ub[(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16) : (uint16_t)0;
             stage = stage == kBStages - 1 ? 0 : stage + 1;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");          // (the next head starts with the first stage again)
@@ -884,8 +889,17 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     // what nothing needs counts as zero
     float *const s = P.scores + at.soff + (long long)b0 * kPBlock;
     const int m = min(nbs * kPBlock, L - b0 * kPBlock);
-    for (int i = tid; i < m; i += kTE)
-        if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
+    if (((uintptr_t)s & 15u) == 0) {
+#pragma unroll 4
+        for (int i = 4 * tid; i + 3 < m; i += 4 * kTE)
+            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i + 3, P.n_scores, kDbgPrune, 10)) *(float4 *)(s + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int i = (m & ~3) + tid;
+        if (tid < (m & 3) && ub[i >> 4] < lo16) s[i] = 0.f;
+    } else {
+#pragma unroll 4
+        for (int i = tid; i < m; i += kTE)
+            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
+    }
 }
 
 // ------------------------------------------------------------------ host side
