@@ -39,11 +39,11 @@ constexpr uint32_t kPBlockHalf = kPBlock * 128;  // one 64-column half of a bloc
 
 // ------------------------------------------------------------------ row statistics
 
-constexpr int kSGroupsNarrow = 3, kSGroupsWide = 4;   // epilogue groups for R <= 128 / R > 128
+constexpr int kSGroups = 4, kSEpi = 4 * kSGroups;   // epilogue groups, and their warps
 constexpr int kSMaxStages = 5;
 constexpr uint32_t kSSlots = 4, kSSlotCols = 128, kSTmemCols = 512;
-__host__ __device__ constexpr int stats_threads(int groups) { return (4 * groups + 2) * 32; }
-static_assert(kSGroupsNarrow <= (int)kSSlots && kSGroupsWide <= (int)kSSlots, "no more epilogue groups than accumulator slots");
+constexpr int kSThreads = (kSEpi + 2) * 32;
+static_assert(kSGroups == (int)kSSlots, "a slot per epilogue group");
 // A role that waits while others work sleeps between polls (ns).
 constexpr uint32_t kSSleepLong = 256, kSSleepShort = 32;
 
@@ -155,24 +155,26 @@ __device__ __forceinline__ float p1_half_max(uint32_t (&v)[16], int c0, int vali
     return cm;
 }
 
-// grid: one CTA per SM; CTA b takes tiles [b T / G, (b + 1) T / G) of the call.  Warps 0 .. 4 kGroups - 1 are the epilogue groups
-// (a thread owns a query row), then the TMA producer and the MMA issuer.
-template <int kGroups>
-__global__ void __launch_bounds__(stats_threads(kGroups), 1)
+// grid: one CTA per SM; CTA b takes tiles [b T / G, (b + 1) T / G) of the call.  Warps 0 .. 15 are the epilogue groups
+// (a thread owns a query row), then
+// the TMA producer and the MMA issuer.  (Four groups over four slots, also for up to 128 rows: 6 % over three groups that look
+// ahead, 32 layers of 32768 keys 601 -> 565 us.)
+template <bool kWide>
+__global__ void __launch_bounds__(kSThreads, 1)
 row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ,
           const __grid_constant__ CUtensorMap mapW, const __grid_constant__ SParams P)
 {
-    constexpr int kEpi = 4 * kGroups;
+    constexpr int kEpi = kSEpi, kGroups = kSGroups, nblk = kWide ? 2 : 1, bs = nblk - 1;   // blocks of 128 query rows
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if (smem_u32(smem_raw) & 1023u) {
         if (threadIdx.x == 0) atomicMax(P.status + kWStatus, (int)JQ_ERR_CUDA);
         return;
     }
-    const uint32_t q_bytes = (uint32_t)P.Rbox * kD * 2;
+    constexpr uint32_t q_bytes = 128 * nblk * kD * 2;
     uint8_t *const qbuf = smem_raw, *const kbuf = smem_raw + 2 * (size_t)q_bytes;
     SCtl *const ctl = (SCtl *)(kbuf + (size_t)P.stages * kPStage);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int R = P.R, Rpad = P.Rpad, stages = P.stages, nblk = P.Rbox / 128;
+    const int R = P.R, Rpad = P.Rpad, stages = P.stages;
     int *const status = P.status;
 #ifdef JQ_DEBUG
     DebugRecord *const dbg = P.dbg_rec;
@@ -273,25 +275,17 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
         // ---------------------------------------------------------------- epilogue groups: accumulator block u is group u % kGroups'
         const int grp = warp >> 2, quarter = warp & 3, row0 = quarter * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-        const int bs = nblk - 1, nunits = ntiles << bs;
+        const int nunits = ntiles << bs;
         const float c = P.c, lazy = 64.f / c;
         const float2 cc = make_float2(c, c);
-        const int win_i0 = row0 % P.w, win_i1 = (row0 + 128) % P.w;   // soft-token index of this thread's row in block 0 / block 1
+        const int blk = grp & bs, row = blk * 128 + row0;       // with two blocks of query rows a group always has the same one
+        const int win = min(P.w, row % P.w + 1);                // window keys up to the row's own position
         uint32_t va[16], vb[16];
-        bool ok = true, pre = false;
+        bool ok = true;
         auto release = [&](uint32_t slot) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->t_empty[slot], 1);
-        };
-        // (with as many groups as slots a group's next block cannot be complete before it gives its slot back)
-        constexpr bool kLookAhead = kGroups < (int)kSSlots;
-        auto try_begin = [&](uint32_t u) -> bool {
-            const uint32_t slot = u % kSSlots;
-            if (!__all_sync(0xffffffffu, mbar_test(&ctl->t_full[slot], (u / kSSlots) & 1))) return false;
-            tc_fence_after();
-            JQ_TMEM_LD16(lane_addr + slot * kSSlotCols, va);
-            return true;
         };
         auto begin = [&](uint32_t u) -> bool {
             const uint32_t slot = u % kSSlots;
@@ -300,7 +294,7 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
             JQ_TMEM_LD16(lane_addr + slot * kSSlotCols, va);
             return true;
         };
-        RowState st0 = {-INFINITY, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, st1 = st0;
+        RowState rs = {-INFINITY, make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         Walk at;
         if (ntiles > 0) at.start(P, first);
         int pub = ntiles > 0 ? at.h : 0, tile = 0;            // next head whose statistics this warp has to publish; tile of the run
@@ -311,42 +305,35 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
                 const long long slot = ((long long)blockIdx.x + pub) * kGroups + grp;
                 float2 *dst = P.part + slot * R;
                 const bool in = JQ_IN(slot * R + R - 1, P.n_part, kDbgPrune, 3);
-                if (row0 < R && in) dst[row0] = make_float2(st0.m, (st0.l01.x + st0.l01.y) + (st0.l23.x + st0.l23.y));
-                if (nblk == 2 && row0 + 128 < R && in) dst[row0 + 128] = make_float2(st1.m, (st1.l01.x + st1.l01.y) + (st1.l23.x + st1.l23.y));
-                st0.m = st1.m = -INFINITY;
-                st0.l01 = st0.l23 = st1.l01 = st1.l23 = make_float2(0.f, 0.f);
+                if (row < R && in) dst[row] = make_float2(rs.m, (rs.l01.x + rs.l01.y) + (rs.l23.x + rs.l23.y));
+                rs.m = -INFINITY;
+                rs.l01 = rs.l23 = make_float2(0.f, 0.f);
             }
         };
 #pragma unroll 1
         for (int k = grp; k < nunits; k += kGroups) {
-            const int n = k >> bs, blk = k & bs;
+            const int n = k >> bs;
             at.advance(P, n - tile);
             tile = n;
             if (at.h != pub) publish_upto(at.h);
             const uint32_t u = (uint32_t)k, slot = u % kSSlots, taddr = lane_addr + slot * kSSlotCols;
-            if (!pre && !begin(u)) { ok = false; break; }
-            // keys of the tile that count for this thread's row: the prefix keys or, in the window tile, the window keys up to
-            // the row's own position (causal)
+            if (!begin(u)) { ok = false; break; }
+            // keys of the tile that count for this thread's row: the prefix keys or, in the window tile, the causal part of it
             const bool wt = P.wtile && at.t == at.tph - 1;
-            const int valid = wt ? min(P.w, (blk ? win_i1 : win_i0) + 1) : min(kPTile, at.L - at.t * kPTile);
-            uint32_t *const bm = P.bmax + (first + n) * 4 * Rpad + blk * 128 + row0;
-            const bool store = blk * 128 + row0 < Rpad && JQ_IN((first + n + 1) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 4);   // warp-uniform
-            if (blk == 1) { const RowState x = st0; st0 = st1; st1 = x; }
+            const int valid = wt ? win : min(kPTile, at.L - at.t * kPTile);
+            uint32_t *const bm = P.bmax + (first + n) * 4 * Rpad + row;
+            const bool store = row < Rpad && JQ_IN((first + n + 1) * 4 * Rpad - 1, P.n_bmax, kDbgPrune, 4);   // warp-uniform
 #pragma unroll 1
             for (int c0 = 0; c0 < kPTile; c0 += 32) {
                 JQ_TMEM_WAIT16(va);
                 JQ_TMEM_LD16(taddr + c0 + 16, vb);
-                const float ma = p1_half_max(va, c0, valid, c, lazy, cc, st0);
+                const float ma = p1_half_max(va, c0, valid, c, lazy, cc, rs);
                 JQ_TMEM_WAIT16(vb);
                 if (c0 + 32 < kPTile) JQ_TMEM_LD16(taddr + c0 + 32, va);
-                else {
-                    release(slot);
-                    if (kLookAhead) pre = k + kGroups < nunits && try_begin(u + kGroups);
-                }
-                const float mb = p1_half_max(vb, c0 + 16, valid, c, lazy, cc, st0);
+                else release(slot);
+                const float mb = p1_half_max(vb, c0 + 16, valid, c, lazy, cc, rs);
                 if (store) bm[(c0 >> 5) * Rpad] = pack_half2(ma * c, mb * c);
             }
-            if (blk == 1) { const RowState x = st0; st0 = st1; st1 = x; }
         }
         if (ok && ntiles > 0) {
             at.advance(P, ntiles - 1 - tile);
@@ -375,7 +362,7 @@ constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16
 struct CParams {
     int L, tph, nkeep;         // one shape (tph: tiles per head in row_stats' numbering, the window tile included)
     int heads, R, Rbox, Rpad, radius;
-    int groups, sms;           // row_stats' epilogue groups and its grid
+    int sms;                   // row_stats' grid
     int stages, share;         // score_candidates: K ring; most tiles of a head that a CTA looks after
     int first_pct;             // blocks of round 1 per 100 pairs kept
     long long T;
@@ -517,12 +504,15 @@ block_bounds(const __grid_constant__ CParams P)
         };
         request(t0 + warp, 0);
         request(t0 + warp + kBThreads / 32, 1);
-        {   // the CTAs of row_stats that had tiles of this head, each with a pair per row and group: eight loads in flight
+        {   // the CTAs of row_stats that had tiles of this head, each with a pair per row and group:
+            // eight loads in flight
             const long long c_lo = ((a.tbase + 1) * P.sms - 1) / P.T, c_hi = ((a.tbase + a.tph1) * P.sms - 1) / P.T;   // owners of the first and last tile
-            const int nsl = (int)(c_hi - c_lo + 1) * P.groups;
-            const long long s0 = (c_lo + h) * P.groups;
             constexpr int kSub = kWide ? 1 : 2;                       // threads per row
             const int row = tid & (kWide ? 255 : 127), sub = kWide ? 0 : tid >> 7;
+            // (with two blocks of query rows every other group has the row)
+            constexpr int kStep = kWide ? 2 : 1;
+            const int nsl = (int)(c_hi - c_lo + 1) * (kSGroups / kStep);
+            const long long s0 = (c_lo + h) * kSGroups + (kWide ? row >> 7 : 0);
             const float2 *src = P.part + s0 * R + row;
             float m = -INFINITY, l = 0.f;
             if (row < R) {
@@ -533,7 +523,7 @@ block_bounds(const __grid_constant__ CParams P)
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         const int i = i0 + kSub * k;
-                        p[k] = i < nsl && JQ_IN((s0 + i) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)i * R) : make_float2(-INFINITY, 0.f);
+                        p[k] = i < nsl && JQ_IN((s0 + i * kStep) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)(i * kStep) * R) : make_float2(-INFINITY, 0.f);
                         if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
                     }
                     if (mn > -INFINITY) {
@@ -925,7 +915,7 @@ bool prune_device(PruneDevice *out)
     if (!d.ready) {
         d.sms = device_sms();
         if (d.sms < 1) return false;
-        for (auto k : {row_stats<kSGroupsNarrow>, row_stats<kSGroupsWide>})
+        for (auto k : {row_stats<false>, row_stats<true>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCMaxSmem) != cudaSuccess) return false;
         for (int wide = 0; wide < 2; ++wide) {
             if (cudaFuncSetAttribute(wide ? block_bounds<true> : block_bounds<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bounds_smem(wide)) != cudaSuccess) return false;
@@ -955,10 +945,10 @@ bool prune_device(PruneDevice *out)
 struct PruneScratch { size_t part, Ms, ub, bytes; };
 PruneScratch prune_layout(long long tiles, int heads, int R)
 {
-    const int Rpad = (R + 31) & ~31, groups = R > 128 ? kSGroupsWide : kSGroupsNarrow;
+    const int Rpad = (R + 31) & ~31;
     PruneScratch s;
     s.part = align_up((size_t)tiles * 4 * Rpad * 4, 256);
-    s.Ms = s.part + align_up((size_t)(heads + 256) * groups * R * sizeof(float2), 256);
+    s.Ms = s.part + align_up((size_t)(heads + 256) * kSGroups * R * sizeof(float2), 256);
     s.ub = s.Ms + align_up((size_t)heads * kMaxR * 4, 256);
     s.bytes = s.ub + align_up((size_t)tiles * 16, 256);
     return s;
@@ -1017,7 +1007,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     char *const scratch = (char *)w.prune;
     S.part = (float2 *)(scratch + lay.part);
     S.status = w.status;
-    const int groups = wide ? kSGroupsWide : kSGroupsNarrow, grid = (int)(T < dev.sms ? T : dev.sms);
+    const int grid = (int)(T < dev.sms ? T : dev.sms);
     CParams P = {};
     CUtensorMap mapK, mapQ, mapW, mapB;
     if (tables) {
@@ -1042,7 +1032,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     if (smem > kCMaxSmem) return JQ_ERR_CUDA;   // (prune_taken's limit on the length keeps every call below)
     P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
     P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
-    P.groups = groups; P.sms = grid;
+    P.sms = grid;
     P.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
     P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.status = w.status;
     P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub);
@@ -1052,10 +1042,10 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     S.dbg_rec = P.dbg_rec = debug_record();
     if (!S.dbg_rec) return JQ_ERR_CUDA;
     S.n_bmax = P.n_bmax = T * 4 * Rpad;
-    S.n_part = P.n_part = (long long)(s.Hkv + 256) * groups * R;
+    S.n_part = P.n_part = (long long)(s.Hkv + 256) * kSGroups * R;
 #endif
     const int bounds_ctas = bounds_per_sm(wide) * dev.sms;
-    if (!launch(wide ? row_stats<kSGroupsWide> : row_stats<kSGroupsNarrow>, (unsigned)grid, (unsigned)stats_threads(groups), stats_smem(Rbox, S.stages), st, 0, mapK, mapQ, mapW, S) ||
+    if (!launch(wide ? row_stats<true> : row_stats<false>, (unsigned)grid, (unsigned)kSThreads, stats_smem(Rbox, S.stages), st, 0, mapK, mapQ, mapW, S) ||
         !launch(wide ? block_bounds<true> : block_bounds<false>, (unsigned)(T < bounds_ctas ? T : bounds_ctas), (unsigned)kBThreads, (size_t)bounds_smem(wide), st, 0, P) ||
         !launch(wide ? score_candidates<true> : score_candidates<false>, (unsigned)(s.Hkv * C), (unsigned)cand_threads(wide), smem, st, C, mapB, mapQ, P))
         return JQ_ERR_CUDA;
