@@ -505,7 +505,8 @@ block_bounds(const __grid_constant__ CParams P)
         request(t0 + warp, 0);
         request(t0 + warp + kBThreads / 32, 1);
         {   // the CTAs of row_stats that had tiles of this head, each with a pair per row and group:
-            // eight loads in flight
+            // kDeep loads in flight (a head that all CTAs share has up to 38 or 76 pairs per row)
+            constexpr int kDeep = 16;
             const long long c_lo = ((a.tbase + 1) * P.sms - 1) / P.T, c_hi = ((a.tbase + a.tph1) * P.sms - 1) / P.T;   // owners of the first and last tile
             constexpr int kSub = kWide ? 1 : 2;                       // threads per row
             const int row = tid & (kWide ? 255 : 127), sub = kWide ? 0 : tid >> 7;
@@ -517,11 +518,11 @@ block_bounds(const __grid_constant__ CParams P)
             float m = -INFINITY, l = 0.f;
             if (row < R) {
 #pragma unroll 1
-                for (int i0 = sub; i0 < nsl; i0 += 8 * kSub) {
-                    float2 p[8];
+                for (int i0 = sub; i0 < nsl; i0 += kDeep * kSub) {
+                    float2 p[kDeep];
                     float mn = m;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
+                    for (int k = 0; k < kDeep; ++k) {
                         const int i = i0 + kSub * k;
                         p[k] = i < nsl && JQ_IN((s0 + i * kStep) * R + row, P.n_part, kDbgPrune, 5) ? __ldcg(src + (size_t)(i * kStep) * R) : make_float2(-INFINITY, 0.f);
                         if (p[k].y > 0.f) mn = fmaxf(mn, p[k].x);
@@ -529,7 +530,7 @@ block_bounds(const __grid_constant__ CParams P)
                     if (mn > -INFINITY) {
                         l *= ex2(P.c * (m - mn));
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) if (p[k].y > 0.f) l = fmaf(p[k].y, ex2(P.c * (p[k].x - mn)), l);
+                        for (int k = 0; k < kDeep; ++k) if (p[k].y > 0.f) l = fmaf(p[k].y, ex2(P.c * (p[k].x - mn)), l);
                         m = mn;
                     }
                 }
@@ -978,14 +979,28 @@ bool launch(void (*kernel)(A...), unsigned grid, unsigned threads, size_t smem, 
 
 size_t prune_bytes(long long tiles, int heads, int R) { return prune_layout(tiles, heads, R).bytes; }
 
-// Whether a call takes this way.  tiles: of all heads; keys: sum of the heads' lengths; kept: sum of what the heads keep.
+// Positions that are kept per block of 16 that holds one, roughly: a peak of the scores lifts the whole window around it.
+static double kept_per_block(int pool) { return pool >= 7 ? 7.0 : pool >= 3 ? 3.5 : 1.3; }
+
+// Whether a call takes this way.  tiles, keys, kept: of all heads, the lengths and what the heads keep.  What it saves is the second
+// pass over the tiles; what it costs is two more launches (with what they have to do before their first byte), and the scores of
+// the candidates, in proportion to the share that is kept.  Both sides were measured over 579 calls (us, two-pass kernel -> this
+// way; keys without structure, and in brackets keys that share directions by segments, which the bounds separate badly), with a
+// window of 7 and 128 query rows:
+//   8 heads x 32768, 65536, 131072 keys, 1 % kept       47 -> 58, 76 -> 75, 128 -> 108
+//   64 x 8192, 16384, 32768, 1 %                         76 -> 71 (92), 137 -> 100 (130), 240 -> 157 (220)
+//   64 x 32768, 3 % and 8 %                              252 -> 188 (240), 272 -> 260 (297)
+//   256 x 4096, 3 %                                      136 -> 114 (148)
+//   64 x 32768, 1.5 %, windows of 1, 3, 13               252 -> 262, 251 -> 179, 256 -> 164
+// With 8 query rows 64 x 32768 keys take 211 -> 141 (1 %), with 256 rows 371 -> 240.  Shorter heads than about 10000 keys gain little
+// and lose most where the bounds separate badly; fewer than 8 rows have not been measured and stay where they were.
 bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L)
 {
-    (void)heads;
     const int R = s.group * s.w;
-    if (R <= 64 || tiles >= (1ll << 30) || max_L > kPBlock * kCMaxBlocks) return false;
-    const double per = s.pool >= 7 ? 6.0 : s.pool >= 3 ? 2.5 : 1.2;    // kept positions per block that holds one
-    return tiles * (R > 128 ? 2 : 1) >= 6000 && kept / per * 16.0 < 0.35 * keys;
+    if (R < 8 || tiles >= (1ll << 30) || max_L > kPBlock * kCMaxBlocks || keys < 10000ll * heads) return false;
+    const double saved = R > 128 ? 9.0e-3 : R > 64 ? 6.2e-3 : 5.5e-3;              // us per tile
+    const double share = (double)kept / (double)keys * 7.0 / kept_per_block(s.pool);
+    return (double)tiles * (saved - 0.08 * share) >= 30.0;
 }
 
 jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const jq_shape &s, void *Kout, void *Vout, int32_t *idx,
@@ -1033,7 +1048,9 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
     P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
     P.sms = grid;
-    P.first_pct = s.pool >= 7 ? 18 : s.pool >= 3 ? 40 : 80;
+    // round 1 should find about as many blocks as hold a kept position: fewer leave the threshold's bound low, more are work that
+    // round 2 would not have asked for
+    P.first_pct = (int)(126.0 / kept_per_block(s.pool));
     P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.status = w.status;
     P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub);
     P.htab = S.htab; P.maps = S.maps;
