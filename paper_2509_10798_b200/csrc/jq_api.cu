@@ -46,15 +46,20 @@ static jq_status check_ws(const jq_shape *s, void *ws, size_t ws_bytes, Workspac
     return ws_bytes < out->bytes ? JQ_ERR_WORKSPACE : JQ_OK;
 }
 
-// One layer that the one-launch pass does not take, in two launches.  src_head_rows, out_head_rows: rows between consecutive heads
-// of K and V / of Kout and Vout when they are not packed; Vwin: the window rows follow the kept ones.
-static jq_status evict_in_two(const void *K, const void *V, const void *Qwin, const jq_shape &s, void *Kout, void *Vout, int32_t *kept_idx,
-                              const Workspace &w, cudaStream_t st, int src_head_rows = 0, int out_head_rows = 0,
-                              const void *Kwin = nullptr, const void *Vwin = nullptr)
+// Whether one pass over the keys and a look at the candidates is the faster way for a layer.
+static bool layer_pruned(const jq_shape &s)
 {
     const long long tiles = (long long)s.Hkv * ((s.L + 127) / 128), keys = (long long)s.Hkv * s.L;
-    const long long kept = (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L);
-    if (prune_taken(s, s.Hkv, tiles, keys, kept, s.L))
+    return prune_taken(s, s.Hkv, tiles, keys, (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L), s.L);
+}
+
+// One layer that the one-launch pass does not take.  src_head_rows, out_head_rows: rows between consecutive heads of K and V / of Kout
+// and Vout when they are not packed; Vwin: the window rows follow the kept ones.
+static jq_status evict_in_steps(const void *K, const void *V, const void *Qwin, const jq_shape &s, void *Kout, void *Vout, int32_t *kept_idx,
+                                const Workspace &w, cudaStream_t st, int src_head_rows = 0, int out_head_rows = 0,
+                                const void *Kwin = nullptr, const void *Vwin = nullptr)
+{
+    if (layer_pruned(s))
         return launch_evict_pruned(K, V, Qwin, s, Kout, Vout, kept_idx, w, st, nullptr, src_head_rows, out_head_rows, Kwin, Vwin);
     const jq_status rc = launch_score_tc(K, Qwin, s, w.scores, w, st, Kwin, nullptr, src_head_rows);
     if (rc != JQ_OK) return rc;
@@ -126,9 +131,9 @@ jq_status jq_evict_layer_windowed(const void *K, const void *V, const void *Qwin
     cudaStream_t st = (cudaStream_t)stream;
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin;
-    bool taken;
-    if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    return evict_in_two(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st, 0, 0, Kwin);
+    bool taken = false;
+    if (!layer_pruned(*s) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
+    return evict_in_steps(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st, 0, 0, Kwin);
 }
 
 jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Qwin, const void *Kwin, const void *Vwin,
@@ -151,10 +156,10 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     const size_t np = (size_t)(sp.budget < s->L ? sp.budget : s->L), nt = np + (size_t)s->w;
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin; src.Vwin = Vwin;
-    bool taken;
-    if ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
+    bool taken = false;
+    if (!layer_pruned(sp) && ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
-    return evict_in_two(K, V, Qwin, sp, Kout, Vout, kept_idx, w, st, 0, (int)nt, Kwin, Vwin);
+    return evict_in_steps(K, V, Qwin, sp, Kout, Vout, kept_idx, w, st, 0, (int)nt, Kwin, Vwin);
 }
 
 jq_status jq_score_fma(const void *K, const void *Qwin, const jq_shape *s, float *scores, void *ws,
@@ -203,9 +208,9 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
     cudaStream_t st = (cudaStream_t)stream;
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L;
-    bool taken;
-    if ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
-    return evict_in_two(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st);
+    bool taken = false;
+    if (!layer_pruned(*s) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
+    return evict_in_steps(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st);
 }
 
 // ---- units of one head geometry in buffers of their own: lengths, budgets and offsets per unit
@@ -407,7 +412,7 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     }
     // 2. the pass over the L = n_old + n_new rows of every head, compacted into the workspace (a row may move
     //    onto a row that another thread still has to read, so the compaction cannot run in place)
-    if ((rc = evict_in_two(Kc, Vc, Qrecent, *s, Ktmp, Vtmp, kept_idx, w, st, cap)) != JQ_OK) return rc;
+    if ((rc = evict_in_steps(Kc, Vc, Qrecent, *s, Ktmp, Vtmp, kept_idx, w, st, cap)) != JQ_OK) return rc;
     // 3. back to the head of the cache
     if (cudaMemcpy2DAsync(Kc, (size_t)cap * row, Ktmp, nkeep * row, nkeep * row, (size_t)s->Hkv, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return JQ_ERR_CUDA;
