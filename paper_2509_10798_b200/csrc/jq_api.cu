@@ -224,6 +224,7 @@ struct RaggedPlan {
     size_t keys = 0;            // sum over units of Hkv * L
     long long rows = 0;         // sum over units of Hkv * nkeep
     int max_L = 0;
+    bool uniform = true;        // one length and one number of kept rows for all units
 };
 
 // Validates the arguments the two ragged entry points share and sums the sizes.  L and budget may be NULL
@@ -234,7 +235,7 @@ jq_status plan_ragged(const jq_shape *common, int nunits, const int *L, const in
     if (nunits < 1) return JQ_ERR_INVALID_ARG;
     if (nunits > kMaxUnits) return JQ_ERR_UNSUPPORTED;
     RaggedPlan pl;
-    int max_keep = 0;
+    int max_keep = 0, L0 = 0, keep0 = 0;
     for (int u = 0; u < nunits; ++u) {
         jq_shape su = *common;
         if (L) su.L = L[u];
@@ -244,6 +245,8 @@ jq_status plan_ragged(const jq_shape *common, int nunits, const int *L, const in
         const int nkeep = su.budget < su.L ? su.budget : su.L;
         pl.keys += (size_t)su.Hkv * su.L;
         pl.rows += (long long)su.Hkv * nkeep;
+        if (u == 0) { L0 = su.L; keep0 = nkeep; }
+        pl.uniform = pl.uniform && su.L == L0 && nkeep == keep0;
         if (su.L > pl.max_L) pl.max_L = su.L;
         if (nkeep > max_keep) max_keep = nkeep;
     }
@@ -356,7 +359,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     t.V = (const void *const *)(tab + maps_bytes + ptr_bytes);
     t.heads = (const HeadRec *)(tab + maps_bytes + 2 * ptr_bytes);
     t.groups = (const GroupRec *)(tab + grp_off);
-    t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows;
+    t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows; t.uniform = pl.uniform;
     if (pruned) return launch_evict_pruned(nullptr, nullptr, nullptr, pl.S, Kout, Vout, kept_idx, w, st, &t);
     if ((rc = launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t)) != JQ_OK) return rc;
     return launch_select(w.scores, pl.S, kept_idx, nullptr, w, st, nullptr, nullptr, Kout, Vout, &t);

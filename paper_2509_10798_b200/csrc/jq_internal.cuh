@@ -91,6 +91,7 @@ struct UnitTables {
     long long total_keys = 0;            // keys of all units (floats in the scores array)
     long long total_rows = 0;            // rows of the stacked outputs
     long long total_tiles = 0;           // tiles of all heads
+    bool uniform = false;                // one length and one number of kept rows for all units
 };
 static inline size_t unit_tables_bytes(int nunits, int hpu)
 {
@@ -124,10 +125,20 @@ jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float
 // src_head_rows: rows between consecutive heads of K and V in memory when the heads are not packed (0: s.L);
 // out_head_rows: rows between consecutive heads of Kout and Vout when more than nkeep (0: nkeep).
 // Kwin, Vwin: with both given, the w window rows of every head follow its kept rows in Kout and Vout.
+// scored: with select_reads_scored_tiles, only the blocks of 16 positions whose bits are set have scores; the others count as zero,
+// and none of the positions that are kept is further than a window from one that is set.
+struct ScoredTiles {
+    const uint8_t *bits = nullptr;   // device: a byte per tile of 128 positions, heads one after the other
+    int tph = 0;                     // tiles from one head's first to the next head's (without tables)
+    int max_tiles = 0;               // of any head
+};
+constexpr int kMaxSparseTiles = 1024;   // (their list is in shared memory; two CTAs to an SM)
+bool select_reads_scored_tiles(const jq_shape &s, int max_L);
 jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, float *pooled,
                         const Workspace &w, cudaStream_t st, const void *K = nullptr, const void *V = nullptr,
                         void *Kout = nullptr, void *Vout = nullptr, const UnitTables *tables = nullptr,
-                        int src_head_rows = 0, int out_head_rows = 0, const void *Kwin = nullptr, const void *Vwin = nullptr);
+                        int src_head_rows = 0, int out_head_rows = 0, const void *Kwin = nullptr, const void *Vwin = nullptr,
+                        const ScoredTiles *scored = nullptr);
 // Scoring, selection and rows in one pass over K and a look at the keys that can be kept (jq_prune.cu), arguments as launch_score_tc
 // and launch_select take them.  prune_taken: whether a call over `heads` heads (tiles, keys and kept pairs of all of them, the
 // longest max_L) is one that this is the faster way for.

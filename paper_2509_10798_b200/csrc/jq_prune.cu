@@ -362,7 +362,7 @@ constexpr int kCMaxBlocks = 32767;               // block numbers are kept in 16
 struct CParams {
     int L, tph, nkeep;         // one shape (tph: tiles per head in row_stats' numbering, the window tile included)
     int heads, R, Rbox, Rpad, radius;
-    int sms;                   // row_stats' grid
+    int sms, hpu;              // row_stats' grid; heads per unit (ragged calls)
     int stages, share;         // score_candidates: K ring; most tiles of a head that a CTA looks after
     int first_pct;             // blocks of round 1 per 100 pairs kept
     long long T;
@@ -371,6 +371,7 @@ struct CParams {
     const uint32_t *bmax;
     float *Ms;                 // [heads][kMaxR]: minus the row normalisers
     uint16_t *ub;              // [tile][8]: bounds of the blocks, upper 16 bits of a float
+    uint8_t *scored;           // [tile]: the blocks that have been scored, as bits (null: the scores of the others are written as zeros)
     float *scores;
     int *status;
     const HeadRec *htab;
@@ -684,9 +685,10 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     const int L = at.L, nkeep = at.nkeep;
     int kv_in = head;
     const CUtensorMap *mb = &mapB, *mq = &mapQ;
-    if (P.htab) {
-        kv_in = P.htab[head].kv_in;
-        mq = P.maps + kMapsPerUnit * (size_t)P.htab[head].unit + 1; mb = mq + 1;
+    if (P.maps) {
+        const int unit = head / P.hpu;
+        kv_in = head - unit * P.hpu;
+        mq = P.maps + kMapsPerUnit * (size_t)unit + 1; mb = mq + 1;
     }
     const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
     const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
@@ -877,20 +879,20 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         return;
     }
 
-    // what nothing needs counts as zero
+    // what nothing needs counts as zero: told to the selection as bits, or written where it reads every score
+    if (P.scored) {
+        for (int t = tid; t < te - ts; t += kTE) {
+            uint32_t m = 0u;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) m |= (uint32_t)(8 * t + e < nbs && ub[8 * t + e] >= lo16) << e;
+            P.scored[at.tbase + ts + t] = (uint8_t)m;
+        }
+        return;
+    }
     float *const s = P.scores + at.soff + (long long)b0 * kPBlock;
     const int m = min(nbs * kPBlock, L - b0 * kPBlock);
-    if (((uintptr_t)s & 15u) == 0) {
-#pragma unroll 4
-        for (int i = 4 * tid; i + 3 < m; i += 4 * kTE)
-            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i + 3, P.n_scores, kDbgPrune, 10)) *(float4 *)(s + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int i = (m & ~3) + tid;
-        if (tid < (m & 3) && ub[i >> 4] < lo16) s[i] = 0.f;
-    } else {
-#pragma unroll 4
-        for (int i = tid; i < m; i += kTE)
-            if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
-    }
+    for (int i = tid; i < m; i += kTE)
+        if (ub[i >> 4] < lo16 && JQ_IN(at.soff + (long long)b0 * kPBlock + i, P.n_scores, kDbgPrune, 14)) s[i] = 0.f;
 }
 
 // ------------------------------------------------------------------ host side
@@ -942,8 +944,8 @@ bool prune_device(PruneDevice *out)
     return true;
 }
 
-// The scratch: maxima, partial statistics, normalisers, bounds.
-struct PruneScratch { size_t part, Ms, ub, bytes; };
+// The scratch: maxima, partial statistics, normalisers, bounds, scored blocks.
+struct PruneScratch { size_t part, Ms, ub, scored, bytes; };
 PruneScratch prune_layout(long long tiles, int heads, int R)
 {
     const int Rpad = (R + 31) & ~31;
@@ -951,7 +953,8 @@ PruneScratch prune_layout(long long tiles, int heads, int R)
     s.part = align_up((size_t)tiles * 4 * Rpad * 4, 256);
     s.Ms = s.part + align_up((size_t)(heads + 256) * kSGroups * R * sizeof(float2), 256);
     s.ub = s.Ms + align_up((size_t)heads * kMaxR * 4, 256);
-    s.bytes = s.ub + align_up((size_t)tiles * 16, 256);
+    s.scored = s.ub + align_up((size_t)tiles * 16, 256);
+    s.bytes = s.scored + align_up((size_t)tiles, 256);
     return s;
 }
 
@@ -1028,7 +1031,8 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     if (tables) {
         memset(&mapK, 0, sizeof mapK);
         mapQ = mapW = mapB = mapK;
-        S.htab = tables->heads; S.maps = (const CUtensorMap *)tables->maps;
+        S.htab = tables->uniform ? nullptr : tables->heads;   // (lengths from the table are a chain of reads before anything starts)
+        S.maps = (const CUtensorMap *)tables->maps;
     } else {
         if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, src_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
             !make_tensor_map(&mapB, K, s.L, s.Hkv, kPBlock, src_head_rows))
@@ -1047,7 +1051,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     if (smem > kCMaxSmem) return JQ_ERR_CUDA;   // (prune_taken's limit on the length keeps every call below)
     P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
     P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
-    P.sms = grid;
+    P.sms = grid; P.hpu = S.hpu;
     // Round 1 should take as many blocks as hold the kept positions.  A peak lifts, within its block, pool - r (r + 1) / 16 positions on
     // average: with fewer blocks than the budget has of those the threshold's bound falls among the positions that are not lifted,
     // and round 2 takes nearly everything (a fifth too few: 32 layers of 32768 keys 600 -> 945 us); more cost next to nothing,
@@ -1056,6 +1060,10 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     P.first_pct = (int)(130.0 / (2 * r + 1 - r * (r + 1) / 16.0));
     P.T = T; P.c = S.c; P.part = S.part; P.bmax = S.bmax; P.scores = w.scores; P.status = w.status;
     P.Ms = (float *)(scratch + lay.Ms); P.ub = (uint16_t *)(scratch + lay.ub);
+    const bool sparse = select_reads_scored_tiles(s, tables ? tables->max_L : s.L);
+    ScoredTiles scored;
+    scored.bits = P.scored = sparse ? (uint8_t *)(scratch + lay.scored) : nullptr;
+    scored.tph = tph; scored.max_tiles = max_tph;
     P.htab = S.htab; P.maps = S.maps;
     P.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
 #ifdef JQ_DEBUG
@@ -1069,7 +1077,8 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
         !launch(wide ? block_bounds<true> : block_bounds<false>, (unsigned)(T < bounds_ctas ? T : bounds_ctas), (unsigned)kBThreads, (size_t)bounds_smem(wide), st, 0, P) ||
         !launch(wide ? score_candidates<true> : score_candidates<false>, (unsigned)(s.Hkv * C), (unsigned)cand_threads(wide), smem, st, C, mapB, mapQ, P))
         return JQ_ERR_CUDA;
-    return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin);
+    return launch_select(w.scores, s, idx, nullptr, w, st, K, V, Kout, Vout, tables, src_head_rows, out_head_rows, Vwin ? Kwin : nullptr, Vwin,
+                         sparse ? &scored : nullptr);
 }
 
 }  // namespace jq

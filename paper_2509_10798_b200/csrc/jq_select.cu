@@ -475,6 +475,7 @@ constexpr int kStrMaxWarps = 32;
 constexpr int kStepQuads = 128;     // quads a warp takes per step
 constexpr int kStageQuads = kStepQuads + 2;
 constexpr int kStreamMinHeads = 128;   // calls with at least this many heads take this kernel
+constexpr int kSparseQuads = 4 * 34;   // (sparse) a step is four tiles of 32 quads, each with a quad of halo on either side
 
 struct StrCtl {
     int scan[kStrMaxWarps + 1];
@@ -515,6 +516,18 @@ __device__ __forceinline__ void stage_issue(float4 *dst, const float *__restrict
             *d = load_quad(s, L, q, vec, soff, ext JQ_DBG_ARG_DEV);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// One quad of a tile into the warp's buffer, if its block is scored; else zeros, as what is not scored counts.
+__device__ __forceinline__ void stage_quad(float4 *d, const float *__restrict__ s, int L, int q, bool scored, bool vec, long long soff,
+                                           const SelExtents &ext JQ_DBG_PARAM)
+{
+    if (!scored)
+        *d = make_float4(0.f, 0.f, 0.f, 0.f);
+    else if (vec && 4 * q + 4 <= L && JQ_IN(soff + 4 * q + 3, ext.scores, kDbgSelect, 22))
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(s + 4 * q) : "memory");
+    else
+        *d = load_quad(s, L, q, vec, soff, ext JQ_DBG_ARG_DEV);
 }
 
 // The staged quads of the step at `base` of the warp's walk over [qa, qb), 128 quads per step: waits for the step's
@@ -571,13 +584,14 @@ __device__ __forceinline__ void hist_add_runs(uint32_t *hist, const uint32_t (&d
 // grid (Hkv), block kThreads = 512 (two CTAs to an SM) or 1024 (one); dynamic shared memory: two staging buffers of
 // kStageQuads float4 per warp.  Arguments as for select_cluster.
 __host__ __device__ constexpr int stream_ctas_per_sm(int threads) { return threads == 512 ? 2 : 1; }
-template <int kThreads>
+template <int kThreads, bool kSparse>
 __global__ void __launch_bounds__(kThreads, stream_ctas_per_sm(kThreads))
 select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, int32_t *__restrict__ idx,
               float *__restrict__ pooled, const uint4 *__restrict__ Kin, const uint4 *__restrict__ Vin,
               uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, const HeadRec *__restrict__ htab,
               const uint4 *const *__restrict__ Ktab, const uint4 *const *__restrict__ Vtab, int src_rows, int out_rows,
-              const WindowRows win, const SelExtents ext JQ_DBG_PARAM)
+              const WindowRows win, const ScoredTiles scored,
+              const SelExtents ext JQ_DBG_PARAM)
 {
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ uint32_t hist[kBins];
@@ -586,7 +600,9 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     __shared__ StrCtl ctl;
     constexpr int T = kThreads, nw = T / 32;
     const int kv = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    float4 *buf = (float4 *)sm + wid * 2 * kStageQuads;   // the warp's two staging buffers
+    constexpr int kBufQuads = kSparse ? kSparseQuads : kStageQuads;
+    float4 *buf = (float4 *)sm + wid * 2 * kBufQuads;     // the warp's two staging buffers
+    uint32_t *const tiles = (uint32_t *)((float4 *)sm + nw * 2 * kBufQuads);   // (sparse) every warp's tiles that take part
     int kv_in = kv;
     long long soff = (long long)kv * L, orow = (long long)kv * nkeep, krow = (long long)kv * out_rows;
     cudaGridDependencySynchronize();   // everything above ran while the previous kernel of the stream was finishing
@@ -602,39 +618,97 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     const bool vec = (((size_t)s) & 15) == 0;
     const int nq = (L + 3) / 4;
     // warp w owns the contiguous quads [qa, qb); every warp makes the same number of steps
-    const int segq = (nq + nw - 1) / nw;
+    const int segq = kSparse ? 32 * (((L + 127) / 128 + nw - 1) / nw) : (nq + nw - 1) / nw;
     const int qa = min(wid * segq, nq), qb = min(qa + segq, nq);
+    int n_tiles = 0;                                           // (sparse) the warp's tiles that take part
+    if (kSparse) {
+        // a tile's entry: its number, its scored blocks, whether the block before it and the one behind it are scored
+        const uint8_t *const from = scored.bits + (htab ? htab[kv].tbase : (long long)kv * scored.tph);
+        const int nt = (L + 127) / 128, ta = min(wid * (segq >> 5), nt), tb = min(ta + (segq >> 5), nt);
+        for (int t0 = ta; t0 < tb; t0 += 32) {
+            const int t = t0 + lane;
+            const uint32_t b = t < tb ? __ldcg(from + t) : 0u;
+            uint32_t before = __shfl_up_sync(0xffffffffu, b, 1) >> 7, behind = __shfl_down_sync(0xffffffffu, b, 1) & 1u;
+            if (lane == 0) before = t > 0 ? (uint32_t)__ldcg(from + t - 1) >> 7 : 0u;
+            if ((lane == 31 || t + 1 >= tb) && t < tb) behind = t + 1 < nt ? (uint32_t)__ldcg(from + t + 1) & 1u : 0u;
+            const bool on = t < tb && (b | before | behind) != 0u;
+            const uint32_t m = __ballot_sync(0xffffffffu, on);
+            const int at = ta + n_tiles + __popc(m & ((1u << lane) - 1u));
+            if (on && JQ_IN(at, scored.max_tiles, kDbgSelect, 36)) tiles[at] = (uint32_t)t | b << 16 | before << 24 | behind << 25;
+            n_tiles += __popc(m);
+        }
+        __syncwarp();
+    }
+    // One walk over the warp's share in order of position: f(q, nval, st) for 32 quads at a time, of which lane l has quad q with
+    // nval positions that take part, staged as st[l + 1] between its neighbours.
+    auto walk = [&](auto f) {
+        if constexpr (kSparse) {
+            const uint32_t *const mine = tiles + min(wid * (segq >> 5), (L + 127) / 128);
+            __syncwarp();                                      // the reads of an earlier walk are done
+            auto request = [&](int i, float4 *to) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (i + u >= n_tiles) break;
+                    const uint32_t e = mine[i + u], t = e & 0xffffu;
+                    float4 *const d = to + 34 * u + 1;
+                    stage_quad(d + lane, s, L, (int)(32 * t) + lane, e >> (16 + (lane >> 2)) & 1u, vec, soff, ext JQ_DBG_ARG_DEV);
+                    if (lane < 2) stage_quad(d + (lane ? 32 : -1), s, L, (int)(32 * t) + (lane ? 32 : -1), e >> (24 + lane) & 1u, vec, soff, ext JQ_DBG_ARG_DEV);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            request(0, buf);
+#pragma unroll 1
+            for (int i = 0; i < n_tiles; i += 4) {
+                const float4 *const cur = buf + (i >> 2 & 1) * kBufQuads;
+                request(i + 4, buf + (~i >> 2 & 1) * kBufQuads);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (i + u >= n_tiles) break;
+                    const uint32_t e = mine[i + u], b = e >> 16 & 0xffu, act = b | b << 1 | b >> 1 | (e >> 24 & 1u) | (e >> 25 & 1u) << 7;
+                    const int q = (int)(32 * (e & 0xffffu)) + lane;
+                    f(q, act >> (lane >> 2) & 1u ? max(0, min(4, L - 4 * q)) : 0, cur + 34 * u);
+                }
+                __syncwarp();
+            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        } else {
+            for (int base = qa; base < qb; base += kStepQuads) {
+                const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int q = base + 32 * u + lane;
+                    f(q, q < qb ? min(4, L - 4 * q) : 0, bf + 32 * u);
+                }
+            }
+        }
+    };
 
     // ---- pass 1: histogram of the top 11 bits of the pooled keys
     for (int i = tid; i < kBins; i += T) hist[i] = 0;
     if (tid == 0) ctl.cand_count = 0;
     __syncthreads();
-    for (int base = qa; base < qb; base += kStepQuads) {
-        const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int q = base + 32 * u + lane;
-            const int nval = q < qb ? min(4, L - 4 * q) : 0;
-            uint32_t key[4];
-            float best[4];
-            pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
-            if (pooled && nval && JQ_IN(soff + 4 * q + nval - 1, ext.scores, kDbgSelect, 25))
-                for (int i = 0; i < nval; ++i) pooled[4 * q + i] = best[i];
-            // one addition per warp when all its positions share the digit (the usual case: 128 neighbouring
-            // positions of similar size), else runs of equal digits per thread
-            const uint32_t d0 = key[0] >> 21;
-            bool same = true;
-            for (int i = 1; i < 4; ++i) if (i < nval && (key[i] >> 21) != d0) same = false;
-            const uint32_t lead = __shfl_sync(0xffffffffu, d0, 0);
-            if (__all_sync(0xffffffffu, nval == 0 || (same && d0 == lead))) {
-                const int tot = __reduce_add_sync(0xffffffffu, nval);
-                if (lane == 0 && tot && JQ_IN(lead, kBins, kDbgSelect, 24)) atomicAdd(&hist[lead], (uint32_t)tot);
-            } else {
-                const uint32_t dg[4] = {key[0] >> 21, key[1] >> 21, key[2] >> 21, key[3] >> 21};
-                hist_add_runs(hist, dg, nval JQ_DBG_ARG_DEV);
-            }
+    walk([&](int q, int nval, const float4 *bf) {
+        uint32_t key[4];
+        float best[4];
+        pooled_quad(bf[lane], bf[lane + 1], bf[lane + 2], radius, key, best);
+        if (pooled && nval && JQ_IN(soff + 4 * q + nval - 1, ext.scores, kDbgSelect, 25))
+            for (int i = 0; i < nval; ++i) pooled[4 * q + i] = best[i];
+        // one addition per warp when all its positions share the digit (the usual case: 128 neighbouring
+        // positions of similar size), else runs of equal digits per thread
+        const uint32_t d0 = key[0] >> 21;
+        bool same = true;
+        for (int i = 1; i < 4; ++i) if (i < nval && (key[i] >> 21) != d0) same = false;
+        const uint32_t lead = __shfl_sync(0xffffffffu, d0, 0);
+        if (__all_sync(0xffffffffu, nval == 0 || (same && d0 == lead))) {
+            const int tot = __reduce_add_sync(0xffffffffu, nval);
+            if (lane == 0 && tot && JQ_IN(lead, kBins, kDbgSelect, 24)) atomicAdd(&hist[lead], (uint32_t)tot);
+        } else {
+            const uint32_t dg[4] = {key[0] >> 21, key[1] >> 21, key[2] >> 21, key[3] >> 21};
+            hist_add_runs(hist, dg, nval JQ_DBG_ARG_DEV);
         }
-    }
+    });
     __syncthreads();
     if (nkeep >= L) {                                          // everything is kept
         for (int e = tid; e < L; e += T) if (JQ_IN(orow + e, ext.out_rows, kDbgSelect, 26)) out[e] = e;
@@ -649,28 +723,22 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
         if (listed) {
             // pass 2: the keys with the winning first digit, with their positions; the warp's keys above that digit
             int hi_cnt = 0;
-            for (int base = qa; base < qb; base += kStepQuads) {
-                const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int q = base + 32 * u + lane;
-                    const int nval = q < qb ? min(4, L - 4 * q) : 0;
-                    if (nval == 0 || (quad_bound_key(bf, 32 * u + lane) >> 21) < pre) continue;
-                    uint32_t key[4];
-                    float best[4];
-                    pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
-                    int nhit = 0;
-                    for (int i = 0; i < 4; ++i) if (i < nval) { nhit += (key[i] >> 21) == pre; hi_cnt += (key[i] >> 21) > pre; }
-                    if (nhit) {
-                        int at = atomicAdd(&ctl.cand_count, nhit);
-                        for (int i = 0; i < 4; ++i)
-                            if (i < nval && (key[i] >> 21) == pre) {
-                                if (JQ_IN(at, kStrCand, kDbgSelect, 27)) { cand_key[at] = key[i]; cand_pos[at] = 4 * q + i; }
-                                ++at;
-                            }
-                    }
+            walk([&](int q, int nval, const float4 *bf) {
+                if (nval == 0 || (quad_bound_key(bf, lane) >> 21) < pre) return;
+                uint32_t key[4];
+                float best[4];
+                pooled_quad(bf[lane], bf[lane + 1], bf[lane + 2], radius, key, best);
+                int nhit = 0;
+                for (int i = 0; i < 4; ++i) if (i < nval) { nhit += (key[i] >> 21) == pre; hi_cnt += (key[i] >> 21) > pre; }
+                if (nhit) {
+                    int at = atomicAdd(&ctl.cand_count, nhit);
+                    for (int i = 0; i < 4; ++i)
+                        if (i < nval && (key[i] >> 21) == pre) {
+                            if (JQ_IN(at, kStrCand, kDbgSelect, 27)) { cand_key[at] = key[i]; cand_pos[at] = 4 * q + i; }
+                            ++at;
+                        }
                 }
-            }
+            });
             hi_cnt = __reduce_add_sync(0xffffffffu, hi_cnt);
             if (lane == 0) ctl.warp_gt[wid] = hi_cnt;
             __syncthreads();
@@ -687,20 +755,14 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
                     if ((k >> (sh + wd)) == pre && JQ_IN((k >> sh) & mask, kBins, kDbgSelect, 24)) atomicAdd(&hist[(k >> sh) & mask], 1u);
                 }
             } else {
-                for (int base = qa; base < qb; base += kStepQuads) {
-                    const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int q = base + 32 * u + lane;
-                        const int nval = q < qb ? min(4, L - 4 * q) : 0;
-                        if (nval == 0 || (quad_bound_key(bf, 32 * u + lane) >> (sh + wd)) < pre) continue;
-                        uint32_t key[4], dg[4];
-                        float best[4];
-                        pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
-                        for (int i = 0; i < 4; ++i) dg[i] = (key[i] >> (sh + wd)) == pre ? ((key[i] >> sh) & mask) : 0xffffffffu;
-                        hist_add_runs(hist, dg, nval JQ_DBG_ARG_DEV);
-                    }
-                }
+                walk([&](int q, int nval, const float4 *bf) {
+                    if (nval == 0 || (quad_bound_key(bf, lane) >> (sh + wd)) < pre) return;
+                    uint32_t key[4], dg[4];
+                    float best[4];
+                    pooled_quad(bf[lane], bf[lane + 1], bf[lane + 2], radius, key, best);
+                    for (int i = 0; i < 4; ++i) dg[i] = (key[i] >> (sh + wd)) == pre ? ((key[i] >> sh) & mask) : 0xffffffffu;
+                    hist_add_runs(hist, dg, nval JQ_DBG_ARG_DEV);
+                });
             }
             __syncthreads();
             find_digit_cta(hist, krem, ctl);
@@ -721,19 +783,13 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
             }
         } else {
             int cgt = 0, ceq = 0;
-            for (int base = qa; base < qb; base += kStepQuads) {
-                const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int q = base + 32 * u + lane;
-                    const int nval = q < qb ? min(4, L - 4 * q) : 0;
-                    if (nval == 0 || quad_bound_key(bf, 32 * u + lane) < tau) continue;
-                    uint32_t key[4];
-                    float best[4];
-                    pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
-                    for (int i = 0; i < 4; ++i) if (i < nval) { cgt += key[i] > tau; ceq += key[i] == tau; }
-                }
-            }
+            walk([&](int q, int nval, const float4 *bf) {
+                if (nval == 0 || quad_bound_key(bf, lane) < tau) return;
+                uint32_t key[4];
+                float best[4];
+                pooled_quad(bf[lane], bf[lane + 1], bf[lane + 2], radius, key, best);
+                for (int i = 0; i < 4; ++i) if (i < nval) { cgt += key[i] > tau; ceq += key[i] == tau; }
+            });
             cgt = __reduce_add_sync(0xffffffffu, cgt);
             ceq = __reduce_add_sync(0xffffffffu, ceq);
             if (lane == 0) { ctl.warp_gt[wid] = cgt; ctl.warp_eq[wid] = ceq; }
@@ -743,42 +799,36 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
         for (int w = 0; w < wid; ++w) { gt_before += ctl.warp_gt[w]; eq_before += ctl.warp_eq[w]; }
 
         // ---- pass 3: ordered compaction (position order = warp, step, quad, position within the quad)
-        for (int base = qa; base < qb; base += kStepQuads) {
-            const float4 *bf = stage_step(buf, s, L, base, qa, qb, vec, soff, ext JQ_DBG_ARG_DEV);
+        walk([&](int q, int nval, const float4 *bf) {
+            const bool may = nval != 0 && quad_bound_key(bf, lane) >= tau;
+            if (!__any_sync(0xffffffffu, may)) return;         // nothing of these 128 quads is at or above tau
+            uint32_t key[4] = {0u, 0u, 0u, 0u};
+            float best[4];
+            if (may) pooled_quad(bf[lane], bf[lane + 1], bf[lane + 2], radius, key, best);
+            int g = 0, e = 0;
+            for (int i = 0; i < 4; ++i) if (may && i < nval) { g += key[i] > tau; e += key[i] == tau; }
+            const int mine = g | (e << 16);
+            int inc = mine;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int q = base + 32 * u + lane;
-                const int nval = q < qb ? min(4, L - 4 * q) : 0;
-                const bool may = nval != 0 && quad_bound_key(bf, 32 * u + lane) >= tau;
-                if (!__any_sync(0xffffffffu, may)) continue;         // nothing of these 128 quads is at or above tau
-                uint32_t key[4] = {0u, 0u, 0u, 0u};
-                float best[4];
-                if (may) pooled_quad(bf[32 * u + lane], bf[32 * u + lane + 1], bf[32 * u + lane + 2], radius, key, best);
-                int g = 0, e = 0;
-                for (int i = 0; i < 4; ++i) if (may && i < nval) { g += key[i] > tau; e += key[i] == tau; }
-                const int mine = g | (e << 16);
-                int inc = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int n = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += n;
-                }
-                const int total = __shfl_sync(0xffffffffu, inc, 31);
-                int g_here = gt_before + ((inc - mine) & 0xffff), e_here = eq_before + ((inc - mine) >> 16);
-                for (int i = 0; i < 4; ++i) {
-                    if (!may || i >= nval) continue;
-                    if (key[i] > tau) {
-                        if (JQ_IN(g_here + min(e_here, need_eq), nkeep, kDbgSelect, 28)) out[g_here + min(e_here, need_eq)] = 4 * q + i;
-                        ++g_here;
-                    } else if (key[i] == tau) {
-                        if (e_here < need_eq && JQ_IN(g_here + e_here, nkeep, kDbgSelect, 29)) out[g_here + e_here] = 4 * q + i;
-                        ++e_here;
-                    }
-                }
-                gt_before += total & 0xffff;
-                eq_before += total >> 16;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int n = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += n;
             }
-        }
+            const int total = __shfl_sync(0xffffffffu, inc, 31);
+            int g_here = gt_before + ((inc - mine) & 0xffff), e_here = eq_before + ((inc - mine) >> 16);
+            for (int i = 0; i < 4; ++i) {
+                if (!may || i >= nval) continue;
+                if (key[i] > tau) {
+                    if (JQ_IN(g_here + min(e_here, need_eq), nkeep, kDbgSelect, 28)) out[g_here + min(e_here, need_eq)] = 4 * q + i;
+                    ++g_here;
+                } else if (key[i] == tau) {
+                    if (e_here < need_eq && JQ_IN(g_here + e_here, nkeep, kDbgSelect, 29)) out[g_here + e_here] = 4 * q + i;
+                    ++e_here;
+                }
+            }
+            gt_before += total & 0xffff;
+            eq_before += total >> 16;
+        });
     }
     if (!Kin) return;
 
@@ -890,14 +940,15 @@ jq_status launch_select_cluster(const float *scores, const jq_shape &s, int nkee
 // when the scores of the heads that 512 would hold in flight (a head is read three times) are far more than the L2.
 jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep, int Lmax, int32_t *idx, float *pooled,
                                cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout, int sms, int dev,
-                               const UnitTables *tables, int src_rows, int out_rows, const WindowRows &win, const SelExtents &ext)
+                               const UnitTables *tables, int src_rows, int out_rows, const WindowRows &win, const ScoredTiles *sparse, const SelExtents &ext)
 {
     const long long resident = (long long)sms * stream_ctas_per_sm(512), inflight = s.Hkv < resident ? s.Hkv : resident;
-    const int threads = inflight * Lmax * 4 <= (96ll << 20) ? 512 : 1024;
-    const auto kernel = threads == 512 ? select_stream<512> : select_stream<1024>;
-    const size_t dyn = (size_t)(threads / 32) * 2 * kStageQuads * sizeof(float4);
-    static bool attr_done[64][2] = {};
-    const int which = threads == 512 ? 0 : 1;
+    const int threads = sparse || inflight * Lmax * 4 <= (96ll << 20) ? 512 : 1024;
+    const auto kernel = sparse ? select_stream<512, true> : threads == 512 ? select_stream<512, false> : select_stream<1024, false>;
+    const size_t dyn = sparse ? (size_t)16 * 2 * kSparseQuads * sizeof(float4) + (size_t)kMaxSparseTiles * 4
+                              : (size_t)(threads / 32) * 2 * kStageQuads * sizeof(float4);
+    static bool attr_done[64][3] = {};
+    const int which = sparse ? 2 : threads == 512 ? 0 : 1;
     if (dev < 0 || dev >= 64) return JQ_ERR_CUDA;
     if (!attr_done[dev][which]) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return JQ_ERR_CUDA;
@@ -916,7 +967,7 @@ jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep
     if (cudaLaunchKernelEx(&cfg, kernel, scores, s.L, nkeep, (s.pool - 1) / 2, idx, pooled, (const uint4 *)K,
                            (const uint4 *)V, (uint4 *)Kout, (uint4 *)Vout, tables ? tables->heads : nullptr,
                            (const uint4 *const *)(tables && Kout ? tables->K : nullptr),
-                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, win, ext JQ_DBG_ARG) != cudaSuccess) {
+                           (const uint4 *const *)(tables && Kout ? tables->V : nullptr), src_rows, out_rows, win, sparse ? *sparse : ScoredTiles(), ext JQ_DBG_ARG) != cudaSuccess) {
         cudaGetLastError();
         return JQ_ERR_CUDA;
     }
@@ -926,9 +977,11 @@ jq_status launch_select_stream(const float *scores, const jq_shape &s, int nkeep
 
 }  // namespace
 
+bool select_reads_scored_tiles(const jq_shape &s, int max_L) { return s.Hkv >= kStreamMinHeads && (s.pool - 1) / 2 <= 4 && max_L <= 128 * kMaxSparseTiles; }
+
 jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, float *pooled,
                         const Workspace &w, cudaStream_t st, const void *K, const void *V, void *Kout, void *Vout,
-                        const UnitTables *tables, int src_head_rows, int out_head_rows, const void *Kwin, const void *Vwin)
+                        const UnitTables *tables, int src_head_rows, int out_head_rows, const void *Kwin, const void *Vwin, const ScoredTiles *sparse)
 {
     const int src_rows = src_head_rows > s.L ? src_head_rows : s.L;
     // with tables: the plan and the shared memory follow the longest head; every head reads its own record
@@ -945,7 +998,7 @@ jq_status launch_select(const float *scores, const jq_shape &s, int32_t *idx, fl
         const int sms = device_sms();
         int dev = 0;
         if (sms < 1 || cudaGetDevice(&dev) != cudaSuccess) return JQ_ERR_CUDA;
-        return launch_select_stream(scores, s, nkeep, Lmax, idx, pooled, st, K, V, Kout, Vout, sms, dev, tables, src_rows, out_rows, win, ext);
+        return launch_select_stream(scores, s, nkeep, Lmax, idx, pooled, st, K, V, Kout, Vout, sms, dev, tables, src_rows, out_rows, win, sparse, ext);
     }
     return launch_select_cluster(scores, s, nkeep, Lmax, idx, pooled, w, st, K, V, Kout, Vout, tables, src_rows, out_rows, win, ext);
 }
