@@ -3,10 +3,10 @@
 //
 // What bounds it: the single read of the two compacted arrays (2 * Hkv * n * 256 bytes) when there are many heads,
 // and the latency of one such read plus the merge when there are few.  So a KV head is one thread-block CLUSTER of
-// 1 to 16 CTAs of eight warps; a warp takes units of 16 keys, keeps a running softmax of its own and never waits for
+// 1 to 16 CTAs of eight or twelve warps; a warp takes units of 16 keys, keeps a running softmax of its own and never waits for
 // another warp before the merge, and both the K and the V rows of a unit go straight from global memory into
 // matrix-instruction fragments (no staging in shared memory, no barrier in the loop: 16 independent 16-byte loads
-// per lane and unit; 182 registers, one CTA to an SM: at 128 registers and two CTAs the spills cost more than they gave).
+// per lane and unit; one CTA to an SM: at 128 registers and two CTAs the spills cost more than they gave).
 //   - logits: S[16 keys x 8 heads] = K q^T, mma.sync m16n8k16.  The order of the 128 dimensions within a dot product is
 //     free, so a lane takes 16 contiguous bytes of a key row as the operands of two steps, and q is permuted alike.
 //     bf16 products, fp32 accumulation.
@@ -15,11 +15,11 @@
 //     product for each; groups of at most 4 heads repeat their heads in the other four columns and so carry two of the
 //     three parts in one product.  (With FMAs the group's 2 x 128 multiply-adds per key and head would bind, and with the
 //     heads as rows of the products, half of them empty, the loop took a quarter longer.)
-//   - merge: the eight warps' (m, l, O) through shared memory, then every CTA pushes its share of each output to the
+//   - merge: the warps' (m, l, O) through shared memory, then every CTA pushes its share of each output to the
 //     CTA of the cluster that writes it (distributed shared memory), one cluster barrier, and the sums are taken in
 //     rank order: deterministic, one launch, no counters in memory.
 // Measured (B200, back-to-back calls; before: one CTA per 64 keys staged in shared memory, FMAs, partials and a ticket in
-// global memory): 8 KV heads x 1024 keys 12.3 -> 4.6 us (latency: 0.9 TB/s), 128 x 2048 186 -> 27 us (4.95 TB/s, 0.77 of
+// global memory): 8 KV heads x 1024 keys 12.3 -> 4.6 us (latency: 0.9 TB/s), 128 x 2048 186 -> 25.2 us (5.3 TB/s, 0.81 of
 // the measured copy bandwidth).
 #include <cuda_bf16.h>
 #include <mutex>
@@ -31,19 +31,19 @@ namespace jq {
 namespace {
 
 constexpr int kDecChunk = 64;       // sizes the caller's workspace (part of the ABI; this kernel keeps its partials on chip)
-constexpr int kDecWarps = 8;
+constexpr int kDecWarps = 8, kDecManyWarps = 12;   // (decode_shape)
 constexpr int kDecResident = 1;     // CTAs per SM
-constexpr int kDecThreads = 32 * kDecWarps;
 constexpr int kDecUnit = 16;        // keys a warp takes at a time
 constexpr int kDecMaxGroup = 8;     // query heads per KV head
 constexpr int kDecMaxCluster = 16;  // CTAs per KV head (more than 8 needs the kernel's opt-in)
 constexpr int kPartial = kD + 2;    // floats per (chunk, head) of the caller's workspace
 constexpr int kOPad = kD + 4;       // row pitch (floats) of a warp's output tile in shared memory
 
+template <int kWarps>
 struct DecSmem {
     __nv_bfloat16 q[kDecMaxGroup * kD];
-    float O[kDecWarps][kDecMaxGroup][kOPad];
-    float m[kDecWarps][kDecMaxGroup], l[kDecWarps][kDecMaxGroup];
+    float O[kWarps][kDecMaxGroup][kOPad];
+    float m[kWarps][kDecMaxGroup], l[kWarps][kDecMaxGroup];
     // what the cluster's CTAs push here: rank r's statistics of every head, and its share of the outputs written here
     float rm[kDecMaxCluster][kDecMaxGroup], rl[kDecMaxCluster][kDecMaxGroup];
     float rO[kDecMaxGroup * kD + kDecMaxCluster];   // [rank][share]: the shares of all ranks make up the head's outputs
@@ -91,19 +91,20 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t v)   // 8 x 8 matrix o
 
 // DUP (groups of at most 4 heads): columns 4 to 7 of the matrix products repeat the heads 0 to 3, so that one product
 // carries two of the three parts of P.
-template <bool DUP>
-__global__ void __launch_bounds__(kDecThreads, kDecResident)
+template <bool DUP, int kWarps>
+__global__ void __launch_bounds__(32 * kWarps, kDecResident)
 decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
             int group, float scale_log2, float *__restrict__ out JQ_DBG_PARAM)
 {
     extern __shared__ __align__(16) uint8_t dec_raw[];
-    DecSmem &sm = *(DecSmem *)dec_raw;
+    DecSmem<kWarps> &sm = *(DecSmem<kWarps> *)dec_raw;
+    constexpr int kThreads = 32 * kWarps;
     uint32_t rank, C;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int kv = blockIdx.x / C;
-    const int nunits = (n + kDecUnit - 1) / kDecUnit, stride = (int)C * kDecWarps;
+    const int nunits = (n + kDecUnit - 1) / kDecUnit, stride = (int)C * kWarps;
     const long long n_rows = (long long)(gridDim.x / C) * n;   // extent, for the bounds-checked build
     (void)n_rows;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // waited for before the first push
@@ -111,7 +112,7 @@ decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
     cudaTriggerProgrammaticLaunchCompletion();   // the stream's next kernel may be set up; it waits for this one's results
 
     const size_t head = (size_t)kv * n;
-    int u = (int)rank * kDecWarps + warp;
+    int u = (int)rank * kWarps + warp;
     uint4 kf[8], vf[8];
     // K: rows g and 8 + g of the unit, 16-byte pieces t, 4 + t, 8 + t, 12 + t (rows past the end are masked below)
     auto load_k = [&](int uu) {
@@ -136,7 +137,7 @@ decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
         }
     };
     if (u < nunits) { load_k(u); load_v(u); }
-    for (int i = tid; i < kDecMaxGroup * kD; i += kDecThreads) {   // (q may be aligned to 2 bytes only)
+    for (int i = tid; i < kDecMaxGroup * kD; i += kThreads) {   // (q may be aligned to 2 bytes only)
         const int src = DUP ? i & (4 * kD - 1) : i;
         sm.q[i] = src < group * kD && JQ_IN(kv * group * kD + src, (long long)(gridDim.x / C) * group * kD, kDbgDecode, 2)
                       ? q[(size_t)kv * group * kD + src] : __float2bfloat16(0.f);
@@ -218,7 +219,7 @@ decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
         l[c] += __shfl_xor_sync(0xffffffffu, l[c], 16);
     }
 
-    // ---- the eight warps of the CTA
+    // ---- the warps of the CTA
     if (g == 0) {
         sm.m[warp][2 * t] = m[0]; sm.m[warp][2 * t + 1] = m[1];
         sm.l[warp][2 * t] = l[0]; sm.l[warp][2 * t + 1] = l[1];
@@ -232,14 +233,14 @@ decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
     __syncthreads();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA of the cluster runs: its memory may be written
     const int items = group * kD, share = (items + (int)C - 1) / (int)C;
-    for (int it = tid; it < items; it += kDecThreads) {
+    for (int it = tid; it < items; it += kThreads) {
         const int h = it / kD, c = it - h * kD;
         float M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < kDecWarps; ++w) M = fmaxf(M, sm.m[w][h]);
+        for (int w = 0; w < kWarps; ++w) M = fmaxf(M, sm.m[w][h]);
         float O = 0.f, Ls = 0.f;
 #pragma unroll
-        for (int w = 0; w < kDecWarps; ++w) {
+        for (int w = 0; w < kWarps; ++w) {
             // a warp without keys has m = -inf and adds nothing (M is -inf too when the whole CTA has none)
             const float f = sm.m[w][h] > -INFINITY ? dec_ex2(sm.m[w][h] - M) : 0.f;
             O = fmaf(DUP ? sm.O[w][h][c] + sm.O[w][h + 4][c] : sm.O[w][h][c], f, O);
@@ -251,7 +252,7 @@ decode_step(const uint4 *Kc, const uint4 *Vc, const __nv_bfloat16 *q, int n,
     }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    for (int i = tid; i < share; i += kDecThreads) {
+    for (int i = tid; i < share; i += kThreads) {
         const int it = (int)rank * share + i, h = it / kD;
         if (it >= items) break;
         float M = -INFINITY, O = 0.f, Ls = 0.f;
@@ -283,19 +284,21 @@ bool decode_plan(DecPlan *out)
     std::lock_guard<std::mutex> lock(mu);
     DecPlan &p = plans[dev];
     if (!p.ready) {
-        for (auto k : {decode_step<true>, decode_step<false>})
+        for (auto k : {decode_step<true, kDecWarps>, decode_step<false, kDecWarps>, decode_step<true, kDecManyWarps>, decode_step<false, kDecManyWarps>})
             if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+        for (auto k : {decode_step<true, kDecManyWarps>, decode_step<false, kDecManyWarps>})   // (eight warps need less than 48 KB)
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecSmem<kDecManyWarps>)) != cudaSuccess) return false;
         for (int C = 1; C <= kDecMaxCluster; ++C) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)C);
-            cfg.blockDim = dim3(kDecThreads);
-            cfg.dynamicSmemBytes = sizeof(DecSmem);
+            cfg.blockDim = dim3(32 * kDecManyWarps);
+            cfg.dynamicSmemBytes = sizeof(DecSmem<kDecManyWarps>);
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&p.resident[C], decode_step<true>, &cfg) != cudaSuccess) { cudaGetLastError(); p.resident[C] = 0; }
+            if (cudaOccupancyMaxActiveClusters(&p.resident[C], decode_step<true, kDecManyWarps>, &cfg) != cudaSuccess) { cudaGetLastError(); p.resident[C] = 0; }
         }
         if (p.resident[1] < 1) return false;
         p.ready = true;
@@ -304,18 +307,25 @@ bool decode_plan(DecPlan *out)
     return true;
 }
 
-int decode_cluster(int Hkv, int n, const DecPlan &p)
+// A CTA has eight warps or twelve: with twelve more of the cache is on its way at a time, which pays where a warp walks through several
+// units (the loop is bound by what a CTA has in flight, 8 KB per warp; a round of units then takes 1.3 times as long), and the merge
+// is larger.  Measured with 8 and 12 warps: 128 heads x 2048 keys 27.2, 25.2 us, 100 x 3000 35.3, 30.1, 90 x 2048 25.8, 22.0,
+// 140 x 4096 49.7, 46.7, 128 x 512 10.9, 10.7; 8 x 1024 5.1, 5.6, 149 x 256 13.1, 13.5.  (Ten: 26.0, 32.1, 23.3, 48.2.)
+struct DecShape { int C; bool many; };
+DecShape decode_shape(int Hkv, int n, const DecPlan &p)
 {
     const int nunits = (n + kDecUnit - 1) / kDecUnit;
-    int best = 1;
-    double best_cost = 0;
-    for (int C = 1; C <= kDecMaxCluster; ++C) {
-        if (p.resident[C] < 1) continue;
-        const int per = kDecWarps * C;
-        const double cost = (double)((Hkv + p.resident[C] - 1) / p.resident[C]) * (3.3 + (nunits + per - 1) / per);
-        // (at equal cost a power of two: the outputs then divide evenly over the CTAs)
-        if (C == 1 || cost < best_cost || (cost == best_cost && (C & (C - 1)) == 0 && (best & (best - 1)) != 0)) { best = C; best_cost = cost; }
-    }
+    DecShape best = {1, false};
+    double best_cost = 1e30;
+    for (int many = 0; many < 2; ++many)
+        for (int C = 1; C <= kDecMaxCluster; ++C) {
+            if (p.resident[C] < 1) continue;
+            const int per = (many ? kDecManyWarps : kDecWarps) * C, units = (nunits + per - 1) / per, rounds = (Hkv + p.resident[C] - 1) / p.resident[C];
+            const double cost = rounds * (many ? 3.35 + 1.3 * units : 3.3 + units) + (rounds > 1 ? 1.0 : 0.0);
+            // (at equal cost a power of two: the outputs then divide evenly over the CTAs)
+            if (cost < best_cost || (cost == best_cost && (C & (C - 1)) == 0 && (best.C & (best.C - 1)) != 0)) { best = {C, many != 0}; best_cost = cost; }
+            if (units == 1) break;   // (more CTAs have nothing to do)
+        }
     return best;
 }
 
@@ -342,12 +352,14 @@ extern "C" jq_status jq_decode_attention(const void *Kc, const void *Vc, const v
     if (!workspace || workspace_bytes < need) return JQ_ERR_WORKSPACE;
     DecPlan plan;
     if (!decode_plan(&plan)) return JQ_ERR_CUDA;
-    const int C = decode_cluster(Hkv, n, plan);
+    const DecShape shape = decode_shape(Hkv, n, plan);
+    const int C = shape.C;
+    const bool many = shape.many;
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)kD);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(Hkv * C));
-    cfg.blockDim = dim3(kDecThreads);
-    cfg.dynamicSmemBytes = sizeof(DecSmem);
+    cfg.blockDim = dim3(32 * (many ? kDecManyWarps : kDecWarps));
+    cfg.dynamicSmemBytes = many ? sizeof(DecSmem<kDecManyWarps>) : sizeof(DecSmem<kDecWarps>);
     cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -356,7 +368,8 @@ extern "C" jq_status jq_decode_attention(const void *Kc, const void *Vc, const v
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, group <= 4 ? decode_step<true> : decode_step<false>, (const uint4 *)Kc, (const uint4 *)Vc, (const __nv_bfloat16 *)q, n, group, scale_log2,
+    if (cudaLaunchKernelEx(&cfg, many ? (group <= 4 ? decode_step<true, kDecManyWarps> : decode_step<false, kDecManyWarps>)
+                                         : (group <= 4 ? decode_step<true, kDecWarps> : decode_step<false, kDecWarps>), (const uint4 *)Kc, (const uint4 *)Vc, (const __nv_bfloat16 *)q, n, group, scale_log2,
                            out JQ_DBG_ARG) != cudaSuccess) {
         cudaGetLastError();
         return JQ_ERR_CUDA;
