@@ -173,8 +173,10 @@ jq_status jq_compact_kv(const void *K, const void *V, const int32_t *kept_idx,
 
 /*
  * The whole pass for one layer, with the results of jq_score -> jq_select_topk -> jq_compact_kv, on one
- * stream: in one launch for short prefixes (at most 12288 keys, where that is the faster way), else in two
- * (the selection kernel also copies the kept rows).  Scores are not handed out.  K may hold several layers of equal shape stacked along the KV-head axis (Hkv = layers x
+ * stream: in one launch for short prefixes (at most 12288 keys, where that is the faster way); in four where
+ * a small share of many keys is kept (one pass over K, bounds, the scores of the keys that can be kept, the
+ * selection); else in two (both passes over K; the selection kernel also copies the kept rows).  Scores are
+ * not handed out.  K may hold several layers of equal shape stacked along the KV-head axis (Hkv = layers x
  * heads per layer, Qwin stacked alike): heads are independent, so one call evicts them all.
  */
 jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const jq_shape *shape,
@@ -182,7 +184,7 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
                          jq_stream_t stream);
 
 /*
- * The pass over several units in ONE call of two launches.  A unit is a layer of a cache, or a layer of one
+ * The pass over several units in ONE call (of two or four launches, as jq_evict_layer).  A unit is a layer of a cache, or a layer of one
  * sequence of a batch: K, V [Hkv, L_u, d] and Qwin [Hq, w, d] in buffers of its own, with a prefix length L_u
  * and a budget B_u of its own; all units share the head geometry of `common` (Hkv, Hq, group, d, w, pool).
  * (Every (unit, KV head) is an independent instance of the pass of the inference section; lengths that differ
@@ -270,7 +272,7 @@ jq_status jq_decode_attention(const void *Kc, const void *Vc, const void *q, int
  * below n_old are old rows).  Rows [nkeep, cap) are unspecified afterwards.  The results of jq_evict_layer on
  * the concatenated tensors.  ws: at least jq_append_workspace_bytes(shape) bytes (it also holds the compacted
  * rows before they are moved to the head of the cache), first 256 bytes initialised by jq_workspace_init.
- * One launch for short caches (as jq_evict_layer), else two launches and up to six strided device copies, all
+ * One launch for short caches, else two or four (as jq_evict_layer) and up to six strided device copies, all
  * on `stream`.
  */
 size_t jq_append_workspace_bytes(const jq_shape *shape);
