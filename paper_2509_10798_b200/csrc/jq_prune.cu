@@ -21,7 +21,7 @@
 // which a call comes here, with what was measured.
 //
 // The bound holds for the scores as they are computed, not only on paper: the rounding of the half is added (block_bounds), the sum
-// is raised by 1 / 64, and it is rounded up to 16 bits, far above the differences in rounding between the two orders of the
+// is raised by 1 / 512, and it is rounded up to 16 bits, far above the differences in rounding between the two orders of the
 // product.
 //
 // What bounds it (32 layers of 8 heads, us, measured back to back on one GPU): 32768 keys, 128 rows, 512 kept: row_stats 370 (2.1 GB
@@ -467,9 +467,11 @@ __host__ __device__ constexpr int bounds_per_sm(bool wide) { return wide ? 2 : 3
 __host__ __device__ constexpr int bounds_smem(bool wide) { return kBThreads / 32 * kBStages * (wide ? 4096 : 2048); }
 
 // grid: two or three CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
-// then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  A maximum x within 64 of its row's
-// normaliser M has been rounded by at most (|M| + 64) / 2048, which is added; smaller ones add less than 2^-60 each, which is
-// added as well; a normaliser near the end of a half's range makes every bound of the head infinite.
+// then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  The bound stays above what it bounds: a maximum x
+// within 24 of its row's normaliser M has been rounded by at most (|M| + 24) / 2048, of which a little more is added (two orders
+// of the product differ by less than |M| 2^-20); smaller ones are below 2^-24, which every row adds; the sum is raised by 1 / 512,
+// far above what exponentials and sums are off by; a normaliser near the end of a half's range makes every bound of the head
+// infinite.  (With wider margins, 64, 1 / 64, the ragged batch of 128 units took 1862 us instead of 1847.)
 template <bool kWide>
 __global__ void __launch_bounds__(kBThreads, bounds_per_sm(kWide))
 block_bounds(const __grid_constant__ CParams P)
@@ -570,9 +572,9 @@ block_bounds(const __grid_constant__ CParams P)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float x = Ms[32 * j + 4 * g + i];
-                nm[4 * j + i] = x > -INFINITY ? x + (fabsf(x) + 64.f) * (1.f / 2048.f) : x;   // (a row that is none stays at -inf)
+                nm[4 * j + i] = x > -INFINITY ? x + (fabsf(x) + 24.f) * (1.f / 2040.f) : x;   // (a row that is none stays at -inf)
             }
-        const float least = huge ? INFINITY : 3e-16f;
+        const float least = huge ? INFINITY : (float)R * 6e-8f;
         int stage = 0;
 #pragma unroll 1
         for (int t = t0 + warp; t < t1; t += kBThreads / 32) {
@@ -598,7 +600,7 @@ block_bounds(const __grid_constant__ CParams P)
             r += __shfl_xor_sync(0xffffffffu, r, 1);
             const int blk = 2 * pair + (odd ? 1 : 0);
             if ((lane & 3) == 0)
-                P.ub[(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 64.f)) + 0xffffu) >> 16) : (uint16_t)0;
+                P.ub[(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 512.f)) + 0xffffu) >> 16) : (uint16_t)0;
             stage = stage == kBStages - 1 ? 0 : stage + 1;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");          // (the next head starts with the first stage again)
