@@ -46,11 +46,16 @@ static jq_status check_ws(const jq_shape *s, void *ws, size_t ws_bytes, Workspac
     return ws_bytes < out->bytes ? JQ_ERR_WORKSPACE : JQ_OK;
 }
 
-// Whether one pass over the keys and a look at the candidates is the faster way for a layer.
-static bool layer_pruned(const jq_shape &s)
+// Whether one pass over the keys and a look at the candidates is the faster way for a layer, and the workspace has room for it; it is
+// then laid out for that (w.prune).
+static bool layer_pruned(const jq_shape &s, void *ws, size_t ws_bytes, Workspace *w)
 {
     const long long tiles = (long long)s.Hkv * ((s.L + 127) / 128), keys = (long long)s.Hkv * s.L;
-    return prune_taken(s, s.Hkv, tiles, keys, (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L), s.L);
+    if (!prune_taken(s, s.Hkv, tiles, keys, (long long)s.Hkv * (s.budget < s.L ? s.budget : s.L), s.L)) return false;
+    const Workspace p = carve_pruned(ws, (size_t)s.Hkv, (size_t)s.group * s.w, (size_t)keys);
+    if (ws_bytes < p.bytes) return false;
+    *w = p;
+    return true;
 }
 
 // One layer that the one-launch pass does not take.  src_head_rows, out_head_rows: rows between consecutive heads of K and V / of Kout
@@ -59,7 +64,7 @@ static jq_status evict_in_steps(const void *K, const void *V, const void *Qwin, 
                                 const Workspace &w, cudaStream_t st, int src_head_rows = 0, int out_head_rows = 0,
                                 const void *Kwin = nullptr, const void *Vwin = nullptr)
 {
-    if (layer_pruned(s))
+    if (w.prune)
         return launch_evict_pruned(K, V, Qwin, s, Kout, Vout, kept_idx, w, st, nullptr, src_head_rows, out_head_rows, Kwin, Vwin);
     const jq_status rc = launch_score_tc(K, Qwin, s, w.scores, w, st, Kwin, nullptr, src_head_rows);
     if (rc != JQ_OK) return rc;
@@ -77,7 +82,7 @@ jq_status jq_check_shape(const jq_shape *s) { return check_shape(s); }
 size_t jq_workspace_bytes(const jq_shape *s)
 {
     if (check_shape(s) != JQ_OK) return 0;
-    return carve(nullptr, *s).bytes;
+    return workspace_need(*s);
 }
 
 int jq_num_kept(const jq_shape *s)
@@ -132,7 +137,7 @@ jq_status jq_evict_layer_windowed(const void *K, const void *V, const void *Qwin
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin;
     bool taken = false;
-    if (!layer_pruned(*s) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
+    if (!layer_pruned(*s, ws, ws_bytes, &w) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
     return evict_in_steps(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st, 0, 0, Kwin);
 }
 
@@ -157,7 +162,7 @@ jq_status jq_evict_layer_window_kept(const void *K, const void *V, const void *Q
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L; src.Kwin = Kwin; src.Vwin = Vwin;
     bool taken = false;
-    if (!layer_pruned(sp) && ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
+    if (!layer_pruned(sp, ws, ws_bytes, &w) && ((rc = launch_fused(sp, src, Qwin, Kout, Vout, (int)nt, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
     // the kept prefix rows of head kv go to rows [kv * nt, kv * nt + np) of the outputs, its window rows behind them
     return evict_in_steps(K, V, Qwin, sp, Kout, Vout, kept_idx, w, st, 0, (int)nt, Kwin, Vwin);
 }
@@ -209,7 +214,7 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
     FusedSource src;
     src.KA = K; src.VA = V; src.LA = s->L;
     bool taken = false;
-    if (!layer_pruned(*s) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
+    if (!layer_pruned(*s, ws, ws_bytes, &w) && ((rc = launch_fused(*s, src, Qwin, Kout, Vout, 0, kept_idx, w, st, &taken)) != JQ_OK || taken)) return rc;
     return evict_in_steps(K, V, Qwin, *s, Kout, Vout, kept_idx, w, st);
 }
 
@@ -266,7 +271,7 @@ size_t jq_ragged_workspace_bytes(const jq_shape *common, int nunits, const int *
 {
     RaggedPlan pl;
     if (plan_ragged(common, nunits, L, nullptr, &pl) != JQ_OK) return 0;
-    return carve(nullptr, (size_t)pl.S.Hkv, (size_t)common->group * common->w, pl.keys).bytes + unit_tables_bytes(nunits, common->Hkv);
+    return workspace_need((size_t)pl.S.Hkv, (size_t)common->group * common->w, pl.keys, pl.max_L) + unit_tables_bytes(nunits, common->Hkv);
 }
 
 long long jq_ragged_output_rows(const jq_shape *common, int nunits, const int *L, const int *budget)
@@ -288,7 +293,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         if (!aligned16(K[u]) || !aligned16(V[u]) || !aligned16(Qwin[u])) return JQ_ERR_INVALID_ARG;
     if (!aligned16(ws) || ((uintptr_t)ws & 255u)) return JQ_ERR_INVALID_ARG;
     const int hpu = common->Hkv, R = common->group * common->w;
-    const Workspace w = carve(ws, (size_t)pl.S.Hkv, (size_t)R, pl.keys);
+    Workspace w = carve(ws, (size_t)pl.S.Hkv, (size_t)R, pl.keys);
     const size_t tab_bytes = unit_tables_bytes(nunits, hpu);
     if (ws_bytes < w.bytes + tab_bytes) return JQ_ERR_WORKSPACE;
     const int sms = score_sms();
@@ -308,7 +313,9 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     GroupRec *h_grp = (GroupRec *)(hb + grp_off);   // last: there are far fewer than there is room for
     UnitTables t;
     for (int u = 0; u < nunits; ++u) t.total_tiles += (long long)hpu * (((L ? L[u] : common->L) + 127) / 128);
-    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L);
+    const Workspace wp = carve_pruned(ws, (size_t)pl.S.Hkv, (size_t)R, pl.keys);
+    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L) && ws_bytes >= wp.bytes + tab_bytes;
+    if (pruned) w = wp;
     long long soff = 0, ooff = 0, tbase = 0;
     int ngroups = 0;
     for (int u = 0; u < nunits; ++u) {
@@ -383,7 +390,7 @@ size_t jq_append_workspace_bytes(const jq_shape *s)
 {
     if (check_shape(s) != JQ_OK) return 0;
     const size_t nkeep = (size_t)(s->budget < s->L ? s->budget : s->L);
-    return carve(nullptr, *s).bytes + 2 * align_up((size_t)s->Hkv * nkeep * s->d * 2, 256);
+    return workspace_need(*s) + 2 * align_up((size_t)s->Hkv * nkeep * s->d * 2, 256);
 }
 
 jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Knew, const void *Vnew, int n_new,
@@ -397,15 +404,16 @@ jq_status jq_evict_append(void *Kc, void *Vc, int cap, int n_old, const void *Kn
     if (n_new > 0 && (!aligned16(Knew) || !aligned16(Vnew))) return JQ_ERR_INVALID_ARG;
     Workspace w;
     if ((rc = check_ws(s, ws, ws_bytes, &w)) != JQ_OK) return rc;
-    if (ws_bytes < jq_append_workspace_bytes(s)) return JQ_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t row = (size_t)s->d * 2, nkeep = (size_t)(s->budget < s->L ? s->budget : s->L);
-    char *Ktmp = (char *)ws + w.bytes, *Vtmp = Ktmp + align_up((size_t)s->Hkv * nkeep * row, 256);
+    const size_t row = (size_t)s->d * 2, nkeep = (size_t)(s->budget < s->L ? s->budget : s->L), rows_bytes = align_up((size_t)s->Hkv * nkeep * row, 256);
+    if (ws_bytes < w.bytes + 2 * rows_bytes) return JQ_ERR_WORKSPACE;
     // a short cache: one launch that reads the two parts where they are and moves the kept rows in place
     FusedSource src;
     src.KA = Kc; src.VA = Vc; src.LA = n_old; src.a_rows = cap; src.KB = Knew; src.VB = Vnew; src.LB = n_new; src.inplace = true;
     bool taken;
     if ((rc = launch_fused(*s, src, Qrecent, Kc, Vc, cap, kept_idx, w, st, &taken)) != JQ_OK || taken) return rc;
+    layer_pruned(*s, ws, ws_bytes - 2 * rows_bytes, &w);
+    char *const Ktmp = (char *)ws + w.bytes, *const Vtmp = Ktmp + rows_bytes;
     // 1. the new rows go behind the retained ones, head by head (the cache keeps `cap` rows per head)
     if (n_new > 0) {
         if (cudaMemcpy2DAsync((char *)Kc + (size_t)n_old * row, (size_t)cap * row, Knew, (size_t)n_new * row, (size_t)n_new * row,
@@ -472,7 +480,7 @@ size_t jq_host_call_bytes(const jq_shape *s)
     b += align_up((size_t)s->Hq * s->w * row, 256);           // Qwin
     b += 2 * align_up((size_t)s->Hkv * nkeep * row, 256);     // Kout, Vout
     b += align_up((size_t)s->Hkv * nkeep * 4, 256) + kHostIdxPad;   // kept_idx, with room to align every chunk's
-    b += carve(nullptr, *s).bytes;
+    b += workspace_need(*s);
     return b;
 }
 
@@ -498,7 +506,7 @@ jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin,
     char *dVo = p;         p += align_up(ob, 256);
     char *dI = p;          p += align_up(ib, 256) + kHostIdxPad;
     char *ws = p;
-    const size_t wsb = carve(nullptr, *s).bytes;
+    const size_t wsb = workspace_need(*s);
     if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return JQ_ERR_CUDA;
     if (cudaMemcpyAsync(dQ, hQwin, qb, cudaMemcpyHostToDevice, st) != cudaSuccess) return JQ_ERR_CUDA;
     // V is read at the kept rows only.  A page-locked host buffer is mapped into the device's address space: the

@@ -18,7 +18,7 @@ struct Workspace {
     float2 *part;       // [Hkv][kSlots][R]   (raw max, sum of exp2(c*(s-max))) per contributing block
     float *scores;      // [Hkv][L]   pre-pool scores (of the two-launch path)
     uint32_t *keys;     // [Hkv][L]   order-preserving bit patterns of the pooled scores (of heads whose keys do not fit on chip)
-    void *prune;        // scratch of the one-pass scoring, in the place of Mrow and part (a call uses one or the other)
+    void *prune;        // scratch of the one-pass eviction, in the place of Mrow and part (carve_pruned; null otherwise)
     size_t bytes;       // total
 };
 // Bytes of that scratch for `tiles` tiles of keys in total (every head's rounded up, window tiles included).
@@ -35,12 +35,11 @@ static inline Workspace carve(void *base, size_t heads, size_t R, size_t keys)
     size_t off = 0;
     w.status = (int *)(p + off);
     off += align_up(kStatusWords * sizeof(int), 256);
-    const size_t mrow = align_up(heads * R * sizeof(float), 256), part = align_up(heads * kSlots * R * sizeof(float2), 256);
-    const size_t prune = prune_bytes((long long)(keys / 128 + 2 * heads), (int)heads, (int)R);
-    w.prune = p + off;
+    w.prune = nullptr;
     w.Mrow = (float *)(p + off);
-    w.part = (float2 *)(p + off + mrow);
-    off += mrow + part > prune ? mrow + part : prune;
+    off += align_up(heads * R * sizeof(float), 256);
+    w.part = (float2 *)(p + off);
+    off += align_up(heads * kSlots * R * sizeof(float2), 256);
     w.scores = (float *)(p + off);
     off += align_up(keys * sizeof(float), 256);
     w.keys = (uint32_t *)(p + off);
@@ -52,6 +51,33 @@ static inline Workspace carve(void *base, const jq_shape &s)
 {
     return carve(base, (size_t)s.Hkv, (size_t)s.group * s.w, (size_t)s.Hkv * s.L);
 }
+// The same for a call that takes the one-pass eviction.  Its scratch can be larger: a workspace that has room for carve() only is as
+// good as any, the call then goes the other way.
+static inline Workspace carve_pruned(void *base, size_t heads, size_t R, size_t keys)
+{
+    Workspace w = {};
+    char *p = (char *)base;
+    size_t off = 0;
+    w.status = (int *)(p + off);
+    off += align_up(kStatusWords * sizeof(int), 256);
+    w.prune = p + off;
+    off += prune_bytes((long long)(keys / 128 + 2 * heads), (int)heads, (int)R);
+    w.scores = (float *)(p + off);
+    off += align_up(keys * sizeof(float), 256);
+    w.keys = (uint32_t *)(p + off);
+    off += align_up(keys * sizeof(uint32_t), 256);
+    w.bytes = off;
+    return w;
+}
+// Bytes of a workspace with which a call over `heads` heads can go either way, whatever its budget.
+bool prune_possible(int heads, int R, long long keys, int max_L);
+static inline size_t workspace_need(size_t heads, size_t R, size_t keys, int max_L)
+{
+    const size_t a = carve(nullptr, heads, R, keys).bytes;
+    const size_t b = prune_possible((int)heads, (int)R, (long long)keys, max_L) ? carve_pruned(nullptr, heads, R, keys).bytes : 0;
+    return a > b ? a : b;
+}
+static inline size_t workspace_need(const jq_shape &s) { return workspace_need((size_t)s.Hkv, (size_t)s.group * s.w, (size_t)s.Hkv * s.L, s.L); }
 
 // Units (layers, sequences) of one head geometry living in buffers of their own, with prefix lengths and
 // budgets of their own (jq_evict_ragged, jq_evict_layers): tables in device memory, behind the workspace proper.

@@ -1007,13 +1007,21 @@ static double kept_per_block(int pool) { return pool >= 7 ? 7.0 : pool >= 3 ? 3.
 //   64 x 32768, 1.5 %, windows of 1, 3, 13               252 -> 262, 251 -> 179, 256 -> 164
 // With 8 query rows 64 x 32768 keys take 211 -> 141 (1 %), with 256 rows 371 -> 240.  Shorter heads than about 10000 keys gain little
 // and lose most where the bounds separate badly; fewer than 8 rows have not been measured and stay where they were.
+static double saved_per_tile(int R) { return R > 128 ? 9.0e-3 : R > 64 ? 6.2e-3 : 5.5e-3; }   // us
+constexpr double kPruneLeast = 30.0;                                                          // us that have to be saved
+
+bool prune_possible(int heads, int R, long long keys, int max_L)
+{
+    const long long tiles = keys / kPTile + heads;
+    return R >= 8 && tiles < (1ll << 30) && max_L <= kPBlock * kCMaxBlocks && keys >= 10000ll * heads && (double)tiles * saved_per_tile(R) >= kPruneLeast;
+}
+
 bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L)
 {
     const int R = s.group * s.w;
-    if (R < 8 || tiles >= (1ll << 30) || max_L > kPBlock * kCMaxBlocks || keys < 10000ll * heads) return false;
-    const double saved = R > 128 ? 9.0e-3 : R > 64 ? 6.2e-3 : 5.5e-3;              // us per tile
+    if (!prune_possible(heads, R, keys, max_L)) return false;
     const double share = (double)kept / (double)keys * 7.0 / kept_per_block(s.pool);
-    return (double)tiles * (saved - 0.08 * share) >= 30.0;
+    return (double)tiles * (saved_per_tile(R) - 0.08 * share) >= kPruneLeast;
 }
 
 jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const jq_shape &s, void *Kout, void *Vout, int32_t *idx,

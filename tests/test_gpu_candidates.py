@@ -159,6 +159,56 @@ def test_append_to_a_long_cache():
     check(K, V, Q, s, Kc[:, :budget], Vc[:, :budget], idx, (3,))
 
 
+def test_a_workspace_without_room_for_it_goes_the_other_way():
+    """What the two-pass kernels need is enough for every call, as it was: status, normalisers, partial statistics, scores, keys."""
+    Hkv, g, w, L, budget = 8, 4, 64, 65537, 500
+    K, V, Q = device_layer(Hkv, g, w, L, 4)
+    s = shape_of(wl_of(Hkv, g, w, L, budget))
+    up = lambda x: (x + 255) // 256 * 256
+    least = 256 + up(Hkv * g * w * 4) + up(Hkv * 640 * g * w * 8) + 2 * up(Hkv * L * 4)
+    assert least < jq.workspace_bytes(s)
+    kept = []
+    for size, launches in ((least, 2), (jq.workspace_bytes(s), LAUNCHES)):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        jq._raise("jq_workspace_init", jq.lib().jq_workspace_init(jq._ptr(ws), ws.numel(), jq._stream(None)))
+        Ko, Vo = (torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        idx = torch.full((Hkv, budget), -1, dtype=torch.int32, device="cuda")
+        n0 = jq.launch_count()
+        jq.evict_layer(K, V, Q, s, Ko, Vo, idx, ws)
+        assert jq.launch_count() - n0 == launches and jq.last_device_status(ws) == jq.JQ_OK
+        check(K, V, Q, s, Ko, Vo, idx, ())
+        kept.append(idx)
+    with pytest.raises(jq.JqError):
+        jq.evict_layer(K, V, Q, s, Ko, Vo, idx, torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+
+
+def test_in_a_graph_and_on_two_streams():
+    """Captured once and replayed on other inputs in the same buffers, while another stream evicts with a workspace of its own."""
+    Hkv, g, w, L, budget = 70, 1, 32, 11264, 64
+    s = shape_of(wl_of(Hkv, g, w, L, budget))
+    A, B, C = (device_layer(Hkv, g, w, L, i) for i in (1, 2, 3))
+    out = [[torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)] + [torch.zeros((Hkv, budget), dtype=torch.int32, device="cuda")] for _ in range(2)]
+    ws = [jq.new_workspace(s) for _ in range(2)]
+    buf = [x.clone() for x in A]
+    jq.evict_layer(*buf, s, *out[0], ws[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        jq.evict_layer(*buf, s, *out[0], ws[0])
+    for x, y in zip(buf, B):
+        x.copy_(y)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    for _ in range(20):
+        graph.replay()
+        with torch.cuda.stream(side):
+            jq.evict_layer(*C, s, *out[1], ws[1])
+    torch.cuda.synchronize()
+    for (K, V, Q), o, x in zip((B, C), out, ws):
+        assert jq.last_device_status(x) == jq.JQ_OK
+        check(K, V, Q, s, o[0], o[1], o[2], ())
+
+
 SWEEP = r'''
 import ctypes, os, sys
 import torch
