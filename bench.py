@@ -592,6 +592,7 @@ def run_ours(args):
                     "peak": peak, "peak_source": peak_src, "unit": "GB/s", "frac": need / call_s / 1e9 / peak, "traffic": None,
                     "bytes_per_launch": need, "ms_per_launch": call_s * 1e3,
                     "layer_formula_gbs": layer_gbs, "layer_frac_of_peak": layer_gbs / peak, "layer_frac_of_8tbs": layer_gbs / 8000.0,
+                    "layer_formula_note": "the formula counts two reads of K, of which this call does one and a small part of the other",
                     "ex2_unit": {"note": "one exponential per query row and key (row_stats); those of the bounds and of the candidates come on top",
                                  "achieved": n_exp1 / call_s / 1e9, "peak": ex2_peak, "unit": "Gexp/s", "frac": n_exp1 / call_s / 1e9 / ex2_peak},
                     "clock_normalised": {"what": "thousands of SM cycles per layer = time x SM MHz sampled while the loop ran", "step": step_kc},
