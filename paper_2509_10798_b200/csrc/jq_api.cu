@@ -2,6 +2,7 @@
 #include "jq_internal.cuh"
 #include <algorithm>
 #include <atomic>
+#include <exception>
 #include <vector>
 
 namespace jq {
@@ -304,7 +305,15 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     // All tables are assembled in one host buffer of the library's own (so that the caller's arrays are only read
     // before the call returns, whatever memory they live in) and go to the device in as few copies as return at once.
     static thread_local std::vector<unsigned char> staging;
-    staging.assign(tab_bytes, 0);
+    static thread_local std::vector<int> order;           // the units by falling length
+    static thread_local std::vector<long long> out_row;   // [unit] its first output row
+    try {
+        staging.assign(tab_bytes, 0);
+        order.resize(nunits);
+        out_row.resize(nunits);
+    } catch (const std::exception &) {   // no host memory: nothing is thrown through the C interface
+        return JQ_ERR_CUDA;
+    }
     unsigned char *hb = staging.data();
     const size_t maps_bytes = align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256), ptr_bytes = align_up((size_t)nunits * sizeof(void *), 256);
     const size_t head_bytes = align_up((size_t)nunits * hpu * sizeof(HeadRec), 256), grp_off = maps_bytes + 2 * ptr_bytes + head_bytes;
@@ -322,9 +331,6 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     // order.  (32 layers of prompts of 32768, 23212, 13655 and 4099 keys, 8 heads each, in the order of the layers: 1920 -> 1865 us,
     // by rising length 1937 -> 1862, by falling length 1862 either way; with few rows, which go the two-pass way, 2095 -> 1835, 1837
     // -> 1826 and 1833.)
-    static thread_local std::vector<int> order;
-    static thread_local std::vector<long long> out_row;
-    order.resize(nunits); out_row.resize(nunits);
     long long soff = 0, ooff = 0, tbase = 0;
     for (int u = 0; u < nunits; ++u) {
         const int Lu = L ? L[u] : common->L, Bu = budget ? budget[u] : common->budget;
