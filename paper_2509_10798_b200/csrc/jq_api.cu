@@ -273,7 +273,8 @@ size_t jq_ragged_workspace_bytes(const jq_shape *common, int nunits, const int *
 {
     RaggedPlan pl;
     if (plan_ragged(common, nunits, L, nullptr, &pl) != JQ_OK) return 0;
-    return workspace_need((size_t)pl.S.Hkv, (size_t)common->group * common->w, pl.keys, pl.max_L) + unit_tables_bytes(nunits, common->Hkv);
+    const UnitTableLayout at = unit_tables(nunits, common->Hkv);
+    return workspace_need((size_t)pl.S.Hkv, (size_t)common->group * common->w, pl.keys, pl.max_L, at.bytes, at.prune_bytes);
 }
 
 long long jq_ragged_output_rows(const jq_shape *common, int nunits, const int *L, const int *budget)
@@ -296,8 +297,8 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     if (!aligned16(ws) || ((uintptr_t)ws & 255u)) return JQ_ERR_INVALID_ARG;
     const int hpu = common->Hkv, R = common->group * common->w;
     Workspace w = carve(ws, (size_t)pl.S.Hkv, (size_t)R, pl.keys);
-    const size_t tab_bytes = unit_tables_bytes(nunits, hpu);
-    if (ws_bytes < w.bytes + tab_bytes) return JQ_ERR_WORKSPACE;
+    const UnitTableLayout at = unit_tables(nunits, hpu);
+    if (ws_bytes < w.bytes + at.bytes) return JQ_ERR_WORKSPACE;
     const int sms = score_sms();
     if (sms < 1) return JQ_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
@@ -308,23 +309,22 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     static thread_local std::vector<int> order;           // the units by falling length
     static thread_local std::vector<long long> out_row;   // [unit] its first output row
     try {
-        staging.assign(tab_bytes, 0);
+        staging.assign(at.bytes > at.prune_bytes ? at.bytes : at.prune_bytes, 0);
         order.resize(nunits);
         out_row.resize(nunits);
     } catch (const std::exception &) {   // no host memory: nothing is thrown through the C interface
         return JQ_ERR_CUDA;
     }
     unsigned char *hb = staging.data();
-    const size_t maps_bytes = align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256), ptr_bytes = align_up((size_t)nunits * sizeof(void *), 256);
-    const size_t head_bytes = align_up((size_t)nunits * hpu * sizeof(HeadRec), 256), grp_off = maps_bytes + 2 * ptr_bytes + head_bytes;
-    unsigned char *h_maps = hb;
-    const void **h_K = (const void **)(hb + maps_bytes), **h_V = (const void **)(hb + maps_bytes + ptr_bytes);
-    HeadRec *h_head = (HeadRec *)(hb + maps_bytes + 2 * ptr_bytes);
-    GroupRec *h_grp = (GroupRec *)(hb + grp_off);   // last: there are far fewer than there is room for
+    unsigned char *h_maps = hb + at.maps, *h_block_maps = hb + at.block_maps;
+    const void **h_K = (const void **)(hb + at.K), **h_V = (const void **)(hb + at.V);
+    HeadRec *h_head = (HeadRec *)(hb + at.heads);
+    GroupRec *h_grp = (GroupRec *)(hb + at.groups);   // last: there are far fewer than there is room for
+    long long *h_tbase = (long long *)(hb + at.tbase);
     UnitTables t;
     for (int u = 0; u < nunits; ++u) t.total_tiles += (long long)hpu * (((L ? L[u] : common->L) + 127) / 128);
     const Workspace wp = carve_pruned(ws, (size_t)pl.S.Hkv, (size_t)R, pl.keys);
-    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L) && ws_bytes >= wp.bytes + tab_bytes;
+    const bool pruned = prune_taken(*common, pl.S.Hkv, t.total_tiles, (long long)pl.keys, pl.rows, pl.max_L) && ws_bytes >= wp.bytes + at.prune_bytes;
     if (pruned) w = wp;
     // The tables hold the units by falling length (equal lengths as given), whatever the order of the call: the kernels that have a
     // CTA per head start the long heads first, and none of those is left to run by itself at the end.  Outputs stay in the call's
@@ -345,7 +345,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         const int nkeep = Bu < Lu ? Bu : Lu;
         unsigned char *const m = h_maps + (size_t)(kMapsPerUnit * i) * kTensorMapBytes;
         if (!make_tensor_map(m, K[u], Lu, hpu, 128) || !make_tensor_map(m + kTensorMapBytes, Qwin[u], R, hpu, R <= 128 ? 128 : 256) ||
-            (pruned && !make_tensor_map(m + 2 * kTensorMapBytes, K[u], Lu, hpu, 16)))
+            (pruned && !make_tensor_map(h_block_maps + (size_t)i * kTensorMapBytes, K[u], Lu, hpu, 16)))
             return JQ_ERR_CUDA;
         h_K[i] = K[u]; h_V[i] = V[u];
         for (int h = 0; h < hpu; ++h) {
@@ -353,7 +353,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
             r.L = Lu; r.nkeep = nkeep; r.unit = i; r.kv_in = h;
             r.soff = soff + (long long)h * Lu;
             r.ooff = out_row[u] + (long long)h * nkeep;
-            r.tbase = tbase + (long long)h * ((Lu + 127) / 128);
+            if (pruned) h_tbase[i * hpu + h] = tbase + (long long)h * ((Lu + 127) / 128);
         }
         tbase += (long long)hpu * ((Lu + 127) / 128);
         soff += (long long)hpu * Lu;
@@ -378,16 +378,18 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
     // Copies from ordinary host memory return at once up to 64 KB; a larger one waits for the stream to reach it, which kept
     // the host from preparing one call while the GPU worked on the one before (128 units: 1.5 ms in the call, and a gap of
     // about 90 us per call of 2.6 ms).
-    const size_t used = grp_off + (size_t)ngroups * sizeof(GroupRec);
+    const size_t used = !pruned ? at.groups + (size_t)ngroups * sizeof(GroupRec) : pl.uniform ? at.tbase : at.prune_bytes;
     for (size_t off = 0; off < used; off += kTablePiece)
         if (cudaMemcpyAsync(tab + off, hb + off, used - off < kTablePiece ? used - off : kTablePiece, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return JQ_ERR_CUDA;
-    t.maps = tab;
-    t.K = (const void *const *)(tab + maps_bytes);
-    t.V = (const void *const *)(tab + maps_bytes + ptr_bytes);
-    t.heads = (const HeadRec *)(tab + maps_bytes + 2 * ptr_bytes);
-    t.groups = (const GroupRec *)(tab + grp_off);
-    t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows; t.uniform = pl.uniform;
+    t.maps = tab + at.maps;
+    t.K = (const void *const *)(tab + at.K);
+    t.V = (const void *const *)(tab + at.V);
+    t.heads = (const HeadRec *)(tab + at.heads);
+    t.groups = (const GroupRec *)(tab + at.groups);
+    t.block_maps = tab + at.block_maps;
+    if (pruned && !pl.uniform) t.tbase = (const long long *)(tab + at.tbase);
+    t.ngroups = ngroups; t.hpu = hpu; t.max_L = pl.max_L; t.total_keys = (long long)pl.keys; t.total_rows = pl.rows;
     if (pruned) return launch_evict_pruned(nullptr, nullptr, nullptr, pl.S, Kout, Vout, kept_idx, w, st, &t);
     if ((rc = launch_score_tc(nullptr, nullptr, pl.S, w.scores, w, st, nullptr, &t)) != JQ_OK) return rc;
     return launch_select(w.scores, pl.S, kept_idx, nullptr, w, st, nullptr, nullptr, Kout, Vout, &t);

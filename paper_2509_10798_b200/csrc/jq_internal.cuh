@@ -71,10 +71,11 @@ static inline Workspace carve_pruned(void *base, size_t heads, size_t R, size_t 
 }
 // Bytes of a workspace with which a call over `heads` heads can go either way, whatever its budget.
 bool prune_possible(int heads, int R, long long keys, int max_L);
-static inline size_t workspace_need(size_t heads, size_t R, size_t keys, int max_L)
+// (tables, prune_tables: bytes of the tables behind it, either way)
+static inline size_t workspace_need(size_t heads, size_t R, size_t keys, int max_L, size_t tables = 0, size_t prune_tables = 0)
 {
-    const size_t a = carve(nullptr, heads, R, keys).bytes;
-    const size_t b = prune_possible((int)heads, (int)R, (long long)keys, max_L) ? carve_pruned(nullptr, heads, R, keys).bytes : 0;
+    const size_t a = carve(nullptr, heads, R, keys).bytes + tables;
+    const size_t b = prune_possible((int)heads, (int)R, (long long)keys, max_L) ? carve_pruned(nullptr, heads, R, keys).bytes + prune_tables : 0;
     return a > b ? a : b;
 }
 static inline size_t workspace_need(const jq_shape &s) { return workspace_need((size_t)s.Hkv, (size_t)s.group * s.w, (size_t)s.Hkv * s.L, s.L); }
@@ -84,7 +85,7 @@ static inline size_t workspace_need(const jq_shape &s) { return workspace_need((
 // KV heads are numbered through all units; unit u owns heads [u * hpu, (u + 1) * hpu).
 constexpr int kMaxUnits = 4096;
 constexpr size_t kTensorMapBytes = 128;
-constexpr int kMapsPerUnit = 3;
+constexpr int kMapsPerUnit = 2;
 // A head group of the scoring kernel: consecutive KV heads of one prefix length whose keys fit a share of the
 // L2.  A group may run over consecutive units of equal length (their scores are consecutive too).
 struct GroupRec {
@@ -103,26 +104,39 @@ struct HeadRec {
     int unit, kv_in;     // the unit and the head's index within it
     long long soff;      // offset (floats / keys) of the head's scores and select keys
     long long ooff;      // offset (rows) of the head's kept indices and compacted rows in the stacked outputs
-    long long tbase;     // tiles of the heads before it
 };
 struct UnitTables {
-    const void *maps = nullptr;          // device: [nunits][kMapsPerUnit] TMA tensor maps (K, Qwin, K in blocks of 16 keys)
+    const void *maps = nullptr;          // device: [nunits][kMapsPerUnit] TMA tensor maps (K, Qwin)
     const void *const *K = nullptr;      // device: [nunits] base of K
     const void *const *V = nullptr;      // device: [nunits] base of V
     const GroupRec *groups = nullptr;    // device: [ngroups]
     const HeadRec *heads = nullptr;      // device: [nunits * hpu]
+    // of the one-pass eviction only, which needs no groups:
+    const void *block_maps = nullptr;    // device: [nunits] TMA tensor maps of K in blocks of 16 keys
+    const long long *tbase = nullptr;    // device: [nunits * hpu] tiles of the heads before it (null: all heads have the same number)
     int ngroups = 0, hpu = 0;            // hpu: KV heads per unit
     int max_group_tiles = 0;             // most tiles in any group (sizes the grid)
     int max_L = 0;                       // longest prefix (sizes the selection kernel's shared memory)
     long long total_keys = 0;            // keys of all units (floats in the scores array)
     long long total_rows = 0;            // rows of the stacked outputs
     long long total_tiles = 0;           // tiles of all heads
-    bool uniform = false;                // one length and one number of kept rows for all units
 };
-static inline size_t unit_tables_bytes(int nunits, int hpu)
+// Where the tables lie, from their first byte on: what both ways of a call read, then the groups of the two passes or the two tables
+// of the one-pass eviction.  A workspace with room for the tables of the two passes is enough for every call.
+struct UnitTableLayout {
+    size_t maps = 0, K, V, heads, groups, block_maps, tbase, bytes, prune_bytes;
+};
+static inline UnitTableLayout unit_tables(int nunits, int hpu)
 {
-    return align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256) + 2 * align_up((size_t)nunits * sizeof(void *), 256) +
-           align_up((size_t)nunits * hpu * sizeof(GroupRec), 256) + align_up((size_t)nunits * hpu * sizeof(HeadRec), 256);
+    UnitTableLayout t;
+    t.K = align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256);
+    t.V = t.K + align_up((size_t)nunits * sizeof(void *), 256);
+    t.heads = t.V + align_up((size_t)nunits * sizeof(void *), 256);
+    t.groups = t.block_maps = t.heads + align_up((size_t)nunits * hpu * sizeof(HeadRec), 256);
+    t.bytes = t.groups + align_up((size_t)nunits * hpu * sizeof(GroupRec), 256);
+    t.tbase = t.block_maps + align_up((size_t)nunits * kTensorMapBytes, 256);
+    t.prune_bytes = t.tbase + align_up((size_t)nunits * hpu * sizeof(long long), 256);
+    return t;
 }
 // One tensor map for a bf16 tensor [heads][rows][128], boxes of 64 columns x box_rows rows (host).
 // (head_rows: rows between consecutive heads in memory when they are not packed).
@@ -155,7 +169,8 @@ jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float
 // and none of the positions that are kept is further than a window from one that is set.
 struct ScoredTiles {
     const uint8_t *bits = nullptr;   // device: a byte per tile of 128 positions, heads one after the other
-    int tph = 0;                     // tiles from one head's first to the next head's (without tables)
+    const long long *tbase = nullptr;   // device: a head's first tile; null: tph of them from one head to the next
+    int tph = 0;
     int max_tiles = 0;               // of any head
 };
 constexpr int kMaxSparseTiles = 1024;   // (their list is in shared memory; two CTAs to an SM)

@@ -76,8 +76,9 @@ struct SParams {
     float2 *part;              // [(CTA + head) * groups + group][R]: the statistics of one CTA's share of a head
     uint32_t *bmax;            // [tile][4][Rpad]: maxima of two blocks of 16 keys each, as halves, times c
     int *status;
-    const HeadRec *htab;       // units in buffers of their own: lengths and first tiles of the heads,
-    const CUtensorMap *maps;   // [units][kMapsPerUnit] tensor maps (K, Qwin, K in blocks)
+    const HeadRec *htab;       // heads of different lengths or budgets (null otherwise): their records,
+    const long long *tbase;    // and first tiles
+    const CUtensorMap *maps;   // units in buffers of their own: [units][kMapsPerUnit] tensor maps (K, Qwin)
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
     long long n_part, n_bmax;
@@ -86,16 +87,16 @@ struct SParams {
 
 // The head that tile `tile` of T belongs to: the last one whose first tile is not past it.  Heads of one length, or nearly, are found
 // at once; the search through the others is a chain of reads from memory.
-__device__ __forceinline__ int head_of_tile(const HeadRec *htab, int heads, long long T, long long tile)
+__device__ __forceinline__ int head_of_tile(const long long *tbase, int heads, long long T, long long tile)
 {
     int lo = 0, hi = heads - 1;
     const int guess = min((int)(tile * heads / T), hi);
-    const long long here = htab[guess].tbase, next = guess < hi ? htab[guess + 1].tbase : T;
+    const long long here = tbase[guess], next = guess < hi ? tbase[guess + 1] : T;
     if (here <= tile && tile < next) return guess;
     if (here <= tile) lo = guess + 1; else hi = guess - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (htab[mid].tbase <= tile) lo = mid; else hi = mid - 1;
+        if (tbase[mid] <= tile) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -117,8 +118,8 @@ struct Walk {
             t = (int)(tile - (long long)h * P.tph);
             return;
         }
-        h = head_of_tile(P.htab, P.heads, P.T, tile);
-        t = (int)(tile - P.htab[h].tbase);
+        h = head_of_tile(P.tbase, P.heads, P.T, tile);
+        t = (int)(tile - P.tbase[h]);
         load(P);
     }
     __device__ __forceinline__ void advance(const SParams &P, int n)   // (never past the last tile of the call)
@@ -383,7 +384,8 @@ struct CParams {
     float *scores;
     int *status;
     const HeadRec *htab;
-    const CUtensorMap *maps;
+    const long long *tbase;
+    const CUtensorMap *maps, *block_maps;   // block_maps: [units]
     long long n_scores;        // floats in the scores array
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
@@ -402,7 +404,7 @@ __device__ __forceinline__ HeadAt head_at(const CParams &P, int h)
     HeadAt a;
     if (P.htab) {
         const HeadRec *r = P.htab + h;
-        a.L = r->L; a.nkeep = r->nkeep; a.soff = r->soff; a.tbase = r->tbase;
+        a.L = r->L; a.nkeep = r->nkeep; a.soff = r->soff; a.tbase = P.tbase[h];
         a.tph1 = (a.L + kPTile - 1) / kPTile;
     } else {
         a.L = P.L; a.nkeep = P.nkeep; a.soff = (long long)h * P.L; a.tbase = (long long)h * P.tph; a.tph1 = P.tph;
@@ -494,7 +496,7 @@ block_bounds(const __grid_constant__ CParams P)
     const long long G = gridDim.x;
     long long f = blockIdx.x * P.T / G;
     const long long end = (blockIdx.x + 1) * P.T / G;
-    int h = P.htab ? head_of_tile(P.htab, P.heads, P.T, f) : (int)(f / P.tph);
+    int h = P.htab ? head_of_tile(P.tbase, P.heads, P.T, f) : (int)(f / P.tph);
 #pragma unroll 1
     for (; f < end; ++h) {
         const HeadAt a = head_at(P, h);
@@ -698,7 +700,7 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     if (P.maps) {
         const int unit = head / P.hpu;
         kv_in = head - unit * P.hpu;
-        mq = P.maps + kMapsPerUnit * (size_t)unit + 1; mb = mq + 1;
+        mq = P.maps + kMapsPerUnit * (size_t)unit + 1; mb = P.block_maps + unit;
     }
     const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
     const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
@@ -1049,7 +1051,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     if (tables) {
         memset(&mapK, 0, sizeof mapK);
         mapQ = mapW = mapB = mapK;
-        S.htab = tables->uniform ? nullptr : tables->heads;   // (lengths from the table are a chain of reads before anything starts)
+        if (tables->tbase) { S.htab = tables->heads; S.tbase = tables->tbase; }   // (lengths from tables are a chain of reads before anything starts)
         S.maps = (const CUtensorMap *)tables->maps;
     } else {
         if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, src_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
@@ -1081,8 +1083,8 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     const bool sparse = select_reads_scored_tiles(s, tables ? tables->max_L : s.L);
     ScoredTiles scored;
     scored.bits = P.scored = sparse ? (uint8_t *)(scratch + lay.scored) : nullptr;
-    scored.tph = tph; scored.max_tiles = max_tph;
-    P.htab = S.htab; P.maps = S.maps;
+    scored.tbase = S.tbase; scored.tph = tph; scored.max_tiles = max_tph;
+    P.htab = S.htab; P.tbase = S.tbase; P.maps = S.maps; P.block_maps = tables ? (const CUtensorMap *)tables->block_maps : nullptr;
     P.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
 #ifdef JQ_DEBUG
     S.dbg_rec = P.dbg_rec = debug_record();

@@ -100,7 +100,7 @@ struct Params {
     int wtile;               // 1 in window-inclusive mode: every head has one more tile, the last, holding the w window keys
     int w;                   // soft-token queries per query head
     // Units in buffers of their own (ragged calls): the head groups, their lengths and score offsets come from
-    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps [units][kMapsPerUnit] (K, Qwin, ...).
+    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps [units][kMapsPerUnit] (K, Qwin).
     const GroupRec *gtab;
     const CUtensorMap *maps;
     int hpu;                 // KV heads per unit (a group may run over consecutive units of one length)

@@ -623,7 +623,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     int n_tiles = 0;                                           // (sparse) the warp's tiles that take part
     if (kSparse) {
         // a tile's entry: its number, its scored blocks, whether the block before it and the one behind it are scored
-        const uint8_t *const from = scored.bits + (htab ? htab[kv].tbase : (long long)kv * scored.tph);
+        const uint8_t *const from = scored.bits + (scored.tbase ? scored.tbase[kv] : (long long)kv * scored.tph);
         const int nt = (L + 127) / 128, ta = min(wid * (segq >> 5), nt), tb = min(ta + (segq >> 5), nt);
         for (int t0 = ta; t0 < tb; t0 += 32) {
             const int t = t0 + lane;

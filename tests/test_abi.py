@@ -106,3 +106,16 @@ def test_pointer_errors_are_caught_on_the_host():
     assert lib.jq_last_device_status(None, None) == jq.JQ_ERR_INVALID_ARG
     assert jq.status_string(jq.JQ_ERR_TIMEOUT) and jq.status_string(99)
     assert jq.launch_count() == 0      # nothing above reached a launch
+
+
+def up(x):
+    return (x + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("n,Hkv,g,w,L", [(2, 2, 4, 16, 2048), (7, 1, 4, 32, 300), (128, 8, 4, 32, 4099), (3, 8, 4, 64, 9000)])
+def test_units_of_the_two_passes_take_no_room_for_another_way(n, Hkv, g, w, L):
+    """Status, normalisers, partial statistics, scores, keys; two tensor maps and two pointers per unit, a group and a head record per head."""
+    heads, R = n * Hkv, g * w
+    tables = up(n * 2 * 128) + 2 * up(n * 8) + up(heads * 40) + up(heads * 32)
+    s = jq.shape(Hkv, Hkv * g, L, w, 64)
+    assert jq.layers_workspace_bytes(s, n) == 256 + up(heads * R * 4) + up(heads * 640 * R * 8) + 2 * up(heads * L * 4) + tables

@@ -182,6 +182,33 @@ def test_a_workspace_without_room_for_it_goes_the_other_way():
         jq.evict_layer(K, V, Q, s, Ko, Vo, idx, torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
 
 
+@pytest.mark.parametrize("Ls,budget,launches", [([80000, 17, 60017], 300, LAUNCHES), ([3000, 130, 5000], 64, 2)])
+def test_units_in_a_workspace_without_room_for_it(Ls, budget, launches):
+    """The same for calls over several units: the tables of the two-pass kernels are all that has to fit behind the scratch."""
+    Hkv, g, w, n = 8, 4, 32, len(Ls)
+    units = [device_layer(Hkv, g, w, L, 21 + i) for i, L in enumerate(Ls)]
+    s = shape_of(wl_of(Hkv, g, w, max(Ls), budget))
+    up = lambda x: (x + 255) // 256 * 256
+    heads, R = n * Hkv, g * w
+    least = 256 + up(heads * R * 4) + up(heads * 640 * R * 8) + 2 * up(Hkv * sum(Ls) * 4)
+    least += up(n * 2 * 128) + 2 * up(n * 8) + up(heads * 40) + up(heads * 32)
+    rows = jq.ragged_output_rows(s, n, Ls, [budget] * n)
+    for size, count in ((least, 2), (jq.ragged_workspace_bytes(s, n, Ls), launches)):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        jq._raise("jq_workspace_init", jq.lib().jq_workspace_init(jq._ptr(ws), ws.numel(), jq._stream(None)))
+        Ko, Vo = (torch.zeros((rows, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        idx = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+        n0 = jq.launch_count()
+        jq.evict_ragged([u[0] for u in units], [u[1] for u in units], [u[2] for u in units], s, Ls, [budget] * n, Ko, Vo, idx, ws)
+        assert jq.launch_count() - n0 == count and jq.last_device_status(ws) == jq.JQ_OK
+        r0 = 0
+        for (K, V, Q), L in zip(units, Ls):
+            k = min(budget, L)
+            r1 = r0 + Hkv * k
+            check(K, V, Q, shape_of(wl_of(Hkv, g, w, L, budget)), Ko[r0:r1].view(Hkv, k, 128), Vo[r0:r1].view(Hkv, k, 128), idx[r0:r1].view(Hkv, k), ())
+            r0 = r1
+
+
 def test_in_a_graph_and_on_two_streams():
     """Captured once and replayed on other inputs in the same buffers, while another stream evicts with a workspace of its own."""
     Hkv, g, w, L, budget = 70, 1, 32, 11264, 64
