@@ -491,11 +491,9 @@ HostPipe *host_pipe()
     return &p;
 }
 
-}  // namespace
-
-size_t jq_host_call_bytes(const jq_shape *s)
+// The device buffer of a call whose workspace, the last part of it, has ws_bytes.
+size_t host_call_bytes(const jq_shape *s, size_t ws_bytes)
 {
-    if (check_shape(s) != JQ_OK) return 0;
     const size_t row = (size_t)s->d * 2;
     const size_t nkeep = (size_t)(s->budget < s->L ? s->budget : s->L);
     size_t b = 0;
@@ -503,9 +501,12 @@ size_t jq_host_call_bytes(const jq_shape *s)
     b += align_up((size_t)s->Hq * s->w * row, 256);           // Qwin
     b += 2 * align_up((size_t)s->Hkv * nkeep * row, 256);     // Kout, Vout
     b += align_up((size_t)s->Hkv * nkeep * 4, 256) + kHostIdxPad;   // kept_idx, with room to align every chunk's
-    b += workspace_need(*s);
-    return b;
+    return b + ws_bytes;
 }
+
+}  // namespace
+
+size_t jq_host_call_bytes(const jq_shape *s) { return check_shape(s) == JQ_OK ? host_call_bytes(s, workspace_need(*s)) : 0; }
 
 jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin, const jq_shape *s,
                               void *hKout, void *hVout, int32_t *hkept_idx, void *dev_buf,
@@ -515,7 +516,7 @@ jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin,
     if (rc != JQ_OK) return rc;
     if (!hK || !hV || !hQwin || !hKout || !hVout || !hkept_idx) return JQ_ERR_INVALID_ARG;
     if (!dev_buf || ((uintptr_t)dev_buf & 255u)) return JQ_ERR_INVALID_ARG;
-    if (dev_buf_bytes < jq_host_call_bytes(s)) return JQ_ERR_WORKSPACE;
+    if (dev_buf_bytes < host_call_bytes(s, carve(nullptr, *s).bytes)) return JQ_ERR_WORKSPACE;   // (what is enough for either way)
     cudaStream_t st = (cudaStream_t)stream;
     const size_t row = (size_t)s->d * 2;
     const size_t nkeep = (size_t)(s->budget < s->L ? s->budget : s->L);
@@ -529,7 +530,7 @@ jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin,
     char *dVo = p;         p += align_up(ob, 256);
     char *dI = p;          p += align_up(ib, 256) + kHostIdxPad;
     char *ws = p;
-    const size_t wsb = workspace_need(*s);
+    const size_t wsb = dev_buf_bytes - (size_t)(ws - (char *)dev_buf);
     if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return JQ_ERR_CUDA;
     if (cudaMemcpyAsync(dQ, hQwin, qb, cudaMemcpyHostToDevice, st) != cudaSuccess) return JQ_ERR_CUDA;
     // V is read at the kept rows only.  A page-locked host buffer is mapped into the device's address space: the

@@ -209,6 +209,25 @@ def test_units_in_a_workspace_without_room_for_it(Ls, budget, launches):
             r0 = r1
 
 
+def test_a_host_call_with_a_buffer_without_room_for_it():
+    """The device buffer of a call on host tensors: K, V, queries, the kept rows, the indices, and what the two-pass kernels need."""
+    Hkv, g, w, L, budget = 8, 4, 64, 65537, 500
+    K, V, Q = device_layer(Hkv, g, w, L, 4)
+    s = shape_of(wl_of(Hkv, g, w, L, budget))
+    up = lambda x: (x + 255) // 256 * 256
+    least = 2 * up(Hkv * L * 256) + up(Hkv * g * w * 256) + 2 * up(Hkv * budget * 256) + up(Hkv * budget * 4) + 256
+    least += 256 + up(Hkv * g * w * 4) + up(Hkv * 640 * g * w * 8) + 2 * up(Hkv * L * 4)
+    assert least < jq.host_call_bytes(s)
+    host = [x.cpu().pin_memory() for x in (K, V, Q)]
+    for size in (least, jq.host_call_bytes(s)):
+        out = [torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16).pin_memory() for _ in range(2)] + [torch.full((Hkv, budget), -1, dtype=torch.int32).pin_memory()]
+        jq.evict_layer_host(*host, s, *out, torch.empty(size, dtype=torch.uint8, device="cuda"))
+        torch.cuda.synchronize()
+        check(K, V, Q, s, *(x.cuda() for x in out), ())
+    with pytest.raises(jq.JqError):
+        jq.evict_layer_host(*host, s, *out, torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+
+
 def test_in_a_graph_and_on_two_streams():
     """Captured once and replayed on other inputs in the same buffers, while another stream evicts with a workspace of its own."""
     Hkv, g, w, L, budget = 70, 1, 32, 11264, 64
