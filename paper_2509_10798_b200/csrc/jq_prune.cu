@@ -15,10 +15,15 @@
 //   the selection     (jq_select.cu) pools, selects and copies the rows as it does behind score_fused.  Its result is the same: every
 //                     position that is kept has the score that it has there.
 //
-// Nothing is assumed about the data: where the bounds do not separate (equal scores), round 2 takes every block and the work is
-// that of the two passes (32 layers of 32768 keys with nearly equal scores: 914 us by the two-pass kernel, 910 this way; of
-// 131072: 5911, 6281; one layer of 8 heads, whose clusters leave a part of the GPU idle: 198, 290).  prune_taken has the rule by
-// which a call comes here, with what was measured.
+// Nothing is assumed about the data for the results; the time depends on it.  Where the bounds do not separate (every query's logits within a
+// few tenths of each other), every block is scored, by the clusters of the heads alone, and a call takes longer than by the two-pass
+// kernels, the more so the fewer heads share the GPU (us, two-pass -> this way; in brackets keys of which some stand out):
+//   32 layers of 8 heads x 32768, 128 rows    985 -> 1055 (945 -> 540)       12 layers of 8 x 131072, 256 rows   2300 -> 2790 (2265 -> 1390)
+//   64 x 16384, 128 rows                       127 -> 147 (124 -> 94)        8 x 131072, 256 rows                 201 -> 277 (191 -> 139)
+//   8 x 131072, 128 rows                       131 -> 199 (127 -> 106)       2 x 300015, 256 rows                 125 -> 310 (123 -> 112)
+// Scoring such heads from end to end with all CTAs that are free (tiles claimed through a list in memory, clusters without a head beside
+// the others) was tried: 277 -> 241 us for 8 x 131072, and 1.5 % slower where the bounds do separate.
+// prune_taken has the rule by which a call comes here, with what was measured.
 //
 // The bound holds for the scores as they are computed, not only on paper: the rounding of the half is added (block_bounds), the sum
 // is raised by 1 / 512, and it is rounded up to 16 bits, far above the differences in rounding between the two orders of the
@@ -915,7 +920,8 @@ constexpr size_t kCMaxSmem = 227 * 1024, kCTwoPerSm = 113 * 1024;
 
 struct PruneDevice {
     int sms = 0;
-    int resident[2][kCMaxCluster + 1] = {};   // [R > 128][C]: clusters of C CTAs that fit at a time
+    int resident[2][kCMaxCluster + 1] = {};   // [R > 128][C]: clusters of C CTAs that fit at a time with an SM for each CTA (what the
+                                              // runtime answers for a kernel that allocates tensor memory, also where two fit)
     bool ready = false;
 };
 
@@ -1067,7 +1073,11 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     P.stages = wide ? 3 : 2;
     while (C < kCMaxCluster && C < max_tph && cand_smem(Rbox, P.stages, (max_tph + C - 1) / C) > (wide ? kCMaxSmem : kCTwoPerSm)) ++C;
     P.share = (max_tph + C - 1) / C;
-    const size_t smem = cand_smem(Rbox, P.stages, P.share);
+    size_t smem = cand_smem(Rbox, P.stages, P.share);
+    // Where an SM each is to be had, no two CTAs share one: set up while block_bounds drains, they would sit in pairs on the SMs that are
+    // free first, with others left empty (64 heads x 16384 keys, 128 CTAs: 16 SMs had two and 36 none, and the calls took 96 us instead of 94, 184
+    // instead of 147 where the scores are nearly equal and all keys are candidates).
+    if (s.Hkv * C <= dev.sms && smem <= kCTwoPerSm) smem = kCTwoPerSm + 1024;
     if (smem > kCMaxSmem) return JQ_ERR_CUDA;   // (prune_taken's limit on the length keeps every call below)
     P.L = s.L; P.tph = tph; P.nkeep = s.budget < s.L ? s.budget : s.L;
     P.heads = s.Hkv; P.R = R; P.Rbox = Rbox; P.Rpad = Rpad; P.radius = (s.pool - 1) / 2;
