@@ -255,6 +255,95 @@ def test_in_a_graph_and_on_two_streams():
         check(K, V, Q, s, o[0], o[1], o[2], ())
 
 
+@pytest.mark.parametrize("Hkv,g,w,L,budget,pool", [(66, 4, 32, 11000, 100, 7), (8, 4, 64, 66000, 300, 7), (130, 2, 16, 10100, 77, 5), (9, 1, 32, 90001, 500, 13)])
+def test_equal_scores_keep_the_lowest_positions(Hkv, g, w, L, budget, pool):
+    """Q = 0: every score is the same number, every block a candidate, and the first `budget` positions stay."""
+    K, V, Q = device_layer(Hkv, g, w, L, 3)
+    s = shape_of(wl_of(Hkv, g, w, L, budget, pool))
+    Ko, Vo = (torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    idx = torch.full((Hkv, budget), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer(K, V, torch.zeros_like(Q), s, Ko, Vo, idx, ws)
+    assert jq.launch_count() - n0 == LAUNCHES and jq.last_device_status(ws) == jq.JQ_OK
+    assert torch.equal(idx, torch.arange(budget, dtype=torch.int32, device="cuda").expand(Hkv, -1))
+    assert torch.equal(Ko, K[:, :budget]) and torch.equal(Vo, V[:, :budget])
+
+
+# logits that are what is left of products that cancel, in the first and the last of eight steps of the product: the sum of |q k| is 2 a b,
+# and what is lost of it in 32 bits is far more than the margin of the bounds (c 2^-24 2 a b against 1 / 512 in the exponent).  The same query
+# in every row, so that a block's bound is the score of its best key and nothing more.
+@pytest.mark.parametrize("a,b", [(256.0, 256.0), (2048.0, 1024.0), (8192.0, 8192.0)])
+def test_logits_that_cancel(a, b):
+    Hkv, g, w, L, budget = 70, 1, 8, 11279, 64
+    K, V, Q = device_layer(Hkv, g, w, L, 6)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    big = (a * (1 + torch.rand((Hkv, L), generator=gen, device="cuda"))).to(torch.bfloat16)
+    Q = Q[:, :1].expand(-1, w, -1).contiguous()
+    K[:, :, 3] = big; K[:, :, 120] = big
+    Q[:, :, 3] = b; Q[:, :, 120] = -b
+    s = shape_of(wl_of(Hkv, g, w, L, budget))
+    Ko, Vo = (torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    idx = torch.full((Hkv, budget), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer(K, V, Q, s, Ko, Vo, idx, ws)
+    assert jq.launch_count() - n0 == LAUNCHES and jq.last_device_status(ws) == jq.JQ_OK
+    check(K, V, Q, s, Ko, Vo, idx, ())
+
+
+@pytest.mark.parametrize("Hkv,g,w,L,budget", [(8, 4, 64, 66001, 400), (130, 2, 16, 10100, 100)])
+def test_windowed(Hkv, g, w, L, budget):
+    K, V, Q = device_layer(Hkv, g, w, L, 5)
+    Kw = torch.randn((Hkv, w, 128), device="cuda").to(torch.bfloat16)
+    s = shape_of(wl_of(Hkv, g, w, L, budget))
+    Ko, Vo = (torch.zeros((Hkv, budget, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    idx = torch.full((Hkv, budget), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_layer_windowed(K, V, Q, Kw, s, Ko, Vo, idx, ws)
+    assert jq.launch_count() - n0 == LAUNCHES and jq.last_device_status(ws) == jq.JQ_OK
+    gi = idx.cpu().numpy()
+    for kv in (0, Hkv - 1):
+        po = oracle.pool(oracle.score_windowed(host_bits(K[kv:kv + 1]), host_bits(Q[kv * g:(kv + 1) * g]), host_bits(Kw[kv:kv + 1])), s.pool)
+        assert_kept_sets_agree(gi[kv:kv + 1], oracle.select(po, budget), po, budget)
+    at = idx.long()[:, :, None].expand(-1, -1, 128)
+    assert torch.equal(Ko, torch.gather(K, 1, at)) and torch.equal(Vo, torch.gather(V, 1, at))
+
+
+# 136 heads in 17 units: the selection reads the scored blocks by their bits, of units of one length and of units whose tiles are
+# numbered in another order than the call's (lengths that are no multiple of 16 or 128, a unit of one key, budgets at and above the length)
+MANY_UNITS = {
+    "one length": ([10100] * 17, [90] * 17),
+    "two budgets": ([10100] * 17, [90, 130] * 8 + [1]),
+    "lengths": ([10017, 20000, 17, 11279, 9001, 1, 30001, 12345, 128, 10100, 16384, 10017, 7777, 25001, 129, 10240, 20033], [90, 200, 17, 100, 64, 5, 300, 1, 1000, 90, 50, 91, 77, 250, 128, 100, 10]),
+}
+
+
+@pytest.mark.parametrize("units", sorted(MANY_UNITS))
+def test_many_units_of_many_heads(units):
+    Hkv, g, w = 8, 4, 32
+    Ls, Bs = MANY_UNITS[units]
+    U = [device_layer(Hkv, g, w, L, 31 + i) for i, L in enumerate(Ls)]
+    s = shape_of(wl_of(Hkv, g, w, Ls[0], Bs[0]))
+    rows = jq.ragged_output_rows(s, len(Ls), Ls, Bs)
+    Ko, Vo = (torch.zeros((rows, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    idx = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_ragged_workspace(s, len(Ls), Ls)
+    n0 = jq.launch_count()
+    if units == "one length":
+        jq.evict_layers([u[0] for u in U], [u[1] for u in U], [u[2] for u in U], s, Ko, Vo, idx, ws)
+    else:
+        jq.evict_ragged([u[0] for u in U], [u[1] for u in U], [u[2] for u in U], s, Ls, Bs, Ko, Vo, idx, ws)
+    assert jq.launch_count() - n0 == LAUNCHES and jq.last_device_status(ws) == jq.JQ_OK
+    r0 = 0
+    for i, ((K, V, Q), L, B) in enumerate(zip(U, Ls, Bs)):
+        n = min(B, L)
+        r1 = r0 + Hkv * n
+        check(K, V, Q, shape_of(wl_of(Hkv, g, w, L, B)), Ko[r0:r1].view(Hkv, n, 128), Vo[r0:r1].view(Hkv, n, 128), idx[r0:r1].view(Hkv, n), (i % Hkv,))
+        r0 = r1
+
+
 SWEEP = r'''
 import ctypes, os, sys
 import torch
@@ -294,6 +383,35 @@ print("DEBUG-SWEEP violations=%%d kernel=%%d site=%%d index=%%d extent=%%d" %% t
 
 def test_no_index_leaves_its_array_in_the_bounds_checked_build():
     out = subprocess.run([sys.executable, "-c", SWEEP % {"root": ROOT}], capture_output=True, text=True, timeout=900)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    line = [ln for ln in out.stdout.splitlines() if ln.startswith("DEBUG-SWEEP")]
+    assert line and line[0].startswith("DEBUG-SWEEP violations=0 "), out.stdout[-2000:]
+
+
+MANY_SWEEP = SWEEP[:SWEEP.index("for Hkv, g, w, L, B, p, scale in")] + r'''
+from test_gpu_candidates import MANY_UNITS
+for Ls, Bs in MANY_UNITS.values():
+    for scale in (1.0, 0.0):
+        u = [device_layer(8, 4, 32, L, 11) for L in Ls]
+        s = shape_of(wl_of(8, 4, 32, Ls[0], Bs[0]))
+        rows = jq.ragged_output_rows(s, len(Ls), Ls, Bs)
+        Ko, Vo = (torch.zeros((rows, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        ws = jq.new_ragged_workspace(s, len(Ls), Ls)
+        n0 = jq.launch_count()
+        jq.evict_ragged([x[0] for x in u], [x[1] for x in u], [(x[2].float() * scale).to(torch.bfloat16) for x in u], s, Ls, Bs, Ko, Vo, torch.zeros((rows,), dtype=torch.int32, device="cuda"), ws)
+        assert jq.launch_count() - n0 == 4 and jq.last_device_status(ws) == jq.JQ_OK
+K, V, Q = device_layer(130, 2, 16, 10100, 5)
+Kw = torch.randn((130, 16, 128), device="cuda").to(torch.bfloat16)
+s = shape_of(wl_of(130, 2, 16, 10100, 100))
+Ko, Vo = (torch.zeros((130, 100, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+ws = jq.new_workspace(s)
+jq.evict_layer_windowed(K, V, Q, Kw, s, Ko, Vo, torch.zeros((130, 100), dtype=torch.int32, device="cuda"), ws)
+assert jq.last_device_status(ws) == jq.JQ_OK
+''' + SWEEP[SWEEP.index("assert lib.jq_debug_read(rec) == 0"):]
+
+
+def test_no_index_leaves_its_array_with_many_units():
+    out = subprocess.run([sys.executable, "-c", MANY_SWEEP % {"root": ROOT}], capture_output=True, text=True, timeout=900)
     assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
     line = [ln for ln in out.stdout.splitlines() if ln.startswith("DEBUG-SWEEP")]
     assert line and line[0].startswith("DEBUG-SWEEP violations=0 "), out.stdout[-2000:]

@@ -304,3 +304,53 @@ def test_calls_over_many_heads_take_the_faster_way(Hkv, g, w, L, launches):
     assert_kept_sets_agree(idx.cpu().numpy(), want.cpu().numpy(), pooled.cpu().numpy().astype(np.float64), 300)
     at = idx.long()[:, :, None].expand(-1, -1, 128)
     assert torch.equal(Ko.view(torch.int16), K.gather(1, at).view(torch.int16)) and torch.equal(Vo.view(torch.int16), V.gather(1, at).view(torch.int16))
+
+
+# CTAs of six tiles and more send their scores to the others as one copy each: lengths that end anywhere in a quad, with the window and
+# without
+@pytest.mark.parametrize("L", [11995, 11997, 11998, 11999])
+@pytest.mark.parametrize("window", [False, True])
+def test_scores_of_many_tiles_between_ctas(L, window):
+    Hkv, g, w, budget = 8, 4, 32, 300
+    wl = wl_of(Hkv, g, w, L, budget)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    Kw = W.make_window_keys(wl, Q)
+    np_ = budget - w if window else budget
+    Ko, Vo, idx = outputs(Hkv, budget, np_)
+    ws = jq.new_workspace(s)
+    n0 = jq.launch_count()
+    if window:
+        jq.evict_layer_window_kept(dev_bf16(K), dev_bf16(V), dev_bf16(Q), dev_bf16(Kw), dev_bf16(Kw), s, Ko, Vo, idx, ws)
+    else:
+        jq.evict_layer(dev_bf16(K), dev_bf16(V), dev_bf16(Q), s, Ko, Vo, idx, ws)
+    assert jq.launch_count() - n0 == 1 and jq.last_device_status(ws) == jq.JQ_OK
+    pooled = oracle.pool(oracle.score_windowed(K, Q, Kw) if window else oracle.score(K, Q), s.pool)
+    gi = idx.cpu().numpy()
+    assert_kept_sets_agree(gi, oracle.select(pooled, np_), pooled, np_)
+    gK, gV = host_bits(Ko), host_bits(Vo)
+    for kv in range(Hkv):
+        assert np.array_equal(gK[kv][:np_], K[kv][gi[kv]]) and np.array_equal(gV[kv][:np_], V[kv][gi[kv]])
+
+
+# the same in two parts: copies where the first part is a multiple of four, four scores at a time where it is not
+@pytest.mark.parametrize("n_old,n_new", [(11000, 997), (11004, 1), (128, 11002), (11001, 996), (11003, 998)])
+def test_scores_of_many_tiles_in_two_parts(n_old, n_new):
+    Hkv, g, w, budget, L = 8, 4, 32, 100, n_old + n_new
+    wl = wl_of(Hkv, g, w, L, budget)
+    K, V, Q, _ = W.make_layer(wl)
+    s = shape_of(wl)
+    Kc, Vc = (torch.zeros((Hkv, L + 3, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    dK, dV = dev_bf16(K), dev_bf16(V)
+    Kc[:, :n_old] = dK[:, :n_old]; Vc[:, :n_old] = dV[:, :n_old]
+    idx = torch.full((Hkv, budget), -1, dtype=torch.int32, device="cuda")
+    ws = jq.new_append_workspace(s)
+    n0 = jq.launch_count()
+    jq.evict_append(Kc, Vc, n_old, dK[:, n_old:].contiguous(), dV[:, n_old:].contiguous(), dev_bf16(Q), s, idx, ws)
+    assert jq.launch_count() - n0 == 1 and jq.last_device_status(ws) == jq.JQ_OK
+    pooled = oracle.pool(oracle.score(K, Q), s.pool)
+    gi = idx.cpu().numpy()
+    assert_kept_sets_agree(gi, oracle.select(pooled, budget), pooled, budget)
+    gK, gV = host_bits(Kc), host_bits(Vc)
+    for kv in range(Hkv):
+        assert np.array_equal(gK[kv][:budget], K[kv][gi[kv]]) and np.array_equal(gV[kv][:budget], V[kv][gi[kv]])
