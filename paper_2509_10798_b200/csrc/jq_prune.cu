@@ -72,7 +72,7 @@ static_assert(sizeof(SCtl) <= kSCtlBytes, "control block");
 
 struct SParams {
     int L, tph;                // one shape: keys and tiles per head (the window tile included)
-    int R, Rbox, Rpad, w;
+    int R, Rpad, w;
     int wtile;                 // every head has one more tile, the last, holding the w window keys
     int stages, hpu;           // hpu: heads per unit (ragged calls)
     long long T;               // tiles of all heads
@@ -442,12 +442,10 @@ __device__ __forceinline__ int scan_threads(int v, int &total, int *sums)
     return before + inc - v;
 }
 
-struct BinAt { int bin, rank, count; };   // a bin, the rank in it of what was looked for, its population
-
 // The same threads: the bin that holds the target-th entry from the top (without so many entries: bin 0).  get(i) gives the
 // counts of bins i, i + 1.
 template <int kThreads, int kN, typename Get>
-__device__ __forceinline__ BinAt find_bin(Get get, int target, BinAt *res, int *sums)
+__device__ __forceinline__ int find_bin(Get get, int target, int *res, int *sums)
 {
     constexpr int per = kN / kThreads;                        // consecutive bins of a thread, from the top
     const int at = kN - per * ((int)threadIdx.x + 1);
@@ -456,11 +454,11 @@ __device__ __forceinline__ BinAt find_bin(Get get, int target, BinAt *res, int *
     for (int i = 0; i < per; i += 2) { const uint2 v = get(at + i); n[i] = (int)v.x; n[i + 1] = (int)v.y; }
 #pragma unroll
     for (int i = 0; i < per; ++i) sum += n[i];
-    if (threadIdx.x == 0) *res = {0, 1, 0};
+    if (threadIdx.x == 0) *res = 0;
     int above = scan_threads<kThreads>(sum, total, sums);
 #pragma unroll
     for (int i = per - 1; i >= 0; --i) {
-        if (above < target && target <= above + n[i]) *res = {at + i, target - above, n[i]};
+        if (above < target && target <= above + n[i]) *res = at + i;
         above += n[i];
     }
     named_sync<kThreads>();
@@ -625,7 +623,7 @@ struct CCtl {
     uint32_t tmem_base;
     int abort_flag;
     int n;                                       // blocks on this CTA's list
-    BinAt found;
+    int found;                                   // (find_bin)
     int sums[16];
     int cnt[kCMaxCluster];                       // candidates of every CTA's share of the head
     alignas(16) float xs[2][2][kPTile];          // (R > 128) the second column half's sums on their way to the first half's threads
@@ -755,7 +753,7 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     for (int round = 0; round < 2; ++round) {
         // ---- the blocks of this round: [lo16, hi16) of the bounds
         if (warp < kEpi) {
-            const uint32_t edge = edge_of(find_bin<kTE, kCBins>(counts, round == 0 ? wanted : nkeep, &ctl->found, ctl->sums).bin);
+            const uint32_t edge = edge_of(find_bin<kTE, kCBins>(counts, round == 0 ? wanted : nkeep, &ctl->found, ctl->sums));
             if (round == 0) { lo16 = edge; hi16 = 0x10000u; }
             else { hi16 = lo16; lo16 = min(edge, lo16); }
             // this CTA's share of them, and their places in the head's list
@@ -1042,7 +1040,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     const int wtile = Kwin ? 1 : 0, tph = (s.L + kPTile - 1) / kPTile + wtile;
     const long long T = tables ? tables->total_tiles : (long long)s.Hkv * tph;
     SParams S = {};
-    S.L = s.L; S.tph = tph; S.R = R; S.Rbox = Rbox; S.Rpad = Rpad; S.w = s.w; S.wtile = wtile;
+    S.L = s.L; S.tph = tph; S.R = R; S.Rpad = Rpad; S.w = s.w; S.wtile = wtile;
     S.stages = wide ? 3 : 5;
     S.T = T; S.heads = s.Hkv; S.hpu = tables ? tables->hpu : s.Hkv;
     S.c = 1.4426950408889634f / sqrtf((float)s.d);

@@ -26,7 +26,6 @@
 // 60000 70 -> 116 -> 75; 8 x 500 with five different scores 9.7 -> 16.2 -> 8.4.
 #include "jq_internal.cuh"
 #include "jq_pool.cuh"
-#include "jq_rows.cuh"
 #include "jq_debug.cuh"
 #include <cooperative_groups.h>
 #include <mutex>
@@ -53,6 +52,16 @@ static_assert(kClMax * kRankMax <= kCandMax, "a place for every CTA's list");
 constexpr int kOwnKey = 0, kOwnPos = kCandMax, kAllKey = 2 * kCandMax, kAllPos = 3 * kCandMax, kListWords = 4 * kCandMax;
 __host__ __device__ constexpr int raw_words(int raw_tile) { return raw_tile + 2 * kHalo > kListWords ? raw_tile + 2 * kHalo : kListWords; }
 static_assert(kBins == 4 * kSelThreads, "a thread takes four bins");
+
+// Extents of what the kernel indexes (read by the bounds-checked build only).
+struct SelExtents {
+    long long scores;     // floats in the scores array (and keys in the global key array)
+    long long out_rows;   // rows of the stacked outputs (kept indices, compacted K and V)
+    long long src_heads;  // heads in one source buffer of K / V
+};
+
+// The window rows that follow every head's kept rows: K, V [Hkv][w] rows (w = 0: none).
+struct WindowRows { const uint4 *K, *V; int w; };
 
 struct SelCtl {
     int digit, krem, count;              // find_digit: the bin of the krem-th key, the rank within it, its population
@@ -134,6 +143,46 @@ __device__ __forceinline__ void find_bin(const uint4 v, int need, SelCtl &ctl)
         above += c[i];
     }
     __syncthreads();
+}
+
+// Rows [r0, r1) of a head's kept rows (256 bytes each: 16 lanes x 16 bytes), four rows of K and V in flight per 16 lanes.
+// kv_in: the head's index within the buffer the rows come from; orow: the head's first row in the outputs.
+__device__ __forceinline__ void copy_rows(const int32_t *out, int r0, int r1, int kv_in, long long orow, int L, const uint4 *__restrict__ Kin,
+                                          const uint4 *__restrict__ Vin, uint4 *__restrict__ Kout, uint4 *__restrict__ Vout, int src_rows,
+                                          const SelExtents &ext JQ_DBG_PARAM)
+{
+    (void)ext;
+    const int lane16 = threadIdx.x & 15, grp = threadIdx.x >> 4, ngrp = blockDim.x >> 4;
+    for (int t0 = r0 + 4 * grp; t0 < r1; t0 += 4 * ngrp) {
+        int j[4];
+        uint4 a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) j[r] = t0 + r < r1 ? min(max(__ldcg(out + t0 + r), 0), L - 1) : 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const size_t src = ((size_t)kv_in * src_rows + j[r]) * 16 + lane16;
+            const bool in = t0 + r < r1 && JQ_IN((long long)kv_in * src_rows + j[r], ext.src_heads * src_rows, kDbgSelect, 1);
+            a[r] = in ? Kin[src] : make_uint4(0u, 0u, 0u, 0u);
+            b[r] = in ? Vin[src] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const size_t dst = (size_t)(orow + t0 + r) * 16 + lane16;
+            if (t0 + r < r1 && JQ_IN(orow + t0 + r, ext.out_rows, kDbgSelect, 2)) { Kout[dst] = a[r]; Vout[dst] = b[r]; }
+        }
+    }
+}
+
+// Window rows [i0, w), every `step`-th group's share, behind the kept rows of head kv (row `row0` of the outputs on).
+__device__ __forceinline__ void copy_window(const WindowRows &win, int kv, long long row0, int first, int step, uint4 *__restrict__ Kout,
+                                            uint4 *__restrict__ Vout, const SelExtents &ext JQ_DBG_PARAM)
+{
+    (void)ext;
+    const int lane16 = threadIdx.x & 15;
+    for (int i = first; i < win.w; i += step) {
+        const size_t src = ((size_t)kv * win.w + i) * 16 + lane16, dst = (size_t)(row0 + i) * 16 + lane16;
+        if (JQ_IN(row0 + i, ext.out_rows, kDbgSelect, 32)) { Kout[dst] = win.K[src]; Vout[dst] = win.V[src]; }
+    }
 }
 
 // grid (Hkv * CL), cluster CL, block 512.  With htab (ragged calls) every head has a length, a budget, offsets
@@ -240,7 +289,7 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
         for (int e = tid; e < n; e += kSelThreads) if (JQ_IN(orow + j0 + e, ext.out_rows, kDbgSelect, 13)) out[j0 + e] = j0 + e;
         if (Kin) {
             cluster.sync();
-            copy_rows(tid, kSelThreads, out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+            copy_rows(out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
             if (win.w) copy_window(win, kv, krow + nkeep, rank * ngrp + (tid >> 4), CL * ngrp, Kout, Vout, ext JQ_DBG_ARG_DEV);
         }
         return;
@@ -451,7 +500,7 @@ select_cluster(const float *__restrict__ scores, int L, int nkeep, int radius, i
     // CTA's list may be being read.)
     cluster.sync();                 // (release and acquire at cluster scope: the readers are in the cluster)
     if (!Kin) return;
-    copy_rows(tid, kSelThreads, out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+    copy_rows(out, r0, r1, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
     if (win.w) copy_window(win, kv, krow + nkeep, rank * ngrp + (tid >> 4), CL * ngrp, Kout, Vout, ext JQ_DBG_ARG_DEV);
 }
 
@@ -834,7 +883,7 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
 
     // ---- the kept rows
     __syncthreads();
-    copy_rows(tid, T, out, 0, nkeep, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
+    copy_rows(out, 0, nkeep, kv_in, krow, L, Kin, Vin, Kout, Vout, src_rows, ext JQ_DBG_ARG_DEV);
     if (win.w) copy_window(win, kv, krow + nkeep, tid >> 4, T >> 4, Kout, Vout, ext JQ_DBG_ARG_DEV);
 }
 
