@@ -1,7 +1,8 @@
 // Bounds-checked build of the kernels (-DJQ_DEBUG; build.build(debug=True) makes libjq_debug.so from the same
-// sources).  It stands in for a memory checker: every index that score_fused, row_stats, score_candidates, evict_fused,
-// select_cluster, select_stream, gather_rows and decode_step compute into global, shared or tensor memory goes through JQ_IN(index,
-// extent, kernel, site) before the access.  An index outside [0, extent) is counted in a record in device memory, the first one is kept
+// sources).  It stands in for a memory checker: every index into global, shared or tensor memory that score_fused, row_stats, block_bounds,
+// score_candidates, evict_fused, select_cluster, select_stream, gather_rows and decode_step compute from lengths, budgets, tiles, lists
+// or scores goes through JQ_IN(index, extent, kernel, site) before the access (not the ones by thread, warp or row number into
+// arrays of that size).  An index outside [0, extent) is counted in a record in device memory, the first one is kept
 // (which kernel, which site, the index and the extent), and the access is skipped: the kernel never traps and
 // always runs to its end.  The host reads the record with jq_debug_read (exported by the debug library only).
 // In the ordinary build JQ_IN is the constant true and the extra kernel parameter does not exist.

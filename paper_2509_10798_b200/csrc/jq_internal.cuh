@@ -172,6 +172,7 @@ struct ScoredTiles {
     const long long *tbase = nullptr;   // device: a head's first tile; null: tph of them from one head to the next
     int tph = 0;
     int max_tiles = 0;               // of any head
+    long long tiles = 0;             // of all heads (read by the bounds-checked build)
 };
 constexpr int kMaxSparseTiles = 1024;   // (their list is in shared memory; two CTAs to an SM)
 bool select_reads_scored_tiles(const jq_shape &s, int max_L);

@@ -567,7 +567,7 @@ block_bounds(const __grid_constant__ CParams P)
                 }
                 Ms[row] = -M;
                 if (!kWide) Ms[128 + row] = -INFINITY;
-                if (t0 == 0) { P.Ms[(size_t)h * kMaxR + row] = -M; if (!kWide) P.Ms[(size_t)h * kMaxR + 128 + row] = -INFINITY; }
+                if (t0 == 0 && JQ_IN(h, P.heads, kDbgPrune, 15)) { P.Ms[(size_t)h * kMaxR + row] = -M; if (!kWide) P.Ms[(size_t)h * kMaxR + 128 + row] = -INFINITY; }
             }
             __syncthreads();
         }
@@ -604,7 +604,7 @@ block_bounds(const __grid_constant__ CParams P)
             r += __shfl_xor_sync(0xffffffffu, r, 2);
             r += __shfl_xor_sync(0xffffffffu, r, 1);
             const int blk = 2 * pair + (odd ? 1 : 0);
-            if ((lane & 3) == 0)
+            if ((lane & 3) == 0 && JQ_IN(a.tbase + t, P.T, kDbgPrune, 16))
                 P.ub[(a.tbase + t) * 8 + blk] = 8 * t + blk < nb ? (uint16_t)((__float_as_uint((r + least) * (1.f + 1.f / 512.f)) + 0xffffu) >> 16) : (uint16_t)0;
             stage = stage == kBStages - 1 ? 0 : stage + 1;
         }
@@ -734,11 +734,11 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
         __syncwarp();
         if (P.maps) tensormap_acquire(mb);                    // (all lanes load)
     } else if (warp < kEpi) {
-        for (int i = tid; i < kMaxR; i += kTE) ctl->Ms[i] = __ldcg(P.Ms + (size_t)head * kMaxR + i);
+        for (int i = tid; i < kMaxR; i += kTE) if (JQ_IN(head, P.heads, kDbgPrune, 17)) ctl->Ms[i] = __ldcg(P.Ms + (size_t)head * kMaxR + i);
         const uint16_t *const src = P.ub + (size_t)(at.tbase + ts) * 8;
         for (int t = tid; t < te - ts; t += kTE) {
+            if (!JQ_IN(t, P.share, kDbgPrune, 7) || !JQ_IN(at.tbase + ts + t, P.T, kDbgPrune, 18)) continue;
             const uint4 v = __ldcg((const uint4 *)src + t);
-            if (!JQ_IN(t, P.share, kDbgPrune, 7)) continue;
             ((uint4 *)ub)[t] = v;
             const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -759,13 +759,13 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
             // this CTA's share of them, and their places in the head's list
             for (int w = warp; w < nw; w += kEpi) {
                 const int i = 32 * w + lane;
-                const uint32_t x = i < nbs ? ub[i] : 0x10000u, m = __ballot_sync(0xffffffffu, x >= lo16 && x < hi16);
-                if (lane == 0) words[w] = m;
+                const uint32_t x = i < nbs && JQ_IN(i, 8 * P.share, kDbgPrune, 19) ? ub[i] : 0x10000u, m = __ballot_sync(0xffffffffu, x >= lo16 && x < hi16);
+                if (lane == 0 && JQ_IN(w, P.share / 4 + 1, kDbgPrune, 20)) words[w] = m;
             }
             named_sync<kTE>();
             int total;
             const int base = scan_threads<kTE>(tid < nw ? __popc(words[tid]) : 0, total, ctl->sums);
-            if (tid < nw) wbase[tid] = base;
+            if (tid < nw && JQ_IN(tid, P.share / 4 + 1, kDbgPrune, 21)) wbase[tid] = base;
             named_sync<kTE>();
             int before = 0, per_cta = 0x40000000;
             if (C > 1) {
@@ -900,7 +900,7 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
             uint32_t m = 0u;
 #pragma unroll
             for (int e = 0; e < 8; ++e) m |= (uint32_t)(8 * t + e < nbs && ub[8 * t + e] >= lo16) << e;
-            P.scored[at.tbase + ts + t] = (uint8_t)m;
+            if (JQ_IN(at.tbase + ts + t, P.T, kDbgPrune, 22)) P.scored[at.tbase + ts + t] = (uint8_t)m;
         }
         return;
     }
@@ -1091,7 +1091,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     const bool sparse = select_reads_scored_tiles(s, tables ? tables->max_L : s.L);
     ScoredTiles scored;
     scored.bits = P.scored = sparse ? (uint8_t *)(scratch + lay.scored) : nullptr;
-    scored.tbase = S.tbase; scored.tph = tph; scored.max_tiles = max_tph;
+    scored.tbase = S.tbase; scored.tph = tph; scored.max_tiles = max_tph; scored.tiles = T;
     P.htab = S.htab; P.tbase = S.tbase; P.maps = S.maps; P.block_maps = tables ? (const CUtensorMap *)tables->block_maps : nullptr;
     P.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
 #ifdef JQ_DEBUG

@@ -672,14 +672,16 @@ select_stream(const float *__restrict__ scores, int L, int nkeep, int radius, in
     int n_tiles = 0;                                           // (sparse) the warp's tiles that take part
     if (kSparse) {
         // a tile's entry: its number, its scored blocks, whether the block before it and the one behind it are scored
-        const uint8_t *const from = scored.bits + (scored.tbase ? scored.tbase[kv] : (long long)kv * scored.tph);
+        const long long tile0 = scored.tbase ? scored.tbase[kv] : (long long)kv * scored.tph;
+        const uint8_t *const from = scored.bits + tile0;
+        auto bits_of = [&](int t) { return JQ_IN(tile0 + t, scored.tiles, kDbgSelect, 37) ? (uint32_t)__ldcg(from + t) : 0u; };
         const int nt = (L + 127) / 128, ta = min(wid * (segq >> 5), nt), tb = min(ta + (segq >> 5), nt);
         for (int t0 = ta; t0 < tb; t0 += 32) {
             const int t = t0 + lane;
-            const uint32_t b = t < tb ? __ldcg(from + t) : 0u;
+            const uint32_t b = t < tb ? bits_of(t) : 0u;
             uint32_t before = __shfl_up_sync(0xffffffffu, b, 1) >> 7, behind = __shfl_down_sync(0xffffffffu, b, 1) & 1u;
-            if (lane == 0) before = t > 0 ? (uint32_t)__ldcg(from + t - 1) >> 7 : 0u;
-            if ((lane == 31 || t + 1 >= tb) && t < tb) behind = t + 1 < nt ? (uint32_t)__ldcg(from + t + 1) & 1u : 0u;
+            if (lane == 0) before = t > 0 ? bits_of(t - 1) >> 7 : 0u;
+            if ((lane == 31 || t + 1 >= tb) && t < tb) behind = t + 1 < nt ? bits_of(t + 1) & 1u : 0u;
             const bool on = t < tb && (b | before | behind) != 0u;
             const uint32_t m = __ballot_sync(0xffffffffu, on);
             const int at = ta + n_tiles + __popc(m & ((1u << lane) - 1u));
