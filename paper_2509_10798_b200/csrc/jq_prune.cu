@@ -1014,12 +1014,15 @@ static double kept_per_block(int pool) { return pool >= 7 ? 7.0 : pool >= 3 ? 3.
 // With 8 query rows 64 x 32768 keys take 211 -> 141 (1 %), with 256 rows 371 -> 240.  Shorter heads than about 10000 keys gain little
 // and lose most where the bounds separate badly; fewer than 8 rows have not been measured and stay where they were.
 static double saved_per_tile(int R) { return R > 128 ? 9.0e-3 : R > 64 ? 6.2e-3 : 5.5e-3; }   // us
-constexpr double kPruneLeast = 30.0;                                                          // us that have to be saved
+// us that have to be saved.  With fewer than four heads the kernels behind row_stats have a cluster or three on the whole GPU and take two to
+// three times as long (1 x 500000, 256 rows 165 -> 166; 2 x 500000, 64, 128, 256 rows 156 -> 161, 166 -> 169, 233 -> 202; 2 x 300015,
+// 256 rows 123 -> 112; 3 x 249386, 64 rows, keys in segments 91 -> 125).
+static double prune_least(int heads, int R) { return heads >= 4 ? 30.0 : R > 128 ? 40.0 : 60.0; }
 
 bool prune_possible(int heads, int R, long long keys, int max_L)
 {
     const long long tiles = keys / kPTile + heads;
-    return R >= 8 && tiles < (1ll << 30) && max_L <= kPBlock * kCMaxBlocks && keys >= 10000ll * heads && (double)tiles * saved_per_tile(R) >= kPruneLeast;
+    return R >= 8 && tiles < (1ll << 30) && max_L <= kPBlock * kCMaxBlocks && keys >= 10000ll * heads && (double)tiles * saved_per_tile(R) >= prune_least(heads, R);
 }
 
 bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, long long kept, int max_L)
@@ -1027,7 +1030,7 @@ bool prune_taken(const jq_shape &s, int heads, long long tiles, long long keys, 
     const int R = s.group * s.w;
     if (!prune_possible(heads, R, keys, max_L)) return false;
     const double share = (double)kept / (double)keys * 7.0 / kept_per_block(s.pool);
-    return (double)tiles * (saved_per_tile(R) - 0.08 * share) >= kPruneLeast;
+    return (double)tiles * (saved_per_tile(R) - 0.08 * share) >= prune_least(heads, R);
 }
 
 jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const jq_shape &s, void *Kout, void *Vout, int32_t *idx,

@@ -112,6 +112,13 @@ def up(x):
     return (x + 255) // 256 * 256
 
 
+@pytest.mark.parametrize("Hkv,g,w,L", [(1, 4, 64, 500000), (2, 4, 16, 500000), (2, 4, 32, 500000), (3, 4, 16, 249386), (3, 4, 63, 165812)])
+def test_few_heads_are_scored_in_two_passes(Hkv, g, w, L):
+    """Calls whose candidates would leave most of the GPU idle have no other way, whatever their workspace."""
+    R = g * w
+    assert jq.workspace_bytes(jq.shape(Hkv, Hkv * g, L, w, 64)) == 256 + up(Hkv * R * 4) + up(Hkv * 640 * R * 8) + 2 * up(Hkv * L * 4)
+
+
 @pytest.mark.parametrize("n,Hkv,g,w,L", [(2, 2, 4, 16, 2048), (7, 1, 4, 32, 300), (128, 8, 4, 32, 4099), (3, 8, 4, 64, 9000)])
 def test_units_of_the_two_passes_take_no_room_for_another_way(n, Hkv, g, w, L):
     """Status, normalisers, partial statistics, scores, keys; two tensor maps and two pointers per unit, a group and a head record per head."""
