@@ -48,7 +48,7 @@ typedef enum {
     JQ_OK = 0,
     JQ_ERR_INVALID_ARG = 1, /* null or misaligned pointer, inconsistent shape                 */
     JQ_ERR_UNSUPPORTED = 2, /* a legal shape the library has no kernel for (d != 128, ...)     */
-    JQ_ERR_WORKSPACE = 3,   /* ws_bytes < jq_workspace_bytes(shape)                            */
+    JQ_ERR_WORKSPACE = 3,   /* less workspace than the call needs (jq_workspace_bytes)         */
     JQ_ERR_CUDA = 4,        /* a CUDA runtime / driver call or a launch failed                 */
     JQ_ERR_TIMEOUT = 5      /* a bounded device-side wait ran out (see jq_last_device_status)  */
 } jq_status;
@@ -67,8 +67,13 @@ typedef struct {
 /* A cudaStream_t, spelled so that this header needs no CUDA header. */
 typedef struct CUstream_st *jq_stream_t;
 
-/* Bytes of device workspace every call below needs for this shape (host-only, no CUDA call);
- * 0 if the shape is invalid or unsupported. */
+/* Bytes of device workspace with which every call below can go its fastest way for this shape (host-only, no
+ * CUDA call); 0 if the shape is invalid or unsupported.  With R = group * w and up(x) = x rounded up to 256,
+ * every call does with 256 + up(4 Hkv R) + up(5120 Hkv R) + 2 up(4 Hkv L) bytes (less: JQ_ERR_WORKSPACE): calls
+ * that keep a small share of many keys then read K twice.  For 32 layers of 8 heads x 131072 keys and 256 rows
+ * those are 576 MiB, against 1290; with many heads of less than about 40000 keys the two are the same.  The
+ * same holds for the other *_bytes functions: of n units the least is that formula with the sums of Hkv and of
+ * Hkv L over the units, and up(256 n) + 2 up(8 n) + up(40 n Hkv) + up(32 n Hkv) bytes of tables. */
 size_t jq_workspace_bytes(const jq_shape *shape);
 
 /*
@@ -198,8 +203,8 @@ jq_status jq_evict_layer(const void *K, const void *V, const void *Qwin, const j
  *   Kout, Vout: device, bf16 [rows, d];  kept_idx: device int32 [rows], where unit u's block of
  *               Hkv * nkeep_u rows (head-major, as jq_evict_layer writes them), nkeep_u = min(B_u, L_u),
  *               starts at row sum_{u' < u} Hkv * nkeep_u' and rows = jq_ragged_output_rows(...);
- *   ws: device, 256-byte aligned, at least jq_ragged_workspace_bytes(common, nunits, L) bytes (0 for arguments
- *       the call would reject), its first 256 bytes initialised by jq_workspace_init.
+ *   ws: device, 256-byte aligned, of jq_ragged_workspace_bytes(common, nunits, L) bytes (0 for arguments the
+ *       call would reject; the least: jq_workspace_bytes), its first 256 bytes initialised by jq_workspace_init.
  * nunits <= 4096 and nunits * Hkv <= 65535, else JQ_ERR_UNSUPPORTED.  The call copies its tables (tensor maps,
  * base pointers, per-head lengths and offsets) from host memory of its own to the device on `stream`, so it
  * cannot be captured into a CUDA graph; capture calls of jq_evict_layer instead.
@@ -213,7 +218,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
 /*
  * jq_evict_ragged for nlayers layers of ONE shape (the usual cache after a prefill): the same call with
  * L = budget = NULL.  Kout, Vout: device, bf16 [nlayers * Hkv, nkeep, d]; kept_idx: device [nlayers * Hkv, nkeep]
- * (layer l at rows l * Hkv ...).  ws: at least jq_layers_workspace_bytes(layer, nlayers) bytes.
+ * (layer l at rows l * Hkv ...).  ws: of jq_layers_workspace_bytes(layer, nlayers) bytes (the least: jq_workspace_bytes).
  */
 size_t jq_layers_workspace_bytes(const jq_shape *layer, int nlayers);
 jq_status jq_evict_layers(const void *const *K, const void *const *V, const void *const *Qwin, int nlayers,
@@ -227,8 +232,8 @@ jq_status jq_evict_layers(const void *const *K, const void *const *V, const void
  * beside it, which `stream` waits for); the call returns without synchronising.  When hV is
  * page-locked memory only its kept rows cross to the device (the kernel reads them in place); hV must
  * then stay unchanged until the stream has passed the call, like every other host buffer.
- * dev_buf is a device buffer of at least jq_host_call_bytes(shape) bytes (it holds the device
- * copies and the workspace).
+ * dev_buf is a device buffer of jq_host_call_bytes(shape) bytes: the device copies and, last, the workspace
+ * (which may be as small as jq_workspace_bytes says).
  */
 size_t jq_host_call_bytes(const jq_shape *shape);
 jq_status jq_evict_layer_host(const void *hK, const void *hV, const void *hQwin,
@@ -270,8 +275,8 @@ jq_status jq_decode_attention(const void *Kc, const void *Vc, const void *q, int
  * L rows of every head, and leaves the min(budget, L) kept rows, in ascending order of their position in
  * that concatenation, in rows [0, nkeep) of Kc and Vc; kept_idx [Hkv, nkeep] holds those positions (values
  * below n_old are old rows).  Rows [nkeep, cap) are unspecified afterwards.  The results of jq_evict_layer on
- * the concatenated tensors.  ws: at least jq_append_workspace_bytes(shape) bytes (it also holds the compacted
- * rows before they are moved to the head of the cache), first 256 bytes initialised by jq_workspace_init.
+ * the concatenated tensors.  ws: of jq_append_workspace_bytes(shape) bytes (a workspace, as small as
+ * jq_workspace_bytes says, and the compacted rows before they are moved to the head of the cache), first 256 bytes initialised by jq_workspace_init.
  * One launch for short caches, else two or four (as jq_evict_layer) and up to six strided device copies, all
  * on `stream`.
  */

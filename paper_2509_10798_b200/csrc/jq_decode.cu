@@ -322,7 +322,9 @@ DecShape decode_shape(int Hkv, int n, const DecPlan &p)
             if (p.resident[C] < 1) continue;
             const int per = (many ? kDecManyWarps : kDecWarps) * C, units = (nunits + per - 1) / per, rounds = (Hkv + p.resident[C] - 1) / p.resident[C];
             const double cost = rounds * (many ? 3.35 + 1.3 * units : 3.3 + units) + (rounds > 1 ? 1.0 : 0.0);
-            // (at equal cost a power of two: the outputs then divide evenly over the CTAs)
+            // (a second round of heads has a start and a merge of its own: 75, 80, 90 heads x 2048 keys take 20.9, 21.6, 21.7 us with a CTA
+            // of twelve warps each, 21.4, 22.0, 23.1 with three in two rounds, which would win by a little without it;
+            // at equal cost a power of two: the outputs then divide evenly over the CTAs)
             if (cost < best_cost || (cost == best_cost && (C & (C - 1)) == 0 && (best.C & (best.C - 1)) != 0)) { best = {C, many != 0}; best_cost = cost; }
             if (units == 1) break;   // (more CTAs have nothing to do)
         }

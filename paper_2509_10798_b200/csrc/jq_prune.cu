@@ -26,13 +26,15 @@
 // prune_taken has the rule by which a call comes here, with what was measured.
 //
 // The bound holds for the scores as they are computed, not only on paper: the rounding of the half is added (block_bounds), the sum
-// is raised by 1 / 512, and it is rounded up to 16 bits, far above the differences in rounding between the two orders of the
-// product.
+// is raised by 1 / 512, and it is rounded up to 16 bits.  The logits that are bounded (Q K^T) and those that are scored (K Q^T) are sums of the
+// same products, added along d in the same steps; that the tensor cores give the same for both is what the margins rely on where
+// large products cancel (within a logit's own size they are far wider than 32-bit rounding), and test_logits_that_cancel holds it to that.
 //
 // What bounds it (32 layers of 8 heads, us, measured back to back on one GPU): 32768 keys, 128 rows, 512 kept: row_stats 370 (2.1 GB
-// of K and 0.13 of maxima: 6.1 TB/s of the 6.5 that a copy reaches), block_bounds 50, score_candidates 50 (the ex2 unit: 5 % of
-// the keys), selection 45; the two-pass kernels 914.  131072 keys, 256 rows, 1024 kept: 2900 (the ex2 unit at 65 %, and the power
-// limit: sustained calls take 7 % longer), 215, 140, 80; before 5900.
+// of K and 0.13 of maxima: 6.1 TB/s of the 6.5 that a copy reaches), block_bounds 50, score_candidates 50, selection 45, the last three chains of
+// dependent steps per head that leave every unit half idle (ex2 54 and 33 %, issue 58 and 24 %, of the first two under ncu); the two-pass
+// kernels 980.  131072 keys, 256 rows, 1024 kept: 2900 (the ex2 unit at 65 %, and the power limit: sustained calls take 7 % longer),
+// 215, 140, 80; before 6000.
 #include "jq_sm100.cuh"
 #include "jq_tmem_ld.cuh"
 #include "jq_debug.cuh"
@@ -472,9 +474,12 @@ __host__ __device__ constexpr int bounds_per_sm(bool wide) { return wide ? 2 : 3
 __host__ __device__ constexpr int bounds_smem(bool wide) { return kBThreads / 32 * kBStages * (wide ? 4096 : 2048); }
 
 // grid: two or three CTAs per SM, CTA b takes tiles [b T / G, (b + 1) T / G).  Per head: the normalisers from row_stats' partial statistics,
-// then a bound per block of 16 keys.  Bound by the read of the maxima from memory.  The bound stays above what it bounds: a maximum x
-// within 24 of its row's normaliser M has been rounded by at most (|M| + 24) / 2048, of which a little more is added (two orders
-// of the product differ by less than |M| 2^-20); smaller ones are below 2^-24, which every row adds; the sum is raised by 1 / 512,
+// then a bound per block of 16 keys.  Neither the read of the maxima bounds it (3.2 TB/s with up to 128 rows, 2.1 with more) nor the
+// exponentials (the ex2 unit 54 and 38 % busy): a CTA does the merge of a head, a chain of loads, before it streams the head's
+// tiles; how the time divides has not been measured.  (The cap of 80 registers for three CTAs costs block_bounds<false> 52 bytes of spills.)
+// The bound stays above what it bounds: a maximum x
+// within 24 of its row's normaliser M has been rounded by at most (|M| + 24) / 2048, of which a little more is added (room for the rounding
+// of x - M); smaller ones are below 2^-24, which every row adds; the sum is raised by 1 / 512,
 // far above what exponentials and sums are off by; a normaliser near the end of a half's range makes every bound of the head
 // infinite.  (With wider margins, 64, 1 / 64, the ragged batch of 128 units took 1862 us instead of 1847.)
 template <bool kWide>
