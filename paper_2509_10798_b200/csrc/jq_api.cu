@@ -316,7 +316,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         return JQ_ERR_CUDA;
     }
     unsigned char *hb = staging.data();
-    unsigned char *h_maps = hb + at.maps, *h_block_maps = hb + at.block_maps;
+    unsigned char *h_maps = hb + at.maps, *h_qmaps = hb + at.qmaps, *h_block_maps = hb + at.block_maps;
     const void **h_K = (const void **)(hb + at.K), **h_V = (const void **)(hb + at.V);
     HeadRec *h_head = (HeadRec *)(hb + at.heads);
     GroupRec *h_grp = (GroupRec *)(hb + at.groups);   // last: there are far fewer than there is room for
@@ -343,9 +343,9 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         const int u = order[i];
         const int Lu = L ? L[u] : common->L, Bu = budget ? budget[u] : common->budget;
         const int nkeep = Bu < Lu ? Bu : Lu;
-        unsigned char *const m = h_maps + (size_t)(kMapsPerUnit * i) * kTensorMapBytes;
-        if (!make_tensor_map(m, K[u], Lu, hpu, 128) || !make_tensor_map(m + kTensorMapBytes, Qwin[u], R, hpu, R <= 128 ? 128 : 256) ||
-            (pruned && !make_tensor_map(h_block_maps + (size_t)i * kTensorMapBytes, K[u], Lu, hpu, 16)))
+        const size_t m = (size_t)i * kTensorMapBytes;
+        if (!make_tensor_map(h_maps + m, K[u], Lu, hpu, 128) || !make_tensor_map(h_qmaps + m, Qwin[u], R, hpu, R <= 128 ? 128 : 256) ||
+            (pruned && !make_tensor_map(h_block_maps + m, K[u], Lu, hpu, 16)))
             return JQ_ERR_CUDA;
         h_K[i] = K[u]; h_V[i] = V[u];
         for (int h = 0; h < hpu; ++h) {
@@ -383,6 +383,7 @@ jq_status jq_evict_ragged(const void *const *K, const void *const *V, const void
         if (cudaMemcpyAsync(tab + off, hb + off, used - off < kTablePiece ? used - off : kTablePiece, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return JQ_ERR_CUDA;
     t.maps = tab + at.maps;
+    t.qmaps = tab + at.qmaps;
     t.K = (const void *const *)(tab + at.K);
     t.V = (const void *const *)(tab + at.V);
     t.heads = (const HeadRec *)(tab + at.heads);

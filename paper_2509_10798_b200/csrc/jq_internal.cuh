@@ -85,7 +85,6 @@ static inline size_t workspace_need(const jq_shape &s) { return workspace_need((
 // KV heads are numbered through all units; unit u owns heads [u * hpu, (u + 1) * hpu).
 constexpr int kMaxUnits = 4096;
 constexpr size_t kTensorMapBytes = 128;
-constexpr int kMapsPerUnit = 2;
 // A head group of the scoring kernel: consecutive KV heads of one prefix length whose keys fit a share of the
 // L2.  A group may run over consecutive units of equal length (their scores are consecutive too).
 struct GroupRec {
@@ -106,7 +105,7 @@ struct HeadRec {
     long long ooff;      // offset (rows) of the head's kept indices and compacted rows in the stacked outputs
 };
 struct UnitTables {
-    const void *maps = nullptr;          // device: [nunits][kMapsPerUnit] TMA tensor maps (K, Qwin)
+    const void *maps = nullptr, *qmaps = nullptr;   // device: [nunits] TMA tensor maps of K, of Qwin
     const void *const *K = nullptr;      // device: [nunits] base of K
     const void *const *V = nullptr;      // device: [nunits] base of V
     const GroupRec *groups = nullptr;    // device: [ngroups]
@@ -124,12 +123,14 @@ struct UnitTables {
 // Where the tables lie, from their first byte on: what both ways of a call read, then the groups of the two passes or the two tables
 // of the one-pass eviction.  A workspace with room for the tables of the two passes is enough for every call.
 struct UnitTableLayout {
-    size_t maps = 0, K, V, heads, groups, block_maps, tbase, bytes, prune_bytes;
+    size_t maps = 0, qmaps, K, V, heads, groups, block_maps, tbase, bytes, prune_bytes;
 };
 static inline UnitTableLayout unit_tables(int nunits, int hpu)
 {
     UnitTableLayout t;
-    t.K = align_up((size_t)nunits * kMapsPerUnit * kTensorMapBytes, 256);
+    t.qmaps = (size_t)nunits * kTensorMapBytes;   // (the two of a unit apart: side by side, 256 bytes to a unit, 16 layers of 8 x 7745 keys took 127.8 us instead
+                                                  // of 126.4, 8 layers of 8 x 4022 54.9 instead of 53.7)
+    t.K = align_up(2 * (size_t)nunits * kTensorMapBytes, 256);
     t.V = t.K + align_up((size_t)nunits * sizeof(void *), 256);
     t.heads = t.V + align_up((size_t)nunits * sizeof(void *), 256);
     t.groups = t.block_maps = t.heads + align_up((size_t)nunits * hpu * sizeof(HeadRec), 256);

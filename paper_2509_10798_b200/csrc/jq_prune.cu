@@ -85,7 +85,7 @@ struct SParams {
     int *status;
     const HeadRec *htab;       // heads of different lengths or budgets (null otherwise): their records,
     const long long *tbase;    // and first tiles
-    const CUtensorMap *maps;   // units in buffers of their own: [units][kMapsPerUnit] tensor maps (K, Qwin)
+    const CUtensorMap *maps, *qmaps;   // units in buffers of their own: [units] tensor maps of K, of Qwin
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
     long long n_part, n_bmax;
@@ -231,7 +231,7 @@ row_stats(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUte
                         const int unit = at.h / P.hpu;
                         c2 = at.h - unit * P.hpu;
                         if (unit != prev_unit) {
-                            mk = P.maps + kMapsPerUnit * (size_t)unit; mq = mk + 1;
+                            mk = P.maps + unit; mq = P.qmaps + unit;
                             tensormap_acquire(mk); tensormap_acquire(mq);
                             prev_unit = unit;
                         }
@@ -392,7 +392,7 @@ struct CParams {
     int *status;
     const HeadRec *htab;
     const long long *tbase;
-    const CUtensorMap *maps, *block_maps;   // block_maps: [units]
+    const CUtensorMap *qmaps, *block_maps;   // [units]
     long long n_scores;        // floats in the scores array
 #ifdef JQ_DEBUG
     DebugRecord *dbg_rec;
@@ -705,10 +705,10 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     const int L = at.L, nkeep = at.nkeep;
     int kv_in = head;
     const CUtensorMap *mb = &mapB, *mq = &mapQ;
-    if (P.maps) {
+    if (P.qmaps) {
         const int unit = head / P.hpu;
         kv_in = head - unit * P.hpu;
-        mq = P.maps + kMapsPerUnit * (size_t)unit + 1; mb = P.block_maps + unit;
+        mq = P.qmaps + unit; mb = P.block_maps + unit;
     }
     const int tph = (L + kPTile - 1) / kPTile, nb = (L + kPBlock - 1) / kPBlock;
     const int ts = (int)((long long)rank * tph / C), te = (int)((long long)(rank + 1) * tph / C);   // tiles of the head that this CTA looks after
@@ -731,13 +731,13 @@ score_candidates(const __grid_constant__ CUtensorMap mapB, const __grid_constant
     uint32_t lo16 = 0u, hi16 = 0u;                            // the blocks of a round: bounds in [lo16, hi16)
     if (warp == kEpi) {
         if (lane == 0) {
-            if (P.maps) { tensormap_acquire(mq); tensormap_acquire(mb); }
+            if (P.qmaps) { tensormap_acquire(mq); tensormap_acquire(mb); }
             mbar_expect_tx(&ctl->q_full, q_bytes);
             tma_load_3d(qbuf, mq, &ctl->q_full, 0, 0, kv_in);
             tma_load_3d(qbuf + q_bytes / 2, mq, &ctl->q_full, 64, 0, kv_in);
         }
         __syncwarp();
-        if (P.maps) tensormap_acquire(mb);                    // (all lanes load)
+        if (P.qmaps) tensormap_acquire(mb);                    // (all lanes load)
     } else if (warp < kEpi) {
         for (int i = tid; i < kMaxR; i += kTE) if (JQ_IN(head, P.heads, kDbgPrune, 17)) ctl->Ms[i] = __ldcg(P.Ms + (size_t)head * kMaxR + i);
         const uint16_t *const src = P.ub + (size_t)(at.tbase + ts) * 8;
@@ -1065,6 +1065,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
         mapQ = mapW = mapB = mapK;
         if (tables->tbase) { S.htab = tables->heads; S.tbase = tables->tbase; }   // (lengths from tables are a chain of reads before anything starts)
         S.maps = (const CUtensorMap *)tables->maps;
+        S.qmaps = (const CUtensorMap *)tables->qmaps;
     } else {
         if (!make_tensor_map(&mapK, K, s.L, s.Hkv, kPTile, src_head_rows) || !make_tensor_map(&mapQ, Q, R, s.Hkv, Rbox) ||
             !make_tensor_map(&mapB, K, s.L, s.Hkv, kPBlock, src_head_rows))
@@ -1100,7 +1101,7 @@ jq_status launch_evict_pruned(const void *K, const void *V, const void *Q, const
     ScoredTiles scored;
     scored.bits = P.scored = sparse ? (uint8_t *)(scratch + lay.scored) : nullptr;
     scored.tbase = S.tbase; scored.tph = tph; scored.max_tiles = max_tph; scored.tiles = T;
-    P.htab = S.htab; P.tbase = S.tbase; P.maps = S.maps; P.block_maps = tables ? (const CUtensorMap *)tables->block_maps : nullptr;
+    P.htab = S.htab; P.tbase = S.tbase; P.qmaps = S.qmaps; P.block_maps = tables ? (const CUtensorMap *)tables->block_maps : nullptr;
     P.n_scores = tables ? tables->total_keys : (long long)s.Hkv * s.L;
 #ifdef JQ_DEBUG
     S.dbg_rec = P.dbg_rec = debug_record();

@@ -100,9 +100,9 @@ struct Params {
     int wtile;               // 1 in window-inclusive mode: every head has one more tile, the last, holding the w window keys
     int w;                   // soft-token queries per query head
     // Units in buffers of their own (ragged calls): the head groups, their lengths and score offsets come from
-    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps [units][kMapsPerUnit] (K, Qwin).
+    // gtab [ngroups] (L, tph, hpg above are then unused) and the tiles through maps, qmaps [units] (K, Qwin).
     const GroupRec *gtab;
-    const CUtensorMap *maps;
+    const CUtensorMap *maps, *qmaps;
     int hpu;                 // KV heads per unit (a group may run over consecutive units of one length)
     uint32_t grid_magic, tph_magic;   // ceil(2^32 / gridDim.x), ceil(2^32 / tph) (see fast_div)
 #ifdef JQ_DEBUG
@@ -303,7 +303,7 @@ score_fused(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
                                 const int du = head_c2 / P.hpu, unit = sg.unit + du;
                                 head_c2 -= du * P.hpu;
                                 if (unit != prev_unit) {
-                                    head_mapK = P.maps + kMapsPerUnit * (size_t)unit; head_mapQ = head_mapK + 1;
+                                    head_mapK = P.maps + unit; head_mapQ = P.qmaps + unit;
                                     tensormap_acquire(head_mapK); tensormap_acquire(head_mapQ);
                                     prev_unit = unit;
                                 }
@@ -839,13 +839,13 @@ jq_status launch_score_tc(const void *K, const void *Q, const jq_shape &s, float
         // every unit has tensor maps of its own in device memory; the three parameter maps are not used
         memset(&mapK, 0, sizeof mapK); mapQ = mapK; mapW = mapK;
         P.L = 0; P.tph = 0; P.hpg = 0;
-        P.gtab = tables->groups; P.maps = (const CUtensorMap *)tables->maps; P.hpu = tables->hpu;
+        P.gtab = tables->groups; P.maps = (const CUtensorMap *)tables->maps; P.qmaps = (const CUtensorMap *)tables->qmaps; P.hpu = tables->hpu;
         P.ngroups = tables->ngroups;
         tmax = tables->max_group_tiles;
     } else {
         P.L = s.L;
         P.tph = (s.L + kTile - 1) / kTile + P.wtile;
-        P.gtab = nullptr; P.maps = nullptr; P.hpu = s.Hkv;
+        P.gtab = nullptr; P.maps = P.qmaps = nullptr; P.hpu = s.Hkv;
         if (!make_map(&mapK, K, s.L, s.Hkv, kTile, k_head_rows) || !make_map(&mapQ, Q, R, s.Hkv, P.Rbox)) return JQ_ERR_CUDA;
         if (Kwin) { if (!make_map(&mapW, Kwin, s.w, s.Hkv, kTile)) return JQ_ERR_CUDA; } else mapW = mapK;
         P.hpg = heads_per_group(s.L, s.Hkv, P.tph, sms, R > 128);
